@@ -19,6 +19,7 @@
 #include "bdss_kalman.h"
 #include "bdss_krylov.h"
 #include "bdss_small.h"
+#include "bdss_tcf.h"
 
 using namespace bdss;
 
@@ -83,6 +84,13 @@ struct bdss_ctx {
   int *Wexp = nullptr;             // (N - 1) x n row exponents
   int schur_emu_ready = 0;
   int schur_emu_on = 0;
+  // n <= 64: factorisation with the coupling solves and Schur products on the
+  // tensor cores (bdss_tcf.cu): buffers of the current level
+  void *tcfX = nullptr;   // (N / 2) x n x n (T)
+  void *tcfC = nullptr;   // (N / 2) x 2 x n x n (T)
+  void *tcfcb = nullptr;  // (N / 2) x 2 x n x d_max (T)
+  int tcf_ready = 0;
+  int tcf_opt = -1;       // BDSS_OPT_SCHUR_EMU at n <= 64: -1 by size, 0 off, 1 on
   // large mixed path: streamed solve passes (maps over Li and Wb)
   CorrMaps corr_maps[3];  // split factors P = 1, 2, 4
   int corr_max_split = 1;
@@ -276,10 +284,26 @@ constexpr int kSmallAutoMaxN = 16;
 constexpr int kSmallAutoPerCta = 8;
 constexpr int kSmallAutoWorkPerCta = 64;
 static bool use_small(const bdss_ctx *h) {
-  if (is_mixed(h) || h->small_cluster < 2 || !h->persistent || h->skip_barrier || h->schur_emu_on) return false;
+  if (is_mixed(h) || h->small_cluster < 2 || !h->persistent || h->skip_barrier || h->tcf_opt == 1) return false;
   if (h->small_opt >= 0) return h->small_opt == 1;
   const int64_t C = h->small_cluster;
   return h->n <= kSmallAutoMaxN && h->N <= kSmallAutoPerCta * C && h->N * h->n <= kSmallAutoWorkPerCta * C;
+}
+
+// Factorisations of n <= 64 blocks with the coupling solves and Schur
+// products on the tensor cores: on request, or by size.  A level costs two
+// launches and the full latency of one block in each, so the path needs many
+// blocks; its gain per block grows with n.  Measured on GB300, d = 1 (the
+// tensor-core path's time over the persistent kernel's): n = 64, N = 4096:
+// 0.57; n = 48, N = 4096: 0.78; n = 32, N = 8192: 0.94, N = 2048: 1.03;
+// n = 24, N = 2000: 1.16.
+constexpr int kTcfMinN = 17;
+constexpr int kTcfAutoMinN = 40;
+constexpr int kTcfAutoMinBlocks = 2048;
+static bool use_tcf(const bdss_ctx *h) {
+  if (h->large || !h->tcf_ready || h->plan.L < 1) return false;
+  if (h->tcf_opt >= 0) return h->tcf_opt == 1;
+  return h->persistent && !h->skip_barrier && h->nstar == 1 && h->n >= kTcfAutoMinN && h->N >= kTcfAutoMinBlocks;
 }
 
 static cudaError_t run_small(bdss_ctx *h, const Args<double> &a, bool factor, bool rhs) {
@@ -345,54 +369,49 @@ static cudaError_t schur_emu_level(bdss_ctx *h, const Args<double> &b, int l) {
   kt_end(h, 1);
   h->launches += 1;
   if (e != cudaSuccess) return e;
-  // the next level's couplings: Eb on the tiled path, region l + 1 of Wb for n <= 64
-  double *En = (h->large ? b.Eb : b.Wb) + (size_t)p.off[l + 1] * nn;
+  double *En = b.Eb + (size_t)p.off[l + 1] * nn;  // the next level's couplings
   kt_begin(h, BDSS_KT_SCHUR_TC);
   e = launch_emu_schur(Nl, p.n, l, h->Wslc, h->Wexp, b.A_diag, b.Ld, En, h->dst, h->timeout_ns, h->sms, h->stream);
   kt_end(h, 1);
   h->launches += 1;
   if (e != cudaSuccess || b.d == 0) return e;
   kt_begin(h, h->kt_cls);
-  if (h->large) {
-    e = launch_large_sub<double>(b, l, kSubBRhsOnly, 1,
-                                 grid_for(h, large_sub_tasks(p, l, kSubBRhsOnly, 1, b.d, 8, 0, 0)), h->smem,
-                                 h->stream);
-  } else {  // phase B without the factor work is the separators' RHS update
-    const int cap = h->bps * h->sms;
-    e = launch_phaseB<double>(b, l, 0, grid_for(h, ((Nl + 1) / 2) * parts_B<double>(p, l, false, cap)), h->smem,
-                              h->stream);
-  }
+  e = launch_large_sub<double>(b, l, kSubBRhsOnly, 1,
+                               grid_for(h, large_sub_tasks(p, l, kSubBRhsOnly, 1, b.d, 8, 0, 0)), h->smem, h->stream);
   kt_end(h, 1);
   h->launches += 1;
   return e;
 }
 
-// FP64 factorisation for n <= 64 with the Schur products on the tensor
-// cores: per level phase A (Cholesky, coupling and RHS substitutions), the
-// slice products, the separators' RHS update; then the top block and the
-// downward pass, one launch each.
-static cudaError_t run_levels_emu_small(bdss_ctx *h, const Args<double> &a, bool rhs) {
+// Factorisation for n <= 64 with the coupling solves and Schur products on
+// the tensor cores: per level the diagonal blocks (ALU), then everything
+// else; the last level's pending updates, the top block and the downward
+// pass, one launch each.
+template <typename T>
+static cudaError_t run_levels_tcf(bdss_ctx *h, const Args<T> &a, bool rhs) {
   const Plan &p = h->plan;
-  const int cap = h->bps * h->sms;
-  Args<double> b = a;
+  Args<T> b = a;
   if (!rhs) b.d = 0;
+  const TcfLevel<T> c{(T *)h->tcfX, (T *)h->tcfC, (T *)h->tcfcb};
   cudaError_t e = cudaSuccess;
   for (int l = 0; l < p.L && e == cudaSuccess; ++l) {
-    const long long nElim = p.Nl[l] / 2;
     kt_begin(h, h->kt_cls);
-    e = launch_phaseA<double>(b, l, 1, grid_for(h, nElim * parts_A<double>(p, l, true, cap)), h->smem, h->stream);
+    e = launch_tcf_diag<T>(b, c, l, 0, h->sms, h->stream);
     kt_end(h, 1);
-    h->launches += 1;
-    if (e == cudaSuccess) e = schur_emu_level(h, b, l);
+    kt_begin(h, BDSS_KT_SCHUR_TC);
+    if (e == cudaSuccess) e = launch_tcf_schur<T>(b, c, l, h->sms, h->stream);
+    kt_end(h, 1);
+    h->launches += 2;
   }
   kt_begin(h, h->kt_cls);
-  if (e == cudaSuccess) e = launch_top<double>(b, 1, h->smem, h->stream);
-  kt_end(h, 1);
-  h->launches += 1;
+  if (e == cudaSuccess) e = launch_tcf_diag<T>(b, c, p.L, 1, h->sms, h->stream);
+  if (e == cudaSuccess) e = launch_top<T>(b, 1, h->smem, h->stream);
+  kt_end(h, 2);
+  h->launches += 2;
   if (rhs)
     for (int l = p.L - 1; l >= 0 && e == cudaSuccess; --l) {
       kt_begin(h, h->kt_cls);
-      e = launch_phaseC<double>(b, l, grid_for(h, p.Nl[l] / 2), h->smem, h->stream);
+      e = launch_phaseC<T>(b, l, grid_for(h, p.Nl[l] / 2), h->smem, h->stream);
       kt_end(h, 1);
       h->launches += 1;
     }
@@ -532,9 +551,7 @@ template <typename T>
 static cudaError_t run_levels(bdss_ctx *h, const Args<T> &a, bool factor, bool rhs) {
   const Plan &p = h->plan;
   if (h->large) return run_levels_large<T>(h, a, factor, rhs);
-  if constexpr (sizeof(T) == 8) {
-    if (factor && h->schur_emu_on) return run_levels_emu_small(h, a, rhs);
-  }
+  if (factor && use_tcf(h)) return run_levels_tcf<T>(h, a, rhs);
   const int cap = h->bps * h->sms;
   if (h->persistent) {
     long long most = 1;  // tasks of the busiest step
@@ -610,6 +627,9 @@ bdss_status bdss_destroy(bdss_handle h) {
   cudaFree(h->emu.xmax);
   cudaFree(h->Wslc);
   cudaFree(h->Wexp);
+  cudaFree(h->tcfX);
+  cudaFree(h->tcfC);
+  cudaFree(h->tcfcb);
   cudaFree(h->Li);
   cudaFree(h->Yt);
   cudaFree(h->Ltinv);
@@ -745,7 +765,7 @@ bdss_status bdss_create(bdss_handle *out, int64_t N, int32_t n, int32_t d_max, b
       }
     }
   }
-  if (ok && prec == BDSS_FP64 && N > 1 && (h->large || n >= 32)) {  // Schur products on the tensor cores
+  if (ok && prec == BDSS_FP64 && N > 1 && h->large) {  // Schur products on the tensor cores
     ok = ws_alloc(h, (void **)&h->Wslc, emu_wslc_bytes(N - 1, n));
     ok = ok && ws_alloc(h, (void **)&h->Wexp, (size_t)(N - 1) * n * sizeof(int));
     if (ok) {
@@ -755,10 +775,20 @@ bdss_status bdss_create(bdss_handle *out, int64_t N, int32_t n, int32_t d_max, b
         return cuda_fail(ec);
       }
       h->schur_emu_ready = 1;
-      // on by default for the tiled path; for n <= 64 the slice products do
-      // not yet beat the FP64 pipe (half of each 128-row tile is padding),
-      // so there the option opts in
-      h->schur_emu_on = h->large ? 1 : 0;
+      h->schur_emu_on = 1;
+    }
+  }
+  if (ok && prec == BDSS_FP64 && N > 1 && !h->large && n >= kTcfMinN) {
+    ok = ws_alloc(h, &h->tcfX, (size_t)(N / 2) * nn * esz);
+    ok = ok && ws_alloc(h, &h->tcfC, (size_t)(N / 2) * 2 * nn * esz);
+    ok = ok && ws_alloc(h, &h->tcfcb, (size_t)(N / 2) * 2 * n * d_max * esz);
+    if (ok) {
+      const cudaError_t ec = tcf_configure<double>(n, d_max);
+      if (ec != cudaSuccess) {
+        bdss_destroy(h);
+        return cuda_fail(ec);
+      }
+      h->tcf_ready = 1;
     }
   }
   if (!ok) {
@@ -840,8 +870,9 @@ bdss_status bdss_set_option(bdss_handle h, bdss_option key, int64_t value) {
       return BDSS_OK;
     case BDSS_OPT_SCHUR_EMU:
       if (value != 0 && value != 1) return BDSS_ERR_INVALID_ARG;
-      if (value && !h->schur_emu_ready) return BDSS_ERR_UNSUPPORTED;
-      h->schur_emu_on = (int)value;
+      if (value && !h->schur_emu_ready && !(h->tcf_ready && !is_mixed(h))) return BDSS_ERR_UNSUPPORTED;
+      if (h->large) h->schur_emu_on = (int)value;
+      else h->tcf_opt = (int)value;
       return BDSS_OK;
     case BDSS_OPT_RESIDUAL_EMU:
       if (value != 0 && value != 1) return BDSS_ERR_INVALID_ARG;

@@ -1,0 +1,212 @@
+// Products of FP64 (or FP32) tiles on the tcgen05 tensor cores at their full
+// accuracy, with the operands cut into digits inside the kernel that uses
+// them (nothing of the digits goes to memory).
+//
+// A row of K <= 64 operand entries gets one binary exponent, the largest of
+// its entries, and every entry becomes the signed integer
+//   q = trunc(v 2^-(exponent) 2^F),  F = 62 bits (FP64) or 30 bits (FP32),
+// written in kDig = 8 (4) base-256 digits q = sum_p d_p 256^(kDig-1-p) with
+// -128 <= d_p <= 127 and |d_0| <= 64, each exact in FP16.  The product of two
+// rows is then
+//   sum_k q_a q_b = sum_t 256^(2 kDig - 2 - t) ACC_t,
+//   ACC_t = sum_{p+q=t} sum_k d_p(a) d_q(b),
+// and only the diagonals t < kDig are formed: the digit pairs left out weigh
+// below 2^-8kDig x 64 x 8, i.e. 2^-57 (2^-25) of the product of the two row
+// maxima at worst and 2^-61 (2^-30) for digits of random sign, beneath the
+// rounding of a chain of 64 FP64 (FP32) multiply-adds.  Every
+// |ACC_t| <= 2 x 64 x 64 x 128 + (t - 1) x 64 x 128 x 128 < 2^23, so the FP32
+// accumulation of the tensor cores is exact whatever its order.
+//
+// One tcgen05.mma (kind::f16, M = 128) per A digit p and K step of 16 covers
+// the B digits q = 0 .. kDig-1-p of up to 32 B rows at once: the B operand
+// stacks the digits (32 rows each), and its D columns start at 32 p, so the
+// pair (p, q) lands on the columns of diagonal p + q.  p = 0 covers every
+// diagonal, so its first K step clears the accumulators.
+#pragma once
+#include <cuda_fp16.h>
+
+#include "bdss_tc.cuh"
+
+namespace bdss {
+
+template <typename T> struct SliceFmt;
+template <> struct SliceFmt<double> { static constexpr int kDig = 8; };
+template <> struct SliceFmt<float> { static constexpr int kDig = 4; };
+
+constexpr int kSlRows = 128;             // A rows of a tile (TMEM lanes)
+constexpr int kSlK = 64;                 // K entries of a tile (128 bytes of FP16)
+constexpr int kSlCols = 32;              // B rows of a column tile
+constexpr int kSlASlab = kSlRows * 128;  // bytes of one digit of the A tile
+constexpr int kSlBSlab = kSlCols * 128;  // bytes of one digit of a B tile
+
+// Exponent field of |v| (0 for zero and subnormals: they count as zero).
+__device__ __forceinline__ int sl_exp(double v) { return (__double2hiint(v) >> 20) & 0x7FF; }
+__device__ __forceinline__ int sl_exp(float v) { return (__float_as_int(v) >> 23) & 0xFF; }
+// The exponent field of infinities and NaN: a row with such an entry poisons
+// every product it takes part in, as a floating-point product would.
+template <typename T> constexpr int kSlPoison = sizeof(T) == 8 ? 0x7FF : 0xFF;
+
+// Biased digits of v under the row exponent field exmax: the byte p from the
+// top is d_p + 128.
+__device__ __forceinline__ unsigned long long sl_biased(double v, int exmax) {
+  const long long b = __double_as_longlong(v);
+  const int ex = (int)(b >> 52) & 0x7FF;
+  unsigned long long m = ((unsigned long long)(b & 0xFFFFFFFFFFFFFLL) | 0x10000000000000ULL) << 9;
+  const int s = exmax - ex;
+  m = (ex == 0) ? 0ULL : (m >> (s > 63 ? 63 : s));
+  return (b < 0 ? 0ULL - m : m) + 0x8080808080808080ULL;
+}
+__device__ __forceinline__ unsigned sl_biased(float v, int exmax) {
+  const int b = __float_as_int(v);
+  const int ex = (b >> 23) & 0xFF;
+  unsigned m = ((unsigned)(b & 0x7FFFFF) | 0x800000u) << 6;
+  const int s = exmax - ex;
+  m = (ex == 0) ? 0u : (m >> (s > 31 ? 31 : s));
+  return (b < 0 ? 0u - m : m) + 0x80808080u;
+}
+
+// Two digits (bytes lo and hi of each half of c) as FP16 pairs: 0x6400 | b is
+// 1024 + b, and subtracting 1152 leaves d = b - 128, both exact.
+__device__ __forceinline__ void sl_half_pairs(unsigned c, unsigned &lo, unsigned &hi) {
+  const __half2 bias = __halves2half2(__ushort_as_half(0x6480), __ushort_as_half(0x6480));
+  unsigned l = __byte_perm(c, 0x64646464u, 0x4240), h = __byte_perm(c, 0x64646464u, 0x4341);
+  __half2 a = *reinterpret_cast<__half2 *>(&l), b = *reinterpret_cast<__half2 *>(&h);
+  a = __hsub2(a, bias);
+  b = __hsub2(b, bias);
+  lo = *reinterpret_cast<unsigned *>(&a);
+  hi = *reinterpret_cast<unsigned *>(&b);
+}
+
+// Two consecutive K entries of one row -> 4 bytes of every digit slab.
+template <typename T>
+__device__ __forceinline__ void sl_store2(T v0, T v1, int exmax, unsigned char *dst, int stride);
+template <>
+__device__ __forceinline__ void sl_store2<double>(double v0, double v1, int exmax, unsigned char *dst, int stride) {
+  const unsigned long long u0 = sl_biased(v0, exmax), u1 = sl_biased(v1, exmax);
+  const unsigned h0 = (unsigned)(u0 >> 32), h1 = (unsigned)(u1 >> 32), l0 = (unsigned)u0, l1 = (unsigned)u1;
+  unsigned w[8];
+  sl_half_pairs(__byte_perm(h0, h1, 0x7632), w[1], w[0]);
+  sl_half_pairs(__byte_perm(h0, h1, 0x5410), w[3], w[2]);
+  sl_half_pairs(__byte_perm(l0, l1, 0x7632), w[5], w[4]);
+  sl_half_pairs(__byte_perm(l0, l1, 0x5410), w[7], w[6]);
+#pragma unroll
+  for (int p = 0; p < 8; ++p) *reinterpret_cast<unsigned *>(dst + p * stride) = w[p];
+}
+template <>
+__device__ __forceinline__ void sl_store2<float>(float v0, float v1, int exmax, unsigned char *dst, int stride) {
+  const unsigned u0 = sl_biased(v0, exmax), u1 = sl_biased(v1, exmax);
+  unsigned w[4];
+  sl_half_pairs(__byte_perm(u0, u1, 0x7632), w[1], w[0]);
+  sl_half_pairs(__byte_perm(u0, u1, 0x5410), w[3], w[2]);
+#pragma unroll
+  for (int p = 0; p < 4; ++p) *reinterpret_cast<unsigned *>(dst + p * stride) = w[p];
+}
+
+// Byte offset of 16-byte group g (K entries 8 g .. 8 g + 7) of row r in a
+// 128-byte-swizzled slab.
+__device__ __forceinline__ int sl_off(int r, int g) { return r * 128 + ((g ^ (r & 7)) << 4); }
+
+// D = FP32, A = B = FP16, both K-major, M = 128 x N.
+__host__ __device__ constexpr uint32_t sl_idesc(int N) {
+  return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kSlRows >> 4) << 24);
+}
+
+__device__ __forceinline__ void sl_mma(uint32_t d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
+      : "memory");
+}
+
+// All digit pairs of A (128 rows) times a B tile of `cols` rows (16 or 32), K
+// steps 0 .. ks - 1, into the accumulators at TMEM address d (diagonal t at
+// columns cols t ..).  One thread; rolled loops, since the code of the digit
+// kernels has to stay in the instruction cache.
+template <typename T>
+__device__ __forceinline__ void sl_issue(uint32_t d, const unsigned char *A, const unsigned char *B, int cols, int ks) {
+  constexpr int kDig = SliceFmt<T>::kDig;
+  const uint64_t ad0 = tc_desc_sw128(A, 0), bd0 = tc_desc_sw128(B, 0);
+#pragma unroll 1
+  for (int p = 0; p < kDig; ++p) {
+    const uint32_t idesc = sl_idesc(cols * (kDig - p)), dp = d + (uint32_t)(cols * p);
+    // the start address field counts 16-byte units: a slab is kSlASlab / 16,
+    // a K step of 16 FP16 entries 2 of them
+    uint64_t ad = ad0 + (uint64_t)(p * (kSlASlab / 16)), bd = bd0;
+    if (ks == 4) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) sl_mma(dp, ad + 2 * k, bd + 2 * k, idesc, (uint32_t)(p | k));
+    } else {
+#pragma unroll 1
+      for (int k = 0; k < ks; ++k, ad += 2, bd += 2) sl_mma(dp, ad, bd, idesc, (uint32_t)(p | k));
+    }
+  }
+}
+
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// An accumulator entry as an integer without the conversion unit (16 lanes a
+// cycle and SM; with eight conversions an entry it set the pace of the
+// drains).  |x| <= 2^22: adding 1.5 * 2^23 puts x in the binade of unit
+// spacing.  |x| < 2^23: 1.5 * 2^24 and a spacing of two, which rounds the last
+// bit away -- used for the two lowest diagonals, where it weighs 2^-60 of the
+// product of the row maxima.
+__device__ __forceinline__ int sl_int22(float x) { return __float_as_int(x + 12582912.0f) - 0x4B400000; }
+__device__ __forceinline__ int sl_int23(float x) { return (__float_as_int(x + 25165824.0f) - 0x4BC00000) * 2; }
+
+// t 2^(be - 1075) for a result outside the normal range.
+__device__ __noinline__ double sl_scale_slow(unsigned long long t, int be) { return scalbn((double)(long long)t, be - 1075); }
+
+// sum_t ACC_t 256^(7-t) 2^(exa + exb - 2112), rounded once to FP64 on the
+// integer pipe (an FP64 instruction holds a warp's FP64 unit for 64 cycles on
+// this GPU; the whole conversion takes about that many integer issue slots for
+// 32 entries).  With |d_0| <= 64 the diagonals are at most 2^18, 2^20, 2^21,
+// 3 2^20, ..., 7 2^20, so neighbouring pairs combine in 32 bits.
+__device__ __forceinline__ double sl_value(const float (&c)[8], int exa, int exb) {
+  const int h01 = sl_int22(c[0]) * 256 + sl_int22(c[1]);
+  const int h23 = sl_int22(c[2]) * 256 + sl_int22(c[3]);
+  const int h45 = sl_int22(c[4]) * 256 + __float2int_rn(c[5]);
+  const int h67 = sl_int23(c[6]) * 256 + sl_int23(c[7]);
+  const long long H = (long long)h01 * 65536 + h23, L = (long long)h45 * 65536 + h67;
+  long long hi = H + (L >> 32);  // value = (hi 2^32 + lo) 2^S
+  unsigned lo = (unsigned)L;
+  int S = exa + exb - 2112;
+  const bool neg = hi < 0;
+  if (neg) {
+    hi = ~hi + (lo == 0u ? 1 : 0);
+    lo = 0u - lo;
+  }
+  if (hi == 0) {
+    hi = (long long)lo;
+    lo = 0u;
+    S -= 32;
+  }
+  if (exa == 0x7FF || exb == 0x7FF) return __longlong_as_double(0x7FF8000000000000LL);
+  if (hi == 0) return 0.0;
+  const int lz = __clzll(hi);  // >= 2
+  const unsigned long long m = ((unsigned long long)hi << lz) | (((unsigned long long)lo << 32) >> (64 - lz));
+  const unsigned long long t = (m >> 11) + ((m >> 10) & 1ULL);  // 53 bits, rounded
+  const int be = 1023 + 63 + 32 - lz + S;
+  if (be < 1 || be > 2046) {  // outside the normal range
+    const double r = sl_scale_slow(t, be);
+    return neg ? -r : r;
+  }
+  const unsigned long long bits = ((unsigned long long)(be - 1) << 52) + t;  // a carry of t raises the exponent
+  return __longlong_as_double((long long)(bits | (neg ? 0x8000000000000000ULL : 0ULL)));
+}
+// The same for FP32: sum_t ACC_t 256^(3-t) 2^(exa + exb - 288).
+__device__ __forceinline__ float sl_value(const float (&c)[4], int exa, int exb) {
+  const int h01 = sl_int22(c[0]) * 256 + sl_int22(c[1]);
+  const int h23 = sl_int22(c[2]) * 256 + sl_int22(c[3]);
+  const float r = fmaf((float)h01, 65536.0f, (float)h23);
+  if (exa == 0xFF || exb == 0xFF) return __int_as_float(0x7FC00000);
+  return ldexpf(r, exa + exb - 288);
+}
+
+}  // namespace bdss

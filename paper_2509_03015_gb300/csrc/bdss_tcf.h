@@ -1,0 +1,31 @@
+// Factorisation of blocks up to n = 64 with the coupling solves and the Schur
+// products on the tensor cores (internal to the library; see bdss_tcf.cu).
+#pragma once
+#include <cuda_runtime.h>
+
+#include "bdss_device.cuh"
+
+namespace bdss {
+
+// Buffers of the current level, one set per eliminated block m: L^{-1}, and the
+// updates it leaves pending on its left and its right separator (n x n
+// diagonal update, lower triangle; n x d right-hand-side update).
+template <typename T>
+struct TcfLevel {
+  T *X;   // [m][n][n], zero above the diagonal
+  T *C;   // [m][2][n][n]
+  T *cb;  // [m][2][n][d]
+};
+
+template <typename T> cudaError_t tcf_configure(int n, int d);
+// Positions of level l: apply the pending updates of level l - 1 to every
+// position; factor the odd ones (L, L^{-1}, y).  fold_all: the updates only
+// (the last level's blocks, before the top block or sweep).
+template <typename T>
+cudaError_t launch_tcf_diag(const Args<T> &a, const TcfLevel<T> &c, int l, int fold_all, int sms, cudaStream_t s);
+// W of level l's eliminated blocks, the updates they leave on their
+// separators and the next level's couplings.
+template <typename T>
+cudaError_t launch_tcf_schur(const Args<T> &a, const TcfLevel<T> &c, int l, int sms, cudaStream_t s);
+
+}  // namespace bdss
