@@ -132,10 +132,10 @@ typedef enum {
                                    (unless BDSS_OPT_REFINE_KRYLOV = 0); the copy of A_diag
                                    (N n^2 doubles) is allocated on first use.
                                    0 = return BDSS_ERR_NOT_SPD */
-  BDSS_OPT_SCHUR_EMU = 13,      /* FP64, N > 1, 17 <= n <= 256: 1 = the factorisation's products
+  BDSS_OPT_SCHUR_EMU = 13,      /* FP64, N > 1, 32 <= n <= 256: 1 = the factorisation's products
                                    on the tensor cores (the separator update of Algorithm 3,
-                                   D - W^T W and -W^T W of Eq. 5's reduced system; for n <= 64
-                                   also the coupling solves of Algorithm 1): each operand row
+                                   D - W^T W and -W^T W of Eq. 5's reduced system; the coupling
+                                   solves of Algorithm 1): each operand row
                                    cut into digits below its maximum (59 bits or more), every
                                    digit product summed exactly in FP32, the result rounded
                                    to FP64; a few launches per level even in persistent mode.

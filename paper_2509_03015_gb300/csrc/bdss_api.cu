@@ -20,6 +20,7 @@
 #include "bdss_krylov.h"
 #include "bdss_small.h"
 #include "bdss_tcf.h"
+#include "bdss_wide.h"
 
 using namespace bdss;
 
@@ -79,11 +80,11 @@ struct bdss_ctx {
   CUtensorMap emu_maps[2];
   int emu_ready = 0;     // buffers allocated and maps encoded
   int emu_on = 0;        // option: use them
-  // FP64 tiled path: Schur products on the tensor cores (digit slices of W)
-  unsigned short *Wslc = nullptr;  // (N - 1) x S x n x np BF16
-  int *Wexp = nullptr;             // (N - 1) x n row exponents
-  int schur_emu_ready = 0;
-  int schur_emu_on = 0;
+  // 64 < n <= 256: factorisation with its products on the tensor cores
+  // (bdss_wide.cu)
+  void *wideX = nullptr;  // inverses of the current panel's diagonal tiles (T)
+  int wide_ready = 0;
+  int wide_on = 0;
   // n <= 64: factorisation with the coupling solves and Schur products on the
   // tensor cores (bdss_tcf.cu): buffers of the current level
   void *tcfX = nullptr;   // (N / 2) x n x n (T)
@@ -297,13 +298,33 @@ static bool use_small(const bdss_ctx *h) {
 // tensor-core path's time over the persistent kernel's): n = 64, N = 4096:
 // 0.57; n = 48, N = 4096: 0.78; n = 32, N = 8192: 0.94, N = 2048: 1.03;
 // n = 24, N = 2000: 1.16.
-constexpr int kTcfMinN = 17;
+constexpr int kTcfMinN = 32;
 constexpr int kTcfAutoMinN = 40;
 constexpr int kTcfAutoMinBlocks = 2048;
+static bool tcf_by_size(const bdss_ctx *h) {
+  return !is_mixed(h) && !h->large && h->n >= kTcfAutoMinN && h->N >= kTcfAutoMinBlocks;
+}
 static bool use_tcf(const bdss_ctx *h) {
-  if (h->large || !h->tcf_ready || h->plan.L < 1) return false;
+  if (!h->tcf_ready || h->plan.L < 1) return false;
   if (h->tcf_opt >= 0) return h->tcf_opt == 1;
-  return h->persistent && !h->skip_barrier && h->nstar == 1 && h->n >= kTcfAutoMinN && h->N >= kTcfAutoMinBlocks;
+  return h->persistent && !h->skip_barrier && h->nstar == 1 && tcf_by_size(h);
+}
+// Its buffers: with the handle where the size selects the path, else when the
+// option asks for it.
+static bdss_status tcf_alloc(bdss_ctx *h) {
+  if (h->tcf_ready) return BDSS_OK;
+  const size_t nn = (size_t)h->n * h->n, m = (size_t)(h->N / 2);
+  bool ok = h->tcfX || ws_alloc(h, &h->tcfX, m * nn * sizeof(double));
+  ok = ok && (h->tcfC || ws_alloc(h, &h->tcfC, m * 2 * nn * sizeof(double)));
+  ok = ok && (h->tcfcb || ws_alloc(h, &h->tcfcb, m * 2 * h->n * h->d_max * sizeof(double)));
+  if (!ok) {
+    cudaGetLastError();
+    return BDSS_ERR_ALLOC;
+  }
+  const cudaError_t e = tcf_configure<double>(h->n, h->d_max);
+  if (e != cudaSuccess) return cuda_fail(e);
+  h->tcf_ready = 1;
+  return BDSS_OK;
 }
 
 static cudaError_t run_small(bdss_ctx *h, const Args<double> &a, bool factor, bool rhs) {
@@ -357,29 +378,47 @@ static Args<T> base_args(bdss_ctx *h) {
   return a;
 }
 
-// Separator update of level l on the tensor cores (FP64 factorisation):
-// slice the level's stored couplings, form D and the next level's E, then the
-// separators' RHS tiles (when the pass carries right-hand sides) on the ALU.
-static cudaError_t schur_emu_level(bdss_ctx *h, const Args<double> &b, int l) {
+// Factorisation for 64 < n <= 256 with its products on the tensor cores: per
+// level and panel the diagonal tiles (ALU) and every other row, then the
+// separators' updates; the top block like an eliminated block without
+// couplings; the downward pass.
+template <typename T>
+static cudaError_t run_levels_wide(bdss_ctx *h, const Args<T> &a, bool rhs) {
   const Plan &p = h->plan;
-  const long long Nl = p.Nl[l];
-  const size_t nn = (size_t)p.n * p.n;
-  kt_begin(h, BDSS_KT_SLICE);
-  cudaError_t e = launch_emu_slice_w(Nl - 1, p.n, b.Wb + (size_t)p.off[l] * nn, h->Wslc, h->Wexp, h->stream);
-  kt_end(h, 1);
-  h->launches += 1;
-  if (e != cudaSuccess) return e;
-  double *En = b.Eb + (size_t)p.off[l + 1] * nn;  // the next level's couplings
-  kt_begin(h, BDSS_KT_SCHUR_TC);
-  e = launch_emu_schur(Nl, p.n, l, h->Wslc, h->Wexp, b.A_diag, b.Ld, En, h->dst, h->timeout_ns, h->sms, h->stream);
-  kt_end(h, 1);
-  h->launches += 1;
-  if (e != cudaSuccess || b.d == 0) return e;
+  Args<T> b = a;
+  if (!rhs) b.d = 0;
+  const WideBuf<T> w{(T *)h->wideX};
+  const int nt = wide_panels(p.n).nt;
   kt_begin(h, h->kt_cls);
-  e = launch_large_sub<double>(b, l, kSubBRhsOnly, 1,
-                               grid_for(h, large_sub_tasks(p, l, kSubBRhsOnly, 1, b.d, 8, 0, 0)), h->smem, h->stream);
+  cudaError_t e = launch_wide_ingest<T>(b, h->sms, h->stream);
   kt_end(h, 1);
   h->launches += 1;
+  for (int l = 0; l <= p.L && e == cudaSuccess; ++l) {
+    for (int k = 0; k < nt && e == cudaSuccess; ++k) {
+      kt_begin(h, h->kt_cls);
+      e = launch_wide_diag<T>(b, w, l, k, h->stream);
+      kt_end(h, 1);
+      kt_begin(h, BDSS_KT_SCHUR_TC);
+      if (e == cudaSuccess) e = launch_wide_panel<T>(b, w, l, k, h->sms, h->stream);
+      kt_end(h, 1);
+      h->launches += 2;
+    }
+    if (l == p.L || e != cudaSuccess) break;
+    kt_begin(h, BDSS_KT_SCHUR_TC);
+    e = launch_wide_schur<T>(b, l, h->sms, h->stream);
+    kt_end(h, 1);
+    h->launches += 1;
+  }
+  // the solve passes read the top factor from Ltop
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(h->Ltop, h->Ld, (size_t)p.n * p.n * sizeof(double), cudaMemcpyDeviceToDevice, h->stream);
+  if (rhs)
+    for (int l = p.L; l >= 0 && e == cudaSuccess; --l) {
+      kt_begin(h, h->kt_cls);
+      e = launch_wide_down<T>(b, l, h->stream);
+      kt_end(h, l < p.L ? 2 : 1);
+      h->launches += l < p.L ? 2 : 1;
+    }
   return e;
 }
 
@@ -484,19 +523,18 @@ static cudaError_t run_levels_large(bdss_ctx *h, const Args<T> &a, bool factor, 
   // Schur-update tiles use that kernel and the Cholesky / substitution tasks
   // keep the two-CTA FP32 kernel.
   const bool tc_factor = sizeof(T) == 4 && h->tf32 && factor;
-  // FP64 factorisation with the Schur products on the tensor cores: sub-phase
-  // by sub-phase as well (the slicing and the product kernels are launches
-  // of their own)
-  const bool emu_factor = sizeof(T) == 8 && factor && h->schur_emu_on;
   const int inv = a.Li ? 1 : 0;
   Args<T> b = a;
   if (!rhs) b.d = 0;
   // solve passes with the stored inverses keep y of the eliminated blocks in Yt
   b.Yt = (!factor && inv) ? (T *)h->Yt : nullptr;
+  if constexpr (sizeof(T) == 8) {
+    if (factor && h->wide_on) return run_levels_wide<T>(h, a, rhs);
+  }
   if constexpr (sizeof(T) == 4) {
     if (!factor && rhs && inv && h->corr_ok && b.d <= kCorrMaxD) return run_corr_passes(h, b);
   }
-  if (h->persistent && !tc_factor && !emu_factor) {
+  if (h->persistent && !tc_factor) {
     long long most = 1;
     for (int l = 0; l < p.L; ++l)
       for (int sub = 0; sub < 4; ++sub) {
@@ -515,12 +553,7 @@ static cudaError_t run_levels_large(bdss_ctx *h, const Args<T> &a, bool factor, 
   cudaError_t e = cudaSuccess;
   for (int l = 0; l < p.L && e == cudaSuccess; ++l)
     for (int sub = factor ? 0 : 1; sub < 3 && e == cudaSuccess; ++sub) {
-      if constexpr (sizeof(T) == 8) {
-        if (emu_factor && sub == 2) {
-          e = schur_emu_level(h, b, l);
-          continue;
-        }
-      } else {
+      if constexpr (sizeof(T) == 4) {
         if (tc_factor && sub == 2 && h->ts_ok) {
           e = schur_tf32_level(h, b, l);
           continue;
@@ -625,8 +658,7 @@ bdss_status bdss_destroy(bdss_handle h) {
   cudaFree(h->emu.Xslc);
   cudaFree(h->emu.xexp);
   cudaFree(h->emu.xmax);
-  cudaFree(h->Wslc);
-  cudaFree(h->Wexp);
+  cudaFree(h->wideX);
   cudaFree(h->tcfX);
   cudaFree(h->tcfC);
   cudaFree(h->tcfcb);
@@ -765,30 +797,23 @@ bdss_status bdss_create(bdss_handle *out, int64_t N, int32_t n, int32_t d_max, b
       }
     }
   }
-  if (ok && prec == BDSS_FP64 && N > 1 && h->large) {  // Schur products on the tensor cores
-    ok = ws_alloc(h, (void **)&h->Wslc, emu_wslc_bytes(N - 1, n));
-    ok = ok && ws_alloc(h, (void **)&h->Wexp, (size_t)(N - 1) * n * sizeof(int));
+  if (ok && prec == BDSS_FP64 && h->large) {
+    ok = ws_alloc(h, &h->wideX, wide_x_bytes<double>(N));
     if (ok) {
-      const cudaError_t ec = emu_configure();
+      const cudaError_t ec = wide_configure<double>();
       if (ec != cudaSuccess) {
         bdss_destroy(h);
         return cuda_fail(ec);
       }
-      h->schur_emu_ready = 1;
-      h->schur_emu_on = 1;
+      h->wide_ready = 1;
+      h->wide_on = 1;
     }
   }
-  if (ok && prec == BDSS_FP64 && N > 1 && !h->large && n >= kTcfMinN) {
-    ok = ws_alloc(h, &h->tcfX, (size_t)(N / 2) * nn * esz);
-    ok = ok && ws_alloc(h, &h->tcfC, (size_t)(N / 2) * 2 * nn * esz);
-    ok = ok && ws_alloc(h, &h->tcfcb, (size_t)(N / 2) * 2 * n * d_max * esz);
-    if (ok) {
-      const cudaError_t ec = tcf_configure<double>(n, d_max);
-      if (ec != cudaSuccess) {
-        bdss_destroy(h);
-        return cuda_fail(ec);
-      }
-      h->tcf_ready = 1;
+  if (ok && tcf_by_size(h)) {
+    const bdss_status st = tcf_alloc(h);
+    if (st != BDSS_OK) {
+      bdss_destroy(h);
+      return st;
     }
   }
   if (!ok) {
@@ -870,9 +895,17 @@ bdss_status bdss_set_option(bdss_handle h, bdss_option key, int64_t value) {
       return BDSS_OK;
     case BDSS_OPT_SCHUR_EMU:
       if (value != 0 && value != 1) return BDSS_ERR_INVALID_ARG;
-      if (value && !h->schur_emu_ready && !(h->tcf_ready && !is_mixed(h))) return BDSS_ERR_UNSUPPORTED;
-      if (h->large) h->schur_emu_on = (int)value;
-      else h->tcf_opt = (int)value;
+      if (value && (is_mixed(h) || h->N < 2 || h->n < kTcfMinN)) return BDSS_ERR_UNSUPPORTED;
+      if (h->large) {
+        h->wide_on = value && h->wide_ready;
+      } else {
+        if (value) {
+          t_alloc_count = 0;
+          const bdss_status st = tcf_alloc(h);
+          if (st != BDSS_OK) return st;
+        }
+        h->tcf_opt = (int)value;
+      }
       return BDSS_OK;
     case BDSS_OPT_RESIDUAL_EMU:
       if (value != 0 && value != 1) return BDSS_ERR_INVALID_ARG;

@@ -553,488 +553,6 @@ cudaError_t encode_bf16_2d(CUtensorMap *out, void *base, unsigned long long cols
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-// ===========================================================================
-// FP64-accurate Schur products of the tiled FP64 factorisation on the tensor
-// cores (the separator update of Algorithm 3, 64 < n <= 256).
-//
-// At level l the stored coupling blocks M_b (b = 0 .. N_l - 2; row m of M_b is
-// column m of the coupling solve W, so D -= M M^T) are cut row by row in the
-// same fixed-point digits as the operator rows of the residual: exponent
-// E_b[m] with max_k |M_b[m][k]| < 2^E and ten planes
-// Wslc[((b S + p) n + m) np + k], zero for k >= n.  Separator s = 2k needs
-//   D_s     = D - M_{s-1} M_{s-1}^T - M_s M_s^T   (lower triangle),
-//   E_{l+1} = - M_{s+1} M_s^T                     (slot k of level l + 1),
-// computed over 128 x 16 output tiles.  Each product M_a M_b^T of a tile is
-// one accumulation round: per K chunk of 64 the B operand is the ten slices
-// of rows c0 .. c0 + 15 of M_b (one 3-D TMA box, N = 160 rows) and the A
-// operand slice p of rows m0 .. m0 + 127 of M_a, written at TMEM column 16 p,
-// so slice pair (p, q) lands on the accumulator of diagonal p + q as in the
-// residual.  With K <= 256, |ACC_t| <= 10 x 256 x 32 x 32 < 2^22: every sum is
-// exact.  The epilogue scales a round by 2^(E_a[r] + E_b[c] - 118) and adds
-// the rounds of a tile in FP64; the only error is the 59-bit cut of the
-// inputs, below an FP64 product's rounding in the normwise sense.
-// ===========================================================================
-constexpr int kSchurN = 16;      // output columns of a tile
-constexpr int kSchurRounds = 2;  // products of one tile at most
-constexpr int kSchurAStages = 10;  // A slabs in flight (one round of ten slices)
-
-// Digit formats of the Schur engine.  Ten signed base-64 digits (59 bits)
-// for K up to 256 (the n > 64 path); eight signed base-256 digits (60 bits)
-// for K = 64 (n <= 64): |ACC_t| <= 8 x 64 x 128 x 128 = 2^23 stays exact in
-// FP32, and 15 diagonals x 16 columns leave room for two accumulators in the
-// 512 TMEM columns, so that a round's epilogue runs under the next round's
-// products.  Diagonal groups of the int64 combination: t <= kG0 (shift kSh0),
-// t <= kG1 (shift kSh1), the rest (shift 0).
-template <int kSl> struct EmuDigits;
-template <> struct EmuDigits<10> {
-  static constexpr int kBits = 6, kFrac = 59, kDg = 19, kG0 = 6, kG1 = 13, kSh0 = 72, kSh1 = 30, kBuf = 1;
-  static constexpr unsigned long long kBias = 32ULL * 18300341342965825ULL;  // 32 (64^10 - 1) / 63
-};
-template <> struct EmuDigits<8> {
-  static constexpr int kBits = 8, kFrac = 60, kDg = 15, kG0 = 4, kG1 = 9, kSh0 = 80, kSh1 = 40, kBuf = 2;
-  static constexpr unsigned long long kBias = 0x8080808080808080ULL;  // 128 (256^8 - 1) / 255
-};
-
-// q = round(v 2^(F - E)) as in emu_fixed, for the format's F.
-template <int kSl>
-__device__ __forceinline__ long long emu_fixed_t(double v, int E) {
-  const long long b = __double_as_longlong(v);
-  const int ex = (int)((b >> 52) & 0x7FF);
-  if (ex == 0 || ex == 0x7FF) return 0;
-  const long long m = (b & 0xFFFFFFFFFFFFFLL) | 0x10000000000000LL;
-  const int sh = ex - 1075 + EmuDigits<kSl>::kFrac - E;
-  long long q;
-  constexpr int cap = EmuDigits<kSl>::kFrac - 53;  // |v| < 2^E keeps sh <= cap
-  if (sh >= 0) q = m << (sh > cap ? cap : sh);
-  else if (sh > -63) q = (m + (1LL << (-sh - 1))) >> (-sh);
-  else q = 0;
-  return b < 0 ? -q : q;
-}
-
-// kSl digit planes of four consecutive entries (the biased digits of
-// u = q + bias, each d + B/2 with B the base, as in emu_store_quad).
-template <int kSl>
-__device__ __forceinline__ void emu_store_quad_t(const double (&v)[4], int E, unsigned short *dst,
-                                                 size_t plane_stride) {
-  constexpr int B = EmuDigits<kSl>::kBits;
-  constexpr unsigned long long mask = (1ULL << B) - 1;
-  constexpr float off = 8388608.0f + (float)(1 << (B - 1));
-  unsigned long long u[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) u[j] = (unsigned long long)emu_fixed_t<kSl>(v[j], E) + EmuDigits<kSl>::kBias;
-#pragma unroll
-  for (int p = 0; p < kSl; ++p) {
-    unsigned h[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int dg = p == 0 ? (int)(u[j] >> (B * (kSl - 1))) : (int)((u[j] >> (B * (kSl - 1 - p))) & mask);
-      h[j] = __float_as_uint(__int_as_float(0x4B000000 + dg) - off) >> 16;
-    }
-    *reinterpret_cast<uint2 *>(dst + (size_t)p * plane_stride) = make_uint2(h[0] | (h[1] << 16), h[2] | (h[3] << 16));
-  }
-}
-
-// One warp per row b n + m of the level's stored blocks.
-template <int kSl>
-__global__ void __launch_bounds__(256) k_emu_slice_w(long long rows, int n, int np, const double *W,
-                                                     unsigned short *Wslc, int *Wexp) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long row = (long long)blockIdx.x * 8 + warp;
-  if (row >= rows) return;
-  const long long b = row / n;
-  const int m = (int)(row - b * n);
-  const double *src = W + (size_t)row * n;
-  double v[2][4];
-  unsigned long long mx = 0;
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int k = 4 * (lane + 32 * i) + t;
-      v[i][t] = k < n ? __ldg(src + k) : 0.0;
-      // |v| as bits: ordered like the values, a NaN above every finite value
-      const unsigned long long bits = (unsigned long long)__double_as_longlong(fabs(v[i][t]));
-      mx = bits > mx ? bits : mx;
-    }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long y = __shfl_xor_sync(0xffffffffu, mx, o);
-    mx = y > mx ? y : mx;
-  }
-  const int E = emu_exp(mx);
-  if (lane == 0) Wexp[row] = E;
-  unsigned short *dst = Wslc + ((size_t)b * kSl * n + m) * np;
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int k = 4 * (lane + 32 * i);
-    if (k < np) emu_store_quad_t<kSl>(v[i], E, dst + k, (size_t)n * np);
-  }
-}
-
-// An accumulator entry: an exact integer |x| < 2^22 held in FP32.  Adding
-// 1.5 * 2^23 puts it in the binade of unit spacing, so its bits minus those
-// of 1.5 * 2^23 are x (integer pipe only).
-__device__ __forceinline__ int emu_acc_int(uint32_t bits) {
-  return __float_as_int(__uint_as_float(bits) + 12582912.0f) - 0x4B400000;
-}
-
-// V 2^E rounded once to FP64 (round to nearest even), built from the bits of
-// the 128-bit integer: the leading one sets the exponent, the next 52 bits the
-// fraction.  Results outside the normal range take the FP64 path.
-__device__ __forceinline__ double emu_i128_to_double(__int128 V, int E) {
-  if (V == 0) return 0.0;
-  const bool neg = V < 0;
-  unsigned __int128 m = neg ? (unsigned __int128)(-V) : (unsigned __int128)V;
-  const unsigned long long hi0 = (unsigned long long)(m >> 64), lo0 = (unsigned long long)m;
-  const int lz = hi0 ? __clzll((long long)hi0) : 64 + __clzll((long long)lo0);
-  m <<= lz;  // leading one at bit 127
-  unsigned long long top = (unsigned long long)(m >> 75);  // 53 bits
-  const unsigned __int128 rem = m & ((((unsigned __int128)1) << 75) - 1);
-  const unsigned __int128 half = ((unsigned __int128)1) << 74;
-  if (rem > half || (rem == half && (top & 1ULL))) ++top;
-  int e2 = 127 - lz + E;
-  if (top >> 53) {
-    top >>= 1;
-    ++e2;
-  }
-  const int be = e2 + 1023;
-  if (be <= 0 || be >= 2047)
-    return scalbn(ldexp((double)(long long)(V >> 64), 64) + (double)(unsigned long long)V, E);
-  const unsigned long long bits =
-      ((unsigned long long)neg << 63) | ((unsigned long long)be << 52) | (top & ((1ULL << 52) - 1));
-  return __longlong_as_double((long long)bits);
-}
-
-__device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, int c0, int c1, int c2,
-                                            uint64_t *bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
-      "[%5];" ::"r"(smem_u32(dst)),
-      "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar))
-      : "memory");
-}
-
-struct EmuSchurArgs {
-  long long Nl;          // positions of level l
-  int n, np, l;
-  const int *Wexp;       // (N_l - 1) x n row exponents of the level's stored blocks
-  const double *A_diag;  // level 0: the separators' D (symmetrised)
-  double *Ld;            // D blocks (slot s << l)
-  double *En;            // E blocks of level l + 1 (slot k)
-  DevStatus *st;
-  long long timeout_ns;
-};
-
-// Column tiles of row tile mt inside D's lower part (c0 < (mt + 1) 128).
-__host__ __device__ inline int schur_d_cols(int n, int mt) {
-  const int CT = (n + kSchurN - 1) / kSchurN, lim = (mt + 1) * kM / kSchurN;
-  return CT < lim ? CT : lim;
-}
-__host__ __device__ inline int schur_tiles_per_sep(int n) {
-  const int MT = (n + kM - 1) / kM, CT = (n + kSchurN - 1) / kSchurN;
-  int t = MT * CT;
-  for (int mt = 0; mt < MT; ++mt) t += schur_d_cols(n, mt);
-  return t;
-}
-
-// Output tile u of the level: separator k, a D tile (lower set) or an E tile,
-// and its rounds (stored blocks of the A and B operands).
-struct SchurTile {
-  long long k, ra0, ra1, rb0, rb1;  // stored blocks of the A and B operands of rounds 0, 1
-  int isD, mt, ct, nr;
-  // scalar fields and selects, so that the tile stays in registers
-  __device__ long long a_of(int r) const { return r == 0 ? ra0 : ra1; }
-  __device__ long long b_of(int r) const { return r == 0 ? rb0 : rb1; }
-};
-__device__ __forceinline__ SchurTile schur_tile(long long u, long long Nl, int n) {
-  SchurTile T;
-  const int per = schur_tiles_per_sep(n);
-  const int MT = (n + kM - 1) / kM, CT = (n + kSchurN - 1) / kSchurN;
-  T.k = u / per;
-  int r = (int)(u - T.k * per);
-  const long long s = 2 * T.k;
-  T.isD = 0;
-  T.mt = 0;
-  T.ct = 0;
-  T.nr = 0;
-  T.ra0 = T.ra1 = T.rb0 = T.rb1 = 0;
-  for (int mt = 0; mt < MT; ++mt) {
-    const int c = schur_d_cols(n, mt);
-    if (r < c) {
-      T.isD = 1;
-      T.mt = mt;
-      T.ct = r;
-      break;
-    }
-    r -= c;
-  }
-  if (T.isD) {
-    const bool hasM = s >= 2, hasP = s + 1 < Nl;
-    // round 0: the left neighbour's block if present, else the right one's
-    T.ra0 = T.rb0 = hasM ? s - 1 : s;
-    T.ra1 = T.rb1 = s;
-    T.nr = (int)hasM + (int)hasP;
-  } else {
-    T.mt = r / CT;
-    T.ct = r - T.mt * CT;
-    if (s + 2 < Nl) {
-      T.ra0 = s + 1;
-      T.rb0 = s;
-      T.nr = 1;
-    }
-  }
-  return T;
-}
-
-// Roles as in the residual kernel: warp 0 TMA, warp 1 MMA, warps 2-5 the
-// epilogue of one TMEM lane quarter each.  Every wait is bounded.
-template <int kSl>
-__global__ void __launch_bounds__(kEmuThreads, 1)
-    k_emu_schur(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
-                const __grid_constant__ EmuSchurArgs a) {
-  using Fm = EmuDigits<kSl>;
-  constexpr int kNs = kSl * kSchurN;           // B rows: the kSl slices of 16 columns stacked (MMA N)
-  constexpr int kBTile = kNs * kEmuKc * 2;     // bytes of one B stage
-  constexpr int kAccCols = Fm::kDg * kSchurN;  // TMEM columns of one accumulator
-  constexpr int kNB = Fm::kBuf;                // accumulators (rounds in flight)
-  constexpr int kAS = kSchurAStages;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ uint64_t a_full[kAS], a_empty[kAS], b_full[kXStages], b_empty[kXStages];
-  __shared__ uint64_t acc_full[2], acc_empty[2], drain;
-  __shared__ uint32_t s_tmem;
-  __shared__ int s_abort;
-  unsigned char *base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  unsigned char *Ast = base;                         // kAS x 16 KB
-  unsigned char *Bst = base + (size_t)kAS * kATile;  // kXStages x kBTile
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n = a.n, kchunks = a.np / kEmuKc;
-  const long long tiles = ((a.Nl + 1) / 2) * schur_tiles_per_sep(n);
-  volatile int *abort = &s_abort;
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kAS; ++s) {
-      mbar_init(&a_full[s], 1);
-      mbar_init(&a_empty[s], 1);
-    }
-    for (int s = 0; s < kXStages; ++s) {
-      mbar_init(&b_full[s], 1);
-      mbar_init(&b_empty[s], 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], 128);
-    }
-    mbar_init(&drain, 1);
-    s_abort = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 1) tmem_alloc(&s_tmem, kTmemCols);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = s_tmem;
-  auto fail = [&]() {
-    *abort = 1;
-    set_status(a.st, kStTimeout, -1, -1);
-  };
-
-  if (warp == 0) {
-    // ---- TMA producer -------------------------------------------------------
-    if (lane == 0) {
-      int as = 0, bs = 0;
-      uint32_t aph = 0, bph = 0;
-      for (long long u = blockIdx.x; u < tiles && !*abort; u += gridDim.x) {
-        const SchurTile T = schur_tile(u, a.Nl, n);
-        for (int r = 0; r < T.nr && !*abort; ++r)
-          for (int kk = 0; kk < kchunks; ++kk) {
-            if (!emu_wait(&b_empty[bs], bph ^ 1, a.timeout_ns, abort)) { fail(); break; }
-            mbar_expect_tx(&b_full[bs], kBTile);
-            tma_load_3d(Bst + (size_t)bs * kBTile, &mapB, kk * kEmuKc, T.ct * kSchurN, (int)(T.b_of(r) * kSl),
-                        &b_full[bs]);
-            if (++bs == kXStages) { bs = 0; bph ^= 1; }
-            for (int p = 0; p < kSl; ++p) {
-              if (!emu_wait(&a_empty[as], aph ^ 1, a.timeout_ns, abort)) { fail(); break; }
-              mbar_expect_tx(&a_full[as], kATile);
-              tma_load_2d(Ast + (size_t)as * kATile, &mapA, kk * kEmuKc, (int)((T.a_of(r) * kSl + p) * n + T.mt * kM),
-                          &a_full[as]);
-              if (++as == kAS) { as = 0; aph ^= 1; }
-            }
-            if (*abort) break;
-          }
-      }
-      for (int s = 0; s < kAS; ++s) {
-        const uint32_t ph = (s < as) ? aph : (aph ^ 1);
-        emu_wait(&a_full[s], ph, a.timeout_ns, nullptr);
-      }
-      for (int s = 0; s < kXStages; ++s) {
-        const uint32_t ph = (s < bs) ? bph : (bph ^ 1);
-        emu_wait(&b_full[s], ph, a.timeout_ns, nullptr);
-      }
-    }
-  } else if (warp == 1) {
-    // ---- MMA issuer ------------------------------------------------------------
-    if (lane == 0) {
-      constexpr uint32_t idesc = emu_idesc(kM, kNs);
-      int as = 0, bs = 0;
-      uint32_t aph = 0, bph = 0;
-      long long i = 0;  // rounds so far: accumulator i % kNB
-      for (long long u = blockIdx.x; u < tiles && !*abort; u += gridDim.x) {
-        const SchurTile T = schur_tile(u, a.Nl, n);
-        for (int r = 0; r < T.nr && !*abort; ++r) {
-          const int ab = (int)(i % kNB);
-          if (!emu_wait(&acc_empty[ab], (uint32_t)((i / kNB) & 1), a.timeout_ns, abort)) { fail(); break; }
-          tc_fence_after();
-          const uint32_t dacc = tmem + (uint32_t)(ab * kAccCols);
-          for (int kk = 0; kk < kchunks; ++kk) {
-            if (!emu_wait(&b_full[bs], bph, a.timeout_ns, abort)) { fail(); break; }
-            const unsigned char *bb = Bst + (size_t)bs * kBTile;
-            for (int p = 0; p < kSl; ++p) {
-              if (!emu_wait(&a_full[as], aph, a.timeout_ns, abort)) { fail(); break; }
-              tc_fence_after();
-              const unsigned char *abuf = Ast + (size_t)as * kATile;
-#pragma unroll
-              for (int ks = 0; ks < kEmuKc / 16; ++ks)
-                emu_mma_bf16(dacc + (uint32_t)(p * kSchurN), tc_desc_sw128(abuf, ks * 32), tc_desc_sw128(bb, ks * 32),
-                             idesc);
-              tc_commit(&a_empty[as]);
-              if (++as == kAS) { as = 0; aph ^= 1; }
-            }
-            tc_commit(&b_empty[bs]);
-            if (++bs == kXStages) { bs = 0; bph ^= 1; }
-            if (*abort) break;
-          }
-          tc_commit(&acc_full[ab]);
-          ++i;
-        }
-      }
-      tc_commit(&drain);
-      emu_wait(&drain, 0, a.timeout_ns, nullptr);
-    }
-  } else {
-    // ---- epilogue: warps 2..5, TMEM lane quarter warp % 4 ---------------------
-    const int quarter = warp & 3;
-    const uint32_t lane_base = tmem + ((uint32_t)(32 * quarter) << 16);
-    auto clear = [&](int b) {
-      for (int t = 0; t < Fm::kDg; ++t) tmem_zero16(lane_base + (uint32_t)(b * kAccCols + t * kSchurN));
-      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-      tc_fence_before();
-      emu_arrive(&acc_empty[b]);
-    };
-    for (int b = 0; b < kNB; ++b) clear(b);
-    long long i = 0;  // rounds so far: accumulator i % kNB
-    const size_t nn = (size_t)n * n;
-    bool stop = false;
-    for (long long u = blockIdx.x; u < tiles && !stop; u += gridDim.x) {
-      const SchurTile T = schur_tile(u, a.Nl, n);
-      if (T.nr == 0) continue;
-      const int row = T.mt * kM + 32 * quarter + lane;
-      double acc[kSchurN];
-#pragma unroll
-      for (int c = 0; c < kSchurN; ++c) acc[c] = 0.0;
-      for (int r = 0; r < T.nr; ++r) {
-        const int ab = (int)(i % kNB);
-        const uint32_t fpar = (uint32_t)((i / kNB) & 1);
-        int ok = 0;
-        if (lane == 0) ok = emu_wait(&acc_full[ab], fpar, a.timeout_ns, abort) ? 1 : 0;
-        ok = __shfl_sync(0xffffffffu, ok, 0);
-        if (!ok) {
-          if (lane == 0) fail();
-          stop = true;
-          break;
-        }
-        if (lane != 0) emu_try(&acc_full[ab], fpar);
-        ++i;
-        tc_fence_after();
-        // the diagonals, combined exactly on the integer pipe: V = sum_t
-        // ACC_t B^(kDg - 1 - t) in three int64 groups, then one 128-bit
-        // integer (|V| < 2^126: a sum of K products of F-bit numbers, K <= 256
-        // for F = 59, K = 64 for F = 60); the FP64 pipe (64 cycles per warp
-        // instruction on this GPU) is left to one add per entry
-        __int128 V[kSchurN];
-        {
-          long long G[kSchurN];
-#pragma unroll
-          for (int c = 0; c < kSchurN; ++c) G[c] = 0;
-          for (int t = 0; t < Fm::kDg; ++t) {
-            uint32_t rr[16];
-            tmem_ld16(lane_base + (uint32_t)(ab * kAccCols + t * kSchurN), rr);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-            for (int c = 0; c < kSchurN; ++c) {
-              // |ACC| < 2^22 (ten digits) takes the integer trick; up to 2^23 a conversion
-              const int x = (kSl == 10) ? emu_acc_int(rr[c]) : __float2int_rn(__uint_as_float(rr[c]));
-              G[c] = G[c] * (1LL << Fm::kBits) + (long long)x;
-            }
-            if (t == Fm::kG0 || t == Fm::kG1 || t == Fm::kDg - 1) {
-              const int sh = t == Fm::kG0 ? Fm::kSh0 : t == Fm::kG1 ? Fm::kSh1 : 0;
-#pragma unroll
-              for (int c = 0; c < kSchurN; ++c) {
-                const __int128 g = (__int128)G[c] << sh;
-                V[c] = (t == Fm::kG0) ? g : V[c] + g;
-                G[c] = 0;
-              }
-            }
-          }
-        }
-        tc_fence_before();
-        clear(ab);
-        const int Ea = row < n ? __ldg(a.Wexp + (size_t)T.a_of(r) * n + row) : 0;
-#pragma unroll
-        for (int c = 0; c < kSchurN; ++c) {
-          const int col = T.ct * kSchurN + c;
-          const int Eb = col < n ? __ldg(a.Wexp + (size_t)T.b_of(r) * n + col) : 0;
-          // an Inf or NaN in either row (exponent field all ones: E = 1025)
-          // poisons the entry, as an FP64 product would
-          acc[c] += (Ea > 1024 || Eb > 1024) ? __longlong_as_double(0x7FF8000000000000LL)
-                                             : emu_i128_to_double(V[c], Ea + Eb - 2 * Fm::kFrac);
-        }
-      }
-      if (stop || row >= n) continue;
-      const long long s = 2 * T.k;
-      if (T.isD) {
-        const long long orig = s << a.l;
-        double *Dg = a.Ld + (size_t)orig * nn + (size_t)row * n;
-        const double *Ag = a.A_diag + (size_t)orig * nn;
-#pragma unroll
-        for (int c = 0; c < kSchurN; ++c) {
-          const int col = T.ct * kSchurN + c;
-          if (col < n && col <= row) {
-            const double b0 = a.l == 0 ? 0.5 * (__ldg(Ag + (size_t)row * n + col) + __ldg(Ag + (size_t)col * n + row))
-                                       : Dg[col];
-            Dg[col] = b0 - acc[c];
-          }
-        }
-      } else {
-        double *Eg = a.En + (size_t)T.k * nn + (size_t)row * n;
-#pragma unroll
-        for (int c = 0; c < kSchurN; ++c) {
-          const int col = T.ct * kSchurN + c;
-          if (col < n) Eg[col] = -acc[c];
-        }
-      }
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  if (warp == 1) tmem_dealloc(tmem, kTmemCols);
-}
-
-cudaError_t encode_bf16_3d(CUtensorMap *out, void *base, unsigned long long cols, unsigned long long rows,
-                           unsigned long long planes, unsigned box_cols, unsigned box_rows, unsigned box_planes) {
-  EncodeTiledFn fn = nullptr;
-  const cudaError_t e = encode_fn(&fn);
-  if (e != cudaSuccess) return e;
-  const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)planes};
-  const cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)cols * rows * 2};
-  const cuuint32_t box[3] = {box_cols, box_rows, box_planes};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
-}
-
-
 }  // namespace
 
 size_t emu_aslc_bytes(long long N, int n) { return (size_t)N * kS * n * 3 * emu_np(n) * 2; }
@@ -1054,8 +572,7 @@ cudaError_t emu_configure() {
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const void *kernels[] = {(const void *)k_emu_residual, (const void *)k_emu_slice_operator,
-                           (const void *)k_emu_slice_x, (const void *)k_emu_schur<10>,
-                           (const void *)k_emu_schur<8>};
+                           (const void *)k_emu_slice_x};
   for (const void *k : kernels) {
     cudaFuncAttributes fa;
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k);
@@ -1104,67 +621,6 @@ cudaError_t launch_emu_residual(long long N, int n, int d, const double *X, cons
   const int grid = (int)(tiles < sms ? tiles : sms);
   k_emu_residual<<<grid, kEmuThreads, kResidualSmem, s>>>(b.maps[0], b.maps[1], k);
   return cudaGetLastError();
-}
-
-size_t emu_wslc_bytes(long long nW, int n) { return (size_t)nW * kS * n * emu_np(n) * 2; }
-
-// Digits of the Schur engine: eight base-256 digits when the whole K = n fits
-// one chunk of 64 (two accumulators in TMEM), else ten base-64 digits.
-static int schur_slices(int n) { return emu_np(n) == kEmuKc ? 8 : 10; }
-
-template <int kSl>
-static size_t schur_smem() {
-  return (size_t)kSchurAStages * kATile + (size_t)kXStages * kSl * kSchurN * kEmuKc * 2 + 1024;
-}
-
-cudaError_t launch_emu_slice_w(long long nW, int n, const double *W, unsigned short *Wslc, int *Wexp,
-                               cudaStream_t s) {
-  if (n > 256) return cudaErrorInvalidValue;
-  const long long rows = nW * n;
-  if (rows <= 0) return cudaSuccess;
-  const unsigned grid = (unsigned)((rows + 7) / 8);
-  if (schur_slices(n) == 8) k_emu_slice_w<8><<<grid, 256, 0, s>>>(rows, n, emu_np(n), W, Wslc, Wexp);
-  else k_emu_slice_w<10><<<grid, 256, 0, s>>>(rows, n, emu_np(n), W, Wslc, Wexp);
-  return cudaGetLastError();
-}
-
-template <int kSl>
-static cudaError_t launch_emu_schur_t(long long Nl, int n, int l, const unsigned short *Wslc, const int *Wexp,
-                                      const double *A_diag, double *Ld, double *En, DevStatus *st,
-                                      long long timeout_ns, int sms, cudaStream_t s) {
-  const int np = emu_np(n);
-  const long long nW = Nl - 1;
-  CUtensorMap mapA, mapB;
-  cudaError_t e = encode_bf16_2d(&mapA, (void *)Wslc, (unsigned long long)np, (unsigned long long)(nW * kSl * n),
-                                 kEmuKc, kM);
-  if (e == cudaSuccess)
-    e = encode_bf16_3d(&mapB, (void *)Wslc, (unsigned long long)np, (unsigned long long)n,
-                       (unsigned long long)(nW * kSl), kEmuKc, kSchurN, kSl);
-  if (e != cudaSuccess) return e;
-  EmuSchurArgs k;
-  k.Nl = Nl;
-  k.n = n;
-  k.np = np;
-  k.l = l;
-  k.Wexp = Wexp;
-  k.A_diag = A_diag;
-  k.Ld = Ld;
-  k.En = En;
-  k.st = st;
-  k.timeout_ns = timeout_ns;
-  const long long tiles = ((Nl + 1) / 2) * schur_tiles_per_sep(n);
-  const int grid = (int)(tiles < sms ? tiles : sms);
-  k_emu_schur<kSl><<<grid, kEmuThreads, schur_smem<kSl>(), s>>>(mapA, mapB, k);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_emu_schur(long long Nl, int n, int l, const unsigned short *Wslc, const int *Wexp,
-                             const double *A_diag, double *Ld, double *En, DevStatus *st, long long timeout_ns,
-                             int sms, cudaStream_t s) {
-  if (Nl < 2 || n > 256) return cudaErrorInvalidValue;
-  if (schur_slices(n) == 8)
-    return launch_emu_schur_t<8>(Nl, n, l, Wslc, Wexp, A_diag, Ld, En, st, timeout_ns, sms, s);
-  return launch_emu_schur_t<10>(Nl, n, l, Wslc, Wexp, A_diag, Ld, En, st, timeout_ns, sms, s);
 }
 
 }  // namespace bdss

@@ -161,7 +161,7 @@ __device__ __forceinline__ int sl_int22(float x) { return __float_as_int(x + 125
 __device__ __forceinline__ int sl_int23(float x) { return (__float_as_int(x + 25165824.0f) - 0x4BC00000) * 2; }
 
 // t 2^(be - 1075) for a result outside the normal range.
-__device__ __noinline__ double sl_scale_slow(unsigned long long t, int be) { return scalbn((double)(long long)t, be - 1075); }
+static __device__ __noinline__ double sl_scale_slow(unsigned long long t, int be) { return scalbn((double)(long long)t, be - 1075); }
 
 // sum_t ACC_t 256^(7-t) 2^(exa + exb - 2112), rounded once to FP64 on the
 // integer pipe (an FP64 instruction holds a warp's FP64 unit for 64 cycles on

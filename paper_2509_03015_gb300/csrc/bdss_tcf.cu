@@ -35,49 +35,6 @@ constexpr int kSchurThreads = 512;
 constexpr uint32_t kTmemAll = 512;
 constexpr uint32_t kBufCols = 256;  // accumulators of one column tile
 
-// X = L^{-1} of the staged factor (reciprocal diagonal), X^T into the upper
-// triangle: X[i][c] at s[c ld + i], c < i.  Rows are taken 8 at a time: the
-// dot products with the rows already inverted run over (column, row) pairs on
-// every thread (n^3/6 multiply-adds: column c starts at its own row), then one
-// thread per column solves the 8 x 8 triangle.  All threads call; ends with a
-// barrier.
-template <typename T>
-__device__ void tri_inverse_upper(T *s, int ld, int n) {
-  constexpr int RB = 8;
-  for (int r0 = 0; r0 < n; r0 += RB) {
-    const int rb = min(RB, n - r0);
-    for (int t = threadIdx.x; t < r0 * RB; t += blockDim.x) {
-      const int i = t % RB, c = t / RB;
-      if (i < rb) {
-        const T *lr = s + (r0 + i) * ld, *xc = s + c * ld;  // xc[p] = X[p][c] for p >= c
-        T acc = T(0);
-        for (int p = c; p < r0; ++p) acc = fma(lr[p], xc[p], acc);
-        s[c * ld + r0 + i] = acc;
-      }
-    }
-    __syncthreads();
-    for (int c = threadIdx.x; c < r0 + rb; c += blockDim.x) {
-      const int cc = c - r0;  // column inside this row block (unit vector) if >= 0
-      T x[RB];
-#pragma unroll
-      for (int i = 0; i < RB; ++i) {
-        x[i] = T(0);
-        if (i < rb && i >= cc) {
-          const T *lr = s + (r0 + i) * ld + r0;
-          T acc = cc < 0 ? s[c * ld + r0 + i] : T(0);
-#pragma unroll
-          for (int q = 0; q < i; ++q) acc = fma(lr[q], x[q], acc);
-          x[i] = (i == cc) ? lr[i] : -acc * lr[i];
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < RB; ++i)
-        if (i < rb && i > cc) s[c * ld + r0 + i] = x[i];
-    }
-    __syncthreads();
-  }
-}
-
 template <typename T>
 __global__ void __launch_bounds__(256) k_tcf_diag(const __grid_constant__ Args<T> a, const TcfLevel<T> w, int l,
                                                   int fold_all) {

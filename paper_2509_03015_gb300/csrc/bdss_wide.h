@@ -1,0 +1,37 @@
+// Factorisation of blocks 64 < n <= 256 with its products on the tensor cores
+// (internal to the library; see bdss_wide.cu).
+#pragma once
+#include <cuda_runtime.h>
+
+#include "bdss_device.cuh"
+
+namespace bdss {
+
+// Panels of a block: nt of them, nb columns each (the last may be narrower).
+struct WidePanels {
+  int nt, nb;
+};
+WidePanels wide_panels(int n);
+
+template <typename T>
+struct WideBuf {
+  T *X;  // [m][64][64]: inverse of the current panel's diagonal tile, per eliminated block of the level
+};
+
+// Bytes of WideBuf::X for a system of N blocks.
+template <typename T> size_t wide_x_bytes(long long N);
+template <typename T> cudaError_t wide_configure();
+
+// Level 0: sym(A_diag) into Ld, the couplings into region 0 of Wb, B into Y.
+template <typename T> cudaError_t launch_wide_ingest(const Args<T> &a, int sms, cudaStream_t s);
+// Panel k of level l's eliminated blocks: the diagonal tile's Cholesky factor
+// and inverse; then every row below it and the rows of W^T and y^T.
+template <typename T> cudaError_t launch_wide_diag(const Args<T> &a, const WideBuf<T> &w, int l, int k, cudaStream_t s);
+template <typename T>
+cudaError_t launch_wide_panel(const Args<T> &a, const WideBuf<T> &w, int l, int k, int sms, cudaStream_t s);
+// The separators' D, the next level's couplings and the separators' b.
+template <typename T> cudaError_t launch_wide_schur(const Args<T> &a, int l, int sms, cudaStream_t s);
+// Downward pass of level l.
+template <typename T> cudaError_t launch_wide_down(const Args<T> &a, int l, cudaStream_t s);
+
+}  // namespace bdss
