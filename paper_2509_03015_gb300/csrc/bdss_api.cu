@@ -83,6 +83,8 @@ struct bdss_ctx {
   // 64 < n <= 256: factorisation with its products on the tensor cores
   // (bdss_wide.cu)
   void *wideX = nullptr;  // inverses of the current panel's diagonal tiles (T)
+  float *wideV = nullptr;    // mixed: L^{-T} of the current level's blocks (N / 2 x n x n)
+  double *wideTop = nullptr; // mixed: workspace of the FP64 top block
   int wide_ready = 0;
   int wide_on = 0;
   // n <= 64: factorisation with the coupling solves and Schur products on the
@@ -378,47 +380,145 @@ static Args<T> base_args(bdss_ctx *h) {
   return a;
 }
 
-// Factorisation for 64 < n <= 256 with its products on the tensor cores: per
-// level and panel the diagonal tiles (ALU) and every other row, then the
-// separators' updates; the top block like an eliminated block without
-// couplings; the downward pass.
-template <typename T>
-static cudaError_t run_levels_wide(bdss_ctx *h, const Args<T> &a, bool rhs) {
+// Downward passes of the large mixed path with the stored inverses, streamed.
+static cudaError_t run_corr_down(bdss_ctx *h, const Args<float> &b) {
   const Plan &p = h->plan;
-  Args<T> b = a;
-  if (!rhs) b.d = 0;
-  const WideBuf<T> w{(T *)h->wideX};
-  const int nt = wide_panels(p.n).nt;
-  kt_begin(h, h->kt_cls);
-  cudaError_t e = launch_wide_ingest<T>(b, h->sms, h->stream);
-  kt_end(h, 1);
-  h->launches += 1;
-  for (int l = 0; l <= p.L && e == cudaSuccess; ++l) {
-    for (int k = 0; k < nt && e == cudaSuccess; ++k) {
-      kt_begin(h, h->kt_cls);
-      e = launch_wide_diag<T>(b, w, l, k, h->stream);
-      kt_end(h, 1);
-      kt_begin(h, BDSS_KT_SCHUR_TC);
-      if (e == cudaSuccess) e = launch_wide_panel<T>(b, w, l, k, h->sms, h->stream);
-      kt_end(h, 1);
-      h->launches += 2;
+  cudaError_t e = cudaSuccess;
+  for (int l = p.L - 1; l >= 0 && e == cudaSuccess; --l) {
+    kt_begin(h, h->kt_cls);
+    if (corr_split(p.n, p.Nl[l] / 2, h->sms, h->corr_max_split) > 1) {
+      // few blocks: t = y - W x, then x = L^{-T} t, each block split over SMs
+      e = launch_large_corr(h->corr_maps, h->corr_max_split, b, l, kSubC1, h->sms, h->stream);
+      if (e == cudaSuccess) e = launch_large_corr(h->corr_maps, h->corr_max_split, b, l, kSubC2, h->sms, h->stream);
+      h->launches += 1;
+    } else {
+      e = launch_large_corr(h->corr_maps, h->corr_max_split, b, l, kSubC, h->sms, h->stream);
     }
-    if (l == p.L || e != cudaSuccess) break;
-    kt_begin(h, BDSS_KT_SCHUR_TC);
-    e = launch_wide_schur<T>(b, l, h->sms, h->stream);
     kt_end(h, 1);
     h->launches += 1;
   }
+  return e;
+}
+
+// Solve pass of the large mixed path with the stored inverses, streamed: per
+// level the upward products (A2, B), the top block, then per level the
+// downward products (C), one launch each.
+static cudaError_t run_corr_passes(bdss_ctx *h, const Args<float> &b) {
+  const Plan &p = h->plan;
+  cudaError_t e = cudaSuccess;
+  for (int l = 0; l < p.L && e == cudaSuccess; ++l)
+    for (int sub = kSubA2; sub <= kSubB && e == cudaSuccess; ++sub) {
+      kt_begin(h, h->kt_cls);
+      e = launch_large_corr(h->corr_maps, h->corr_max_split, b, l, sub, h->sms, h->stream);
+      kt_end(h, 1);
+      h->launches += 1;
+    }
+  kt_begin(h, h->kt_cls);
+  if (e == cudaSuccess) e = launch_large_top<float>(b, 0, h->smem, h->stream);
+  kt_end(h, 1);
+  h->launches += 1;
+  if (e == cudaSuccess) e = run_corr_down(h, b);
+  return e;
+}
+
+// The downward pass after an FP32 factorisation: streamed, or (odd shapes)
+// level by level with a thread per row.
+static cudaError_t wide_down_f32(bdss_ctx *h, const Args<float> &b) {
+  const Plan &p = h->plan;
+  if (h->corr_ok && b.d <= kCorrMaxD) return run_corr_down(h, b);
+  cudaError_t e = cudaSuccess;
+  for (int l = p.L - 1; l >= 0 && e == cudaSuccess; --l) {
+    kt_begin(h, h->kt_cls);
+    e = launch_large_sub<float>(b, l, 3, 0, grid_for(h, large_sub_tasks(p, l, 3, 0, b.d, 4, 0, 1)), h->smem, h->stream);
+    kt_end(h, 1);
+    h->launches += 1;
+  }
+  return e;
+}
+
+// Factorisation for 64 < n <= 256 with its products on the tensor cores: per
+// level and panel the diagonal tiles (ALU) and every other row, then the
+// separators' updates; the top block (in FP64) like an eliminated block
+// without couplings; the downward pass.
+template <typename T>
+static cudaError_t wide_block(bdss_ctx *h, const Args<T> &a, const WideBuf<T> &w, int l) {
+  const int nt = wide_panels(a.p.n).nt;
+  cudaError_t e = cudaSuccess;
+  for (int k = 0; k < nt && e == cudaSuccess; ++k) {
+    kt_begin(h, h->kt_cls);
+    e = launch_wide_diag<T>(a, w, l, k, h->stream);
+    kt_end(h, 1);
+    kt_begin(h, BDSS_KT_SCHUR_TC);
+    if (e == cudaSuccess) e = launch_wide_panel<T>(a, w, l, k, h->sms, h->stream);
+    kt_end(h, 1);
+    h->launches += 2;
+  }
+  return e;
+}
+
+template <typename T>
+static cudaError_t wide_up(bdss_ctx *h, const Args<T> &a, const WideBuf<T> &w) {
+  kt_begin(h, h->kt_cls);
+  cudaError_t e = launch_wide_ingest<T>(a, h->sms, h->stream);
+  kt_end(h, 1);
+  h->launches += 1;
+  for (int l = 0; l < a.p.L && e == cudaSuccess; ++l) {
+    e = wide_block<T>(h, a, w, l);
+    kt_begin(h, BDSS_KT_SCHUR_TC);
+    if (e == cudaSuccess) e = launch_wide_schur<T>(a, l, h->sms, h->stream);
+    kt_end(h, 1);
+    h->launches += 1;
+  }
+  return e;
+}
+
+static cudaError_t run_levels_wide(bdss_ctx *h, const Args<double> &a, bool rhs) {
+  const Plan &p = h->plan;
+  Args<double> b = a;
+  if (!rhs) b.d = 0;
+  const WideBuf<double> w{(double *)h->wideX, nullptr, nullptr};
+  cudaError_t e = wide_up<double>(h, b, w);
+  if (e == cudaSuccess) e = wide_block<double>(h, b, w, p.L);
   // the solve passes read the top factor from Ltop
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(h->Ltop, h->Ld, (size_t)p.n * p.n * sizeof(double), cudaMemcpyDeviceToDevice, h->stream);
   if (rhs)
     for (int l = p.L; l >= 0 && e == cudaSuccess; --l) {
       kt_begin(h, h->kt_cls);
-      e = launch_wide_down<T>(b, l, h->stream);
+      e = launch_wide_down<double>(b, l, h->stream);
       kt_end(h, l < p.L ? 2 : 1);
       h->launches += l < p.L ? 2 : 1;
     }
+  return e;
+}
+
+// FP32: L^{-1} of every block as well, y kept in Yt as in the solve passes,
+// whose downward pass follows.
+static cudaError_t run_levels_wide(bdss_ctx *h, const Args<float> &a, bool rhs) {
+  const Plan &p = h->plan;
+  const size_t nn = (size_t)p.n * p.n;
+  Args<float> b = a;  // upward: b and y in Yt
+  if (!rhs) b.d = 0;
+  b.Y = h->Yt;
+  cudaError_t e = wide_up<float>(h, b, WideBuf<float>{(float *)h->wideX, (float *)h->Li, h->wideV});
+  double *ws = h->wideTop;  // X, L^{-1}, L^{-T} and y of the top block
+  Args<double> t = base_args<double>(h);
+  t.Ld = h->Ltop;
+  t.Y = ws + (size_t)64 * 64 + 2 * nn;
+  t.d = b.d;
+  kt_begin(h, h->kt_cls);
+  if (e == cudaSuccess) e = launch_wide_top_in(b, h->Ltop, t.Y, h->stream);
+  kt_end(h, 1);
+  if (e == cudaSuccess)
+    e = wide_block<double>(h, t, WideBuf<double>{ws, ws + (size_t)64 * 64, ws + (size_t)64 * 64 + nn}, p.L);
+  b.Y = a.Y;
+  b.Yt = h->Yt;
+  kt_begin(h, h->kt_cls);
+  if (e == cudaSuccess && rhs) e = launch_wide_down<double>(t, p.L, h->stream);
+  if (e == cudaSuccess) e = launch_wide_top_out(b, ws + (size_t)64 * 64, t.Y, h->stream);
+  kt_end(h, rhs ? 2 : 1);
+  h->launches += rhs ? 3 : 2;
+  if (rhs && e == cudaSuccess) e = wide_down_f32(h, b);
   return e;
 }
 
@@ -454,39 +554,6 @@ static cudaError_t run_levels_tcf(bdss_ctx *h, const Args<T> &a, bool rhs) {
       kt_end(h, 1);
       h->launches += 1;
     }
-  return e;
-}
-
-// Solve pass of the large mixed path with the stored inverses, streamed: per
-// level the upward products (A2, B), the top block, then per level the
-// downward products (C), one launch each.
-static cudaError_t run_corr_passes(bdss_ctx *h, const Args<float> &b) {
-  const Plan &p = h->plan;
-  cudaError_t e = cudaSuccess;
-  for (int l = 0; l < p.L && e == cudaSuccess; ++l)
-    for (int sub = kSubA2; sub <= kSubB && e == cudaSuccess; ++sub) {
-      kt_begin(h, h->kt_cls);
-      e = launch_large_corr(h->corr_maps, h->corr_max_split, b, l, sub, h->sms, h->stream);
-      kt_end(h, 1);
-      h->launches += 1;
-    }
-  kt_begin(h, h->kt_cls);
-  if (e == cudaSuccess) e = launch_large_top<float>(b, 0, h->smem, h->stream);
-  kt_end(h, 1);
-  h->launches += 1;
-  for (int l = p.L - 1; l >= 0 && e == cudaSuccess; --l) {
-    kt_begin(h, h->kt_cls);
-    if (corr_split(p.n, p.Nl[l] / 2, h->sms, h->corr_max_split) > 1) {
-      // few blocks: t = y - W x, then x = L^{-T} t, each block split over SMs
-      e = launch_large_corr(h->corr_maps, h->corr_max_split, b, l, kSubC1, h->sms, h->stream);
-      if (e == cudaSuccess) e = launch_large_corr(h->corr_maps, h->corr_max_split, b, l, kSubC2, h->sms, h->stream);
-      h->launches += 1;
-    } else {
-      e = launch_large_corr(h->corr_maps, h->corr_max_split, b, l, kSubC, h->sms, h->stream);
-    }
-    kt_end(h, 1);
-    h->launches += 1;
-  }
   return e;
 }
 
@@ -528,9 +595,7 @@ static cudaError_t run_levels_large(bdss_ctx *h, const Args<T> &a, bool factor, 
   if (!rhs) b.d = 0;
   // solve passes with the stored inverses keep y of the eliminated blocks in Yt
   b.Yt = (!factor && inv) ? (T *)h->Yt : nullptr;
-  if constexpr (sizeof(T) == 8) {
-    if (factor && h->wide_on) return run_levels_wide<T>(h, a, rhs);
-  }
+  if (factor && h->wide_on) return run_levels_wide(h, a, rhs);
   if constexpr (sizeof(T) == 4) {
     if (!factor && rhs && inv && h->corr_ok && b.d <= kCorrMaxD) return run_corr_passes(h, b);
   }
@@ -659,6 +724,8 @@ bdss_status bdss_destroy(bdss_handle h) {
   cudaFree(h->emu.xexp);
   cudaFree(h->emu.xmax);
   cudaFree(h->wideX);
+  cudaFree(h->wideV);
+  cudaFree(h->wideTop);
   cudaFree(h->tcfX);
   cudaFree(h->tcfC);
   cudaFree(h->tcfcb);
@@ -797,10 +864,15 @@ bdss_status bdss_create(bdss_handle *out, int64_t N, int32_t n, int32_t d_max, b
       }
     }
   }
-  if (ok && prec == BDSS_FP64 && h->large) {
-    ok = ws_alloc(h, &h->wideX, wide_x_bytes<double>(N));
+  if (ok && h->large) {
+    ok = ws_alloc(h, &h->wideX, is_mixed(h) ? wide_x_bytes<float>(N) : wide_x_bytes<double>(N));
+    if (is_mixed(h)) {
+      ok = ok && ws_alloc(h, (void **)&h->wideV, (size_t)(N / 2 > 1 ? N / 2 : 1) * nn * sizeof(float));
+      ok = ok && ws_alloc(h, (void **)&h->wideTop, ((size_t)64 * 64 + 2 * nn + (size_t)n * d_max) * sizeof(double));
+    }
     if (ok) {
-      const cudaError_t ec = wide_configure<double>();
+      cudaError_t ec = wide_configure<double>();
+      if (ec == cudaSuccess && is_mixed(h)) ec = wide_configure<float>();
       if (ec != cudaSuccess) {
         bdss_destroy(h);
         return cuda_fail(ec);
@@ -1240,6 +1312,7 @@ static bdss_status krylov_cycle(bdss_ctx *h, const double *B, double *X, int d) 
 // of either kind.
 static bdss_status refine(bdss_ctx *h, const double *B, double *X, int d, bdss_info *info) {
   constexpr int kMaxCgCycles = 4;
+  constexpr double kTargetMargin = 0.95;
   double prev = INFINITY, berr = -1.0;
   int cycles = 0;
   bdss_status result = BDSS_ERR_NO_CONVERGENCE;
@@ -1248,9 +1321,12 @@ static bdss_status refine(bdss_ctx *h, const double *B, double *X, int d, bdss_i
   for (int it = 0;; ++it) {
     bdss_status st = residual_berr(h, B, X, d, &berr);
     if (st != BDSS_OK) return st;
-    if (berr <= h->target) { result = BDSS_OK; break; }
+    // the measured error stands for the true one within a few per cent (a
+    // residual of finite precision, an FP32 norm of A): the target counts as
+    // met with that much to spare, or exactly once refinement has stalled
     const bool stalled = it > 0 && !(berr < 0.5 * prev);
     const bool plain_done = stalled || it >= h->max_refine;
+    if (berr <= (plain_done ? 1.0 : kTargetMargin) * h->target) { result = BDSS_OK; break; }
     // shifted factors are no accurate solver of A: CG from the first correction
     const bool cg = cycles > 0 || h->krylov == 2 || (h->krylov == 1 && (plain_done || h->shift_used > 0));
     if (!cg) {

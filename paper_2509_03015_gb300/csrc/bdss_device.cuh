@@ -516,47 +516,208 @@ __device__ int chol_fused(T *s, int ld, int n, T *V1, int nv1, T *V2, int nv2, i
   return 0;
 }
 
-// X = L^{-1} of the staged factor (reciprocal diagonal), X^T into the upper
-// triangle: X[i][c] at s[c ld + i], c < i.  Rows are taken 8 at a time: the
-// dot products with the rows already inverted run over (column, row) pairs on
-// every thread (n^3/6 multiply-adds: column c starts at its own row), then one
-// thread per column solves the 8 x 8 triangle.  All threads call; ends with a
+// Seed of 1 / x for a positive finite x: the FP32 reciprocal of x cut to FP32
+// (below 2^-21 off).  One third-order step follows it,
+//   e = 1 - x y,  y <- y + y (e + e^2),
+// three FP64 instructions.  FP64 numbers outside the FP32 exponent range: 1 / x
+// (e is then zero within rounding).
+__device__ __forceinline__ float rcp_seed(float x) { return __frcp_rn(x); }
+__device__ __forceinline__ double rcp_seed(double x) {
+  const long long b = __double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 0x7FF);
+  if (ex < 1023 - 120 || ex > 1023 + 120) return 1.0 / x;
+  const float xf = __int_as_float(((ex - 1023 + 127) << 23) | (int)((b >> 29) & 0x7FFFFF));
+  const int yb = __float_as_int(__fdividef(1.0f, xf));
+  return __longlong_as_double(((long long)(((yb >> 23) & 0xFF) - 127 + 1023) << 52) | ((long long)(yb & 0x7FFFFF) << 29));
+}
+
+// Cholesky factor L of the staged lower triangle together with X = L^{-1}: on
+// exit the lower triangle holds L, the diagonal 1 / L_kk and the upper triangle
+// X^T (X[i][c] at s[c ld + i], c < i).  n is a multiple of 8 (the caller pads
+// with unit diagonal entries) up to 64, ld >= n.
+//
+// Panels of 8 columns.  A panel is factored in registers by up to three warps,
+// a lane per row; each warp repeats the 8 x 8 diagonal part in its lanes 0 .. 7,
+// so the pivot chain needs no barrier, and it runs in the form without square
+// roots (d_k the pivot, c = column / d_k; the columns are scaled by d_k^{-1/2}
+// at the end).  Its rank-8 update is applied to the next panel's columns by
+// all warps, then to the rest in 8 x 8 tiles drawn from a counter while the
+// next panel's chain runs.  X then grows from the 8 x 8 diagonal inverses by
+// doubling, X_21 = -X_22 (L_21 X_11), lanes along the dimension in which the
+// triangular dot products are equally long.
+//
+// What bounds it: FP64, the pipe (n^3/3 multiply-adds, 2 a cycle) and the
+// pivot chain, six dependent instructions of 64 cycles a column; FP32, the
+// chain and the barriers.  The column-by-column sweep with a separate
+// inversion took 90 us (FP64) and 60 us (FP32) for a 64 x 64 block.
+// cbuf: 17 x 64 entries, cnt: 8 integers (shared).  At least four warps.
+// Returns the first failing column + 1, or 0.  All threads call; ends with a
 // barrier.
 template <typename T>
-__device__ void tri_inverse_upper(T *s, int ld, int n) {
-  constexpr int RB = 8;
-  for (int r0 = 0; r0 < n; r0 += RB) {
-    const int rb = min(RB, n - r0);
-    for (int t = threadIdx.x; t < r0 * RB; t += blockDim.x) {
-      const int i = t % RB, c = t / RB;
-      if (i < rb) {
-        const T *lr = s + (r0 + i) * ld, *xc = s + c * ld;  // xc[p] = X[p][c] for p >= c
-        T acc = T(0);
-        for (int p = c; p < r0; ++p) acc = fma(lr[p], xc[p], acc);
-        s[c * ld + r0 + i] = acc;
+__device__ int chol_inverse(T *s, int ld, int n, T *cbuf, int *cnt, int *s_flag) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5, np = n >> 3;
+  T *dv = cbuf + 16 * kMaxN;  // pivots
+  if (threadIdx.x < 8) cnt[threadIdx.x] = 0;
+  if (threadIdx.x == 0) *s_flag = 0;
+  // factor panel p (warps 0 .. 2)
+  auto panel = [&](int p) {
+    const int k0 = 8 * p;
+    T *cb = cbuf + (p & 1) * 8 * kMaxN;
+    if (warp > 2 || (warp > 0 && k0 + 8 + 24 * warp >= n)) return;
+    const int row = lane < 8 ? k0 + lane : k0 + 24 * warp + lane;
+    const bool live = row < n, own = live && (lane >= 8 || warp == 0);
+    T a[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) a[q] = live ? s[row * ld + k0 + q] : T(0);
+    // every warp has read the diagonal rows before warp 0 writes them
+    const int warps = 1 + (k0 + 32 < n) + (k0 + 56 < n);
+    if (warps > 1) asm volatile("bar.sync 2, %0;" ::"r"(32 * warps) : "memory");
+    // The updates of the columns q + 1 .. wait for the reciprocal's steps of
+    // column q: an FP64 instruction holds the pipe as long as its latency, so
+    // each fills the gap before the next step of the chain.
+    T pa = T(0), pc = T(0);  // the column before: its entry and coefficient of this lane's row
+    auto update = [&](int r) {
+      const T cr = __shfl_sync(0xffffffffu, pc, r & 7);
+      if (r < 8) a[r & 7] = fma(-pa, cr, a[r & 7]);
+    };
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      T d = __shfl_sync(0xffffffffu, a[q], q);
+      if (!pivot_ok(d)) {  // the sweep runs on with a harmless pivot
+        if (warp == 0 && lane == 0 && *s_flag == 0) *s_flag = k0 + q + 1;
+        d = T(1);
+      }
+      T y = rcp_seed(d);
+      if (q > 0) update(q + 1);
+      if constexpr (sizeof(T) == 8) {
+        const T e = fma(-d, y, T(1));
+        if (q > 0) update(q + 2);
+        const T f = fma(e, e, e);
+        if (q > 0) update(q + 3);
+        y = fma(y, f, y);
+      } else if (q > 0) {
+        update(q + 2);
+        update(q + 3);
+      }
+      if (q > 0) update(q + 4);
+      const T c = a[q] * y;
+      if (q > 0) {
+        update(q + 5);
+        update(q + 6);
+      }
+      pa = a[q];
+      pc = c;
+      if (q < 7) {  // the next column at once
+        const T cr = __shfl_sync(0xffffffffu, c, q + 1);
+        a[q + 1] = fma(-a[q], cr, a[q + 1]);
+      }
+      if (own) {
+        cb[q * kMaxN + row] = c;
+        if (lane >= q) s[row * ld + k0 + q] = a[q];
+        if (lane == q && warp == 0) dv[k0 + q] = d;
       }
     }
+  };
+  // rank-8 update of tile (R, C) by panel p
+  auto tile = [&](int R, int C, int p) {
+    const int i = 8 * R + (lane >> 2), j = 8 * C + 2 * (lane & 3);
+    const T *x = s + i * ld + 8 * p, *y = cbuf + (p & 1) * 8 * kMaxN + j;
+    T z0 = s[i * ld + j], z1 = s[i * ld + j + 1];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      z0 = fma(-x[q], y[q * kMaxN], z0);
+      z1 = fma(-x[q], y[q * kMaxN + 1], z1);
+    }
+    s[i * ld + j] = z0;
+    s[i * ld + j + 1] = z1;
+  };
+  __syncthreads();
+  panel(0);
+  __syncthreads();
+  for (int p = 0; p + 1 < np; ++p) {
+    for (int R = p + 1 + warp; R < np; R += nw) tile(R, p + 1, p);
+    const int m = np - p - 2, tiles = m * (m + 1) / 2;
     __syncthreads();
-    for (int c = threadIdx.x; c < r0 + rb; c += blockDim.x) {
-      const int cc = c - r0;  // column inside this row block (unit vector) if >= 0
-      T x[RB];
-#pragma unroll
-      for (int i = 0; i < RB; ++i) {
-        x[i] = T(0);
-        if (i < rb && i >= cc) {
-          const T *lr = s + (r0 + i) * ld + r0;
-          T acc = cc < 0 ? s[c * ld + r0 + i] : T(0);
-#pragma unroll
-          for (int q = 0; q < i; ++q) acc = fma(lr[q], x[q], acc);
-          x[i] = (i == cc) ? lr[i] : -acc * lr[i];
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < RB; ++i)
-        if (i < rb && i > cc) s[c * ld + r0 + i] = x[i];
+    panel(p + 1);
+    for (;;) {
+      int t = 0;
+      if (lane == 0) t = atomicAdd(cnt + p, 1);
+      t = __shfl_sync(0xffffffffu, t, 0);
+      if (t >= tiles) break;
+      int a, b;
+      tri_index(t, a, b);
+      tile(p + 2 + a, p + 2 + b, p);
     }
     __syncthreads();
   }
+  // square roots, all at once; columns scaled
+  T *rs = cbuf;
+  if (threadIdx.x < n) rs[threadIdx.x] = rsqrt_pivot(dv[threadIdx.x]);
+  __syncthreads();
+  {
+    const int j = threadIdx.x & (kMaxN - 1);
+    if (j < n) {
+      const T r = rs[j];
+      for (int i = threadIdx.x / kMaxN; i < n; i += blockDim.x / kMaxN)
+        if (i >= j) s[i * ld + j] = i == j ? r : s[i * ld + j] * r;
+    }
+  }
+  __syncthreads();
+  // 8 x 8 diagonal inverses: a lane per column
+  for (int t = warp; t < np; t += nw) {
+    if (lane < 8) {
+      T *b = s + 8 * t * ld + 8 * t;  // this diagonal tile
+      T x[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        T acc = T(0);
+#pragma unroll
+        for (int q = 0; q < i; ++q) acc = fma(b[i * ld + q], x[q], acc);
+        const T r = b[i * ld + i];
+        x[i] = i == lane ? r : i > lane ? -acc * r : T(0);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (i > lane) b[lane * ld + i] = x[i];
+    }
+  }
+  __syncthreads();
+  for (int h = 8; h < n; h *= 2) {
+    const int b0 = 2 * h * (lane / h), e = lane % h;  // this lane's pair of h x h blocks
+    T v[8];
+    // T = L_21 X_11, into the place of X_21^T: column c the same for a warp
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int c = nw * u + (u & 1 ? nw - 1 - warp : warp);
+      if (nw * u < h && c < h && b0 + h + e < n) {
+        const T *lr = s + (b0 + h + e) * ld + b0, *xr = s + (b0 + c) * ld + b0;
+        T acc = T(0);
+        for (int q = c; q < h; ++q) acc = fma(lr[q], xr[q], acc);
+        s[(b0 + c) * ld + b0 + h + e] = acc;
+      }
+    }
+    __syncthreads();
+    // X_21 = -X_22 T: row i the same for a warp
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = nw * u + (u & 1 ? nw - 1 - warp : warp);
+      v[u] = T(0);
+      if (nw * u < h && i < h && b0 + h + i < n) {
+        const T *xc = s + (b0 + h) * ld + b0 + h + i, *tr = s + (b0 + e) * ld + b0 + h;
+        T acc = T(0);
+        for (int q = 0; q <= i; ++q) acc = fma(xc[q * ld], tr[q], acc);
+        v[u] = -acc;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = nw * u + (u & 1 ? nw - 1 - warp : warp);
+      if (nw * u < h && i < h && b0 + h + i < n) s[(b0 + e) * ld + b0 + h + i] = v[u];
+    }
+    __syncthreads();
+  }
+  return *s_flag;
 }
 
 // Warp-cooperative substitutions for a few right-hand sides (n <= 64): lane

@@ -1,28 +1,39 @@
-// Products of FP64 (or FP32) tiles on the tcgen05 tensor cores at their full
-// accuracy, with the operands cut into digits inside the kernel that uses
-// them (nothing of the digits goes to memory).
+// Products of FP64 and FP32 tiles on the tcgen05 tensor cores at their full
+// accuracy, with the operands cut into parts inside the kernel that uses them
+// (nothing of the parts goes to memory).
 //
-// A row of K <= 64 operand entries gets one binary exponent, the largest of
-// its entries, and every entry becomes the signed integer
-//   q = trunc(v 2^-(exponent) 2^F),  F = 62 bits (FP64) or 30 bits (FP32),
-// written in kDig = 8 (4) base-256 digits q = sum_p d_p 256^(kDig-1-p) with
+// FP64.  A row of K <= 64 operand entries gets one binary exponent, the
+// largest of its entries, and every entry becomes the signed integer
+//   q = trunc(v 2^-(exponent) 2^62),
+// written in kDig = 8 base-256 digits q = sum_p d_p 256^(7-p) with
 // -128 <= d_p <= 127 and |d_0| <= 64, each exact in FP16.  The product of two
 // rows is then
-//   sum_k q_a q_b = sum_t 256^(2 kDig - 2 - t) ACC_t,
+//   sum_k q_a q_b = sum_t 256^(14 - t) ACC_t,
 //   ACC_t = sum_{p+q=t} sum_k d_p(a) d_q(b),
-// and only the diagonals t < kDig are formed: the digit pairs left out weigh
-// below 2^-8kDig x 64 x 8, i.e. 2^-57 (2^-25) of the product of the two row
-// maxima at worst and 2^-61 (2^-30) for digits of random sign, beneath the
-// rounding of a chain of 64 FP64 (FP32) multiply-adds.  Every
+// and only the diagonals t < 8 are formed: the digit pairs left out weigh
+// below 2^-64 x 64 x 8, i.e. 2^-57 of the product of the two row maxima at
+// worst and 2^-61 for digits of random sign, beneath the rounding of a chain
+// of 64 FP64 multiply-adds.  Every
 // |ACC_t| <= 2 x 64 x 64 x 128 + (t - 1) x 64 x 128 x 128 < 2^23, so the FP32
 // accumulation of the tensor cores is exact whatever its order.
 //
-// One tcgen05.mma (kind::f16, M = 128) per A digit p and K step of 16 covers
-// the B digits q = 0 .. kDig-1-p of up to 32 B rows at once: the B operand
-// stacks the digits (32 rows each), and its D columns start at 32 p, so the
+// FP32.  An entry is the sum of kDig = 3 BF16 numbers: h, its rounding to a
+// multiple of 2^-8 times the power of two above the row's largest entry, and
+// two roundings of what is left (25 bits or more below the row maximum).  The
+// products of parts p + q <= 2 are summed, each p + q in an accumulator of its
+// own; the ones left out are below 2^-26 of the product of the row maxima.  The
+// tensor cores truncate where they add in FP32, which on sums of 256 BF16
+// products cost three bits against a chain of FP32 multiply-adds; the sum of
+// the products h h is an integer below 2^16 x 64 and exact, and the others'
+// truncation weighs 2^-8 as much.
+//
+// One tcgen05.mma (kind::f16, M = 128) per A part p and K step of 16 covers
+// the B parts q = 0 .. kDig-1-p of up to 32 B rows at once: the B operand
+// stacks the parts (32 rows each), and its D columns start at 32 p, so the
 // pair (p, q) lands on the columns of diagonal p + q.  p = 0 covers every
 // diagonal, so its first K step clears the accumulators.
 #pragma once
+#include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
 #include "bdss_tc.cuh"
@@ -31,7 +42,7 @@ namespace bdss {
 
 template <typename T> struct SliceFmt;
 template <> struct SliceFmt<double> { static constexpr int kDig = 8; };
-template <> struct SliceFmt<float> { static constexpr int kDig = 4; };
+template <> struct SliceFmt<float> { static constexpr int kDig = 3; };
 
 constexpr int kSlRows = 128;             // A rows of a tile (TMEM lanes)
 constexpr int kSlK = 64;                 // K entries of a tile (128 bytes of FP16)
@@ -42,10 +53,6 @@ constexpr int kSlBSlab = kSlCols * 128;  // bytes of one digit of a B tile
 // Exponent field of |v| (0 for zero and subnormals: they count as zero).
 __device__ __forceinline__ int sl_exp(double v) { return (__double2hiint(v) >> 20) & 0x7FF; }
 __device__ __forceinline__ int sl_exp(float v) { return (__float_as_int(v) >> 23) & 0xFF; }
-// The exponent field of infinities and NaN: a row with such an entry poisons
-// every product it takes part in, as a floating-point product would.
-template <typename T> constexpr int kSlPoison = sizeof(T) == 8 ? 0x7FF : 0xFF;
-
 // Biased digits of v under the row exponent field exmax: the byte p from the
 // top is d_p + 128.
 __device__ __forceinline__ unsigned long long sl_biased(double v, int exmax) {
@@ -56,15 +63,6 @@ __device__ __forceinline__ unsigned long long sl_biased(double v, int exmax) {
   m = (ex == 0) ? 0ULL : (m >> (s > 63 ? 63 : s));
   return (b < 0 ? 0ULL - m : m) + 0x8080808080808080ULL;
 }
-__device__ __forceinline__ unsigned sl_biased(float v, int exmax) {
-  const int b = __float_as_int(v);
-  const int ex = (b >> 23) & 0xFF;
-  unsigned m = ((unsigned)(b & 0x7FFFFF) | 0x800000u) << 6;
-  const int s = exmax - ex;
-  m = (ex == 0) ? 0u : (m >> (s > 31 ? 31 : s));
-  return (b < 0 ? 0u - m : m) + 0x80808080u;
-}
-
 // Two digits (bytes lo and hi of each half of c) as FP16 pairs: 0x6400 | b is
 // 1024 + b, and subtracting 1152 leaves d = b - 128, both exact.
 __device__ __forceinline__ void sl_half_pairs(unsigned c, unsigned &lo, unsigned &hi) {
@@ -92,23 +90,37 @@ __device__ __forceinline__ void sl_store2<double>(double v0, double v1, int exma
 #pragma unroll
   for (int p = 0; p < 8; ++p) *reinterpret_cast<unsigned *>(dst + p * stride) = w[p];
 }
+// The BF16 parts of two entries, one pair per part.
+__device__ __forceinline__ void sl_parts(float v0, float v1, int exmax, unsigned (&w)[3]) {
+  // adding 1.5 x 2^23 units rounds to the unit (2^-7 of the row exponent)
+  const float C = __int_as_float((min(exmax + 16, 254) << 23) | 0x400000);
+  float h0 = (v0 + C) - C, h1 = (v1 + C) - C;
+#pragma unroll
+  for (int p = 0; p < 3; ++p) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(h0, h1);
+    w[p] = *reinterpret_cast<const unsigned *>(&h);
+    v0 -= __low2float(h);
+    v1 -= __high2float(h);
+    h0 = v0;
+    h1 = v1;
+  }
+}
 template <>
 __device__ __forceinline__ void sl_store2<float>(float v0, float v1, int exmax, unsigned char *dst, int stride) {
-  const unsigned u0 = sl_biased(v0, exmax), u1 = sl_biased(v1, exmax);
-  unsigned w[4];
-  sl_half_pairs(__byte_perm(u0, u1, 0x7632), w[1], w[0]);
-  sl_half_pairs(__byte_perm(u0, u1, 0x5410), w[3], w[2]);
+  unsigned w[3];
+  sl_parts(v0, v1, exmax, w);
 #pragma unroll
-  for (int p = 0; p < 4; ++p) *reinterpret_cast<unsigned *>(dst + p * stride) = w[p];
+  for (int p = 0; p < 3; ++p) *reinterpret_cast<unsigned *>(dst + p * stride) = w[p];
 }
 
 // Byte offset of 16-byte group g (K entries 8 g .. 8 g + 7) of row r in a
 // 128-byte-swizzled slab.
 __device__ __forceinline__ int sl_off(int r, int g) { return r * 128 + ((g ^ (r & 7)) << 4); }
 
-// D = FP32, A = B = FP16, both K-major, M = 128 x N.
+// D = FP32, A = B = FP16 (FP64 digits) or BF16 (FP32 parts), both K-major, M = 128 x N.
+template <typename T>
 __host__ __device__ constexpr uint32_t sl_idesc(int N) {
-  return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kSlRows >> 4) << 24);
+  return (1u << 4) | (sizeof(T) == 4 ? (1u << 7) | (1u << 10) : 0u) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kSlRows >> 4) << 24);
 }
 
 __device__ __forceinline__ void sl_mma(uint32_t d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
@@ -129,7 +141,7 @@ __device__ __forceinline__ void sl_issue(uint32_t d, const unsigned char *A, con
   const uint64_t ad0 = tc_desc_sw128(A, 0), bd0 = tc_desc_sw128(B, 0);
 #pragma unroll 1
   for (int p = 0; p < kDig; ++p) {
-    const uint32_t idesc = sl_idesc(cols * (kDig - p)), dp = d + (uint32_t)(cols * p);
+    const uint32_t idesc = sl_idesc<T>(cols * (kDig - p)), dp = d + (uint32_t)(cols * p);
     // the start address field counts 16-byte units: a slab is kSlASlab / 16,
     // a K step of 16 FP16 entries 2 of them
     uint64_t ad = ad0 + (uint64_t)(p * (kSlASlab / 16)), bd = bd0;
@@ -200,13 +212,7 @@ __device__ __forceinline__ double sl_value(const float (&c)[8], int exa, int exb
   const unsigned long long bits = ((unsigned long long)(be - 1) << 52) + t;  // a carry of t raises the exponent
   return __longlong_as_double((long long)(bits | (neg ? 0x8000000000000000ULL : 0ULL)));
 }
-// The same for FP32: sum_t ACC_t 256^(3-t) 2^(exa + exb - 288).
-__device__ __forceinline__ float sl_value(const float (&c)[4], int exa, int exb) {
-  const int h01 = sl_int22(c[0]) * 256 + sl_int22(c[1]);
-  const int h23 = sl_int22(c[2]) * 256 + sl_int22(c[3]);
-  const float r = fmaf((float)h01, 65536.0f, (float)h23);
-  if (exa == 0xFF || exb == 0xFF) return __int_as_float(0x7FC00000);
-  return ldexpf(r, exa + exb - 288);
-}
+// The same for FP32: the smaller parts' products first.
+__device__ __forceinline__ float sl_value(const float (&c)[3], int, int) { return c[0] + (c[1] + c[2]); }
 
 }  // namespace bdss

@@ -39,17 +39,17 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_tcf_diag(const __grid_constant__ Args<T> a, const TcfLevel<T> w, int l,
                                                   int fold_all) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int s_flag, s_go;
+  __shared__ int s_flag, s_go, s_cnt[8];
   if (threadIdx.x == 0) s_go = ld_relaxed_i32(&a.st->status) == 0;
   __syncthreads();
   if (!s_go) return;
-  const int n = a.p.n, d = a.d, ld = ldstride(n);
+  const int n = a.p.n, d = a.d, np = (n + 7) & ~7, ld = ldstride(np);
   const size_t nn = (size_t)n * n, nd = (size_t)n * d;
   const long long Nl = a.p.Nl[l], nE = Nl / 2, t = blockIdx.x;
   const bool elim = !fold_all && t < nE;
   const long long j = fold_all ? t : elim ? 2 * t + 1 : 2 * (t - nE);
   const long long orig = j << l;
-  T *s = reinterpret_cast<T *>(smem_raw), *sB = s + (size_t)n * ld;
+  T *s = reinterpret_cast<T *>(smem_raw), *sB = s + (size_t)np * ld, *cbuf = sB + (size_t)d * ld;
   // the eliminated neighbours at level l - 1 are its blocks m = j - 1 (this
   // position is its right separator) and m = j (its left one)
   const bool hasM = l > 0 && j >= 1, hasP = l > 0 && j < a.p.Nl[l > 0 ? l - 1 : 0] / 2;
@@ -83,11 +83,14 @@ __global__ void __launch_bounds__(256) k_tcf_diag(const __grid_constant__ Args<T
   __syncthreads();
   T *Lg = a.Ld + (size_t)orig * nn;
   if (elim) {
-    if (chol_fused(s, ld, n, s, 0, sB, d, &s_flag)) {
+    for (int e = threadIdx.x; e < (np - n) * np; e += blockDim.x) {
+      const int i = n + e / np, c = e % np;
+      if (c <= i) s[i * ld + c] = T(i == c);
+    }
+    if (chol_inverse(s, ld, np, cbuf, s_cnt, &s_flag)) {
       if (threadIdx.x == 0) set_status(a.st, kStNotSPD, l, orig);
       return;
     }
-    tri_inverse_upper(s, ld, n);
     T *Xg = w.X + (size_t)t * nn;
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
       const int i = e / n, c = e - i * n;
@@ -102,8 +105,16 @@ __global__ void __launch_bounds__(256) k_tcf_diag(const __grid_constant__ Args<T
     }
   }
   for (int e = threadIdx.x; e < n * d; e += blockDim.x) {
-    const int i = e / d, c = e - i * d;
-    a.Y[(size_t)orig * nd + e] = sB[c * ld + i];
+    if (elim) {  // y = L^{-1} b, threads along the rows: X[i][q] is s[q ld + i]
+      const int c = e / n, i = e - c * n;
+      const T *b = sB + c * ld;
+      T v = T(0);
+      for (int q = 0; q <= i; ++q) v = fma(s[q * ld + i], b[q], v);
+      a.Y[(size_t)orig * nd + (size_t)i * d + c] = v;
+    } else {
+      const int i = e / d, c = e - i * d;
+      a.Y[(size_t)orig * nd + e] = sB[c * ld + i];
+    }
   }
 }
 
@@ -449,7 +460,8 @@ __global__ void __launch_bounds__(kSchurThreads, 1)
   if (warp == 0) tmem_dealloc(tmem, kTmemAll);
 }
 
-size_t diag_smem(int n, int d, size_t esz) { return ((size_t)(n + d) * ldstride(n) + 8) * esz; }
+size_t diag_smem(int n, int d, size_t esz) { const int np = (n + 7) & ~7;
+  return ((size_t)(np + d) * ldstride(np) + 17 * kMaxN) * esz; }
 
 }  // namespace
 

@@ -21,23 +21,12 @@
 // diagonal), where a diagonal tile keeps X_kk^T above its diagonal for the
 // downward pass.
 #include "bdss_launch.h"
-#include "bdss_slice.cuh"
+#include "bdss_slice_cta.cuh"
 #include "bdss_wide.h"
 
 namespace bdss {
 
 namespace {
-
-constexpr int kWdThreads = 512;
-constexpr int kWdWarps = kWdThreads / 32;
-constexpr int kWdTile = 64;  // rows of a slot, columns of an output tile
-template <typename T> constexpr int kWdStageRow = sizeof(T) == 8 ? 48 : 16;  // bytes of a staged output row
-template <typename T> constexpr uint32_t kWdBufCols = SliceFmt<T>::kDig * kSlCols;  // accumulators of 32 columns
-template <typename T> constexpr uint32_t kWdTmem = 2 * kWdBufCols<T>;
-template <typename T> constexpr int kWdBBytes = SliceFmt<T>::kDig * kSlBSlab;
-template <typename T> constexpr size_t wd_smem() {
-  return (size_t)SliceFmt<T>::kDig * (kSlASlab + 2 * kSlBSlab) + (size_t)kWdWarps * 32 * kWdStageRow<T> + 1024;
-}
 
 // Panels: equal widths rounded up to 8 columns, so that the diagonal tiles'
 // pivot chains, which are the critical path, are equally long.
@@ -51,38 +40,14 @@ __host__ __device__ inline WidePanels panels_of(int n) {
 template <typename T>
 struct Slot {
   T *p;
-  long long rs, cs;
+  int rs, cs;
   int rows;
+  int q = -1;  // >= 0: unit rows, the q-th block row of the identity (zero before column q nb)
 };
 
 template <typename T>
 __device__ __forceinline__ Slot<T> no_slot() {
   return {nullptr, 0, 0, 0};
-}
-
-template <typename T>
-struct WdCta {
-  unsigned char *A, *B, *stage;  // digit slabs, this warp's output stage
-  uint32_t tmem;
-  uint64_t *bar;
-  int *exA, *exB, *exP, *s_ok;   // row exponents: A (128), B (64), partial (4 x 128)
-  uint32_t ph;
-  long long timeout_ns;
-};
-
-template <typename T>
-__device__ __forceinline__ void load2(const T *p, T &x, T &y);
-template <>
-__device__ __forceinline__ void load2<double>(const double *p, double &x, double &y) {
-  const double2 v = __ldcg(reinterpret_cast<const double2 *>(p));
-  x = v.x;
-  y = v.y;
-}
-template <>
-__device__ __forceinline__ void load2<float>(const float *p, float &x, float &y) {
-  const float2 v = __ldcg(reinterpret_cast<const float2 *>(p));
-  x = v.x;
-  y = v.y;
 }
 
 // Digits of the K columns [0, kc) of the slots a0, a1 (A rows 0 .. 63, 64 ..
@@ -99,7 +64,7 @@ __device__ __forceinline__ void wd_cut(const WdCta<T> &w, const Slot<T> &a0, con
     const int r = (u & 3) * kWdWarps + warp;
     v[u][0] = v[u][1] = T(0);
     if ((u < 8 ? do_a : do_b) && r < s.rows && k < kc) {
-      const T *p = s.p + (long long)r * s.rs + (long long)k * s.cs;
+      const T *p = s.p + (r * s.rs + k * s.cs);
       if (pairs && s.cs == 1) {
         load2(p, v[u][0], v[u][1]);
       } else {
@@ -125,193 +90,12 @@ __device__ __forceinline__ void wd_cut(const WdCta<T> &w, const Slot<T> &a0, con
   }
 }
 
-// Eight consecutive K entries of one row -> 16 bytes of every digit slab.
+// Slot i of the rows below panel k of block j (the level's m-th): block rows
+// k + 1 .. of D, then W_L, W_R, the right-hand sides and, where L^{-1} is
+// wanted, the first k block rows of the identity, which become L^{-T}.
 template <typename T>
-__device__ __forceinline__ void store8(const T *v, int ex, unsigned char *dst, int stride);
-template <>
-__device__ __forceinline__ void store8<double>(const double *v, int ex, unsigned char *dst, int stride) {
-  unsigned w[4][8];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const unsigned long long u0 = sl_biased(v[2 * i], ex), u1 = sl_biased(v[2 * i + 1], ex);
-    const unsigned h0 = (unsigned)(u0 >> 32), h1 = (unsigned)(u1 >> 32), l0 = (unsigned)u0, l1 = (unsigned)u1;
-    sl_half_pairs(__byte_perm(h0, h1, 0x7632), w[i][1], w[i][0]);
-    sl_half_pairs(__byte_perm(h0, h1, 0x5410), w[i][3], w[i][2]);
-    sl_half_pairs(__byte_perm(l0, l1, 0x7632), w[i][5], w[i][4]);
-    sl_half_pairs(__byte_perm(l0, l1, 0x5410), w[i][7], w[i][6]);
-  }
-#pragma unroll
-  for (int p = 0; p < 8; ++p)
-    *reinterpret_cast<uint4 *>(dst + p * stride) = make_uint4(w[0][p], w[1][p], w[2][p], w[3][p]);
-}
-template <>
-__device__ __forceinline__ void store8<float>(const float *v, int ex, unsigned char *dst, int stride) {
-  unsigned w[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const unsigned u0 = sl_biased(v[2 * i], ex), u1 = sl_biased(v[2 * i + 1], ex);
-    sl_half_pairs(__byte_perm(u0, u1, 0x7632), w[i][1], w[i][0]);
-    sl_half_pairs(__byte_perm(u0, u1, 0x5410), w[i][3], w[i][2]);
-  }
-#pragma unroll
-  for (int p = 0; p < 4; ++p)
-    *reinterpret_cast<uint4 *>(dst + p * stride) = make_uint4(w[0][p], w[1][p], w[2][p], w[3][p]);
-}
-
-// The A rows from registers: this thread's 16 columns of its row.  Contains
-// CTA barriers.
-template <typename T>
-__device__ __forceinline__ void wd_cut_regs(const WdCta<T> &w, const T (&v)[16], int row, int hw) {
-  int ex = 0;
-#pragma unroll
-  for (int i = 0; i < 16; ++i) ex = max(ex, sl_exp(v[i]));
-  w.exP[hw * kSlRows + row] = ex;
-  __syncthreads();
-#pragma unroll
-  for (int q = 0; q < 4; ++q) ex = max(ex, w.exP[q * kSlRows + row]);
-  if (hw == 0) w.exA[row] = ex;
-#pragma unroll
-  for (int i = 0; i < 2; ++i) store8<T>(v + 8 * i, ex, w.A + sl_off(row, 2 * hw + i), kSlASlab);
-}
-
-// The product of the cut operands, waited for.  cols2: the second 32 columns
-// as well; ks0 / ks1: K steps of either column tile.  False after a timeout.
-template <typename T>
-__device__ __forceinline__ bool wd_product(WdCta<T> &w, bool cols2, int ks0, int ks1) {
-  // every thread's operands before the products that read them, its TMEM
-  // reads before the products that overwrite them
-  fence_proxy_async_smem();
-  tc_fence_before();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    tc_fence_after();
-    sl_issue<T>(w.tmem, w.A, w.B, kSlCols, ks0);
-    if (cols2) sl_issue<T>(w.tmem + kWdBufCols<T>, w.A, w.B + kWdBBytes<T>, kSlCols, ks1);
-    tc_commit(w.bar);
-  }
-  if (!mbar_wait_cta(w.bar, w.ph, w.timeout_ns, w.s_ok)) {
-    // wait again (bounded) for the products in flight before TMEM is freed
-    mbar_wait_cta(w.bar, w.ph, w.timeout_ns, w.s_ok);
-    return false;
-  }
-  w.ph ^= 1;
-  tc_fence_after();
-  return true;
-}
-
-// Four columns of the product from TMEM address `at`, as values.
-template <typename T>
-__device__ __forceinline__ void wd_drain4(uint32_t at, int ea, const int *exb, T (&v)[4]) {
-  constexpr int kDig = SliceFmt<T>::kDig;
-  uint32_t acc[kDig][4];
-#pragma unroll
-  for (int q = 0; q < kDig; ++q) tmem_ld4(at + (uint32_t)(q * kSlCols), acc[q]);
-  tmem_ld_wait();
-#pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    float f[kDig];
-#pragma unroll
-    for (int q = 0; q < kDig; ++q) f[q] = __uint_as_float(acc[q][e]);
-    v[e] = sl_value(f, ea, exb[e]);
-  }
-}
-
-// Four columns of a warp's 32 rows to memory through the warp's stage, in
-// 16-byte pieces where rows allow it.  dst: the warp's first row, first
-// column; rows / cols: how many of them exist.  sub: subtract from what is
-// there instead.
-template <typename T>
-__device__ __forceinline__ void wd_store4(unsigned char *stage, const T (&v)[4], T *dst, long long ld, int rows,
-                                          int cols, bool segs, bool sub) {
-  constexpr int kPiece = 16 / sizeof(T), PR = 4 / kPiece;
-  const int lane = threadIdx.x & 31;
-  __syncwarp();
-#pragma unroll
-  for (int e = 0; e < PR; ++e)
-    *reinterpret_cast<uint4 *>(stage + lane * kWdStageRow<T> + 16 * e) = *reinterpret_cast<const uint4 *>(v + e * kPiece);
-  __syncwarp();
-  if (segs) {
-#pragma unroll
-    for (int u = 0; u < PR; ++u) {
-      const int rr = (32 / PR) * u + lane / PR, pc = lane % PR;
-      uint4 x = *reinterpret_cast<const uint4 *>(stage + rr * kWdStageRow<T> + 16 * pc);
-      if (rr < rows && pc * kPiece < cols) {
-        uint4 *at = reinterpret_cast<uint4 *>(dst + rr * ld + pc * kPiece);
-        if (sub) {
-          uint4 o = __ldcg(at);
-          T *ov = reinterpret_cast<T *>(&o);
-          const T *xv = reinterpret_cast<const T *>(&x);
-#pragma unroll
-          for (int i = 0; i < kPiece; ++i) ov[i] -= xv[i];
-          x = o;
-        }
-        *at = x;
-      }
-    }
-  } else {
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int rr = 8 * u + (lane >> 2), c = lane & 3;
-      const T x = *reinterpret_cast<const T *>(stage + rr * kWdStageRow<T> + c * sizeof(T));
-      if (rr < rows && c < cols) {
-        T *at = dst + rr * ld + c;
-        *at = sub ? ldcg(at) - x : x;
-      }
-    }
-  }
-}
-
-// Set up and release of the CTA's tensor-core state.  All threads call.
-template <typename T>
-__device__ __forceinline__ void wd_begin(WdCta<T> &w, unsigned char *smem_raw, uint64_t *bar, uint32_t *s_tmem,
-                                         int *exA, int *exB, int *exP, int *s_ok, long long timeout_ns) {
-  w.A = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  w.B = w.A + (size_t)SliceFmt<T>::kDig * kSlASlab;
-  w.stage = w.B + 2 * kWdBBytes<T> + (threadIdx.x >> 5) * 32 * kWdStageRow<T>;
-  w.bar = bar;
-  w.exA = exA;
-  w.exB = exB;
-  w.exP = exP;
-  w.s_ok = s_ok;
-  w.ph = 0;
-  w.timeout_ns = timeout_ns;
-  if (threadIdx.x == 0) {
-    mbar_init(bar, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (threadIdx.x < 32) tmem_alloc(s_tmem, kWdTmem<T>);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  w.tmem = *s_tmem;
-}
-template <typename T>
-__device__ __forceinline__ void wd_end(const WdCta<T> &w) {
-  tc_fence_before();
-  __syncthreads();
-  if (threadIdx.x < 32) tmem_dealloc(w.tmem, kWdTmem<T>);
-}
-
-#define WD_CTA_SETUP(T)                                                                                   \
-  extern __shared__ __align__(16) unsigned char smem_raw[];                                               \
-  __shared__ uint64_t s_bar;                                                                              \
-  __shared__ uint32_t s_tmem;                                                                             \
-  __shared__ int s_ok, s_go, s_exA[kSlRows], s_exB[kWdTile], s_exP[4 * kSlRows];                          \
-  if (threadIdx.x == 0) s_go = ld_relaxed_i32(&a.st->status) == 0;                                        \
-  __syncthreads();                                                                                        \
-  if (!s_go) return;                                                                                      \
-  WdCta<T> w;                                                                                             \
-  wd_begin(w, smem_raw, &s_bar, &s_tmem, s_exA, s_exB, s_exP, &s_ok, a.timeout_ns);                       \
-  /* this thread drains row `row` (slot row >> 6), 16 columns from 16 hw */                               \
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, hw = warp >> 2, row0 = 32 * (warp & 3),     \
-            row = row0 + lane;                                                                            \
-  const uint32_t lane_base = w.tmem + ((uint32_t)row0 << 16);                                             \
-  const uint32_t acc16 = lane_base + (uint32_t)(hw >> 1) * kWdBufCols<T> + (uint32_t)(16 * (hw & 1));
-
-// Slot i of the rows below panel k of block j: block rows k + 1 .. of D, then
-// W_L, W_R and the right-hand sides.
-template <typename T>
-__device__ __forceinline__ Slot<T> panel_slot(const Args<T> &a, const WidePanels &P, int l, long long j, int k, int i) {
+__device__ __forceinline__ Slot<T> panel_slot(const Args<T> &a, const WideBuf<T> &wb, const WidePanels &P, int l,
+                                              long long j, long long m, int k, int i) {
   const int n = a.p.n;
   const size_t nn = (size_t)n * n;
   const long long orig = j << l;
@@ -326,12 +110,14 @@ __device__ __forceinline__ Slot<T> panel_slot(const Args<T> &a, const WidePanels
     if (side && j + 1 >= a.p.Nl[l]) return no_slot<T>();
     return {a.Wb + (size_t)(a.p.off[l] + j - 1 + side) * nn + (size_t)q * P.nb * n, n, 1, min(P.nb, n - q * P.nb)};
   }
-  if (i == 2 * nW && a.d > 0) return {a.Y + (size_t)orig * n * a.d, 1, a.d, a.d};
+  i -= 2 * nW;
+  if (a.d > 0 && i-- == 0) return {a.Y + (size_t)orig * n * a.d, 1, a.d, a.d};
+  if (wb.Li && i < k) return {wb.V + (size_t)m * nn + (size_t)i * P.nb * n, n, 1, P.nb, i};
   return no_slot<T>();
 }
 // Slots of a panel: the D rows alone are the last panel's ones without couplings.
-__host__ __device__ inline int panel_slots(const WidePanels &P, bool couplings, int k, int d) {
-  return P.nt - 1 - k + (couplings ? 2 * P.nt : 0) + (d > 0 ? 1 : 0);
+__host__ __device__ inline int panel_slots(const WidePanels &P, bool couplings, int k, int d, bool inverse) {
+  return P.nt - 1 - k + (couplings ? 2 * P.nt : 0) + (d > 0 ? 1 : 0) + (inverse ? k : 0);
 }
 
 template <typename T>
@@ -342,14 +128,14 @@ __global__ void __launch_bounds__(kWdThreads, sizeof(T) == 8 ? 1 : 2)
   const WidePanels P = panels_of(n);
   const bool top = l == a.p.L;
   const long long nE = top ? 1 : a.p.Nl[l] / 2;
-  const int tiles = (panel_slots(P, !top, k, a.d) + 1) / 2;
+  const int tiles = (panel_slots(P, !top, k, a.d, wb.Li != nullptr) + 1) / 2;
   const bool pairs = (n & 1) == 0, segs = ((n * (int)sizeof(T)) & 15) == 0;
   const int kb = min(P.nb, n - k * P.nb);  // columns of this panel
   bool ok = true;
   for (long long t = blockIdx.x; t < nE * tiles && ok; t += gridDim.x) {
     const long long m = t / tiles, j = top ? 0 : 2 * m + 1;
     const int i0 = 2 * (int)(t - m * tiles);
-    const Slot<T> s0 = panel_slot(a, P, l, j, k, i0), s1 = panel_slot(a, P, l, j, k, i0 + 1);
+    const Slot<T> s0 = panel_slot(a, wb, P, l, j, m, k, i0), s1 = panel_slot(a, wb, P, l, j, m, k, i0 + 1);
     if (s0.rows == 0 && s1.rows == 0) continue;
     const int nD = P.nt - 1 - k - i0;  // this tile's slots of D
     const T *Lk = a.Ld + ((size_t)(j << l) * n + (size_t)k * P.nb) * n;
@@ -361,18 +147,22 @@ __global__ void __launch_bounds__(kWdThreads, sizeof(T) == 8 ? 1 : 2)
       const int c0 = rd < k ? rd * P.nb : k * P.nb;  // the chunk's first column
       if (rd <= k) {
         Slot<T> c_0 = s0, c_1 = s1;
-        c_0.p += (long long)c0 * s0.cs;
-        c_1.p += (long long)c0 * s1.cs;
+        c_0.p += c0 * s0.cs;
+        c_1.p += c0 * s1.cs;
+        if (rd < s0.q) c_0.rows = 0;
+        if (rd < s1.q) c_1.rows = 0;
         Slot<T> b = rd < k ? Slot<T>{const_cast<T *>(Lk) + c0, n, 1, kb}
                            : Slot<T>{wb.X + (size_t)m * kWdTile * kWdTile, kWdTile, 1, kWdTile};
         wd_cut<T>(w, c_0, c_1, b, rd < k || k == 0, true, rd < k ? P.nb : kb, pairs);
       }
       if ((rd == k && k > 0) || rd == k + 1) {
         if (rd == k) {  // S - sum of the products
-          const T *src = mine.p + (long long)r * mine.rs + (long long)(k * P.nb + 16 * hw) * mine.cs;
+          const T *src = mine.p + (r * mine.rs + (k * P.nb + 16 * hw) * mine.cs);
 #pragma unroll
           for (int i = 0; i < 16; ++i)
-            acc[i] = (r < mine.rows && 16 * hw + i < kb) ? ldcg(src + i * mine.cs) - acc[i] : T(0);
+            acc[i] = mine.q >= 0                             ? -acc[i]
+                     : r < mine.rows && 16 * hw + i < kb ? ldcg(src + i * mine.cs) - acc[i]
+                                                         : T(0);
         }
         wd_cut_regs<T>(w, acc, row, hw);
         if (rd == k + 1) __syncthreads();
@@ -407,12 +197,18 @@ __global__ void __launch_bounds__(kWdThreads, sizeof(T) == 8 ? 1 : 2)
             if (rd == k) {
               const int col = k * P.nb + 16 * hw + c;
               if (mine.cs == 1) {
-                wd_store4<T>(w.stage, v, mine.p + (long long)(row0 & 63) * mine.rs + col, mine.rs, wrows,
+                wd_store4<T>(w.stage, v, mine.p + (row0 & 63) * mine.rs + col, mine.rs, wrows,
                              kb - 16 * hw - c, segs, false);
+                if (mine.q >= 0 && r < mine.rows) {  // L^{-1}: a warp's rows are consecutive columns
+                  T *o = wb.Li + (size_t)(j << l) * n * n + (size_t)col * n + mine.q * P.nb + r;
+#pragma unroll
+                  for (int e = 0; e < 4; ++e)
+                    if (16 * hw + c + e < kb) o[(size_t)e * n] = v[e];
+                }
               } else if (r < mine.rows) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
-                  if (16 * hw + c + e < kb) mine.p[(long long)(col + e) * mine.cs + r * mine.rs] = v[e];
+                  if (16 * hw + c + e < kb) mine.p[(col + e) * mine.cs + r * mine.rs] = v[e];
               }
             }
           } else {
@@ -431,7 +227,7 @@ __global__ void __launch_bounds__(kWdThreads, sizeof(T) == 8 ? 1 : 2)
             wd_drain4<T>(lane_base + (uint32_t)(row >> 6) * kWdBufCols<T> + (uint32_t)(8 * hw + c), ea,
                          w.exA + (row & 64) + col, v);
             const int ib = k + 1 + i0 + (row >> 6);
-            wd_store4<T>(w.stage, v, mine.p + (long long)(row0 & 63) * mine.rs + ib * P.nb + col, mine.rs, wrows,
+            wd_store4<T>(w.stage, v, mine.p + (row0 & 63) * mine.rs + ib * P.nb + col, mine.rs, wrows,
                          mine.rows - col, segs, true);
           }
         }
@@ -565,34 +361,66 @@ template <typename T>
 __global__ void __launch_bounds__(kDiagThreads) k_wide_diag(const __grid_constant__ Args<T> a, const WideBuf<T> wb,
                                                            int l, int k) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int s_flag, s_go;
+  __shared__ int s_flag, s_go, s_cnt[8];
   if (threadIdx.x == 0) s_go = ld_relaxed_i32(&a.st->status) == 0;
   __syncthreads();
   if (!s_go) return;
   const int n = a.p.n;
   const WidePanels P = panels_of(n);
-  const int kb = min(P.nb, n - k * P.nb), ld = ldstride(kb);
+  const int kb = min(P.nb, n - k * P.nb), kp = (kb + 7) & ~7, ld = ldstride(kp);
   const long long m = blockIdx.x, orig = (l == a.p.L ? 0 : 2 * m + 1) << l;
-  T *s = reinterpret_cast<T *>(smem_raw);
+  T *s = reinterpret_cast<T *>(smem_raw), *cbuf = s + (size_t)kp * ld;
   T *Lg = a.Ld + (size_t)orig * n * n + ((size_t)k * P.nb) * n + k * P.nb;
-  for (int e = threadIdx.x; e < kb * kb; e += blockDim.x) {
-    const int i = e / kb, c = e - i * kb;
-    if (c <= i) s[i * ld + c] = ldcg(Lg + (size_t)i * n + c);
+  // a thread takes a column of the tile, every fourth row
+  const int c = threadIdx.x & (kWdTile - 1), i0 = threadIdx.x / kWdTile;
+  constexpr int kStep = kDiagThreads / kWdTile;
+#pragma unroll
+  for (int u = 0; u < kWdTile / kStep; ++u) {
+    const int i = i0 + u * kStep;
+    if (i < kp && c <= i) s[i * ld + c] = i < kb ? ldcg(Lg + (size_t)i * n + c) : T(i == c);
   }
-  __syncthreads();
-  if (chol_fused(s, ld, kb, s, 0, s, 0, &s_flag)) {
+  if (chol_inverse(s, ld, kp, cbuf, s_cnt, &s_flag)) {
     if (threadIdx.x == 0) set_status(a.st, kStNotSPD, l, orig);
     return;
   }
-  tri_inverse_upper(s, ld, kb);
   T *Xg = wb.X + (size_t)m * kWdTile * kWdTile;
-  for (int e = threadIdx.x; e < kWdTile * kWdTile; e += blockDim.x) {
-    const int i = e / kWdTile, c = e - i * kWdTile;
-    Xg[e] = (c <= i && i < kb) ? s[c * ld + i] : T(0);  // X[i][c] is in the upper triangle
+  // L^{-1}: the tile, zeros to its right; the same tile of L^{-T}
+  const int k0 = k * P.nb;
+  T *Li = wb.Li + (size_t)orig * n * n + (size_t)k0 * n + k0, *V = wb.V + (size_t)m * n * n + (size_t)k0 * n + k0;
+#pragma unroll 4
+  for (int u = 0; u < kWdTile / kStep; ++u) {
+    const int i = i0 + u * kStep;
+    const bool in = i < kb && c < kb;
+    const T x = in && c <= i ? s[c * ld + i] : T(0);  // X[i][c] is in the upper triangle
+    Xg[i * kWdTile + c] = x;
+    if (in) {
+      Lg[(size_t)i * n + c] = s[i * ld + c];
+      if (wb.Li) V[(size_t)i * n + c] = i <= c ? s[i * ld + c] : T(0);
+    }
+    if (wb.Li && i < kb)
+      for (int z = c; z < n - k0; z += kWdTile) Li[(size_t)i * n + z] = z == c && in ? x : T(0);
   }
-  for (int e = threadIdx.x; e < kb * kb; e += blockDim.x) {
-    const int i = e / kb, c = e - i * kb;
-    Lg[(size_t)i * n + c] = s[i * ld + c];
+}
+
+// The FP64 top block of an FP32 factorisation: D_0 (lower) and b_0 to FP64.
+__global__ void __launch_bounds__(256) k_wide_top_in(const __grid_constant__ Args<float> a, double *D, double *y) {
+  const int n = a.p.n;
+  for (int e = blockIdx.x * 256 + threadIdx.x; e < n * n; e += gridDim.x * 256) D[e] = e % n <= e / n ? (double)ldcg(a.Ld + e) : 0.0;
+  for (int e = blockIdx.x * 256 + threadIdx.x; e < n * a.d; e += gridDim.x * 256) y[e] = (double)ldcg(a.Y + e);
+}
+// Its results: float(L) and float(L^{-1}) for the solve passes, x_0.
+__global__ void __launch_bounds__(256) k_wide_top_out(const __grid_constant__ Args<float> a, const double *Li,
+                                                      const double *x) {
+  if (ld_relaxed_i32(&a.st->status) != 0) return;
+  const int n = a.p.n;
+  for (int e = blockIdx.x * 256 + threadIdx.x; e < n * n; e += gridDim.x * 256) {
+    a.Ltinv[e] = e % n <= e / n ? (float)__ldcg(a.Ltop + e) : 0.0f;
+    a.Ltinv[n * n + e] = (float)__ldcg(Li + e);
+  }
+  for (int e = blockIdx.x * 256 + threadIdx.x; e < n * a.d; e += gridDim.x * 256) {
+    const double v = __ldcg(x + e);
+    a.Y[e] = (float)v;
+    if (a.X64) a.X64[e] = a.x_accumulate ? a.X64[e] + v : v;
   }
 }
 
@@ -808,7 +636,7 @@ cudaError_t launch_wide_ingest(const Args<T> &a, int sms, cudaStream_t s) {
 template <typename T>
 cudaError_t launch_wide_diag(const Args<T> &a, const WideBuf<T> &w, int l, int k, cudaStream_t s) {
   const long long nE = l == a.p.L ? 1 : a.p.Nl[l] / 2;
-  const size_t smem = (size_t)kWdTile * ldstride(kWdTile) * sizeof(T);
+  const size_t smem = ((size_t)kWdTile * ldstride(kWdTile) + 17 * kMaxN) * sizeof(T);
   k_wide_diag<T><<<(unsigned)nE, kDiagThreads, smem, s>>>(a, w, l, k);
   return cudaGetLastError();
 }
@@ -817,7 +645,7 @@ template <typename T>
 cudaError_t launch_wide_panel(const Args<T> &a, const WideBuf<T> &w, int l, int k, int sms, cudaStream_t s) {
   const WidePanels P = panels_of(a.p.n);
   const bool top = l == a.p.L;
-  const long long tasks = (top ? 1 : a.p.Nl[l] / 2) * ((panel_slots(P, !top, k, a.d) + 1) / 2);
+  const long long tasks = (top ? 1 : a.p.Nl[l] / 2) * ((panel_slots(P, !top, k, a.d, w.Li != nullptr) + 1) / 2);
   if (tasks == 0) return cudaSuccess;  // the last panel of the top block without right-hand sides
   k_wide_panel<T><<<wd_grid(tasks, sizeof(T) == 8 ? sms : 2 * sms), kWdThreads, wd_smem<T>(), s>>>(a, w, l, k);
   return cudaGetLastError();
@@ -830,6 +658,15 @@ cudaError_t launch_wide_schur(const Args<T> &a, int l, int sms, cudaStream_t s) 
   return cudaGetLastError();
 }
 
+cudaError_t launch_wide_top_in(const Args<float> &a, double *D, double *y, cudaStream_t s) {
+  k_wide_top_in<<<64, 256, 0, s>>>(a, D, y);
+  return cudaGetLastError();
+}
+cudaError_t launch_wide_top_out(const Args<float> &a, const double *Li, const double *x, cudaStream_t s) {
+  k_wide_top_out<<<64, 256, 0, s>>>(a, Li, x);
+  return cudaGetLastError();
+}
+
 template <typename T>
 cudaError_t launch_wide_down(const Args<T> &a, int l, cudaStream_t s) {
   const long long nE = l == a.p.L ? 1 : a.p.Nl[l] / 2;
@@ -838,14 +675,15 @@ cudaError_t launch_wide_down(const Args<T> &a, int l, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-#define BDSS_WIDE_INSTANTIATE(T)                                                                                   \
-  template size_t wide_x_bytes<T>(long long);                                                                     \
-  template cudaError_t wide_configure<T>();                                                                       \
-  template cudaError_t launch_wide_ingest<T>(const Args<T> &, int, cudaStream_t);                                 \
-  template cudaError_t launch_wide_diag<T>(const Args<T> &, const WideBuf<T> &, int, int, cudaStream_t);          \
-  template cudaError_t launch_wide_panel<T>(const Args<T> &, const WideBuf<T> &, int, int, int, cudaStream_t);    \
-  template cudaError_t launch_wide_schur<T>(const Args<T> &, int, int, cudaStream_t);                             \
-  template cudaError_t launch_wide_down<T>(const Args<T> &, int, cudaStream_t);
+#define BDSS_WIDE_INSTANTIATE(T)                                                                                  \
+  template size_t wide_x_bytes<T>(long long);                                                                    \
+  template cudaError_t wide_configure<T>();                                                                      \
+  template cudaError_t launch_wide_ingest<T>(const Args<T> &, int, cudaStream_t);                                \
+  template cudaError_t launch_wide_diag<T>(const Args<T> &, const WideBuf<T> &, int, int, cudaStream_t);         \
+  template cudaError_t launch_wide_panel<T>(const Args<T> &, const WideBuf<T> &, int, int, int, cudaStream_t);   \
+  template cudaError_t launch_wide_schur<T>(const Args<T> &, int, int, cudaStream_t);
 BDSS_WIDE_INSTANTIATE(double)
+BDSS_WIDE_INSTANTIATE(float)
+template cudaError_t launch_wide_down<double>(const Args<double> &, int, cudaStream_t);
 
 }  // namespace bdss

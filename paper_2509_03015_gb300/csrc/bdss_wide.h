@@ -16,6 +16,9 @@ WidePanels wide_panels(int n);
 template <typename T>
 struct WideBuf {
   T *X;  // [m][64][64]: inverse of the current panel's diagonal tile, per eliminated block of the level
+  // both or neither (FP32, whose solve passes stream L^{-1}):
+  T *Li;  // L^{-1} of every eliminated block (slot of its original index), zero above the diagonal
+  T *V;   // [m][n][n]: L^{-T} of the level's blocks, as far as formed
 };
 
 // Bytes of WideBuf::X for a system of N blocks.
@@ -31,6 +34,10 @@ template <typename T>
 cudaError_t launch_wide_panel(const Args<T> &a, const WideBuf<T> &w, int l, int k, int sms, cudaStream_t s);
 // The separators' D, the next level's couplings and the separators' b.
 template <typename T> cudaError_t launch_wide_schur(const Args<T> &a, int l, int sms, cudaStream_t s);
+// The top block of an FP32 factorisation is factored in FP64: D_0 and b_0 (in
+// a.Y) to FP64; its factor (a.Ltop), inverse and solution back.
+cudaError_t launch_wide_top_in(const Args<float> &a, double *D, double *y, cudaStream_t s);
+cudaError_t launch_wide_top_out(const Args<float> &a, const double *Li, const double *x, cudaStream_t s);
 // Downward pass of level l.
 template <typename T> cudaError_t launch_wide_down(const Args<T> &a, int l, cudaStream_t s);
 

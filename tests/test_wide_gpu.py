@@ -81,3 +81,21 @@ def test_bad_pivot_is_reported(what):
     assert e.value.status == 2
     if what == "not_spd":
         assert e.value.info.block == 6 and e.value.info.level == 1
+
+
+# FP32 factors refined to a backward error of 1e-14 (the call fails otherwise);
+# kappa(A) below 1e3 then bounds the forward error by 1e-11.  Shapes whose
+# inverse is streamed and shapes (n % 4, d > 16) whose is not; N = 1: the FP64
+# top block alone.
+@pytest.mark.parametrize("N,n,d", [(1, 100, 2), (2, 65, 1), (3, 66, 3), (5, 128, 16), (6, 132, 17), (9, 193, 2),
+                                   (4, 256, 1), (17, 256, 16)])
+def test_mixed_precision_matches_oracle(oracle_mod, N, n, d):
+    s = inputs.random_btd(N, n, d, seed=800 + N + n)
+    X, X2, ld = _solve(s, precision="fp32_ir")
+    Xo = oracle_mod.solve_system(s["A_diag"], s["A_sub"], s["B"])
+    for x in (X, X2):
+        assert oracle_mod.forward_error(x, Xo) <= 1e-11
+        assert oracle_mod.backward_error(s["A_diag"], s["A_sub"], x, s["B"]) <= 1e-14
+    L, _ = oracle_mod.factor(s["A_diag"], s["A_sub"])
+    # each of the N n pivots' logarithms is within a few FP32 roundings
+    assert abs(ld - oracle_mod.logdet(L)) <= N * n * 2.0 ** -20
