@@ -1480,22 +1480,29 @@ bdss_status bdss_kalman_assemble(int64_t N, int32_t n, int32_t m, int32_t rinv_d
   a.A_diag = A_diag;
   a.A_sub = N > 1 ? A_sub : nullptr;
   a.B = B;
-  const size_t words = (size_t)N * ((size_t)m * n + m + n);
+  const size_t words = (size_t)N * ((size_t)m * n + m + n), bytes = words * sizeof(double) + sizeof(DevStatus);
+  int dev = 0, sms = 0, status = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return cuda_fail(cudaGetLastError());
   void *ws = nullptr;
   t_alloc_count = 0;
-  if (inject_alloc_failure() || cudaMallocAsync(&ws, words * sizeof(double), s) != cudaSuccess) {
+  if (inject_alloc_failure() || cudaMallocAsync(&ws, bytes, s) != cudaSuccess) {
     cudaGetLastError();
     return BDSS_ERR_ALLOC;
   }
   a.U = static_cast<double *>(ws);
   a.v = a.U + (size_t)N * m * n;
   a.w = a.v + (size_t)N * m;
-  cudaError_t e = launch_kalman_assemble(a, s);
+  DevStatus *st = reinterpret_cast<DevStatus *>(a.v + (size_t)N * (m + n));
+  cudaError_t e = cudaMemsetAsync(st, 0, kStatusCoreBytes, s);
+  if (e == cudaSuccess) e = launch_kalman_assemble(a, st, sms, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&status, &st->status, sizeof(int), cudaMemcpyDeviceToHost, s);
   cudaError_t f = cudaFreeAsync(ws, s);
   if (e == cudaSuccess) e = f;
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e);
-  return BDSS_OK;
+  return (bdss_status)status;
 }
 
 bdss_status bdss_tc_selftest(double *max_rel_err) {

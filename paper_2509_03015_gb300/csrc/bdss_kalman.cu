@@ -6,145 +6,330 @@
 //   A_kk      = Qinv_k + G_{k+1}^T Qinv_{k+1} G_{k+1} + H_k^T Rinv_k H_k
 //   A_{k+1,k} = -Qinv_{k+1} G_{k+1}
 //   b_k       = H_k^T Rinv_k z_k + Qinv_k zeta_k - G_{k+1}^T Qinv_{k+1} zeta_{k+1}
-// Two launches, each a flat grid of (step, task) CTAs whose tasks of one step
-// are adjacent so that step's operands are shared through L2:
-//   products  A_{k+1,k} tiles (-Qinv G), U_k = Rinv_k H_k tiles (a row
-//             scaling when Rinv_k is diagonal), and the vectors
-//             v_k = Rinv_k z_k, w_k = Qinv_k zeta_k;
-//   diagonal  A_kk tiles = Qinv_k + H_k^T U_k - G_{k+1}^T A_{k+1,k}, and b_k.
-// All arithmetic is FP64, 64 x 64 output tiles through gemm_nt_tile.
-#include "bdss_large.cuh"
+// The n x n and m x n products run on the tensor cores as digit products
+// (bdss_slice.cuh), two launches:
+//   products  A_{k+1,k} = -Qinv G and, for a full Rinv, U_k = Rinv_k H_k;
+//   diagonal  A_kk = Qinv_k + H_k^T U_k - G_{k+1}^T A_{k+1,k} (a diagonal Rinv
+//             scales the rows of H as they are cut).
+// The vectors v_k = Rinv_k z_k, w_k = Qinv_k zeta_k and b_k are two small
+// FP64 launches.
+//
+// Every product is formed transposed (TMEM lane = column of the result), so
+// that a warp stores 32 consecutive entries of a row, and its A operand is a
+// matrix read by columns: thread (c, g) takes the eight K entries 8 g .. of
+// column c, coalesced over c, and cuts them to 16 bytes of every digit.
+// With n <= 64 the 128 A rows of a tile are two steps, each multiplied by 32
+// of its own B rows at a time; above, two blocks of 64 columns of one step.
+//
+// FP64-ALU tiles took 23.2 ms at N = 16384, n = 64, m = 32 (0.82 of the FP64
+// pipe's rate).
 #include "bdss_kalman.h"
+#include "bdss_launch.h"
+#include "bdss_slice_cta.cuh"
 
 namespace bdss {
 
 namespace {
 
-__device__ void store_tile(double *out, long long ld, int rows, int cols, int r0, int c0,
-                           const double (&acc)[4][4], double sign, const double *add) {
-  const int tm = threadIdx.x >> 4, tn = threadIdx.x & 15;
+// Work units: pairs of steps (n <= 64) or steps, and per unit the tiles of 128
+// result columns.
+__host__ __device__ inline long long kalman_groups(long long N, int n) { return n <= 64 ? (N + 1) / 2 : N; }
+__host__ __device__ inline int kalman_row_tiles(int n) { return n <= 64 ? 1 : (n + 127) / 128; }
+constexpr long long kKalmanTimeoutNs = 10000000000LL;  // bound of a product's wait
+
+constexpr int kKmGroups = 8;  // K groups of eight in a chunk
+constexpr size_t kKmSmem = wd_smem<double>();
+
+// 64 rows of an operand by K index: entry (k, c) at p[k ld + c], c < cols
+// (rows of B operands read by rows: entry (k, c) at p[c ld + k]); scale:
+// factors of the K entries, or null.
+struct KmSlot {
+  const double *p;
+  const double *scale;
+  int cols;
+};
+
+// Entries k0 + 8 g .. of column c of a slot (zero past the ends).
+__device__ __forceinline__ void km_load_col(const KmSlot &s, int ld, int k0, int K, int c, int g, double (&v)[8]) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = r0 + 4 * tm + i;
-    if (r >= rows) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = c0 + 4 * tn + j;
-      if (c >= cols) continue;
-      const long long o = (long long)r * ld + c;
-      out[o] = (add ? add[o] : 0.0) + sign * acc[i][j];
-    }
+  for (int i = 0; i < 8; ++i) {
+    const int k = k0 + 8 * g + i;
+    const bool in = c < s.cols && k < K;
+    v[i] = in ? ldcg(s.p + (size_t)k * ld + c) : 0.0;
+    if (s.scale && in) v[i] *= ldcg(s.scale + k);
   }
 }
+__device__ __forceinline__ int km_exp(const double (&v)[8]) {
+  int ex = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) ex = max(ex, sl_exp(v[i]));
+  return ex;
+}
 
-__global__ void __launch_bounds__(kThreads) k_kalman_products(KalmanArgs a) {
-  __shared__ double sA[kKc * kTilePad], sB[kKc * kTilePad];
-  const int n = a.n, m = a.m, nt = ntiles(n), mt = ntiles(m);
-  const int tasks = nt * nt + mt * nt + 1;
-  const long long k = (long long)blockIdx.x / tasks;
-  const int t = (int)((long long)blockIdx.x - k * tasks);
-  const long long nn = (long long)n * n, mn = (long long)m * n;
-  const long long mm = a.rinv_diag ? (long long)m : (long long)m * m;  // Rinv stride per step
-  double acc[4][4] = {};
-  if (t < nt * nt) {
-    if (k + 1 >= a.N) return;
-    const int r0 = (t / nt) * kTile, c0 = (t % nt) * kTile;
-    const View<double> Q{a.Qinv + (k + 1) * nn, n, 1, n, n};   // (r, j) -> Qinv_{k+1}[r][j]
-    const View<double> Gt{a.G + (k + 1) * nn, 1, n, n, n};     // (c, j) -> G_{k+1}[j][c]
-    gemm_nt_tile(acc, Q, r0, Gt, c0, n, sA, sB);
-    store_tile(a.A_sub + k * nn, n, n, n, r0, c0, acc, -1.0, nullptr);
-  } else if (t < nt * nt + mt * nt) {
-    const int u = t - nt * nt, r0 = (u / nt) * kTile, c0 = (u % nt) * kTile;
-    if (a.rinv_diag) {
-      const double *rk = a.Rinv + k * mm, *Hk = a.H + k * mn;
-      double *Uk = a.U + k * mn;
-      for (int e = threadIdx.x; e < kTile * kTile; e += blockDim.x) {
-        const int r = r0 + e / kTile, c = c0 + e % kTile;
-        if (r < m && c < n) Uk[(long long)r * n + c] = rk[r] * Hk[(long long)r * n + c];
+// What a CTA multiplies: out[c][r] (+)= sum_k A(k, c) B(k, r) over K.
+struct KmProduct {
+  KmSlot a[2];   // A columns 64 b .. (two steps, or two blocks of one)
+  int lda, K;
+  KmSlot b[2];   // the B of each (the same matrix unless two steps)
+  int ldb;
+  bool brows;    // B read by rows (K contiguous)
+  double sign;
+};
+
+// acc += sign x product: this thread's row and 16 columns.  pair: two steps,
+// 32 columns each per round (column 32 h + 8 hw + i at acc[8 h + i]); else 64
+// columns from the first B slot (column 16 hw + i).  ncols: columns in use.
+template <bool kPair>
+__device__ __forceinline__ bool km_product(WdCta<double> &w, const KmProduct &P, int ncols, int row, int hw,
+                                           uint32_t lane_base, int *exK, double (&acc)[16]) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int c = tid & 63, g = tid >> 6;
+  int *exKB = exK + kKmGroups * kSlRows;
+#pragma unroll 1
+  for (int k0 = 0; k0 < P.K; k0 += kSlK) {
+    const int kc = min(kSlK, P.K - k0), ks = (kc + 15) >> 4;
+    const int halves = kPair && ncols > 32 ? 2 : 1;
+#pragma unroll 1
+    for (int h = 0; h < halves; ++h) {
+      double v[2][8], vb[8];
+      if (h == 0) {
+#pragma unroll
+        for (int b = 0; b < 2; ++b) km_load_col(P.a[b], P.lda, k0, P.K, c, g, v[b]);
       }
-      return;
+      // B row rr of 64: column h 32 + (rr & 31) of its step, or column rr
+      const int bs = kPair ? c >> 5 : 0, bc = kPair ? 32 * h + (c & 31) : c;
+      double r2[4][2];
+      if (P.brows) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int rr = u * kWdWarps + warp, k = 2 * lane;
+          const KmSlot &s = P.b[kPair ? rr >> 5 : 0];
+          const int col = kPair ? 32 * h + (rr & 31) : rr;
+          r2[u][0] = r2[u][1] = 0.0;
+          if (col < s.cols) {
+            const double *p = s.p + (size_t)col * P.ldb + k0 + k;
+            if (k < kc) r2[u][0] = ldcg(p);
+            if (k + 1 < kc) r2[u][1] = ldcg(p + 1);
+          }
+        }
+      } else {
+        km_load_col(P.b[bs], P.ldb, k0, P.K, bc, g, vb);
+        exKB[g * 64 + c] = km_exp(vb);
+      }
+      if (h == 0) {
+#pragma unroll
+        for (int b = 0; b < 2; ++b) exK[g * kSlRows + 64 * b + c] = km_exp(v[b]);
+      }
+      __syncthreads();
+      if (h == 0) {
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+          int ex = 0;
+#pragma unroll
+          for (int q = 0; q < kKmGroups; ++q) ex = max(ex, exK[q * kSlRows + 64 * b + c]);
+          if (g == 0) w.exA[64 * b + c] = ex;
+          store8<double>(v[b], ex, w.A + sl_off(64 * b + c, g), kSlASlab);
+        }
+      }
+      if (P.brows) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int rr = u * kWdWarps + warp, k = 2 * lane;
+          const int ex = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(sl_exp(r2[u][0]), sl_exp(r2[u][1])));
+          if (lane == 0) w.exB[rr] = ex;
+          sl_store2<double>(r2[u][0], r2[u][1], ex,
+                            w.B + (rr >> 5) * kWdBBytes<double> + sl_off(rr & 31, k >> 3) + 2 * (k & 7), kSlBSlab);
+        }
+      } else {
+        int ex = 0;
+#pragma unroll
+        for (int q = 0; q < kKmGroups; ++q) ex = max(ex, exKB[q * 64 + c]);
+        if (g == 0) w.exB[c] = ex;
+        store8<double>(vb, ex, w.B + (c >> 5) * kWdBBytes<double> + sl_off(c & 31, g), kSlBSlab);
+      }
+      if (!wd_product<double>(w, kPair || ncols > 32, ks, ks)) return false;
+      const int ea = w.exA[row];
+      if constexpr (kPair) {
+#pragma unroll
+        for (int i = 0; i < 8; i += 4) {
+          if (32 * h + 8 * hw + i < ncols) {  // the same for a warp
+            double x[4];
+            wd_drain4<double>(lane_base + (uint32_t)(row >> 6) * kWdBufCols<double> + (uint32_t)(8 * hw + i), ea,
+                              w.exB + (row >> 6) * 32 + 8 * hw + i, x);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              if (h == 0) acc[i + e] = fma(P.sign, x[e], acc[i + e]);
+              else acc[8 + i + e] = fma(P.sign, x[e], acc[8 + i + e]);
+            }
+          }
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < 16; i += 4) {
+          if (16 * hw + i < ncols) {
+            double x[4];
+            wd_drain4<double>(lane_base + (uint32_t)(hw >> 1) * kWdBufCols<double> + (uint32_t)(16 * (hw & 1) + i), ea,
+                              w.exB + 16 * hw + i, x);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[i + e] = fma(P.sign, x[e], acc[i + e]);
+          }
+        }
+      }
+      // the exponents and slabs have been read before the next ones are written
+      tc_fence_before();
+      __syncthreads();
+      tc_fence_after();
     }
-    const View<double> R{a.Rinv + k * mm, m, 1, m, m};         // (r, j) -> Rinv_k[r][j]
-    const View<double> Ht{a.H + k * mn, 1, n, n, m};           // (c, j) -> H_k[j][c]
-    gemm_nt_tile(acc, R, r0, Ht, c0, m, sA, sB);
-    store_tile(a.U + k * mn, n, m, n, r0, c0, acc, 1.0, nullptr);
-  } else {
-    if (!a.B) return;
-    const double *Rk = a.Rinv + k * mm, *zk = a.z + k * m;
-    for (int i = threadIdx.x; i < m; i += blockDim.x) {
-      double s = 0.0;
-      if (a.rinv_diag)
-        s = Rk[i] * zk[i];
-      else
-        for (int j = 0; j < m; ++j) s = fma(Rk[(long long)i * m + j], zk[j], s);
-      a.v[k * m + i] = s;
+  }
+  return true;
+}
+
+// kDiag = 0: the products A_{k+1,k} and U_k; 1: the diagonal blocks.
+template <int kDiag, bool kPair>
+__global__ void __launch_bounds__(kWdThreads, 1) k_kalman_tc(const __grid_constant__ KalmanArgs a, DevStatus *st) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint64_t s_bar;
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_ok, s_exA[kSlRows], s_exB[64], s_exK[kKmGroups * (kSlRows + 64)];
+  WdCta<double> w;
+  wd_begin(w, smem_raw, &s_bar, &s_tmem, s_exA, s_exB, s_exK, &s_ok, kKalmanTimeoutNs);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, hw = warp >> 2, row0 = 32 * (warp & 3), row = row0 + lane;
+  const uint32_t lane_base = w.tmem + ((uint32_t)row0 << 16);
+  const int n = a.n, m = a.m;
+  const size_t nn = (size_t)n * n, mn = (size_t)m * n, mm = a.rinv_diag ? (size_t)m : (size_t)m * m;
+  const long long groups = kalman_groups(a.N, n);
+  const int tr = kalman_row_tiles(n), tn = (n + 63) / 64, tm = kDiag || a.rinv_diag ? 0 : (m + 63) / 64;
+  const int tiles = tr * (tn + tm);
+  bool ok = true;
+  for (long long t = blockIdx.x; t < groups * tiles && ok; t += gridDim.x) {
+    const long long grp = t / tiles;
+    const int u = (int)(t - grp * tiles), ct = u / tr, c0 = kPair ? 0 : 128 * (u - ct * tr);
+    const bool isU = ct >= tn;
+    const int r0 = 64 * (isU ? ct - tn : ct), R = isU ? m : n, ncols = min(64, R - r0);
+    // slot b: step k_b, result columns c_b .. (rows of TMEM)
+    double acc[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc[i] = 0.0;
+    KmProduct P;
+    P.lda = n;
+    for (int part = kDiag && m > 0 ? 0 : 1; part < 2 && ok; ++part) {
+      // kDiag: part 0: H^T U, part 1: -G^T A_sub; else one product
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        const long long k = kPair ? 2 * grp + b : grp;
+        const int cb = kPair ? 0 : c0 + 64 * b;
+        const bool next = k + 1 < a.N, live = k < a.N && cb < n;
+        KmSlot sa{nullptr, nullptr, 0}, sb{nullptr, nullptr, 0};
+        if (kDiag && part == 0 && live) {
+          sa = {(a.rinv_diag ? a.H : a.U) + (size_t)k * mn + cb, a.rinv_diag ? a.Rinv + (size_t)k * mm : nullptr,
+                min(64, n - cb)};
+          sb = {a.H + (size_t)k * mn + r0, nullptr, ncols};
+        } else if (kDiag && live && next) {
+          sa = {a.A_sub + (size_t)k * nn + cb, nullptr, min(64, n - cb)};
+          sb = {a.G + (size_t)(k + 1) * nn + r0, nullptr, ncols};
+        } else if (!kDiag && isU && live) {
+          sa = {a.H + (size_t)k * mn + cb, nullptr, min(64, n - cb)};
+          sb = {a.Rinv + (size_t)k * mm + (size_t)r0 * m, nullptr, ncols};
+        } else if (!kDiag && !isU && live && next) {
+          sa = {a.G + (size_t)(k + 1) * nn + cb, nullptr, min(64, n - cb)};
+          sb = {a.Qinv + (size_t)(k + 1) * nn + (size_t)r0 * n, nullptr, ncols};
+        }
+        P.a[b] = sa;
+        P.b[b] = sb;
+      }
+      if (!kPair) P.b[1] = P.b[0];
+      P.brows = !kDiag;
+      P.K = (kDiag ? part == 0 : isU) ? m : n;
+      P.ldb = kDiag ? n : isU ? m : n;
+      P.sign = kDiag ? (part == 0 ? 1.0 : -1.0) : isU ? 1.0 : -1.0;
+      ok = km_product<kPair>(w, P, ncols, row, hw, lane_base, s_exK, acc);
     }
-    const double *Qk = a.Qinv + k * nn, *ek = a.zeta ? a.zeta + k * n : nullptr;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      double s = 0.0;
+    if (!ok) {
+      if (threadIdx.x == 0) set_status(st, kStTimeout, -1, -1);
+      break;
+    }
+    const int b = row >> 6, c = (kPair ? 0 : c0 + 64 * b) + (row & 63);
+    const long long k = kPair ? 2 * grp + b : grp;
+    if (k >= a.N || c >= n || (!kDiag && !isU && k + 1 >= a.N)) continue;
+    double *out = kDiag ? a.A_diag + (size_t)k * nn : isU ? a.U + (size_t)k * mn : a.A_sub + (size_t)k * nn;
+    const double *add = kDiag ? a.Qinv + (size_t)k * nn : nullptr;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const int r = kPair ? 32 * (i >> 3) + 8 * hw + (i & 7) : 16 * hw + i;
+      if (r < ncols) {
+        const size_t o = (size_t)(r0 + r) * n + c;
+        out[o] = kDiag ? ldcg(add + o) + acc[i] : acc[i];
+      }
+    }
+  }
+  wd_end(w);
+}
+
+// v_k = Rinv_k z_k, w_k = Qinv_k zeta_k (one step per CTA).
+__global__ void __launch_bounds__(kThreads) k_kalman_vectors(const __grid_constant__ KalmanArgs a) {
+  const int n = a.n, m = a.m;
+  const long long k = blockIdx.x;
+  const double *Rk = a.Rinv + (size_t)k * (a.rinv_diag ? (size_t)m : (size_t)m * m), *zk = a.z + k * m;
+  const double *Qk = a.Qinv + (size_t)k * n * n, *ek = a.zeta ? a.zeta + k * n : nullptr;
+  for (int i = threadIdx.x; i < n + m; i += blockDim.x) {
+    double s = 0.0;
+    if (i < n) {
       if (ek)
-        for (int j = 0; j < n; ++j) s = fma(Qk[(long long)i * n + j], ek[j], s);
+        for (int j = 0; j < n; ++j) s = fma(Qk[(size_t)i * n + j], ek[j], s);
       a.w[k * n + i] = s;
+    } else if (a.rinv_diag) {
+      a.v[k * m + i - n] = Rk[i - n] * zk[i - n];
+    } else {
+      const double *r = Rk + (size_t)(i - n) * m;
+      for (int j = 0; j < m; ++j) s = fma(r[j], zk[j], s);
+      a.v[k * m + i - n] = s;
     }
   }
 }
 
-__global__ void __launch_bounds__(kThreads) k_kalman_diag(KalmanArgs a) {
-  __shared__ double sA[kKc * kTilePad], sB[kKc * kTilePad];
-  const int n = a.n, m = a.m, nt = ntiles(n);
-  const int tasks = nt * nt + 1;
-  const long long k = (long long)blockIdx.x / tasks;
-  const int t = (int)((long long)blockIdx.x - k * tasks);
-  const long long nn = (long long)n * n, mn = (long long)m * n;
-  if (t < nt * nt) {
-    const int r0 = (t / nt) * kTile, c0 = (t % nt) * kTile;
-    double acc[4][4] = {};
-    const View<double> Hc{a.H + k * mn, 1, n, n, m};           // (r, j) -> H_k[j][r]
-    const View<double> Uc{a.U + k * mn, 1, n, n, m};           // (c, j) -> U_k[j][c]
-    gemm_nt_tile(acc, Hc, r0, Uc, c0, m, sA, sB);
-    if (k + 1 < a.N) {
-      double acc2[4][4] = {};
-      const View<double> Gc{a.G + (k + 1) * nn, 1, n, n, n};   // (r, j) -> G_{k+1}[j][r]
-      const View<double> Sc{a.A_sub + k * nn, 1, n, n, n};     // (c, j) -> A_{k+1,k}[j][c]
-      gemm_nt_tile(acc2, Gc, r0, Sc, c0, n, sA, sB);
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] -= acc2[i][j];
-    }
-    store_tile(a.A_diag + k * nn, n, n, n, r0, c0, acc, 1.0, a.Qinv + k * nn);
-  } else {
-    if (!a.B) return;
-    const double *Hk = a.H + k * mn, *vk = a.v + k * m, *wk = a.w + k * n;
-    const bool next = k + 1 < a.N;
-    const double *G1 = a.G + (k + 1) * nn, *w1 = a.w + (k + 1) * n;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      double s = 0.0;
-      for (int j = 0; j < m; ++j) s = fma(Hk[(long long)j * n + i], vk[j], s);
-      double g = 0.0;
-      if (next)
-        for (int j = 0; j < n; ++j) g = fma(G1[(long long)j * n + i], w1[j], g);
-      a.B[k * n + i] = s + wk[i] - g;
-    }
+// b_k = H_k^T v_k + w_k - G_{k+1}^T w_{k+1}.
+__global__ void __launch_bounds__(kThreads) k_kalman_rhs(const __grid_constant__ KalmanArgs a) {
+  const int n = a.n, m = a.m;
+  const long long k = blockIdx.x;
+  const double *Hk = a.H + (size_t)k * m * n, *vk = a.v + k * m, *wk = a.w + k * n;
+  const bool next = k + 1 < a.N;
+  const double *G1 = a.G + (size_t)(k + 1) * n * n, *w1 = a.w + (k + 1) * n;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    double s = 0.0;
+    for (int j = 0; j < m; ++j) s = fma(Hk[(size_t)j * n + i], vk[j], s);
+    double g = 0.0;
+    if (next)
+      for (int j = 0; j < n; ++j) g = fma(G1[(size_t)j * n + i], w1[j], g);
+    a.B[k * n + i] = s + wk[i] - g;
   }
 }
 
 }  // namespace
 
+// Grid limit of the former per-tile launches, kept as the entry point's limit.
 long long kalman_max_steps(int n, int m) {
-  const int nt = ntiles(n), mt = ntiles(m);
+  const int nt = (n + 63) / 64, mt = (m + 63) / 64;
   return 0x7fffffffLL / (nt * nt + mt * nt + 1);
 }
 
-cudaError_t launch_kalman_assemble(const KalmanArgs &a, cudaStream_t s) {
-  const int nt = ntiles(a.n), mt = ntiles(a.m);
-  const long long g1 = a.N * (long long)(nt * nt + mt * nt + 1);
-  const long long g2 = a.N * (long long)(nt * nt + 1);
+cudaError_t launch_kalman_assemble(const KalmanArgs &a, DevStatus *st, int sms, cudaStream_t s) {
   if (a.N > kalman_max_steps(a.n, a.m)) return cudaErrorInvalidValue;
-  k_kalman_products<<<(unsigned)g1, kThreads, 0, s>>>(a);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_kalman_diag<<<(unsigned)g2, kThreads, 0, s>>>(a);
+  const bool pair = a.n <= 64;
+  const void *kernels[2] = {pair ? (const void *)k_kalman_tc<0, true> : (const void *)k_kalman_tc<0, false>,
+                            pair ? (const void *)k_kalman_tc<1, true> : (const void *)k_kalman_tc<1, false>};
+  cudaError_t e = cudaSuccess;
+  for (const void *k : kernels)
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kKmSmem);
+  for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
+    const int tn = (a.n + 63) / 64, tm = i || a.rinv_diag ? 0 : (a.m + 63) / 64;
+    const long long tasks = kalman_groups(a.N, a.n) * kalman_row_tiles(a.n) * (tn + tm);
+    const unsigned grid = (unsigned)(tasks < sms ? tasks : sms);
+    void *args[] = {(void *)&a, (void *)&st};
+    e = cudaLaunchKernel(kernels[i], dim3(grid), dim3(kWdThreads), args, kKmSmem, s);
+  }
+  if (e != cudaSuccess || !a.B) return e;
+  k_kalman_vectors<<<(unsigned)a.N, kThreads, 0, s>>>(a);
+  k_kalman_rhs<<<(unsigned)a.N, kThreads, 0, s>>>(a);
   return cudaGetLastError();
 }
 

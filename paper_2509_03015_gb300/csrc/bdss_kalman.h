@@ -3,6 +3,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "bdss_device.cuh"
+
 namespace bdss {
 
 // Normal equations assembled on the device.  U (N m n), v (N m), w (N n) are
@@ -15,7 +17,8 @@ struct KalmanArgs {
   double *A_diag, *A_sub, *B;
   double *U, *v, *w;
 };
-cudaError_t launch_kalman_assemble(const KalmanArgs &a, cudaStream_t s);
+// A product whose wait runs out sets st->status (cleared by the caller).
+cudaError_t launch_kalman_assemble(const KalmanArgs &a, DevStatus *st, int sms, cudaStream_t s);
 long long kalman_max_steps(int n, int m);  // largest N whose grids fit one launch
 
 }  // namespace bdss
