@@ -93,6 +93,7 @@ struct bdss_ctx {
   void *tcfC = nullptr;   // (N / 2) x 2 x n x n (T)
   void *tcfcb = nullptr;  // (N / 2) x 2 x n x d_max (T)
   int tcf_ready = 0;
+  bool tcf_factored = false;  // the stored factors are that path's
   int tcf_opt = -1;       // BDSS_OPT_SCHUR_EMU at n <= 64: -1 by size, 0 off, 1 on
   // large mixed path: streamed solve passes (maps over Li and Wb)
   CorrMaps corr_maps[3];  // split factors P = 1, 2, 4
@@ -302,9 +303,13 @@ static bool use_small(const bdss_ctx *h) {
 // n = 24, N = 2000: 1.16.
 constexpr int kTcfMinN = 32;
 constexpr int kTcfAutoMinN = 40;
-constexpr int kTcfAutoMinBlocks = 2048;
+constexpr int kTcfAutoMinBlocks = 1536;
+constexpr int kTcfAutoMinN32 = 24;
+constexpr int kTcfAutoMinBlocks32 = 32;
 static bool tcf_by_size(const bdss_ctx *h) {
-  return !is_mixed(h) && !h->large && h->n >= kTcfAutoMinN && h->N >= kTcfAutoMinBlocks;
+  if (h->large) return false;
+  if (is_mixed(h)) return h->n >= kTcfAutoMinN32 && h->N >= kTcfAutoMinBlocks32;
+  return h->n >= kTcfAutoMinN && h->N >= kTcfAutoMinBlocks;
 }
 static bool use_tcf(const bdss_ctx *h) {
   if (!h->tcf_ready || h->plan.L < 1) return false;
@@ -316,14 +321,15 @@ static bool use_tcf(const bdss_ctx *h) {
 static bdss_status tcf_alloc(bdss_ctx *h) {
   if (h->tcf_ready) return BDSS_OK;
   const size_t nn = (size_t)h->n * h->n, m = (size_t)(h->N / 2);
-  bool ok = h->tcfX || ws_alloc(h, &h->tcfX, m * nn * sizeof(double));
-  ok = ok && (h->tcfC || ws_alloc(h, &h->tcfC, m * 2 * nn * sizeof(double)));
-  ok = ok && (h->tcfcb || ws_alloc(h, &h->tcfcb, m * 2 * h->n * h->d_max * sizeof(double)));
+  const size_t esz = is_mixed(h) ? sizeof(float) : sizeof(double);
+  bool ok = h->tcfX || ws_alloc(h, &h->tcfX, m * nn * esz);
+  ok = ok && (h->tcfC || ws_alloc(h, &h->tcfC, m * 2 * nn * esz));
+  ok = ok && (h->tcfcb || ws_alloc(h, &h->tcfcb, m * 2 * h->n * h->d_max * esz));
   if (!ok) {
     cudaGetLastError();
     return BDSS_ERR_ALLOC;
   }
-  const cudaError_t e = tcf_configure<double>(h->n, h->d_max);
+  const cudaError_t e = is_mixed(h) ? tcf_configure<float>(h->n, h->d_max) : tcf_configure<double>(h->n, h->d_max);
   if (e != cudaSuccess) return cuda_fail(e);
   h->tcf_ready = 1;
   return BDSS_OK;
@@ -522,6 +528,17 @@ static cudaError_t run_levels_wide(bdss_ctx *h, const Args<float> &a, bool rhs) 
   return e;
 }
 
+// Downward pass over factors that hold their inverses (bdss_tcf.cu).
+template <typename T>
+static cudaError_t tcf_down(bdss_ctx *h, const Args<T> &b) {
+  cudaError_t e = cudaSuccess;
+  kt_begin(h, h->kt_cls);
+  for (int l = h->plan.L - 1; l >= 0 && e == cudaSuccess; --l) e = launch_tcf_down<T>(b, l, h->stream);
+  kt_end(h, h->plan.L);
+  h->launches += h->plan.L;
+  return e;
+}
+
 // Factorisation for n <= 64 with the coupling solves and Schur products on
 // the tensor cores: per level the diagonal blocks (ALU), then everything
 // else; the last level's pending updates, the top block and the downward
@@ -542,19 +559,31 @@ static cudaError_t run_levels_tcf(bdss_ctx *h, const Args<T> &a, bool rhs) {
     kt_end(h, 1);
     h->launches += 2;
   }
+  const bool one = p.Nl[p.L] == 1;
   kt_begin(h, h->kt_cls);
-  if (e == cudaSuccess) e = launch_tcf_diag<T>(b, c, p.L, 1, h->sms, h->stream);
-  if (e == cudaSuccess) e = launch_top<T>(b, 1, h->smem, h->stream);
-  kt_end(h, 2);
-  h->launches += 2;
-  if (rhs)
-    for (int l = p.L - 1; l >= 0 && e == cudaSuccess; --l) {
-      kt_begin(h, h->kt_cls);
-      e = launch_phaseC<T>(b, l, grid_for(h, p.Nl[l] / 2), h->smem, h->stream);
-      kt_end(h, 1);
-      h->launches += 1;
-    }
-  return e;
+  if (one) {
+    if (e == cudaSuccess) e = launch_tcf_top<T>(b, c, h->stream);
+  } else {
+    if (e == cudaSuccess) e = launch_tcf_diag<T>(b, c, p.L, 1, h->sms, h->stream);
+    if (e == cudaSuccess) e = launch_top<T>(b, 1, h->smem, h->stream);
+  }
+  kt_end(h, one ? 1 : 2);
+  h->launches += one ? 1 : 2;
+  h->tcf_factored = true;
+  return e == cudaSuccess && rhs ? tcf_down<T>(h, b) : e;
+}
+
+// Solve pass over the factors of run_levels_tcf.
+template <typename T>
+static cudaError_t run_solve_tcf(bdss_ctx *h, const Args<T> &b) {
+  const Plan &p = h->plan;
+  kt_begin(h, h->kt_cls);
+  cudaError_t e = launch_tcf_up<T>(b, 0, 1, h->stream);
+  for (int l = 0; l < p.L && e == cudaSuccess; ++l) e = launch_tcf_up<T>(b, l, 0, h->stream);
+  if (e == cudaSuccess) e = launch_top<T>(b, 0, h->smem, h->stream);
+  kt_end(h, p.L + 2);
+  h->launches += p.L + 2;
+  return e == cudaSuccess ? tcf_down<T>(h, b) : e;
 }
 
 // Separator update of level l in the TF32 mode: the D and E tiles on the
@@ -649,7 +678,9 @@ template <typename T>
 static cudaError_t run_levels(bdss_ctx *h, const Args<T> &a, bool factor, bool rhs) {
   const Plan &p = h->plan;
   if (h->large) return run_levels_large<T>(h, a, factor, rhs);
+  if (factor) h->tcf_factored = false;
   if (factor && use_tcf(h)) return run_levels_tcf<T>(h, a, rhs);
+  if (!factor && h->tcf_factored && use_tcf(h)) return run_solve_tcf<T>(h, a);
   const int cap = h->bps * h->sms;
   if (h->persistent) {
     long long most = 1;  // tasks of the busiest step

@@ -32,8 +32,9 @@ namespace {
 
 constexpr int kDiagThreads = 128;   // levels of many blocks: several CTAs share an SM
 constexpr int kSchurThreads = 512;
-constexpr uint32_t kTmemAll = 512;
-constexpr uint32_t kBufCols = 256;  // accumulators of one column tile
+template <typename T> constexpr uint32_t kBufCols = SliceFmt<T>::kDig * kSlCols;  // accumulators of one column tile
+template <typename T> constexpr uint32_t kTmem = sizeof(T) == 8 ? 512 : 256;       // a power of two
+template <typename T> constexpr int kSchurCtas = sizeof(T) == 8 ? 1 : 2;            // per SM
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_tcf_diag(const __grid_constant__ Args<T> a, const TcfLevel<T> w, int l,
@@ -96,7 +97,9 @@ __global__ void __launch_bounds__(256) k_tcf_diag(const __grid_constant__ Args<T
       const int i = e / n, c = e - i * n;
       const T x = c <= i ? s[c * ld + i] : T(0);  // X[i][c] is in the upper triangle
       Xg[e] = x;
-      if (c <= i) Lg[e] = kStoreInverse<T> ? x : s[i * ld + c];
+      // FP64: L with X^T above it; FP32: X
+      if (!kStoreInverse<T>) Lg[e] = s[i * ld + c];
+      else if (c <= i) Lg[e] = x;
     }
   } else {
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
@@ -121,8 +124,12 @@ __global__ void __launch_bounds__(256) k_tcf_diag(const __grid_constant__ Args<T
 constexpr int kStageRow = 48;               // bytes of a staged output row: 32 and a pad
 constexpr int kStageWarp = 32 * kStageRow;  // bytes of a warp's output stage
 constexpr int kWarps = kSchurThreads / 32;
+// the column tiles' space, which also holds P (128 x 64) between its rounds
+template <typename T> constexpr size_t kBSpace =
+    (size_t)SliceFmt<T>::kDig * 2 * kSlBSlab > 128 * 64 * sizeof(T) ? (size_t)SliceFmt<T>::kDig * 2 * kSlBSlab
+                                                                    : 128 * 64 * sizeof(T);
 template <typename T> constexpr size_t schur_smem() {
-  return (size_t)SliceFmt<T>::kDig * (kSlASlab + 2 * kSlBSlab) + kWarps * kStageWarp + 1024;
+  return (size_t)SliceFmt<T>::kDig * kSlASlab + kBSpace<T> + kWarps * kStageWarp + 1024;
 }
 
 template <typename T> struct Pair { T x, y; };
@@ -171,7 +178,7 @@ __device__ __forceinline__ Pair<T> load_pair(const S *p, int k, int n, bool pair
 // instructions, every pass over a tile missed the instruction cache, and a
 // tile took 117,000 cycles.
 template <typename T, int kNP>
-__global__ void __launch_bounds__(kSchurThreads, 1)
+__global__ void __launch_bounds__(kSchurThreads, kSchurCtas<T>)
     k_tcf_schur(const __grid_constant__ Args<T> a, const TcfLevel<T> w, int l) {
   constexpr int kDig = SliceFmt<T>::kDig;
   constexpr int G = 64 / kNP;             // blocks per tile
@@ -192,7 +199,7 @@ __global__ void __launch_bounds__(kSchurThreads, 1)
   unsigned char *A = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   unsigned char *B0 = A + (size_t)kDig * kSlASlab;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  unsigned char *stage = B0 + 2 * kBBytes + warp * kStageWarp;
+  unsigned char *stage = B0 + kBSpace<T> + warp * kStageWarp;
   T *raw = reinterpret_cast<T *>(B0);
   const int n = a.p.n, d = a.d, KS = (n + 15) / 16;
   const size_t nn = (size_t)n * n, nd = (size_t)n * d;
@@ -204,7 +211,7 @@ __global__ void __launch_bounds__(kSchurThreads, 1)
     mbar_init(&s_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0) tmem_alloc(&s_tmem, kTmemAll);
+  if (warp == 0) tmem_alloc(&s_tmem, kTmem<T>);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -351,7 +358,7 @@ __global__ void __launch_bounds__(kSchurThreads, 1)
         const int cols = rd < 3 ? kSlCols : 16;
         // kNP = 64: rows 0 .. 31 of the lower triangular X have 32 entries
         sl_issue<T>(tmem, A, B0, cols, rd == 0 ? min(KS, 2) : KS);
-        if (rd < 3 || G > 1) sl_issue<T>(tmem + kBufCols, A, B0 + kBBytes, cols, KS);
+        if (rd < 3 || G > 1) sl_issue<T>(tmem + kBufCols<T>, A, B0 + kBBytes, cols, KS);
         tc_commit(&s_bar);
       }
       if (!mbar_wait_cta(&s_bar, ph, a.timeout_ns, &s_ok)) {
@@ -385,7 +392,7 @@ __global__ void __launch_bounds__(kSchurThreads, 1)
         cols = 4;
         if (!wlive || d0 + 4 * hw >= d) cols = 0;
       }
-      const uint32_t acc_base = lane_base + (uint32_t)(rd < 3 ? ctile : rblk) * kBufCols +
+      const uint32_t acc_base = lane_base + (uint32_t)(rd < 3 ? ctile : rblk) * kBufCols<T> +
                                 (uint32_t)(rd < 3 ? tcol : 4 * hw);
       const int tstep = rd < 3 ? kSlCols : 16;
       // exponents of the columns this thread drains
@@ -457,7 +464,154 @@ __global__ void __launch_bounds__(kSchurThreads, 1)
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem, kTmemAll);
+  if (warp == 0) tmem_dealloc(tmem, kTmem<T>);
+}
+
+// The top block (one block left at level L): the last level's pending update,
+// its FP64 factor and inverse, x_0 = X^T (X b_0).
+template <typename T>
+__global__ void __launch_bounds__(256) k_tcf_top(const __grid_constant__ Args<T> a, const TcfLevel<T> w) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int s_flag, s_go, s_cnt[8];
+  if (threadIdx.x == 0) s_go = ld_relaxed_i32(&a.st->status) == 0;
+  __syncthreads();
+  if (!s_go) return;
+  const int n = a.p.n, d = a.d, np = (n + 7) & ~7, ld = ldstride(np), L = a.p.L;
+  double *s = reinterpret_cast<double *>(smem_raw), *sB = s + (size_t)np * ld, *cbuf = sB + (size_t)2 * d * ld;
+  for (int e = threadIdx.x; e < np * np; e += blockDim.x) {
+    const int i = e / np, c = e - i * np;
+    if (c > i) continue;
+    double v = i == c;
+    if (i < n) {
+      T x = L > 1 ? ldcg(a.Ld + (size_t)i * n + c)
+                  : T(0.5) * ((T)ldcg(a.A_diag + (size_t)i * n + c) + (T)ldcg(a.A_diag + (size_t)c * n + i));
+      x -= ldcg(w.C + (size_t)i * n + c);
+      v = (double)x;
+    }
+    s[i * ld + c] = v;
+  }
+  for (int e = threadIdx.x; e < n * d; e += blockDim.x) {
+    const int i = e / d, c = e - i * d;
+    T v = L > 1 ? ldcg(a.Y + e) : a.B64 ? (T)ldcg(a.B64 + e) : ldcg(a.Bt + e);
+    v -= ldcg(w.cb + e);
+    sB[c * ld + i] = (double)v;
+  }
+  if (chol_inverse(s, ld, np, cbuf, s_cnt, &s_flag)) {
+    if (threadIdx.x == 0) set_status(a.st, kStNotSPD, L, 0);
+    return;
+  }
+  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
+    const int i = e / n, c = e - i * n;
+    a.Ltop[e] = c <= i ? s[i * ld + c] : 0.0;
+  }
+  double *sY = sB + (size_t)d * ld;
+  for (int e = threadIdx.x; e < n * d; e += blockDim.x) {  // X[i][q] is s[q ld + i]
+    const int c = e / n, i = e - c * n;
+    double v = 0.0;
+    for (int q = 0; q <= i; ++q) v = fma(s[q * ld + i], sB[c * ld + q], v);
+    sY[c * ld + i] = v;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < n * d; e += blockDim.x) {
+    const int c = e / n, i = e - c * n;
+    double v = 0.0;
+    for (int q = i; q < n; ++q) v = fma(s[i * ld + q], sY[c * ld + q], v);
+    const size_t o = (size_t)i * d + c;
+    a.Y[o] = (T)v;
+    if (a.X64) a.X64[o] = a.x_accumulate ? a.X64[o] + v : v;
+  }
+}
+
+// One level of a solve with the stored inverses.
+//   kUp:   separator s: b_s -= Wt(s-1) y_{s-1} + Wt(s) y_{s+1}; if s is eliminated
+//          at the next level, y_s = X_s b_s.  first: no level before the first
+//          elimination yet, y_j = X_j b_j of level 0.
+//   down:  eliminated j: t = y_j - Wt(j-1)^T x_{j-1} - Wt(j)^T x_{j+1}, x_j = X_j^T t.
+// Thread (i, g): row i of the result, a quarter of either sum; it loads all of
+// its matrix entries at once, before any of them is used, and keeps them for
+// every four columns of the right-hand sides.
+//
+// What bounds it: few blocks, two trips to memory and four barriers (a level of
+// one 64 x 64 block: substitutions by one warp took 74 us); many, the FP64 pipe
+// (5 n^2 d / 2 multiply-adds a block on the way down).
+constexpr int kSolveCols = 4;
+template <typename T, bool kUp>
+__global__ void __launch_bounds__(256, 2) k_tcf_solve(const __grid_constant__ Args<T> a, int l, int first) {
+  __shared__ T sV[2][kMaxN][kSolveCols], sR[4][kMaxN][kSolveCols], sT[kMaxN][kSolveCols];
+  if (ld_relaxed_i32(&a.st->status) != 0) return;
+  const int n = a.p.n, d = a.d, i = threadIdx.x & (kMaxN - 1), g = threadIdx.x / kMaxN;
+  const size_t nn = (size_t)n * n, nd = (size_t)n * d;
+  const long long m = blockIdx.x, Nl = a.p.Nl[l];
+  const long long pos = kUp && !first ? 2 * m : 2 * m + 1, orig = pos << l;
+  const bool hasM = !first && pos >= 1, hasP = !first && pos + 1 < Nl;
+  const bool tri = !kUp || first || (m & 1);  // a triangular product follows
+  const bool raw = kUp && l == 0 && (a.B64 || a.Bt);
+  // matrix entries: W of slot pos - 1 (g < 2) or pos (g >= 2), X of this block
+  T wv[kMaxN / 2], xv[kMaxN / 4];
+  const bool mine = i < n && (g < 2 ? hasM : hasP);
+  const T *Wg = a.Wb + (size_t)(a.p.off[l] + pos - (g < 2 ? 1 : 0)) * nn;
+#pragma unroll
+  for (int u = 0; u < kMaxN / 2; ++u) {
+    const int v = (g & 1) * (kMaxN / 2) + u;
+    wv[u] = mine && v < n ? (kUp ? Wg[(size_t)i * n + v] : Wg[(size_t)v * n + i]) : T(0);
+  }
+  // FP64 keeps X^T above the diagonal of Ld (1 / L_ii on it), FP32 X below
+  const T *Xg = a.Ld + (size_t)orig * nn;
+#pragma unroll
+  for (int u = 0; u < kMaxN / 4; ++u) {
+    const int c = 4 * u + g;
+    const bool in = tri && i < n && c < n && (kUp ? c <= i : c >= i);
+    const int r0 = kUp ? i : c, c0 = kUp ? c : i;  // X[r0][c0]
+    xv[u] = in ? (kStoreInverse<T> ? Xg[(size_t)r0 * n + c0] : Xg[(size_t)c0 * n + r0]) : T(0);
+  }
+  for (int d0 = 0; d0 < d; d0 += kSolveCols) {
+    const int dc = min(kSolveCols, d - d0);
+    for (int e = threadIdx.x; e < 2 * kMaxN * kSolveCols; e += 256) {
+      const int side = e / (kMaxN * kSolveCols), v = (e / kSolveCols) % kMaxN, c = e % kSolveCols;
+      const bool in = v < n && c < dc && (side ? hasP : hasM);
+      sV[side][v][c] = in ? ldcg(a.Y + (size_t)((side ? pos + 1 : pos - 1) << l) * nd + (size_t)v * d + d0 + c) : T(0);
+    }
+    __syncthreads();
+    T acc[kSolveCols] = {};
+    if (hasM || hasP) {
+#pragma unroll
+      for (int u = 0; u < kMaxN / 2; ++u)
+#pragma unroll
+        for (int c = 0; c < kSolveCols; ++c)
+          if (c < dc) acc[c] = fma(wv[u], sV[g >> 1][(g & 1) * (kMaxN / 2) + u][c], acc[c]);
+    }
+#pragma unroll
+    for (int c = 0; c < kSolveCols; ++c) sR[g][i][c] = acc[c];
+    __syncthreads();
+    if (i < n && g < dc) {  // thread (i, g): column g
+      const size_t o = (size_t)orig * nd + (size_t)i * d + d0 + g;
+      const T base = !raw ? ldcg(a.Y + o) : a.B64 ? (T)ldcg(a.B64 + o) : ldcg(a.Bt + o);
+      const T t = base - ((sR[0][i][g] + sR[1][i][g]) + (sR[2][i][g] + sR[3][i][g]));
+      sT[i][g] = t;
+      if (!tri) a.Y[o] = t;
+    } else {
+      sT[i][g] = T(0);
+    }
+    __syncthreads();
+    if (!tri) continue;
+#pragma unroll
+    for (int c = 0; c < kSolveCols; ++c) acc[c] = T(0);
+#pragma unroll
+    for (int u = 0; u < kMaxN / 4; ++u)
+#pragma unroll
+      for (int c = 0; c < kSolveCols; ++c)
+        if (c < dc) acc[c] = fma(xv[u], sT[4 * u + g][c], acc[c]);
+#pragma unroll
+    for (int c = 0; c < kSolveCols; ++c) sR[g][i][c] = acc[c];
+    __syncthreads();
+    if (i < n && g < dc) {
+      const size_t o = (size_t)orig * nd + (size_t)i * d + d0 + g;
+      const T x = (sR[0][i][g] + sR[1][i][g]) + (sR[2][i][g] + sR[3][i][g]);
+      a.Y[o] = x;
+      if (!kUp && a.X64) a.X64[o] = a.x_accumulate ? a.X64[o] + (double)x : (double)x;
+    }
+    // sR and sT are next written after two barriers
+  }
 }
 
 size_t diag_smem(int n, int d, size_t esz) { const int np = (n + 7) & ~7;
@@ -470,14 +624,14 @@ cudaError_t tcf_configure(int n, int d) {
   int dev = 0, optin = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  const void *kernels[] = {(const void *)k_tcf_diag<T>, (const void *)k_tcf_schur<T, 32>,
+  const void *kernels[] = {(const void *)k_tcf_diag<T>, (const void *)k_tcf_top<T>, (const void *)k_tcf_schur<T, 32>,
                            (const void *)k_tcf_schur<T, 64>};
   for (const void *k : kernels) {
     cudaFuncAttributes fa;
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
-    if (e == cudaSuccess && k != kernels[0] && schur_smem<T>() > (size_t)optin - fa.sharedSizeBytes)
+    if (e == cudaSuccess && k != kernels[0] && k != kernels[1] && schur_smem<T>() > (size_t)optin - fa.sharedSizeBytes)
       e = cudaErrorInvalidConfiguration;
   }
   if (e == cudaSuccess && diag_smem(n, d, sizeof(T)) > (size_t)optin - 64) e = cudaErrorInvalidConfiguration;
@@ -500,16 +654,40 @@ cudaError_t launch_tcf_schur(const Args<T> &a, const TcfLevel<T> &c, int l, int 
   const long long nE = a.p.Nl[l] / 2;
   const int G = a.p.n <= 32 ? 2 : 1;
   const long long tasks = (nE + G - 1) / G;
-  const unsigned grid = (unsigned)(tasks < sms ? tasks : sms);
+  const long long most = (long long)kSchurCtas<T> * sms;
+  const unsigned grid = (unsigned)(tasks < most ? tasks : most);
   if (G == 2) k_tcf_schur<T, 32><<<grid, kSchurThreads, schur_smem<T>(), s>>>(a, c, l);
   else k_tcf_schur<T, 64><<<grid, kSchurThreads, schur_smem<T>(), s>>>(a, c, l);
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_tcf_top(const Args<T> &a, const TcfLevel<T> &c, cudaStream_t s) {
+  const int np = (a.p.n + 7) & ~7;
+  const size_t smem = ((size_t)(np + 2 * a.d) * ldstride(np) + 17 * kMaxN) * sizeof(double);
+  k_tcf_top<T><<<1, 256, smem, s>>>(a, c);
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_tcf_up(const Args<T> &a, int l, int first, cudaStream_t s) {
+  k_tcf_solve<T, true><<<(unsigned)(first ? a.p.Nl[l] / 2 : (a.p.Nl[l] + 1) / 2), 256, 0, s>>>(a, l, first);
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_tcf_down(const Args<T> &a, int l, cudaStream_t s) {
+  k_tcf_solve<T, false><<<(unsigned)(a.p.Nl[l] / 2), 256, 0, s>>>(a, l, 0);
   return cudaGetLastError();
 }
 
 #define BDSS_TCF_INSTANTIATE(T)                                                                       \
   template cudaError_t tcf_configure<T>(int, int);                                                    \
   template cudaError_t launch_tcf_diag<T>(const Args<T> &, const TcfLevel<T> &, int, int, int, cudaStream_t); \
-  template cudaError_t launch_tcf_schur<T>(const Args<T> &, const TcfLevel<T> &, int, int, cudaStream_t);
+  template cudaError_t launch_tcf_schur<T>(const Args<T> &, const TcfLevel<T> &, int, int, cudaStream_t);        \
+  template cudaError_t launch_tcf_top<T>(const Args<T> &, const TcfLevel<T> &, cudaStream_t);                     \
+  template cudaError_t launch_tcf_up<T>(const Args<T> &, int, int, cudaStream_t);                                 \
+  template cudaError_t launch_tcf_down<T>(const Args<T> &, int, cudaStream_t);
 BDSS_TCF_INSTANTIATE(double)
 BDSS_TCF_INSTANTIATE(float)
 

@@ -82,3 +82,20 @@ def test_bad_pivot_is_reported(what):
     assert e.value.status == 2
     if what == "not_spd":
         assert e.value.info.block == 6 and e.value.info.level == 1
+
+
+# mixed precision takes the path by size; the call refines to a backward error
+# of 1e-14, and kappa(A) below 1e3 then bounds the forward error by 1e-11
+@pytest.mark.parametrize("N,n,d,precision", [(2048, 40, 1, "fp32_ir"), (2049, 63, 3, "tf32_ir"),
+                                             (2100, 64, 17, "fp32_ir")])
+def test_mixed_precision_matches_oracle(oracle_mod, N, n, d, precision):
+    from paper_2509_03015_gb300 import Solver
+    s = inputs.random_btd(N, n, d, seed=N + n)
+    sol = Solver(N, n, d_max=d, precision=precision)
+    X = sol.factor_solve(_dev(s["A_diag"]), _dev(s["A_sub"]), _dev(s["B"])).cpu().numpy()
+    X2 = sol.solve(_dev(s["B"])).cpu().numpy()
+    sol.close()
+    Xo = oracle_mod.solve_system(s["A_diag"], s["A_sub"], s["B"])
+    for x in (X, X2):
+        assert oracle_mod.forward_error(x, Xo) <= 1e-11
+        assert oracle_mod.backward_error(s["A_diag"], s["A_sub"], x, s["B"]) <= 1.1e-14
