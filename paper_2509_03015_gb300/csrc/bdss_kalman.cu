@@ -76,14 +76,15 @@ struct KmProduct {
   double sign;
 };
 
-// acc += sign x product: this thread's row and 16 columns.  pair: two steps,
-// 32 columns each per round (column 32 h + 8 hw + i at acc[8 h + i]); else 64
-// columns from the first B slot (column 16 hw + i).  ncols: columns in use.
+// acc += sign x product: this thread's row and 8 columns.  pair: two steps, 32
+// columns each per round (column 32 h + 4 hw + i at acc[4 h + i]); else 64
+// columns from the first B slot (column 8 hw + i).  ncols: columns in use.
 template <bool kPair>
 __device__ __forceinline__ bool km_product(WdCta<double> &w, const KmProduct &P, int ncols, int row, int hw,
-                                           uint32_t lane_base, int *exK, double (&acc)[16]) {
+                                           uint32_t lane_base, int *exK, double (&acc)[8]) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int c = tid & 63, g = tid >> 6;
+  const int c = tid & 63, g = (tid >> 6) & 7, half = tid >> 9;  // half: this thread's A slot
+  constexpr int kR = 64 / kWdWarps<double>;
   int *exKB = exK + kKmGroups * kSlRows;
 #pragma unroll 1
   for (int k0 = 0; k0 < P.K; k0 += kSlK) {
@@ -91,19 +92,15 @@ __device__ __forceinline__ bool km_product(WdCta<double> &w, const KmProduct &P,
     const int halves = kPair && ncols > 32 ? 2 : 1;
 #pragma unroll 1
     for (int h = 0; h < halves; ++h) {
-      double v[2][8], vb[8];
-      if (h == 0) {
-#pragma unroll
-        for (int b = 0; b < 2; ++b) km_load_col(P.a[b], P.lda, k0, P.K, c, g, v[b]);
-      }
-      // B row rr of 64: column h 32 + (rr & 31) of its step, or column rr
-      const int bs = kPair ? c >> 5 : 0, bc = kPair ? 32 * h + (c & 31) : c;
-      double r2[4][2];
+      double v[8], vb[8], r2[kR][2];
+      const KmSlot sa = half ? P.a[1] : P.a[0];
+      if (h == 0) km_load_col(sa, P.lda, k0, P.K, c, g, v);
+      // B row rr of 64: column 32 h + (rr & 31) of its step, or column rr
       if (P.brows) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int rr = u * kWdWarps + warp, k = 2 * lane;
-          const KmSlot &s = P.b[kPair ? rr >> 5 : 0];
+        for (int u = 0; u < kR; ++u) {
+          const int rr = u * kWdWarps<double> + warp, k = 2 * lane;
+          const KmSlot s = kPair && rr >= 32 ? P.b[1] : P.b[0];
           const int col = kPair ? 32 * h + (rr & 31) : rr;
           r2[u][0] = r2[u][1] = 0.0;
           if (col < s.cols) {
@@ -112,73 +109,67 @@ __device__ __forceinline__ bool km_product(WdCta<double> &w, const KmProduct &P,
             if (k + 1 < kc) r2[u][1] = ldcg(p + 1);
           }
         }
-      } else {
-        km_load_col(P.b[bs], P.ldb, k0, P.K, bc, g, vb);
+      } else if (half == 0) {
+        const KmSlot sb = kPair && c >= 32 ? P.b[1] : P.b[0];
+        km_load_col(sb, P.ldb, k0, P.K, kPair ? 32 * h + (c & 31) : c, g, vb);
         exKB[g * 64 + c] = km_exp(vb);
       }
-      if (h == 0) {
-#pragma unroll
-        for (int b = 0; b < 2; ++b) exK[g * kSlRows + 64 * b + c] = km_exp(v[b]);
-      }
+      if (h == 0) exK[g * kSlRows + 64 * half + c] = km_exp(v);
       __syncthreads();
       if (h == 0) {
+        int ex = 0;
 #pragma unroll
-        for (int b = 0; b < 2; ++b) {
-          int ex = 0;
-#pragma unroll
-          for (int q = 0; q < kKmGroups; ++q) ex = max(ex, exK[q * kSlRows + 64 * b + c]);
-          if (g == 0) w.exA[64 * b + c] = ex;
-          store8<double>(v[b], ex, w.A + sl_off(64 * b + c, g), kSlASlab);
-        }
+        for (int q = 0; q < kKmGroups; ++q) ex = max(ex, exK[q * kSlRows + 64 * half + c]);
+        if (g == 0) w.exA[64 * half + c] = sl_row_exp<double>(ex);
+        store8<double>(v, ex, w.A + sl_off(64 * half + c, g), kSlASlab);
       }
       if (P.brows) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int rr = u * kWdWarps + warp, k = 2 * lane;
+        for (int u = 0; u < kR; ++u) {
+          const int rr = u * kWdWarps<double> + warp, k = 2 * lane;
           const int ex = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(sl_exp(r2[u][0]), sl_exp(r2[u][1])));
-          if (lane == 0) w.exB[rr] = ex;
+          if (lane == 0) w.exB[rr] = sl_row_exp<double>(ex);
           sl_store2<double>(r2[u][0], r2[u][1], ex,
                             w.B + (rr >> 5) * kWdBBytes<double> + sl_off(rr & 31, k >> 3) + 2 * (k & 7), kSlBSlab);
         }
-      } else {
+      } else if (half == 0) {
         int ex = 0;
 #pragma unroll
         for (int q = 0; q < kKmGroups; ++q) ex = max(ex, exKB[q * 64 + c]);
-        if (g == 0) w.exB[c] = ex;
+        if (g == 0) w.exB[c] = sl_row_exp<double>(ex);
         store8<double>(vb, ex, w.B + (c >> 5) * kWdBBytes<double> + sl_off(c & 31, g), kSlBSlab);
       }
-      if (!wd_product<double>(w, kPair || ncols > 32, ks, ks)) return false;
+      const bool cols2 = kPair || ncols > 32;
+      wd_issue<double>(w, cols2, ks, ks);
       const int ea = w.exA[row];
+      bool ok = true;
       if constexpr (kPair) {
+        if (32 * h + 4 * hw < ncols) {  // the same for a warp
+          ok = wd_wait<double>(w, row >> 6);
+          double x[4];
+          if (ok)
+            wd_drain4<double>(lane_base + (uint32_t)(row >> 6) * kWdBufCols<double> + (uint32_t)(4 * hw), ea,
+                              w.exB + (row >> 6) * 32 + 4 * hw, x);
 #pragma unroll
-        for (int i = 0; i < 8; i += 4) {
-          if (32 * h + 8 * hw + i < ncols) {  // the same for a warp
-            double x[4];
-            wd_drain4<double>(lane_base + (uint32_t)(row >> 6) * kWdBufCols<double> + (uint32_t)(8 * hw + i), ea,
-                              w.exB + (row >> 6) * 32 + 8 * hw + i, x);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              if (h == 0) acc[i + e] = fma(P.sign, x[e], acc[i + e]);
-              else acc[8 + i + e] = fma(P.sign, x[e], acc[8 + i + e]);
-            }
+          for (int e = 0; e < 4; ++e) {
+            if (h == 0) acc[e] = fma(P.sign, x[e], acc[e]);
+            else acc[4 + e] = fma(P.sign, x[e], acc[4 + e]);
           }
         }
-      } else {
+      } else if (8 * hw < ncols) {
+        ok = wd_wait<double>(w, hw >> 2);
 #pragma unroll
-        for (int i = 0; i < 16; i += 4) {
-          if (16 * hw + i < ncols) {
-            double x[4];
-            wd_drain4<double>(lane_base + (uint32_t)(hw >> 1) * kWdBufCols<double> + (uint32_t)(16 * (hw & 1) + i), ea,
-                              w.exB + 16 * hw + i, x);
+        for (int i = 0; i < 8; i += 4) {
+          double x[4];
+          if (ok)
+            wd_drain4<double>(lane_base + (uint32_t)(hw >> 2) * kWdBufCols<double> + (uint32_t)(8 * (hw & 3) + i), ea,
+                              w.exB + 8 * hw + i, x);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) acc[i + e] = fma(P.sign, x[e], acc[i + e]);
-          }
+          for (int e = 0; e < 4; ++e) acc[i + e] = fma(P.sign, x[e], acc[i + e]);
         }
       }
       // the exponents and slabs have been read before the next ones are written
-      tc_fence_before();
-      __syncthreads();
-      tc_fence_after();
+      if (!wd_round_end<double>(w, cols2, ok)) return false;
     }
   }
   return true;
@@ -186,13 +177,13 @@ __device__ __forceinline__ bool km_product(WdCta<double> &w, const KmProduct &P,
 
 // kDiag = 0: the products A_{k+1,k} and U_k; 1: the diagonal blocks.
 template <int kDiag, bool kPair>
-__global__ void __launch_bounds__(kWdThreads, 1) k_kalman_tc(const __grid_constant__ KalmanArgs a, DevStatus *st) {
+__global__ void __launch_bounds__(kWdThreads<double>, 1) k_kalman_tc(const __grid_constant__ KalmanArgs a, DevStatus *st) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ uint64_t s_bar;
+  __shared__ uint64_t s_bar[2];
   __shared__ uint32_t s_tmem;
-  __shared__ int s_ok, s_exA[kSlRows], s_exB[64], s_exK[kKmGroups * (kSlRows + 64)];
+  __shared__ int s_exA[kSlRows], s_exB[64], s_exK[kKmGroups * (kSlRows + 64)];
   WdCta<double> w;
-  wd_begin(w, smem_raw, &s_bar, &s_tmem, s_exA, s_exB, s_exK, &s_ok, kKalmanTimeoutNs);
+  wd_begin(w, smem_raw, s_bar, &s_tmem, s_exA, s_exB, s_exK, kKalmanTimeoutNs);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, hw = warp >> 2, row0 = 32 * (warp & 3), row = row0 + lane;
   const uint32_t lane_base = w.tmem + ((uint32_t)row0 << 16);
   const int n = a.n, m = a.m;
@@ -207,9 +198,9 @@ __global__ void __launch_bounds__(kWdThreads, 1) k_kalman_tc(const __grid_consta
     const bool isU = ct >= tn;
     const int r0 = 64 * (isU ? ct - tn : ct), R = isU ? m : n, ncols = min(64, R - r0);
     // slot b: step k_b, result columns c_b .. (rows of TMEM)
-    double acc[16];
+    double acc[8];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) acc[i] = 0.0;
+    for (int i = 0; i < 8; ++i) acc[i] = 0.0;
     KmProduct P;
     P.lda = n;
     for (int part = kDiag && m > 0 ? 0 : 1; part < 2 && ok; ++part) {
@@ -254,8 +245,8 @@ __global__ void __launch_bounds__(kWdThreads, 1) k_kalman_tc(const __grid_consta
     double *out = kDiag ? a.A_diag + (size_t)k * nn : isU ? a.U + (size_t)k * mn : a.A_sub + (size_t)k * nn;
     const double *add = kDiag ? a.Qinv + (size_t)k * nn : nullptr;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const int r = kPair ? 32 * (i >> 3) + 8 * hw + (i & 7) : 16 * hw + i;
+    for (int i = 0; i < 8; ++i) {
+      const int r = kPair ? 32 * (i >> 2) + 4 * hw + (i & 3) : 8 * hw + i;
       if (r < ncols) {
         const size_t o = (size_t)(r0 + r) * n + c;
         out[o] = kDiag ? ldcg(add + o) + acc[i] : acc[i];
@@ -325,7 +316,7 @@ cudaError_t launch_kalman_assemble(const KalmanArgs &a, DevStatus *st, int sms, 
     const long long tasks = kalman_groups(a.N, a.n) * kalman_row_tiles(a.n) * (tn + tm);
     const unsigned grid = (unsigned)(tasks < sms ? tasks : sms);
     void *args[] = {(void *)&a, (void *)&st};
-    e = cudaLaunchKernel(kernels[i], dim3(grid), dim3(kWdThreads), args, kKmSmem, s);
+    e = cudaLaunchKernel(kernels[i], dim3(grid), dim3(kWdThreads<double>), args, kKmSmem, s);
   }
   if (e != cudaSuccess || !a.B) return e;
   k_kalman_vectors<<<(unsigned)a.N, kThreads, 0, s>>>(a);

@@ -53,6 +53,13 @@ constexpr int kSlBSlab = kSlCols * 128;  // bytes of one digit of a B tile
 // Exponent field of |v| (0 for zero and subnormals: they count as zero).
 __device__ __forceinline__ int sl_exp(double v) { return (__double2hiint(v) >> 20) & 0x7FF; }
 __device__ __forceinline__ int sl_exp(float v) { return (__float_as_int(v) >> 23) & 0xFF; }
+// The row exponent that enters sl_value: a row with an infinity or NaN poisons
+// every product it takes part in, as a floating-point product would.
+constexpr int kSlPoisonEx = 1 << 16;
+template <typename T>
+__device__ __forceinline__ int sl_row_exp(int ex) {
+  return sizeof(T) == 8 && ex == 0x7FF ? kSlPoisonEx : ex;
+}
 // Biased digits of v under the row exponent field exmax: the byte p from the
 // top is d_p + 128.
 __device__ __forceinline__ unsigned long long sl_biased(double v, int exmax) {
@@ -164,53 +171,64 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // An accumulator entry as an integer without the conversion unit (16 lanes a
-// cycle and SM; with eight conversions an entry it set the pace of the
-// drains).  |x| <= 2^22: adding 1.5 * 2^23 puts x in the binade of unit
-// spacing.  |x| < 2^23: 1.5 * 2^24 and a spacing of two, which rounds the last
-// bit away -- used for the two lowest diagonals, where it weighs 2^-60 of the
-// product of the row maxima.
-__device__ __forceinline__ int sl_int22(float x) { return __float_as_int(x + 12582912.0f) - 0x4B400000; }
-__device__ __forceinline__ int sl_int23(float x) { return (__float_as_int(x + 25165824.0f) - 0x4BC00000) * 2; }
+// cycle and SM): |x| <= 2^22, adding 1.5 * 2^23 puts x in the binade of unit
+// spacing, and the bits are kSlBias + x.  |x| < 2^23: 1.5 * 2^24 and a spacing of
+// two (bits kSlBias2 + x / 2), which rounds the last bit away -- used for the
+// two lowest diagonals, where it weighs 2^-60 of the product of the row maxima.
+constexpr unsigned kSlBias = 0x4B400000u, kSlBias2 = 0x4BC00000u;
+__device__ __forceinline__ unsigned sl_bits22(float x) { return (unsigned)__float_as_int(x + 12582912.0f); }
+__device__ __forceinline__ unsigned sl_bits23(float x) { return (unsigned)__float_as_int(x + 25165824.0f); }
 
-// t 2^(be - 1075) for a result outside the normal range.
-static __device__ __noinline__ double sl_scale_slow(unsigned long long t, int be) { return scalbn((double)(long long)t, be - 1075); }
+// (-1)^neg (m2 2^64 + m1 2^32 + m0) 2^S rounded to FP64, whatever the range
+// (zero, subnormal and infinite results; a poisoned row's exponent is out of it).
+static __device__ __noinline__ double sl_value_slow(unsigned m2, unsigned m1, unsigned m0, bool neg, int S) {
+  if (S > kSlPoisonEx / 2) return __longlong_as_double(0x7FF8000000000000LL);
+  if ((m2 | m1 | m0) == 0u) return 0.0;
+  unsigned long long hi = ((unsigned long long)m2 << 32) | m1;
+  double r;
+  if (hi == 0) {
+    r = scalbn((double)m0, S);
+  } else {  // 64 leading bits, the last one sticky
+    const int lz = __clzll((long long)hi);
+    unsigned long long m = lz == 0 ? hi : (hi << lz) | (((unsigned long long)m0 << 32) >> (64 - lz));
+    if (lz < 32 && (unsigned)(m0 << lz) != 0u) m |= 1ULL;
+    r = scalbn(__ull2double_rn(m), S + 32 - lz);
+  }
+  return neg ? -r : r;
+}
 
 // sum_t ACC_t 256^(7-t) 2^(exa + exb - 2112), rounded once to FP64 on the
-// integer pipe (an FP64 instruction holds a warp's FP64 unit for 64 cycles on
-// this GPU; the whole conversion takes about that many integer issue slots for
-// 32 entries).  With |d_0| <= 64 the diagonals are at most 2^18, 2^20, 2^21,
+// integer pipes (an FP64 instruction holds a warp's FP64 unit for 64 cycles on
+// this GPU).  With |d_0| <= 64 the diagonals are at most 2^18, 2^20, 2^21,
 // 3 2^20, ..., 7 2^20, so neighbouring pairs combine in 32 bits.
+//
+// The logic pipe (half rate) sets the pace of the drains, so additions that
+// can be multiply-adds are, the biases of the pairs are subtracted once, the
+// sign is taken off by complement (one unit of 2^-62 of the row maxima), and
+// everything unusual goes to sl_value_slow: about 30 logic instructions an
+// entry, half of a conversion through 64-bit shifts and selects (the products
+// of a 128 x 64 tile took 9,200 of a round's 24,700 cycles to drain).
 __device__ __forceinline__ double sl_value(const float (&c)[8], int exa, int exb) {
-  const int h01 = sl_int22(c[0]) * 256 + sl_int22(c[1]);
-  const int h23 = sl_int22(c[2]) * 256 + sl_int22(c[3]);
-  const int h45 = sl_int22(c[4]) * 256 + __float2int_rn(c[5]);
-  const int h67 = sl_int23(c[6]) * 256 + sl_int23(c[7]);
+  const int h01 = (int)(sl_bits22(c[0]) * 256u + sl_bits22(c[1]) - kSlBias * 257u);
+  const int h23 = (int)(sl_bits22(c[2]) * 256u + sl_bits22(c[3]) - kSlBias * 257u);
+  const int h45 = (int)(sl_bits22(c[4]) * 256u + (unsigned)__float2int_rn(c[5]) - kSlBias * 256u);
+  const int h67 = (int)(sl_bits23(c[6]) * 512u + sl_bits23(c[7]) * 2u - kSlBias2 * 514u);
   const long long H = (long long)h01 * 65536 + h23, L = (long long)h45 * 65536 + h67;
-  long long hi = H + (L >> 32);  // value = (hi 2^32 + lo) 2^S
-  unsigned lo = (unsigned)L;
-  int S = exa + exb - 2112;
-  const bool neg = hi < 0;
-  if (neg) {
-    hi = ~hi + (lo == 0u ? 1 : 0);
-    lo = 0u - lo;
-  }
-  if (hi == 0) {
-    hi = (long long)lo;
-    lo = 0u;
-    S -= 32;
-  }
-  if (exa == 0x7FF || exb == 0x7FF) return __longlong_as_double(0x7FF8000000000000LL);
-  if (hi == 0) return 0.0;
-  const int lz = __clzll(hi);  // >= 2
-  const unsigned long long m = ((unsigned long long)hi << lz) | (((unsigned long long)lo << 32) >> (64 - lz));
-  const unsigned long long t = (m >> 11) + ((m >> 10) & 1ULL);  // 53 bits, rounded
-  const int be = 1023 + 63 + 32 - lz + S;
-  if (be < 1 || be > 2046) {  // outside the normal range
-    const double r = sl_scale_slow(t, be);
-    return neg ? -r : r;
-  }
-  const unsigned long long bits = ((unsigned long long)(be - 1) << 52) + t;  // a carry of t raises the exponent
-  return __longlong_as_double((long long)(bits | (neg ? 0x8000000000000000ULL : 0ULL)));
+  const long long hi = H + (int)(L >> 32);  // value = (hi 2^32 + lo) 2^S
+  const int sgn = (int)(hi >> 63);
+  const unsigned m2 = (unsigned)((int)(hi >> 32) ^ sgn), m1 = (unsigned)((int)hi ^ sgn), m0 = (unsigned)((int)L ^ sgn);
+  // 96 bits; the leading word is m2 or m1
+  const bool p = m2 != 0;
+  const unsigned w2 = p ? m2 : m1, w1 = p ? m1 : m0, w0 = p ? m0 : 0u;
+  const int z = __clz((int)w2);
+  const unsigned a1 = __funnelshift_l(w1, w2, z), a0 = __funnelshift_l(w0, w1, z);
+  // exponent field of the result, less one: the mantissa's leading bit adds it
+  const int S = exa + exb - 2112, be = S + (p ? 1023 + 95 - 1 : 1023 + 63 - 1) - z;
+  if (w2 == 0u || (unsigned)be > 2044u) return sl_value_slow(m2, m1, m0, sgn != 0, S);
+  const unsigned t0 = __funnelshift_r(a0, a1, 11), rb = (a0 >> 10) & 1u;
+  const unsigned long long bits =
+      (((unsigned long long)((unsigned)be * 0x100000u + (a1 >> 11)) << 32) | t0) + rb;  // a carry raises the exponent
+  return __longlong_as_double((long long)(bits | ((unsigned long long)((unsigned)sgn & 0x80000000u) << 32)));
 }
 // The same for FP32: the smaller parts' products first.
 __device__ __forceinline__ float sl_value(const float (&c)[3], int, int) { return c[0] + (c[1] + c[2]); }

@@ -6,24 +6,29 @@
 
 namespace bdss {
 
-constexpr int kWdThreads = 512;
-constexpr int kWdWarps = kWdThreads / 32;
+// FP64: one CTA of 32 warps per SM (its digit slabs fill the shared memory);
+// FP32: two of 16.
+template <typename T> constexpr int kWdThreads = sizeof(T) == 8 ? 1024 : 512;
+template <typename T> constexpr int kWdWarps = kWdThreads<T> / 32;
+template <typename T> constexpr int kWdCols = 8192 / kWdThreads<T>;  // columns of an output row per thread
 constexpr int kWdTile = 64;  // rows of a slot, columns of an output tile
-template <typename T> constexpr int kWdStageRow = sizeof(T) == 8 ? 48 : 16;  // bytes of a staged output row
 template <typename T> constexpr uint32_t kWdBufCols = SliceFmt<T>::kDig * kSlCols;  // accumulators of 32 columns
 template <typename T> constexpr uint32_t kWdTmem = sizeof(T) == 8 ? 512 : 256;  // a power of two
 template <typename T> constexpr int kWdBBytes = SliceFmt<T>::kDig * kSlBSlab;
+constexpr int kWdStage = 32 * 4;  // entries of a warp's output stage: 32 rows of four
 template <typename T> constexpr size_t wd_smem() {
-  return (size_t)SliceFmt<T>::kDig * (kSlASlab + 2 * kSlBSlab) + (size_t)kWdWarps * 32 * kWdStageRow<T> + 1024;
+  return (size_t)SliceFmt<T>::kDig * (kSlASlab + 2 * kSlBSlab) + 1024;
 }
 
 template <typename T>
 struct WdCta {
-  unsigned char *A, *B, *stage;  // digit slabs, this warp's output stage
+  // digit slabs; this warp's output stage, in the first B tile's place, whose
+  // products are complete whenever there is something to put out
+  unsigned char *A, *B, *stage;
   uint32_t tmem;
-  uint64_t *bar;
-  int *exA, *exB, *exP, *s_ok;   // row exponents: A (128), B (64), partial (4 x 128)
-  uint32_t ph;
+  uint64_t *bar;               // one per column tile
+  int *exA, *exB, *exP;        // row exponents: A (128), B (64), partial (64 / kWdCols x 128)
+  uint32_t ph0, ph1;
   long long timeout_ns;
 };
 
@@ -71,26 +76,27 @@ __device__ __forceinline__ void store8<float>(const float *v, int ex, unsigned c
     *reinterpret_cast<uint4 *>(dst + p * stride) = make_uint4(w[0][p], w[1][p], w[2][p], w[3][p]);
 }
 
-// The A rows from registers: this thread's 16 columns of its row.  Contains a
+// The A rows from registers: this thread's kWdCols columns of its row.  Contains a
 // CTA barrier.
 template <typename T>
-__device__ __forceinline__ void wd_cut_regs(const WdCta<T> &w, const T (&v)[16], int row, int hw) {
+__device__ __forceinline__ void wd_cut_regs(const WdCta<T> &w, const T (&v)[kWdCols<T>], int row, int hw) {
+  constexpr int kGroups = kWdCols<T> / 8;
   int ex = 0;
 #pragma unroll
-  for (int i = 0; i < 16; ++i) ex = max(ex, sl_exp(v[i]));
+  for (int i = 0; i < kWdCols<T>; ++i) ex = max(ex, sl_exp(v[i]));
   w.exP[hw * kSlRows + row] = ex;
   __syncthreads();
 #pragma unroll
-  for (int q = 0; q < 4; ++q) ex = max(ex, w.exP[q * kSlRows + row]);
-  if (hw == 0) w.exA[row] = ex;
+  for (int q = 0; q < 64 / kWdCols<T>; ++q) ex = max(ex, w.exP[q * kSlRows + row]);
+  if (hw == 0) w.exA[row] = sl_row_exp<T>(ex);
 #pragma unroll
-  for (int i = 0; i < 2; ++i) store8<T>(v + 8 * i, ex, w.A + sl_off(row, 2 * hw + i), kSlASlab);
+  for (int i = 0; i < kGroups; ++i) store8<T>(v + 8 * i, ex, w.A + sl_off(row, kGroups * hw + i), kSlASlab);
 }
 
-// The product of the cut operands, waited for.  cols2: the second 32 columns
-// as well; ks0 / ks1: K steps of either column tile.  False after a timeout.
+// Issue the product of the cut operands.  cols2: the second 32 columns as
+// well; ks0 / ks1: K steps of either column tile.
 template <typename T>
-__device__ __forceinline__ bool wd_product(WdCta<T> &w, bool cols2, int ks0, int ks1) {
+__device__ __forceinline__ void wd_issue(WdCta<T> &w, bool cols2, int ks0, int ks1) {
   // every thread's operands before the products that read them, its TMEM
   // reads before the products that overwrite them
   fence_proxy_async_smem();
@@ -99,33 +105,58 @@ __device__ __forceinline__ bool wd_product(WdCta<T> &w, bool cols2, int ks0, int
   if (threadIdx.x == 0) {
     tc_fence_after();
     sl_issue<T>(w.tmem, w.A, w.B, kSlCols, ks0);
-    if (cols2) sl_issue<T>(w.tmem + kWdBufCols<T>, w.A, w.B + kWdBBytes<T>, kSlCols, ks1);
     tc_commit(w.bar);
+    if (cols2) {
+      sl_issue<T>(w.tmem + kWdBufCols<T>, w.A, w.B + kWdBBytes<T>, kSlCols, ks1);
+      tc_commit(w.bar + 1);
+    }
   }
-  if (!mbar_wait_cta(w.bar, w.ph, w.timeout_ns, w.s_ok)) {
-    // wait again (bounded) for the products in flight before TMEM is freed
-    mbar_wait_cta(w.bar, w.ph, w.timeout_ns, w.s_ok);
-    return false;
-  }
-  w.ph ^= 1;
+  __syncwarp();
+}
+// Wait (bounded) for a column tile's product, a warp at a time: the warps of
+// the first tile drain it while the second is multiplied.  False after a
+// timeout; wd_round_end makes that the whole CTA's.
+template <typename T>
+__device__ __forceinline__ bool wd_wait(const WdCta<T> &w, int tile) {
+  const bool ok = mbar_wait(w.bar + tile, tile ? w.ph1 : w.ph0, w.timeout_ns);
   tc_fence_after();
-  return true;
+  return __all_sync(0xffffffffu, ok);
+}
+// End of a round: what it left in shared memory and TMEM has been read.
+template <typename T>
+__device__ __forceinline__ bool wd_round_end(WdCta<T> &w, bool cols2, bool ok) {
+  tc_fence_before();
+  ok = __syncthreads_and(ok);
+  tc_fence_after();
+  if (!ok) {  // once more (bounded), so that no product is in flight when TMEM is freed
+    mbar_wait(w.bar, w.ph0, w.timeout_ns);
+    if (cols2) mbar_wait(w.bar + 1, w.ph1, w.timeout_ns);
+  }
+  w.ph0 ^= 1;
+  w.ph1 ^= cols2 ? 1u : 0u;
+  return ok;
 }
 
 // Four columns of the product from TMEM address `at`, as values.
+__device__ __forceinline__ void tmem_ld2(uint32_t taddr, uint32_t (&r)[2]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(taddr) : "memory");
+}
 template <typename T>
 __device__ __forceinline__ void wd_drain4(uint32_t at, int ea, const int *exb, T (&v)[4]) {
   constexpr int kDig = SliceFmt<T>::kDig;
-  uint32_t acc[kDig][4];
 #pragma unroll
-  for (int q = 0; q < kDig; ++q) tmem_ld4(at + (uint32_t)(q * kSlCols), acc[q]);
-  tmem_ld_wait();
+  for (int c = 0; c < 4; c += 2) {  // two at a time: registers
+    uint32_t acc[kDig][2];
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    float f[kDig];
+    for (int q = 0; q < kDig; ++q) tmem_ld2(at + (uint32_t)(q * kSlCols + c), acc[q]);
+    tmem_ld_wait();
 #pragma unroll
-    for (int q = 0; q < kDig; ++q) f[q] = __uint_as_float(acc[q][e]);
-    v[e] = sl_value(f, ea, exb[e]);
+    for (int e = 0; e < 2; ++e) {
+      float f[kDig];
+#pragma unroll
+      for (int q = 0; q < kDig; ++q) f[q] = __uint_as_float(acc[q][e]);
+      v[c + e] = sl_value(f, ea, exb[c + e]);
+    }
   }
 }
 
@@ -138,37 +169,39 @@ __device__ __forceinline__ void wd_store4(unsigned char *stage, const T (&v)[4],
                                           int cols, bool segs, bool sub) {
   constexpr int kPiece = 16 / sizeof(T), PR = 4 / kPiece;
   const int lane = threadIdx.x & 31;
+  // row r, piece pc: neighbouring groups of four rows swap their pieces, so
+  // that eight lanes meet eight different bank groups
+  auto at = [&](int r, int pc) { return stage + (r * PR + (PR == 2 ? pc ^ ((r >> 2) & 1) : pc)) * 16; };
   __syncwarp();
 #pragma unroll
-  for (int e = 0; e < PR; ++e)
-    *reinterpret_cast<uint4 *>(stage + lane * kWdStageRow<T> + 16 * e) = *reinterpret_cast<const uint4 *>(v + e * kPiece);
+  for (int e = 0; e < PR; ++e) *reinterpret_cast<uint4 *>(at(lane, e)) = *reinterpret_cast<const uint4 *>(v + e * kPiece);
   __syncwarp();
   if (segs) {
 #pragma unroll
     for (int u = 0; u < PR; ++u) {
       const int rr = (32 / PR) * u + lane / PR, pc = lane % PR;
-      uint4 x = *reinterpret_cast<const uint4 *>(stage + rr * kWdStageRow<T> + 16 * pc);
+      uint4 x = *reinterpret_cast<const uint4 *>(at(rr, pc));
       if (rr < rows && pc * kPiece < cols) {
-        uint4 *at = reinterpret_cast<uint4 *>(dst + rr * ld + pc * kPiece);
+        uint4 *o4 = reinterpret_cast<uint4 *>(dst + rr * ld + pc * kPiece);
         if (sub) {
-          uint4 o = __ldcg(at);
+          uint4 o = __ldcg(o4);
           T *ov = reinterpret_cast<T *>(&o);
           const T *xv = reinterpret_cast<const T *>(&x);
 #pragma unroll
           for (int i = 0; i < kPiece; ++i) ov[i] -= xv[i];
           x = o;
         }
-        *at = x;
+        *o4 = x;
       }
     }
   } else {
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int rr = 8 * u + (lane >> 2), c = lane & 3;
-      const T x = *reinterpret_cast<const T *>(stage + rr * kWdStageRow<T> + c * sizeof(T));
+      const T x = *reinterpret_cast<const T *>(at(rr, c / kPiece) + (c % kPiece) * sizeof(T));
       if (rr < rows && c < cols) {
-        T *at = dst + rr * ld + c;
-        *at = sub ? ldcg(at) - x : x;
+        T *o = dst + rr * ld + c;
+        *o = sub ? ldcg(o) - x : x;
       }
     }
   }
@@ -177,19 +210,20 @@ __device__ __forceinline__ void wd_store4(unsigned char *stage, const T (&v)[4],
 // Set up and release of the CTA's tensor-core state.  All threads call.
 template <typename T>
 __device__ __forceinline__ void wd_begin(WdCta<T> &w, unsigned char *smem_raw, uint64_t *bar, uint32_t *s_tmem,
-                                         int *exA, int *exB, int *exP, int *s_ok, long long timeout_ns) {
+                                         int *exA, int *exB, int *exP, long long timeout_ns) {
   w.A = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   w.B = w.A + (size_t)SliceFmt<T>::kDig * kSlASlab;
-  w.stage = w.B + 2 * kWdBBytes<T> + (threadIdx.x >> 5) * 32 * kWdStageRow<T>;
+  w.stage = w.B + (threadIdx.x >> 5) * kWdStage * sizeof(T);
+  static_assert(kWdWarps<T> * kWdStage * sizeof(T) <= (size_t)kWdBBytes<T>, "the stages fit the first B tile");
   w.bar = bar;
   w.exA = exA;
   w.exB = exB;
   w.exP = exP;
-  w.s_ok = s_ok;
-  w.ph = 0;
+  w.ph0 = w.ph1 = 0;
   w.timeout_ns = timeout_ns;
   if (threadIdx.x == 0) {
     mbar_init(bar, 1);
+    mbar_init(bar + 1, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (threadIdx.x < 32) tmem_alloc(s_tmem, kWdTmem<T>);
@@ -207,18 +241,18 @@ __device__ __forceinline__ void wd_end(const WdCta<T> &w) {
 
 #define WD_CTA_SETUP(T)                                                                                   \
   extern __shared__ __align__(16) unsigned char smem_raw[];                                               \
-  __shared__ uint64_t s_bar;                                                                              \
+  __shared__ uint64_t s_bar[2];                                                                           \
   __shared__ uint32_t s_tmem;                                                                             \
-  __shared__ int s_ok, s_go, s_exA[kSlRows], s_exB[kWdTile], s_exP[4 * kSlRows];                          \
+  __shared__ int s_go, s_exA[kSlRows], s_exB[kWdTile], s_exP[64 / kWdCols<T> * kSlRows];                  \
   if (threadIdx.x == 0) s_go = ld_relaxed_i32(&a.st->status) == 0;                                        \
   __syncthreads();                                                                                        \
   if (!s_go) return;                                                                                      \
   WdCta<T> w;                                                                                             \
-  wd_begin(w, smem_raw, &s_bar, &s_tmem, s_exA, s_exB, s_exP, &s_ok, a.timeout_ns);                       \
-  /* this thread drains row `row` (slot row >> 6), 16 columns from 16 hw */                               \
+  wd_begin(w, smem_raw, s_bar, &s_tmem, s_exA, s_exB, s_exP, a.timeout_ns);                               \
+  /* this thread drains row `row` (slot row >> 6), kWdCols columns from column cb */                      \
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, hw = warp >> 2, row0 = 32 * (warp & 3),     \
-            row = row0 + lane;                                                                            \
+            row = row0 + lane, cb = kWdCols<T> * hw, ctile = cb >> 5;                                     \
   const uint32_t lane_base = w.tmem + ((uint32_t)row0 << 16);                                             \
-  const uint32_t acc16 = lane_base + (uint32_t)(hw >> 1) * kWdBufCols<T> + (uint32_t)(16 * (hw & 1));
+  const uint32_t accb = lane_base + (uint32_t)ctile * kWdBufCols<T> + (uint32_t)(cb & 31);
 
 }  // namespace bdss

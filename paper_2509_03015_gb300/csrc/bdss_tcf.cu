@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(kSchurThreads, kSchurCtas<T>)
 #pragma unroll
       for (int o = 1; o < LPR; o <<= 1) ex = max(ex, __shfl_xor_sync(0xffffffffu, ex, o));
     }
-    if (k == 0) *ex_at = ex;
+    if (k == 0) *ex_at = sl_row_exp<T>(ex);
     return ex;
   };
 

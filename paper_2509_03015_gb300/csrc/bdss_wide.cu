@@ -50,20 +50,29 @@ __device__ __forceinline__ Slot<T> no_slot() {
   return {nullptr, 0, 0, 0};
 }
 
+template <typename T>
+__device__ __forceinline__ void load2_cached(const T *p, T &x, T &y) {
+  struct alignas(2 * sizeof(T)) Two { T x, y; };
+  const Two v = *reinterpret_cast<const Two *>(p);
+  x = v.x;
+  y = v.y;
+}
+
 // Digits of the K columns [0, kc) of the slots a0, a1 (A rows 0 .. 63, 64 ..
 // 127; skipped unless do_a) and b (B rows), a warp per row: all loads of the
 // 192 rows first, then the cutting.
 template <typename T>
 __device__ __forceinline__ void wd_cut(const WdCta<T> &w, const Slot<T> &a0, const Slot<T> &a1, const Slot<T> &b,
                                        bool do_a, bool do_b, int kc, bool pairs) {
+  constexpr int kR = 64 / kWdWarps<T>;  // rows of a slot per warp
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, k = 2 * lane;
-  T v[12][2];
+  T v[3 * kR][2];
 #pragma unroll
-  for (int u = 0; u < 12; ++u) {
-    const Slot<T> &s = u < 4 ? a0 : u < 8 ? a1 : b;
-    const int r = (u & 3) * kWdWarps + warp;
+  for (int u = 0; u < 3 * kR; ++u) {
+    const Slot<T> &s = u < kR ? a0 : u < 2 * kR ? a1 : b;
+    const int r = (u % kR) * kWdWarps<T> + warp;
     v[u][0] = v[u][1] = T(0);
-    if ((u < 8 ? do_a : do_b) && r < s.rows && k < kc) {
+    if ((u < 2 * kR ? do_a : do_b) && r < s.rows && k < kc) {
       const T *p = s.p + (r * s.rs + k * s.cs);
       if (pairs && s.cs == 1) {
         load2(p, v[u][0], v[u][1]);
@@ -74,16 +83,16 @@ __device__ __forceinline__ void wd_cut(const WdCta<T> &w, const Slot<T> &a0, con
     }
   }
 #pragma unroll
-  for (int u = 0; u < 12; ++u) {
-    if (!(u < 8 ? do_a : do_b)) continue;
-    const int r = (u & 3) * kWdWarps + warp;
+  for (int u = 0; u < 3 * kR; ++u) {
+    if (!(u < 2 * kR ? do_a : do_b)) continue;
+    const int r = (u % kR) * kWdWarps<T> + warp;
     const int ex = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(sl_exp(v[u][0]), sl_exp(v[u][1])));
-    if (u < 8) {
-      const int ra = 64 * (u >> 2) + r;
-      if (lane == 0) w.exA[ra] = ex;
+    if (u < 2 * kR) {
+      const int ra = 64 * (u / kR) + r;
+      if (lane == 0) w.exA[ra] = sl_row_exp<T>(ex);
       sl_store2<T>(v[u][0], v[u][1], ex, w.A + sl_off(ra, k >> 3) + 2 * (k & 7), kSlASlab);
     } else {
-      if (lane == 0) w.exB[r] = ex;
+      if (lane == 0) w.exB[r] = sl_row_exp<T>(ex);
       sl_store2<T>(v[u][0], v[u][1], ex, w.B + (r >> 5) * kWdBBytes<T> + sl_off(r & 31, k >> 3) + 2 * (k & 7),
                    kSlBSlab);
     }
@@ -121,7 +130,7 @@ __host__ __device__ inline int panel_slots(const WidePanels &P, bool couplings, 
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kWdThreads, sizeof(T) == 8 ? 1 : 2)
+__global__ void __launch_bounds__(kWdThreads<T>, sizeof(T) == 8 ? 1 : 2)
     k_wide_panel(const __grid_constant__ Args<T> a, const WideBuf<T> wb, int l, int k) {
   WD_CTA_SETUP(T)
   const int n = a.p.n;
@@ -141,7 +150,7 @@ __global__ void __launch_bounds__(kWdThreads, sizeof(T) == 8 ? 1 : 2)
     const T *Lk = a.Ld + ((size_t)(j << l) * n + (size_t)k * P.nb) * n;
     const Slot<T> mine = row < 64 ? s0 : s1;
     const int r = row & 63, wrows = mine.rows - (row0 & 63);  // rows of this warp
-    T acc[16];
+    T acc[kWdCols<T>];
 #pragma unroll 1
     for (int rd = 0; rd < k + (nD > 0 ? 3 : 1); ++rd) {
       const int c0 = rd < k ? rd * P.nb : k * P.nb;  // the chunk's first column
@@ -157,12 +166,21 @@ __global__ void __launch_bounds__(kWdThreads, sizeof(T) == 8 ? 1 : 2)
       }
       if ((rd == k && k > 0) || rd == k + 1) {
         if (rd == k) {  // S - sum of the products
-          const T *src = mine.p + (r * mine.rs + (k * P.nb + 16 * hw) * mine.cs);
+          const T *src = mine.p + (r * mine.rs + (k * P.nb + cb) * mine.cs);
 #pragma unroll
-          for (int i = 0; i < 16; ++i)
-            acc[i] = mine.q >= 0                             ? -acc[i]
-                     : r < mine.rows && 16 * hw + i < kb ? ldcg(src + i * mine.cs) - acc[i]
-                                                         : T(0);
+          for (int i = 0; i < kWdCols<T>; i += 2) {  // (plain loads: a sector serves several of them)
+            T x0 = T(0), x1 = T(0);
+            if (mine.q < 0 && r < mine.rows) {
+              if (pairs && mine.cs == 1) {
+                if (cb + i < kb) load2_cached(src + i, x0, x1);
+              } else {
+                if (cb + i < kb) x0 = src[i * mine.cs];
+                if (cb + i + 1 < kb) x1 = src[(i + 1) * mine.cs];
+              }
+            }
+            acc[i] = x0 - acc[i];
+            acc[i + 1] = x1 - acc[i + 1];
+          }
         }
         wd_cut_regs<T>(w, acc, row, hw);
         if (rd == k + 1) __syncthreads();
@@ -171,7 +189,7 @@ __global__ void __launch_bounds__(kWdThreads, sizeof(T) == 8 ? 1 : 2)
         // B tiles: rows 32 h .. 32 h + 31 of either slot
         const int h = rd - k - 1;
 #pragma unroll 4
-        for (int e = threadIdx.x; e < SliceFmt<T>::kDig * 64 * 8; e += kWdThreads) {
+        for (int e = threadIdx.x; e < SliceFmt<T>::kDig * 64 * 8; e += kWdThreads<T>) {
           const int p = e >> 9, rr = (e >> 3) & 63, g = e & 7;
           const int src = 64 * (rr >> 5) + 32 * h + (rr & 31);
           *reinterpret_cast<uint4 *>(w.B + (rr >> 5) * kWdBBytes<T> + p * kSlBSlab + (rr & 31) * 128 + g * 16) =
@@ -179,52 +197,56 @@ __global__ void __launch_bounds__(kWdThreads, sizeof(T) == 8 ? 1 : 2)
         }
       }
       const int ks = ((rd < k ? P.nb : kb) + 15) >> 4;
+      const bool cols2 = rd <= k ? kb > 32 : nD > 1;
       // X is lower triangular: its first 32 rows have 32 columns
-      if (!wd_product<T>(w, rd <= k ? kb > 32 : nD > 1, rd == k ? min(ks, 2) : ks, ks)) {
-        if (threadIdx.x == 0) set_status(a.st, kStTimeout, l, -1);
-        ok = false;
-        break;
-      }
+      wd_issue<T>(w, cols2, rd == k ? min(ks, 2) : ks, ks);
       const int ea = w.exA[row];
       if (rd <= k) {
+        if (cb < kb && wrows > 0) {  // the same for a warp
+          ok = wd_wait<T>(w, ctile);
 #pragma unroll
-        for (int c = 0; c < 16; c += 4) {
-          if (16 * hw + c < kb && wrows > 0) {  // the same for a warp
-            T v[4];
-            wd_drain4<T>(acc16 + c, ea, w.exB + 16 * hw + c, v);
+          for (int c = 0; c < kWdCols<T>; c += 4) {
+            if (cb + c < kb && ok) {
+              T v[4];
+              wd_drain4<T>(accb + c, ea, w.exB + cb + c, v);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) acc[c + e] = rd > 0 && rd < k ? acc[c + e] + v[e] : v[e];
-            if (rd == k) {
-              const int col = k * P.nb + 16 * hw + c;
-              if (mine.cs == 1) {
-                wd_store4<T>(w.stage, v, mine.p + (row0 & 63) * mine.rs + col, mine.rs, wrows,
-                             kb - 16 * hw - c, segs, false);
-                if (mine.q >= 0 && r < mine.rows) {  // L^{-1}: a warp's rows are consecutive columns
-                  T *o = wb.Li + (size_t)(j << l) * n * n + (size_t)col * n + mine.q * P.nb + r;
+              for (int e = 0; e < 4; ++e) acc[c + e] = rd > 0 && rd < k ? acc[c + e] + v[e] : v[e];
+              if (rd == k) {
+                const int col = k * P.nb + cb + c;
+                if (mine.cs == 1) {
+                  wd_store4<T>(w.stage, v, mine.p + (row0 & 63) * mine.rs + col, mine.rs, wrows, kb - cb - c, segs,
+                               false);
+                  if (mine.q >= 0 && r < mine.rows) {  // L^{-1}: a warp's rows are consecutive columns
+                    T *o = wb.Li + (size_t)(j << l) * n * n + (size_t)col * n + mine.q * P.nb + r;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                      if (cb + c + e < kb) o[(size_t)e * n] = v[e];
+                  }
+                } else if (r < mine.rows) {
 #pragma unroll
                   for (int e = 0; e < 4; ++e)
-                    if (16 * hw + c + e < kb) o[(size_t)e * n] = v[e];
+                    if (cb + c + e < kb) mine.p[(col + e) * mine.cs + r * mine.rs] = v[e];
                 }
-              } else if (r < mine.rows) {
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                  if (16 * hw + c + e < kb) mine.p[(col + e) * mine.cs + r * mine.rs] = v[e];
               }
-            }
-          } else {
+            } else {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) acc[c + e] = T(0);
+              for (int e = 0; e < 4; ++e) acc[c + e] = T(0);
+            }
           }
+        } else {
+#pragma unroll
+          for (int c = 0; c < kWdCols<T>; ++c) acc[c] = T(0);
         }
       } else if ((row >> 6) < nD) {
         // columns 32 h .. of the diagonal tile of each slot of D, lower part
-        const int h = rd - k - 1;
+        const int h = rd - k - 1, cd = kWdCols<T> / 2 * hw;
+        ok = wd_wait<T>(w, row >> 6);
 #pragma unroll
-        for (int c = 0; c < 8; c += 4) {
-          const int col = 32 * h + 8 * hw + c;
-          if (col < mine.rows && wrows > 0 && col <= (r | 31)) {
+        for (int c = 0; c < kWdCols<T> / 2; c += 4) {
+          const int col = 32 * h + cd + c;
+          if (ok && col < mine.rows && wrows > 0 && col <= (r | 31)) {
             T v[4];
-            wd_drain4<T>(lane_base + (uint32_t)(row >> 6) * kWdBufCols<T> + (uint32_t)(8 * hw + c), ea,
+            wd_drain4<T>(lane_base + (uint32_t)(row >> 6) * kWdBufCols<T> + (uint32_t)(cd + c), ea,
                          w.exA + (row & 64) + col, v);
             const int ib = k + 1 + i0 + (row >> 6);
             wd_store4<T>(w.stage, v, mine.p + (row0 & 63) * mine.rs + ib * P.nb + col, mine.rs, wrows,
@@ -232,10 +254,12 @@ __global__ void __launch_bounds__(kWdThreads, sizeof(T) == 8 ? 1 : 2)
           }
         }
       }
-      // the exponents and slabs of the round have been read before the next one's
-      tc_fence_before();
-      __syncthreads();
-      tc_fence_after();
+      // the exponents, slabs and stages of the round have been read before the next one's
+      ok = wd_round_end<T>(w, cols2, ok);
+      if (!ok) {
+        if (threadIdx.x == 0) set_status(a.st, kStTimeout, l, -1);
+        break;
+      }
     }
   }
   wd_end(w);
@@ -254,7 +278,7 @@ __host__ __device__ inline int schur_tiles(int nt, int d) {
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kWdThreads, sizeof(T) == 8 ? 1 : 2)
+__global__ void __launch_bounds__(kWdThreads<T>, sizeof(T) == 8 ? 1 : 2)
     k_wide_schur(const __grid_constant__ Args<T> a, int l) {
   WD_CTA_SETUP(T)
   const int n = a.p.n, d = a.d;
@@ -294,9 +318,9 @@ __global__ void __launch_bounds__(kWdThreads, sizeof(T) == 8 ? 1 : 2)
     const int bcols = isR ? d : min(nb, n - jb * nb);  // output columns
     const int first = (isE || hasM) ? 0 : nt, last = (isE || !hasP) ? nt : 2 * nt;
     const int r = row & 63, rows = row < 64 ? rows0 : rows1, wrows = rows - (row0 & 63);
-    T acc[16];
+    T acc[kWdCols<T>];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) acc[i] = T(0);
+    for (int i = 0; i < kWdCols<T>; ++i) acc[i] = T(0);
 #pragma unroll 1
     for (int rd = first; rd < last; ++rd) {
       const int second = rd >= nt, p = rd - second * nt, c0 = p * nb, kc = min(nb, n - c0);
@@ -312,45 +336,48 @@ __global__ void __launch_bounds__(kWdThreads, sizeof(T) == 8 ? 1 : 2)
       }
       wd_cut<T>(w, s0, s1, b, true, true, kc, pairs);
       const int ks = (kc + 15) >> 4;
-      if (!wd_product<T>(w, bcols > 32, ks, ks)) {
+      const bool cols2 = bcols > 32;
+      wd_issue<T>(w, cols2, ks, ks);
+      const int ea = w.exA[row];
+      if (cb < bcols && wrows > 0) {  // the same for a warp
+        ok = wd_wait<T>(w, ctile);
+#pragma unroll
+        for (int c = 0; c < kWdCols<T>; c += 4)
+          if (cb + c < bcols && ok) {
+            T v[4];
+            wd_drain4<T>(accb + c, ea, w.exB + cb + c, v);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[c + e] += v[e];
+          }
+      }
+      ok = wd_round_end<T>(w, cols2, ok);
+      if (!ok) {
         if (threadIdx.x == 0) set_status(a.st, kStTimeout, l, -1);
-        ok = false;
         break;
       }
-      const int ea = w.exA[row];
-#pragma unroll
-      for (int c = 0; c < 16; c += 4)
-        if (16 * hw + c < bcols && wrows > 0) {
-          T v[4];
-          wd_drain4<T>(acc16 + c, ea, w.exB + 16 * hw + c, v);
-#pragma unroll
-          for (int e = 0; e < 4; ++e) acc[c + e] += v[e];
-        }
-      tc_fence_before();
-      __syncthreads();
-      tc_fence_after();
     }
     if (!ok) break;
     if (isR) {
       if (r < rows) {
-        T *y = a.Y + ((size_t)orig * n + ra + (row & 64 ? nb : 0) + r) * d + 16 * hw;
+        T *y = a.Y + ((size_t)orig * n + ra + (row & 64 ? nb : 0) + r) * d + cb;
 #pragma unroll
-        for (int i = 0; i < 16; ++i)
-          if (16 * hw + i < d) y[i] = ldcg(y + i) - acc[i];
+        for (int i = 0; i < kWdCols<T>; ++i)
+          if (cb + i < d) y[i] = ldcg(y + i) - acc[i];
       }
       continue;
     }
     T *dst = isE ? a.Wb + ((size_t)a.p.off[l + 1] + (size_t)q) * nn : a.Ld + (size_t)orig * nn;
     const int rw = ra + (row & 64 ? nb : 0) + (row0 & 63);  // the warp's first row
 #pragma unroll
-    for (int c = 0; c < 16; c += 4) {
-      const int col = jb * nb + 16 * hw + c;
-      if (16 * hw + c >= bcols || wrows <= 0 || (isD && col > rw + 31)) continue;  // the same for a warp
+    for (int c = 0; c < kWdCols<T>; c += 4) {
+      const int col = jb * nb + cb + c;
+      if (cb + c >= bcols || wrows <= 0 || (isD && col > rw + 31)) continue;  // the same for a warp
       T v[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) v[e] = isE ? -acc[c + e] : acc[c + e];
-      wd_store4<T>(w.stage, v, dst + (size_t)rw * n + col, n, wrows, bcols - 16 * hw - c, segs, isD);
+      wd_store4<T>(w.stage, v, dst + (size_t)rw * n + col, n, wrows, bcols - cb - c, segs, isD);
     }
+    __syncthreads();  // the stages have been read before the next task's B digits take their place
   }
   wd_end(w);
 }
@@ -647,14 +674,14 @@ cudaError_t launch_wide_panel(const Args<T> &a, const WideBuf<T> &w, int l, int 
   const bool top = l == a.p.L;
   const long long tasks = (top ? 1 : a.p.Nl[l] / 2) * ((panel_slots(P, !top, k, a.d, w.Li != nullptr) + 1) / 2);
   if (tasks == 0) return cudaSuccess;  // the last panel of the top block without right-hand sides
-  k_wide_panel<T><<<wd_grid(tasks, sizeof(T) == 8 ? sms : 2 * sms), kWdThreads, wd_smem<T>(), s>>>(a, w, l, k);
+  k_wide_panel<T><<<wd_grid(tasks, sizeof(T) == 8 ? sms : 2 * sms), kWdThreads<T>, wd_smem<T>(), s>>>(a, w, l, k);
   return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_wide_schur(const Args<T> &a, int l, int sms, cudaStream_t s) {
   const long long tasks = (a.p.Nl[l] + 1) / 2 * schur_tiles(panels_of(a.p.n).nt, a.d);
-  k_wide_schur<T><<<wd_grid(tasks, sizeof(T) == 8 ? sms : 2 * sms), kWdThreads, wd_smem<T>(), s>>>(a, l);
+  k_wide_schur<T><<<wd_grid(tasks, sizeof(T) == 8 ? sms : 2 * sms), kWdThreads<T>, wd_smem<T>(), s>>>(a, l);
   return cudaGetLastError();
 }
 
