@@ -533,7 +533,7 @@ template <typename T>
 static cudaError_t tcf_down(bdss_ctx *h, const Args<T> &b) {
   cudaError_t e = cudaSuccess;
   kt_begin(h, h->kt_cls);
-  for (int l = h->plan.L - 1; l >= 0 && e == cudaSuccess; --l) e = launch_tcf_down<T>(b, l, h->stream);
+  for (int l = h->plan.L - 1; l >= 0 && e == cudaSuccess; --l) e = launch_tcf_down<T>(b, l, h->sms, h->stream);
   kt_end(h, h->plan.L);
   h->launches += h->plan.L;
   return e;
@@ -578,8 +578,8 @@ template <typename T>
 static cudaError_t run_solve_tcf(bdss_ctx *h, const Args<T> &b) {
   const Plan &p = h->plan;
   kt_begin(h, h->kt_cls);
-  cudaError_t e = launch_tcf_up<T>(b, 0, 1, h->stream);
-  for (int l = 0; l < p.L && e == cudaSuccess; ++l) e = launch_tcf_up<T>(b, l, 0, h->stream);
+  cudaError_t e = launch_tcf_up<T>(b, 0, 1, h->sms, h->stream);
+  for (int l = 0; l < p.L && e == cudaSuccess; ++l) e = launch_tcf_up<T>(b, l, 0, h->sms, h->stream);
   if (e == cudaSuccess) e = launch_top<T>(b, 0, h->smem, h->stream);
   kt_end(h, p.L + 2);
   h->launches += p.L + 2;

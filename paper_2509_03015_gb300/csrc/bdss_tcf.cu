@@ -23,7 +23,7 @@
 // eliminated blocks) are left transposed, so that every row of the second
 // kernel's operands is contiguous.
 #include "bdss_launch.h"
-#include "bdss_slice.cuh"
+#include "bdss_slice_cta.cuh"
 #include "bdss_tcf.h"
 
 namespace bdss {
@@ -614,6 +614,167 @@ __global__ void __launch_bounds__(256, 2) k_tcf_solve(const __grid_constant__ Ar
   }
 }
 
+// k_tcf_solve for many right-hand sides (FP64): the products with W as digit
+// products, 16 columns at a time, the triangular one on the ALU.  One block a
+// tile: its 128 A rows are the rows (up) or columns (down) of its two W, each
+// multiplied by its own neighbour's vectors (B tile 0 or 1), so the halves of
+// the result are added.
+//
+// With 16 columns the FP64 ALU needs 2.5 n^2 d multiply-adds a block and way
+// (82,000 cycles at n = 64); here cutting W (the same for any d) and 16k cycles
+// of triangular product remain.
+constexpr int kTcRhs = 16;
+constexpr int kTcLdX = kMaxN + 1;
+constexpr size_t kTcSolveSmem = 8 * kSlASlab + 2 * 8 * kTcRhs * 128 +
+                                (size_t)(kSlRows * kTcRhs + kMaxN * kTcRhs + kMaxN * kTcLdX) * sizeof(double) + 1024;
+template <bool kUp>
+__global__ void __launch_bounds__(1024, 1) k_tcf_solve_tc(const __grid_constant__ Args<double> a, int l, int first) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint64_t s_bar[2];
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_go, s_exA[kSlRows], s_exB[2 * kTcRhs], s_exP[8 * kSlRows];
+  if (threadIdx.x == 0) s_go = ld_relaxed_i32(&a.st->status) == 0;
+  __syncthreads();
+  if (!s_go) return;
+  WdCta<double> w;
+  wd_begin(w, smem_raw, s_bar, &s_tmem, s_exA, s_exB, s_exP, a.timeout_ns);
+  constexpr int kTileB = 8 * kTcRhs * 128;  // bytes of a B tile's digits
+  double *red = reinterpret_cast<double *>(w.B + 2 * kTileB), *sT = red + kSlRows * kTcRhs, *sX = sT + kMaxN * kTcRhs;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, hw = warp >> 2, row0 = 32 * (warp & 3), row = row0 + lane;
+  const uint32_t lane_base = w.tmem + ((uint32_t)row0 << 16);
+  const int n = a.p.n, d = a.d, ks = (n + 15) >> 4;
+  const size_t nn = (size_t)n * n, nd = (size_t)n * d;
+  const long long Nl = a.p.Nl[l], count = !kUp || first ? Nl / 2 : (Nl + 1) / 2;
+  const bool pairs = (n & 1) == 0;
+  bool ok = true;
+  for (long long m = blockIdx.x; m < count && ok; m += gridDim.x) {
+    const long long pos = kUp && !first ? 2 * m : 2 * m + 1, orig = pos << l;
+    const bool hasM = !first && pos >= 1, hasP = !first && pos + 1 < Nl;
+    const bool tri = !kUp || first || (m & 1), raw = kUp && l == 0 && (a.B64 || a.Bt);
+    const double *W0 = a.Wb + (size_t)(a.p.off[l] + pos - 1) * nn, *W1 = W0 + nn;
+    // X (FP64 keeps X^T above the diagonal of Ld): X[i][q] at sX[q kTcLdX + i], q <= i
+    double xv[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int q = (tid >> 6) + 16 * u, i = tid & 63;
+      xv[u] = tri && i < n && q <= i ? ldcg(a.Ld + (size_t)orig * nn + (size_t)q * n + i) : 0.0;
+    }
+    if (hasM || hasP) {
+      if constexpr (kUp) {  // rows of W^T, a warp per row
+        double v[4][2];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int r = 32 * u + warp, k = 2 * lane, i = r & 63;
+          const double *src = (r < 64 ? W0 : W1) + (size_t)i * n + k;
+          v[u][0] = v[u][1] = 0.0;
+          if ((r < 64 ? hasM : hasP) && i < n && k < n) {
+            if (pairs) {
+              const double2 x = __ldcg(reinterpret_cast<const double2 *>(src));
+              v[u][0] = x.x;
+              v[u][1] = x.y;
+            } else {
+              v[u][0] = ldcg(src);
+              if (k + 1 < n) v[u][1] = ldcg(src + 1);
+            }
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int r = 32 * u + warp, k = 2 * lane;
+          const int ex = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(sl_exp(v[u][0]), sl_exp(v[u][1])));
+          if (lane == 0) w.exA[r] = sl_row_exp<double>(ex);
+          sl_store2<double>(v[u][0], v[u][1], ex, w.A + sl_off(r, k >> 3) + 2 * (k & 7), kSlASlab);
+        }
+      } else {  // columns of W^T: thread (column, eight K entries)
+        const int c = tid & 63, g = (tid >> 6) & 7, half = tid >> 9;
+        const double *src = half ? W1 : W0;
+        double v[8];
+        int ex = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int p = 8 * g + i;
+          v[i] = (half ? hasP : hasM) && c < n && p < n ? ldcg(src + (size_t)p * n + c) : 0.0;
+          ex = max(ex, sl_exp(v[i]));
+        }
+        w.exP[g * kSlRows + 64 * half + c] = ex;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 8; ++q) ex = max(ex, w.exP[q * kSlRows + 64 * half + c]);
+        if (g == 0) w.exA[64 * half + c] = sl_row_exp<double>(ex);
+        store8<double>(v, ex, w.A + sl_off(64 * half + c, g), kSlASlab);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) sX[((tid >> 6) + 16 * u) * kTcLdX + (tid & 63)] = xv[u];
+    for (int d0 = 0; d0 < d && ok; d0 += kTcRhs) {
+      const int i = tid >> 4, c = tid & 15;  // the result entry this thread forms
+      const bool in = i < n && d0 + c < d;
+      const size_t o = (size_t)orig * nd + (size_t)i * d + d0 + c;
+      double t = !in ? 0.0 : !raw ? ldcg(a.Y + o) : a.B64 ? ldcg(a.B64 + o) : ldcg(a.Bt + o);
+      if (hasM || hasP) {
+        // B row of this warp: column d0 + r of the neighbour's vectors
+        const int r = warp & 15, side = warp >> 4, k = 2 * lane;
+        const double *src = a.Y + (size_t)((side ? pos + 1 : pos - 1) << l) * nd + d0 + r;
+        const bool live = (side ? hasP : hasM) && d0 + r < d;
+        const double v0 = live && k < n ? src[(size_t)k * d] : 0.0, v1 = live && k + 1 < n ? src[(size_t)(k + 1) * d] : 0.0;
+        const int ex = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(sl_exp(v0), sl_exp(v1)));
+        if (lane == 0) w.exB[warp] = sl_row_exp<double>(ex);
+        sl_store2<double>(v0, v1, ex, w.B + side * kTileB + sl_off(r, k >> 3) + 2 * (k & 7), kTcRhs * 128);
+        fence_proxy_async_smem();
+        tc_fence_before();
+        __syncthreads();
+        if (tid == 0) {
+          tc_fence_after();
+          sl_issue<double>(w.tmem, w.A, w.B, kTcRhs, ks);
+          sl_issue<double>(w.tmem + 256, w.A, w.B + kTileB, kTcRhs, ks);
+          tc_commit(w.bar);
+        }
+        __syncwarp();
+        ok = wd_wait<double>(w, 0);
+        if (ok) {
+          uint32_t acc[8][2];
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            tmem_ld2(lane_base + (uint32_t)((row >> 6) * 256 + q * kTcRhs + 2 * hw), acc[q]);
+          tmem_ld_wait();
+          const int ea = w.exA[row];
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            float f[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) f[q] = __uint_as_float(acc[q][e]);
+            red[row * kTcRhs + 2 * hw + e] = sl_value(f, ea, w.exB[(row >> 6) * kTcRhs + 2 * hw + e]);
+          }
+        }
+        ok = wd_round_end<double>(w, false, ok);
+        if (!ok) {
+          if (tid == 0) set_status(a.st, kStTimeout, l, -1);
+          break;
+        }
+        t -= red[i * kTcRhs + c] + red[(64 + i) * kTcRhs + c];
+      }
+      if (!tri) {
+        if (in) a.Y[o] = t;
+      } else {
+        sT[i * kTcRhs + c] = in ? t : 0.0;
+        __syncthreads();
+        if (in) {
+          double x = 0.0;
+          if constexpr (kUp) {
+            for (int q = 0; q <= i; ++q) x = fma(sX[q * kTcLdX + i], sT[q * kTcRhs + c], x);
+          } else {
+            for (int q = i; q < n; ++q) x = fma(sX[i * kTcLdX + q], sT[q * kTcRhs + c], x);
+          }
+          a.Y[o] = x;
+          if (!kUp && a.X64) a.X64[o] = a.x_accumulate ? a.X64[o] + x : x;
+        }
+      }
+      __syncthreads();
+    }
+  }
+  wd_end(w);
+}
+
 size_t diag_smem(int n, int d, size_t esz) { const int np = (n + 7) & ~7;
   return ((size_t)(np + d) * ldstride(np) + 17 * kMaxN) * esz; }
 
@@ -633,6 +794,14 @@ cudaError_t tcf_configure(int n, int d) {
       e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
     if (e == cudaSuccess && k != kernels[0] && k != kernels[1] && schur_smem<T>() > (size_t)optin - fa.sharedSizeBytes)
       e = cudaErrorInvalidConfiguration;
+  }
+  if (sizeof(T) == 8) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute((const void *)k_tcf_solve_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)kTcSolveSmem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute((const void *)k_tcf_solve_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)kTcSolveSmem);
   }
   if (e == cudaSuccess && diag_smem(n, d, sizeof(T)) > (size_t)optin - 64) e = cudaErrorInvalidConfiguration;
   return e;
@@ -669,15 +838,33 @@ cudaError_t launch_tcf_top(const Args<T> &a, const TcfLevel<T> &c, cudaStream_t 
   return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_tcf_up(const Args<T> &a, int l, int first, cudaStream_t s) {
-  k_tcf_solve<T, true><<<(unsigned)(first ? a.p.Nl[l] / 2 : (a.p.Nl[l] + 1) / 2), 256, 0, s>>>(a, l, first);
+// Solve passes with more than kTcMinRhs right-hand sides take the digit
+// products (measured at N = 4096, n = 64, both passes: d = 16, see k_tcf_solve_tc).
+constexpr int kTcMinRhs = 8;
+template <bool kUp>
+static cudaError_t launch_solve_tc(const Args<double> &a, int l, int first, long long count, int sms, cudaStream_t s) {
+  const unsigned grid = (unsigned)(count < sms ? count : sms);
+  k_tcf_solve_tc<kUp><<<grid, 1024, kTcSolveSmem, s>>>(a, l, first);
   return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t launch_tcf_down(const Args<T> &a, int l, cudaStream_t s) {
-  k_tcf_solve<T, false><<<(unsigned)(a.p.Nl[l] / 2), 256, 0, s>>>(a, l, 0);
+cudaError_t launch_tcf_up(const Args<T> &a, int l, int first, int sms, cudaStream_t s) {
+  const long long count = first ? a.p.Nl[l] / 2 : (a.p.Nl[l] + 1) / 2;
+  if constexpr (sizeof(T) == 8) {
+    if (a.d > kTcMinRhs) return launch_solve_tc<true>(a, l, first, count, sms, s);
+  }
+  k_tcf_solve<T, true><<<(unsigned)count, 256, 0, s>>>(a, l, first);
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_tcf_down(const Args<T> &a, int l, int sms, cudaStream_t s) {
+  const long long count = a.p.Nl[l] / 2;
+  if constexpr (sizeof(T) == 8) {
+    if (a.d > kTcMinRhs) return launch_solve_tc<false>(a, l, 0, count, sms, s);
+  }
+  k_tcf_solve<T, false><<<(unsigned)count, 256, 0, s>>>(a, l, 0);
   return cudaGetLastError();
 }
 
@@ -686,8 +873,8 @@ cudaError_t launch_tcf_down(const Args<T> &a, int l, cudaStream_t s) {
   template cudaError_t launch_tcf_diag<T>(const Args<T> &, const TcfLevel<T> &, int, int, int, cudaStream_t); \
   template cudaError_t launch_tcf_schur<T>(const Args<T> &, const TcfLevel<T> &, int, int, cudaStream_t);        \
   template cudaError_t launch_tcf_top<T>(const Args<T> &, const TcfLevel<T> &, cudaStream_t);                     \
-  template cudaError_t launch_tcf_up<T>(const Args<T> &, int, int, cudaStream_t);                                 \
-  template cudaError_t launch_tcf_down<T>(const Args<T> &, int, cudaStream_t);
+  template cudaError_t launch_tcf_up<T>(const Args<T> &, int, int, int, cudaStream_t);                                 \
+  template cudaError_t launch_tcf_down<T>(const Args<T> &, int, int, cudaStream_t);
 BDSS_TCF_INSTANTIATE(double)
 BDSS_TCF_INSTANTIATE(float)
 

@@ -31,7 +31,7 @@ cudaError_t launch_tcf_schur(const Args<T> &a, const TcfLevel<T> &c, int l, int 
 template <typename T> cudaError_t launch_tcf_top(const Args<T> &a, const TcfLevel<T> &c, cudaStream_t s);
 // One level of a solve pass over stored factors that hold X (after launch_tcf_diag;
 // in FP32 after any factorisation): up (first: y of level 0) and down.
-template <typename T> cudaError_t launch_tcf_up(const Args<T> &a, int l, int first, cudaStream_t s);
-template <typename T> cudaError_t launch_tcf_down(const Args<T> &a, int l, cudaStream_t s);
+template <typename T> cudaError_t launch_tcf_up(const Args<T> &a, int l, int first, int sms, cudaStream_t s);
+template <typename T> cudaError_t launch_tcf_down(const Args<T> &a, int l, int sms, cudaStream_t s);
 
 }  // namespace bdss
