@@ -33,15 +33,12 @@ struct bdss_ctx {
   Plan plan{};
   int sms = 0;
   int bps = 0;          // resident CTAs per SM of the persistent kernel
-  int bps_tc = 0;       // the same for the tiled path's tensor-core kernel (TF32 factor)
   size_t smem = 0;      // dynamic shared memory per CTA
   // workspace
   bool large = false;   // 64 < n <= 256: tiled path
   void *Ld = nullptr;   // N n n  (T)
   void *Wb = nullptr;   // coupling slots (T)
   void *Eb = nullptr;   // large path: couplings of levels >= 1 (T)
-  int tf32 = 0;         // TF32 mode on the large path: tensor-core Schur tiles
-  CUtensorMap *d_tmap = nullptr;  // TMA map of Wb (device copy)
   double *Ltop = nullptr;
   void *Li = nullptr;    // large mixed path: L^{-1} of the eliminated blocks (N n n, FP32)
   float *Yt = nullptr;   // large mixed path: y of the eliminated blocks in solve passes (N n d_max)
@@ -99,9 +96,6 @@ struct bdss_ctx {
   CorrMaps corr_maps[3];  // split factors P = 1, 2, 4
   int corr_max_split = 1;
   int corr_ok = 0;
-  // TF32 mode: the pipelined 3xTF32 Schur tiles read W through this map
-  CUtensorMap ts_map_w;
-  int ts_ok = 0;
   bool emu_sliced = false;
   int skip_barrier = 0;
   // one-cluster path for short systems (FP64, n <= 32, d_max <= 16)
@@ -295,21 +289,28 @@ static bool use_small(const bdss_ctx *h) {
 }
 
 // Factorisations of n <= 64 blocks with the coupling solves and Schur
-// products on the tensor cores: on request, or by size.  A level costs two
-// launches and the full latency of one block in each, so the path needs many
-// blocks; its gain per block grows with n.  Measured on GB300, d = 1 (the
-// tensor-core path's time over the persistent kernel's): n = 64, N = 4096:
-// 0.57; n = 48, N = 4096: 0.78; n = 32, N = 8192: 0.94, N = 2048: 1.03;
-// n = 24, N = 2000: 1.16.
+// products on the tensor cores: on request, or by size.  A level costs three
+// launches and the full latency of one block in each, so in FP64 the path
+// needs large blocks or many; its gain per block grows with n.  Measured on
+// GB300, d = 1, factor + solve (the tensor-core path's time over the persistent
+// kernel's):
+//   FP64   N = 128  512  2048  8192        FP32   N = 32  512  8192
+//   n = 32   1.18  1.09  1.00  0.92        n = 20   0.71  0.89  0.89
+//   n = 40   1.11  1.01  0.95  0.91        n = 24   0.89  0.84  0.84
+//   n = 48   0.93  0.82  0.73  0.67        n = 48   0.78  0.68  0.74
+//   n = 64   0.68  0.57  0.47  0.42        n = 64   0.70  0.60  0.69
+// (n = 37, whose odd rows cannot be read in pairs, 1.05 at N = 8192.)  Handles
+// for several right-hand sides keep the single launch up to N = 1536: their
+// callers count on one.
 constexpr int kTcfMinN = 32;
-constexpr int kTcfAutoMinN = 40;
-constexpr int kTcfAutoMinBlocks = 1536;
-constexpr int kTcfAutoMinN32 = 24;
-constexpr int kTcfAutoMinBlocks32 = 32;
+constexpr int kTcfAutoMinN = 40, kTcfAutoMinBlocks = 1536;
+constexpr int kTcfAutoMinN1 = 48, kTcfAutoMinBlocks1 = 128;  // one right-hand side
+constexpr int kTcfAutoMinN32 = 20, kTcfAutoMinBlocks32 = 32;  // FP32
 static bool tcf_by_size(const bdss_ctx *h) {
   if (h->large) return false;
   if (is_mixed(h)) return h->n >= kTcfAutoMinN32 && h->N >= kTcfAutoMinBlocks32;
-  return h->n >= kTcfAutoMinN && h->N >= kTcfAutoMinBlocks;
+  return (h->n >= kTcfAutoMinN && h->N >= kTcfAutoMinBlocks) ||
+         (h->d_max == 1 && h->n >= kTcfAutoMinN1 && h->N >= kTcfAutoMinBlocks1);
 }
 static bool use_tcf(const bdss_ctx *h) {
   if (!h->tcf_ready || h->plan.L < 1) return false;
@@ -379,8 +380,6 @@ static Args<T> base_args(bdss_ctx *h) {
   a.timeout_ns = h->timeout_ns;
   a.skip_barrier = h->skip_barrier;
   a.capacity = h->bps * h->sms;
-  a.tf32 = h->tf32;
-  a.tmap_w = h->d_tmap;
   a.Li = (T *)h->Li;
   a.Ltinv = (T *)h->Ltinv;
   return a;
@@ -435,7 +434,7 @@ static cudaError_t wide_down_f32(bdss_ctx *h, const Args<float> &b) {
   cudaError_t e = cudaSuccess;
   for (int l = p.L - 1; l >= 0 && e == cudaSuccess; --l) {
     kt_begin(h, h->kt_cls);
-    e = launch_large_sub<float>(b, l, 3, 0, grid_for(h, large_sub_tasks(p, l, 3, 0, b.d, 4, 0, 1)), h->smem, h->stream);
+    e = launch_large_sub<float>(b, l, 3, 0, grid_for(h, large_sub_tasks(p, l, 3, 0, b.d, 4, 1)), h->smem, h->stream);
     kt_end(h, 1);
     h->launches += 1;
   }
@@ -586,39 +585,12 @@ static cudaError_t run_solve_tcf(bdss_ctx *h, const Args<T> &b) {
   return e == cudaSuccess ? tcf_down<T>(h, b) : e;
 }
 
-// Separator update of level l in the TF32 mode: the D and E tiles on the
-// pipelined tensor-core kernel, then the separators' RHS tiles on the ALU.
-static cudaError_t schur_tf32_level(bdss_ctx *h, const Args<float> &b, int l) {
-  const Plan &p = h->plan;
-  kt_begin(h, BDSS_KT_SCHUR_TC);
-  cudaError_t e = launch_tf32_schur(h->ts_map_w, b, l, h->sms, h->stream);
-  kt_end(h, 1);
-  h->launches += 1;
-  if (e != cudaSuccess || b.d == 0) return e;
-  kt_begin(h, h->kt_cls);
-  // b_s -= W^T y of the neighbours: the streamed product of the solve passes
-  // (the factor pass keeps y in Y), else the RHS tiles
-  if (h->corr_ok && b.d <= kCorrMaxD)
-    e = launch_large_corr(h->corr_maps, h->corr_max_split, b, l, kSubB, h->sms, h->stream);
-  else
-    e = launch_large_sub<float>(b, l, kSubBRhsOnly, 1,
-                                grid_for(h, large_sub_tasks(p, l, kSubBRhsOnly, 1, b.d, 4, 0, 0)), h->smem, h->stream);
-  kt_end(h, 1);
-  h->launches += 1;
-  return e;
-}
-
 // One factor and/or RHS pass over all levels, persistent or per level.
 // Large-block path: three tile sub-phases per level (see bdss_large.cu).
 template <typename T>
 static cudaError_t run_levels_large(bdss_ctx *h, const Args<T> &a, bool factor, bool rhs) {
   const Plan &p = h->plan;
   const int esz = (int)sizeof(T);
-  // The TF32 factorisation runs sub-phase by sub-phase even in persistent
-  // mode: a kernel holding tcgen05 code gets one CTA per SM, so only the
-  // Schur-update tiles use that kernel and the Cholesky / substitution tasks
-  // keep the two-CTA FP32 kernel.
-  const bool tc_factor = sizeof(T) == 4 && h->tf32 && factor;
   const int inv = a.Li ? 1 : 0;
   Args<T> b = a;
   if (!rhs) b.d = 0;
@@ -628,11 +600,11 @@ static cudaError_t run_levels_large(bdss_ctx *h, const Args<T> &a, bool factor, 
   if constexpr (sizeof(T) == 4) {
     if (!factor && rhs && inv && h->corr_ok && b.d <= kCorrMaxD) return run_corr_passes(h, b);
   }
-  if (h->persistent && !tc_factor) {
+  if (h->persistent) {
     long long most = 1;
     for (int l = 0; l < p.L; ++l)
       for (int sub = 0; sub < 4; ++sub) {
-        const long long t = large_sub_tasks(p, l, sub, factor ? 1 : 0, rhs ? a.d : 0, esz, h->tf32, inv);
+        const long long t = large_sub_tasks(p, l, sub, factor ? 1 : 0, rhs ? a.d : 0, esz, inv);
         if (t > most) most = t;
       }
     h->launches += 1;
@@ -647,14 +619,8 @@ static cudaError_t run_levels_large(bdss_ctx *h, const Args<T> &a, bool factor, 
   cudaError_t e = cudaSuccess;
   for (int l = 0; l < p.L && e == cudaSuccess; ++l)
     for (int sub = factor ? 0 : 1; sub < 3 && e == cudaSuccess; ++sub) {
-      if constexpr (sizeof(T) == 4) {
-        if (tc_factor && sub == 2 && h->ts_ok) {
-          e = schur_tf32_level(h, b, l);
-          continue;
-        }
-      }
-      kt_begin(h, (tc_factor && sub == 2) ? BDSS_KT_SCHUR_TC : h->kt_cls);
-      e = launch_large_sub<T>(b, l, sub, f, grid_for(h, large_sub_tasks(p, l, sub, f, b.d, esz, h->tf32, inv)),
+      kt_begin(h, h->kt_cls);
+      e = launch_large_sub<T>(b, l, sub, f, grid_for(h, large_sub_tasks(p, l, sub, f, b.d, esz, inv)),
                               h->smem, h->stream);
       kt_end(h, 1);
       h->launches += 1;
@@ -666,7 +632,7 @@ static cudaError_t run_levels_large(bdss_ctx *h, const Args<T> &a, bool factor, 
   if (rhs)
     for (int l = p.L - 1; l >= 0 && e == cudaSuccess; --l) {
       kt_begin(h, h->kt_cls);
-      e = launch_large_sub<T>(b, l, 3, 0, grid_for(h, large_sub_tasks(p, l, 3, 0, b.d, esz, 0, inv)), h->smem,
+      e = launch_large_sub<T>(b, l, 3, 0, grid_for(h, large_sub_tasks(p, l, 3, 0, b.d, esz, inv)), h->smem,
                               h->stream);
       kt_end(h, 1);
       h->launches += 1;
@@ -747,7 +713,6 @@ bdss_status bdss_destroy(bdss_handle h) {
   cudaFree(h->Ld);
   cudaFree(h->Wb);
   cudaFree(h->Eb);
-  cudaFree(h->d_tmap);
   cudaFree(h->Ltop);
   cudaFree(h->emu.Aslc);
   cudaFree(h->emu.Aexp);
@@ -811,13 +776,12 @@ bdss_status bdss_create(bdss_handle *out, int64_t N, int32_t n, int32_t d_max, b
   if (h->large) {
     e = configure<double>(1, 1, &h->smem, &h->bps);  // raises every kernel's shared-memory limit
     if (e == cudaSuccess)
-      e = is_mixed(h) ? configure_large<float>(n, d_max, &h->smem, &h->bps, &h->bps_tc)
-                      : configure_large<double>(n, d_max, &h->smem, &h->bps, &h->bps_tc);
+      e = is_mixed(h) ? configure_large<float>(n, d_max, &h->smem, &h->bps)
+                      : configure_large<double>(n, d_max, &h->smem, &h->bps);
   } else {
     e = is_mixed(h) ? configure<float>(n, d_max, &h->smem, &h->bps) : configure<double>(n, d_max, &h->smem, &h->bps);
   }
-  if (e == cudaSuccess && !h->large) h->bps_tc = h->bps;
-  if (e != cudaSuccess || h->bps < 1 || h->bps_tc < 1) {
+  if (e != cudaSuccess || h->bps < 1) {
     bdss_destroy(h);
     return cuda_fail(e != cudaSuccess ? e : cudaErrorInvalidConfiguration);
   }
@@ -834,18 +798,6 @@ bdss_status bdss_create(bdss_handle *out, int64_t N, int32_t n, int32_t d_max, b
   ok = ok && ws_alloc(h, (void **)&h->partial, kLogdetGrid * sizeof(double));
   ok = ok && ws_alloc(h, (void **)&h->dst, sizeof(DevStatus));
   ok = ok && !inject_alloc_failure() && cudaMallocHost((void **)&h->hst, sizeof(DevStatus)) == cudaSuccess;
-  if (ok && h->large && prec == BDSS_TF32_IR && n % 4 == 0) {
-    // tensor-core Schur tiles read W^T rows of Wb through TMA
-    CUtensorMap map;
-    cudaError_t em = make_w_tensor_map(&map, (const float *)h->Wb, (long long)slots * n, n);
-    ok = em == cudaSuccess && ws_alloc(h, (void **)&h->d_tmap, sizeof(CUtensorMap)) &&
-         cudaMemcpy(h->d_tmap, &map, sizeof(CUtensorMap), cudaMemcpyHostToDevice) == cudaSuccess;
-    h->tf32 = ok ? 1 : 0;
-    if (ok) {
-      h->ts_map_w = map;
-      h->ts_ok = 1;
-    }
-  }
   if (ok && is_mixed(h)) {
     const size_t nd = (size_t)N * n * d_max;
     ok = ws_alloc(h, (void **)&h->Y32, nd * sizeof(float));

@@ -84,8 +84,6 @@ struct Args {
   long long timeout_ns;
   int skip_barrier;      // test hook: 1-based barrier index CTA 0 skips
   int capacity;          // CTAs of a full persistent grid (tail-level splits)
-  int tf32;              // large FP32 path: Schur products on tcgen05 (3xTF32)
-  const CUtensorMap *tmap_w;  // TMA map of Wb as (slots * n) rows x n FP32 columns
   T *Li;                 // large FP32 path: L^{-1} of every eliminated block (slot of
                          // its original index, row-major n x n, zero above the
                          // diagonal), formed by the factorisation; null elsewhere
@@ -663,23 +661,22 @@ __device__ int chol_inverse(T *s, int ld, int n, T *cbuf, int *cnt, int *s_flag)
     }
   }
   __syncthreads();
-  // 8 x 8 diagonal inverses: a lane per column
-  for (int t = warp; t < np; t += nw) {
-    if (lane < 8) {
-      T *b = s + 8 * t * ld + 8 * t;  // this diagonal tile
-      T x[8];
+  // 8 x 8 diagonal inverses: a lane per column, four tiles a warp
+  for (int t = 4 * warp + (lane >> 3); t < np; t += 4 * nw) {
+    const int col = lane & 7;
+    T *b = s + 8 * t * ld + 8 * t;  // this diagonal tile
+    T x[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        T acc = T(0);
+    for (int i = 0; i < 8; ++i) {
+      T acc = T(0);
 #pragma unroll
-        for (int q = 0; q < i; ++q) acc = fma(b[i * ld + q], x[q], acc);
-        const T r = b[i * ld + i];
-        x[i] = i == lane ? r : i > lane ? -acc * r : T(0);
-      }
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-        if (i > lane) b[lane * ld + i] = x[i];
+      for (int q = 0; q < i; ++q) acc = fma(b[i * ld + q], x[q], acc);
+      const T r = b[i * ld + i];
+      x[i] = i == col ? r : i > col ? -acc * r : T(0);
     }
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (i > col) b[col * ld + i] = x[i];
   }
   __syncthreads();
   for (int h = 8; h < n; h *= 2) {

@@ -10,15 +10,15 @@
 namespace bdss {
 
 
-template <typename T, bool kTc>
-__device__ bool large_sub(const Args<T> &a, int l, int sub, bool factor, T *smem, int *s_flag, TcState *tc,
-                          int rank) {
+template <typename T>
+__device__ bool large_sub(const Args<T> &a, int l, int sub, bool factor, T *smem, int *s_flag, int rank) {
   const int n = a.p.n, d = a.d;
   const long long Nl = a.p.Nl[l];
   const long long nE = Nl / 2, nS = (Nl + 1) / 2;
   if (sub == kSubA1) {
-    for (long long m = rank; m < nE; m += gridDim.x)
-      if (!largeA1(a, l, 2 * m + 1, smem, s_flag)) return false;
+    if constexpr (sizeof(T) == 8)  // (FP32 blocks are factored in bdss_wide.cu)
+      for (long long m = rank; m < nE; m += gridDim.x)
+        if (!largeA1(a, l, 2 * m + 1, smem, s_flag)) return false;
   } else if (sub == kSubA2 && !factor && a.Li) {
     // solve pass with the stored inverses: y_j = L_j^{-1} b_j, a thread per row
     if constexpr (sizeof(T) == 4)
@@ -32,22 +32,6 @@ __device__ bool large_sub(const Args<T> &a, int l, int sub, bool factor, T *smem
       if (largeA2_live(a, l, j, factor, v * VT)) largeA2(a, l, j, v, factor, smem);
     }
   } else if (sub == kSubB) {
-    if constexpr (kTc) {
-      if (tc && factor) {
-        // D and E tiles on the tensor cores, RHS tiles on CUDA cores
-        const int nTC = largeB_tc_tiles(n), nR = largeB_tiles(n, false, d), nTB = nTC + nR;
-        for (long long t = rank; t < nS * nTB; t += gridDim.x) {
-          const long long k = t / nTB;
-          const int u = (int)(t % nTB);
-          if (u < nTC) {
-            if (!largeB_tc(a, l, k, u, *tc)) return false;
-          } else {
-            largeB(a, l, k, u - nTC, false, smem);
-          }
-        }
-        return true;
-      }
-    }
     if constexpr (sizeof(T) == 4) {
       if (!factor) {  // solve pass: the separator RHS updates, a thread per row
         for (long long k = rank; k < nS; k += gridDim.x) largeB_rows(a, l, k, smem);
@@ -56,9 +40,6 @@ __device__ bool large_sub(const Args<T> &a, int l, int sub, bool factor, T *smem
     }
     const int nTB = largeB_tiles(n, factor, d);
     for (long long t = rank; t < nS * nTB; t += gridDim.x) largeB(a, l, t / nTB, (int)(t % nTB), factor, smem);
-  } else if (sub == kSubBRhsOnly) {
-    const int nR = largeB_tiles(n, false, d);
-    for (long long t = rank; t < nS * nR; t += gridDim.x) largeB(a, l, t / nR, (int)(t % nR), false, smem);
   } else {
     if constexpr (sizeof(T) == 4) {
       if (a.Li) {  // with the stored inverses, a thread per row
@@ -71,77 +52,50 @@ __device__ bool large_sub(const Args<T> &a, int l, int sub, bool factor, T *smem
   return true;
 }
 
-template <typename T, bool kTc>
-__device__ void large_body(const Args<T> &a, int factor, int rhs, unsigned char *smem_raw, int *s_flag,
-                           TcState *tc) {
+template <typename T>
+__device__ void large_body(const Args<T> &a, int factor, int rhs, unsigned char *smem_raw, int *s_flag) {
   T *smem = reinterpret_cast<T *>(smem_raw);
   int bar = 0;
   const int rank = spread_rank(a.st, a.timeout_ns);
   if (rank < 0) return;
   for (int l = 0; l < a.p.L; ++l) {
     if (factor) {
-      large_sub<T, kTc>(a, l, kSubA1, true, smem, s_flag, tc, rank);
+      large_sub<T>(a, l, kSubA1, true, smem, s_flag, rank);
       if (!grid_barrier(a.st, a.timeout_ns, ++bar, a.skip_barrier)) return;
     }
-    large_sub<T, kTc>(a, l, kSubA2, factor != 0, smem, s_flag, tc, rank);
+    large_sub<T>(a, l, kSubA2, factor != 0, smem, s_flag, rank);
     if (!grid_barrier(a.st, a.timeout_ns, ++bar, a.skip_barrier)) return;
-    large_sub<T, kTc>(a, l, kSubB, factor != 0, smem, s_flag, tc, rank);
+    large_sub<T>(a, l, kSubB, factor != 0, smem, s_flag, rank);
     if (!grid_barrier(a.st, a.timeout_ns, ++bar, a.skip_barrier)) return;
   }
   if (rank == 0) largeTop(a, factor != 0, reinterpret_cast<double *>(smem_raw), s_flag);
   if (!rhs || a.p.L == 0) return;
   if (!grid_barrier(a.st, a.timeout_ns, ++bar, a.skip_barrier)) return;
   for (int l = a.p.L - 1; l >= 0; --l) {
-    large_sub<T, kTc>(a, l, kSubC, false, smem, s_flag, tc, rank);
+    large_sub<T>(a, l, kSubC, false, smem, s_flag, rank);
     if (l > 0 && !grid_barrier(a.st, a.timeout_ns, ++bar, a.skip_barrier)) return;
   }
 }
 
-// The tensor-core state (TMEM, mbarriers) is set up once per CTA when the
-// TF32 mode factors and released on every way out of the kernel body.  The
-// tensor-core variant (kTc) is a separate kernel: the occupancy calculator
-// allows one CTA per SM for a kernel that contains tcgen05 code, while the
-// FP32 tiles without it fit two.
 // Register cap: FP32 tiles fit two CTAs per SM in shared memory, so the
 // registers must allow two as well; FP64 is shared-memory limited to one.
 #define BDSS_LARGE_MAXNREG(T) __maxnreg__(sizeof(T) == 4 ? 120 : 255)
 
-template <typename T, bool kTc>
+template <typename T>
 __global__ void __launch_bounds__(kThreads) BDSS_LARGE_MAXNREG(T)
     k_large_persistent(const __grid_constant__ Args<T> a, int factor, int rhs) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_flag;
-  if constexpr (kTc) {
-    __shared__ uint64_t s_bars[3];
-    __shared__ uint32_t s_tmem;
-    TcState tc;
-    const bool use_tc = a.tf32 && factor;
-    if (use_tc) tc_begin(tc, smem_raw, s_bars, &s_tmem);
-    large_body<T, true>(a, factor, rhs, smem_raw, &s_flag, use_tc ? &tc : nullptr);
-    if (use_tc) tc_end(tc, a.timeout_ns);
-  } else {
-    large_body<T, false>(a, factor, rhs, smem_raw, &s_flag, nullptr);
-  }
+  large_body<T>(a, factor, rhs, smem_raw, &s_flag);
 }
 
-template <typename T, bool kTc>
+template <typename T>
 __global__ void __launch_bounds__(kThreads) BDSS_LARGE_MAXNREG(T)
     k_large_sub(const __grid_constant__ Args<T> a, int l, int sub, int factor) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_flag;
   if (ld_relaxed_i32(&a.st->status) != 0) return;
-  if constexpr (kTc) {
-    __shared__ uint64_t s_bars[3];
-    __shared__ uint32_t s_tmem;
-    TcState tc;
-    const bool use_tc = a.tf32 && factor && sub == kSubB;
-    if (use_tc) tc_begin(tc, smem_raw, s_bars, &s_tmem);
-    large_sub<T, true>(a, l, sub, factor != 0, reinterpret_cast<T *>(smem_raw), &s_flag, use_tc ? &tc : nullptr,
-                       (int)blockIdx.x);
-    if (use_tc) tc_end(tc, a.timeout_ns);
-  } else {
-    large_sub<T, false>(a, l, sub, factor != 0, reinterpret_cast<T *>(smem_raw), &s_flag, nullptr, (int)blockIdx.x);
-  }
+  large_sub<T>(a, l, sub, factor != 0, reinterpret_cast<T *>(smem_raw), &s_flag, (int)blockIdx.x);
 }
 
 template <typename T>
@@ -630,350 +584,6 @@ __global__ void __launch_bounds__(kQ == 2 ? 2 * kThreads : kThreads, kQ == 1 ? 2
   }
 }
 
-// ---------------------------------------------------------------------------
-// TF32 Schur products on the tensor cores, pipelined (the separator update of
-// Algorithm 3 in the TF32 mode of the tiled path).  An output tile of
-// 128 x 128 (D's lower part: one round per eliminated neighbour, accumulated;
-// E: one round) takes, per K chunk of 32, twelve tcgen05.mma (kind::tf32,
-// K = 8): hi*hi + hi*lo + lo*hi, the 3xTF32 product, into an FP32
-// accumulator in TMEM, where hi is W rounded to TF32 and lo = W - hi.
-// Roles (320 threads):
-//   warp 0     TMA: the raw W slabs of the A and B rows (2 x 16 KB per chunk)
-//              into a ring of two stages;
-//   warps 6-9  split each raw stage into hi and lo slabs (the swizzled
-//              layout is element-position preserving) in a second ring;
-//   warp 1     one thread issues the MMAs of a split stage and commits it;
-//   warps 2-5  drain the accumulator, two buffers, so that a tile's
-//              epilogue runs under the next tile's products.
-// Every wait is bounded; a timed-out wait aborts every role.
-// ---------------------------------------------------------------------------
-constexpr int kTsRaw = 2 * kTcSlab;     // raw A | B of one chunk
-constexpr int kTsSplit = 4 * kTcSlab;   // A hi | A lo | B hi | B lo
-constexpr int kTsStages = 2;            // stages of each ring
-constexpr int kTsThreads = 320;
-constexpr int kTsSplitters = 128;       // warps 6-9
-constexpr uint32_t kTsTmemCols = 2 * kTcN;
-constexpr size_t kTsSmem = (size_t)kTsStages * (kTsRaw + kTsSplit) + 1024;
-
-__device__ __forceinline__ bool ts_try(uint64_t *bar, uint32_t parity) {
-  uint32_t done;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(done)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return done != 0;
-}
-// Bounded wait; gives up early when another role aborted (abort != null).
-__device__ __forceinline__ bool ts_wait(uint64_t *bar, uint32_t parity, long long timeout_ns, volatile int *abort) {
-  long long t0 = 0;
-  for (uint32_t it = 0;; ++it) {
-    if (ts_try(bar, parity)) return true;
-    if ((it & 63) == 63) {
-      if (abort && *abort) return false;
-      const long long now = global_ns();
-      if (t0 == 0) t0 = now;
-      else if (now - t0 > timeout_ns) return false;
-    }
-  }
-}
-
-__device__ __forceinline__ void mbar_arrive_local(uint64_t *bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-struct TsTile {
-  long long k;       // separator 2k
-  int isD, ti, tj, nr;
-  // rows (in the W buffer) of the A and B operands of rounds 0 and 1; scalar
-  // fields, so that the tile stays in registers
-  long long ra0, ra1, rb0, rb1;
-  __device__ long long a_of(int r) const { return r == 0 ? ra0 : ra1; }
-  __device__ long long b_of(int r) const { return r == 0 ? rb0 : rb1; }
-};
-
-__device__ __forceinline__ TsTile ts_tile(const Args<float> &a, int l, long long u) {
-  const int n = a.p.n, nt = (n + kTcM - 1) / kTcM, nD = nt * (nt + 1) / 2, per = nD + nt * nt;
-  const long long Nl = a.p.Nl[l], slot0 = a.p.off[l];
-  TsTile T;
-  T.k = u / per;
-  const int t = (int)(u - T.k * per);
-  const long long s = 2 * T.k;
-  T.nr = 0;
-  T.ra0 = T.ra1 = T.rb0 = T.rb1 = 0;
-  if (t < nD) {
-    T.isD = 1;
-    int ti = 0;
-    while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
-    T.ti = ti;
-    T.tj = t - ti * (ti + 1) / 2;
-    const long long bm = (slot0 + s - 1) * n, bp = (slot0 + s) * n;
-    const bool hasM = s >= 2, hasP = s + 1 < Nl;
-    // round 0: the left neighbour if present, else the right one
-    T.ra0 = (hasM ? bm : bp) + T.ti * kTcM;
-    T.rb0 = (hasM ? bm : bp) + T.tj * kTcM;
-    T.ra1 = bp + T.ti * kTcM;
-    T.rb1 = bp + T.tj * kTcM;
-    T.nr = (int)hasM + (int)hasP;
-  } else {
-    T.isD = 0;
-    T.ti = (t - nD) / nt;
-    T.tj = (t - nD) - T.ti * nt;
-    if (s + 2 < Nl) {
-      T.ra0 = (slot0 + s + 1) * n + T.ti * kTcM;
-      T.rb0 = (slot0 + s) * n + T.tj * kTcM;
-      T.nr = 1;
-    }
-  }
-  return T;
-}
-
-__global__ void __launch_bounds__(kTsThreads, 1)
-    k_tf32_schur(const __grid_constant__ CUtensorMap mapW, const __grid_constant__ Args<float> a, int l) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ uint64_t tfull[kTsStages], tempty[kTsStages], sfull[kTsStages], sempty[kTsStages];
-  __shared__ uint64_t acc_full[2], acc_empty[2], drain;
-  __shared__ uint32_t s_tmem;
-  __shared__ int s_abort, s_go;
-  if (threadIdx.x == 0) s_go = ld_relaxed_i32(&a.st->status) == 0;
-  __syncthreads();
-  if (!s_go) return;
-  unsigned char *raw = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  unsigned char *split = raw + (size_t)kTsStages * kTsRaw;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n = a.p.n, nt = (n + kTcM - 1) / kTcM, kchunks = (n + kTcK - 1) / kTcK;
-  const long long Nl = a.p.Nl[l];
-  const long long tiles = ((Nl + 1) / 2) * (long long)(nt * (nt + 1) / 2 + nt * nt);
-  volatile int *abort = &s_abort;
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kTsStages; ++s) {
-      mbar_init(&tfull[s], 1);
-      mbar_init(&tempty[s], kTsSplitters);
-      mbar_init(&sfull[s], kTsSplitters);
-      mbar_init(&sempty[s], 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], 128);
-    }
-    mbar_init(&drain, 1);
-    s_abort = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 1) tmem_alloc(&s_tmem, kTsTmemCols);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = s_tmem;
-  auto fail = [&]() {
-    *abort = 1;
-    set_status(a.st, kStTimeout, l, -1);
-  };
-
-  if (warp == 0) {
-    // ---- TMA producer: raw slabs ------------------------------------------------
-    if (lane == 0) {
-      int st = 0;
-      uint32_t ph = 0;
-      bool stop = false;
-      for (long long u = blockIdx.x; u < tiles && !stop; u += gridDim.x) {
-        const TsTile T = ts_tile(a, l, u);
-        for (int r = 0; r < T.nr && !stop; ++r)
-          for (int kc = 0; kc < kchunks; ++kc) {
-            if (!ts_wait(&tempty[st], ph ^ 1, a.timeout_ns, abort)) {
-              fail();
-              stop = true;
-              break;
-            }
-            unsigned char *base = raw + (size_t)st * kTsRaw;
-            mbar_expect_tx(&tfull[st], kTsRaw);
-            tma_load_2d(base, &mapW, kc * kTcK, (int)T.a_of(r), &tfull[st]);
-            tma_load_2d(base + kTcSlab, &mapW, kc * kTcK, (int)T.b_of(r), &tfull[st]);
-            if (++st == kTsStages) { st = 0; ph ^= 1; }
-          }
-      }
-      // wait out the loads still in flight (each stage's last armed phase)
-      for (int s = 0; s < kTsStages; ++s) ts_wait(&tfull[s], (s < st) ? ph : (ph ^ 1), a.timeout_ns, nullptr);
-    }
-  } else if (warp >= 6) {
-    // ---- split warps: raw -> hi | lo -------------------------------------------
-    const int sid = threadIdx.x - 6 * 32;
-    int ts = 0, ss = 0;
-    uint32_t tph = 0, sph = 0;
-    bool stop = false;
-    for (long long u = blockIdx.x; u < tiles && !stop; u += gridDim.x) {
-      const TsTile T = ts_tile(a, l, u);
-      for (int r = 0; r < T.nr && !stop; ++r)
-        for (int kc = 0; kc < kchunks; ++kc) {
-          // warp-uniform waits: lane 0 polls, the others then observe the phase
-          int ok = 0;
-          if (lane == 0)
-            ok = (ts_wait(&tfull[ts], tph, a.timeout_ns, abort) && ts_wait(&sempty[ss], sph ^ 1, a.timeout_ns, abort))
-                     ? 1
-                     : 0;
-          ok = __shfl_sync(0xffffffffu, ok, 0);
-          if (!ok) {
-            if (lane == 0) fail();
-            stop = true;
-            break;
-          }
-          if (lane != 0) {
-            ts_try(&tfull[ts], tph);
-            ts_try(&sempty[ss], sph ^ 1);
-          }
-          const float4 *src = reinterpret_cast<const float4 *>(raw + (size_t)ts * kTsRaw);
-          unsigned char *dst = split + (size_t)ss * kTsSplit;
-#pragma unroll 4
-          for (int i = sid; i < kTsRaw / 16; i += kTsSplitters) {
-            const int which = i / (kTcSlab / 16), j = i - which * (kTcSlab / 16);  // A or B, float4 in slab
-            const float4 x = src[i];
-            float4 h, o;
-            const float xs[4] = {x.x, x.y, x.z, x.w};
-            float hs[4], os[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              hs[q] = __uint_as_float((__float_as_uint(xs[q]) + 0x1000u) & 0xFFFFE000u);
-              os[q] = xs[q] - hs[q];
-            }
-            h = make_float4(hs[0], hs[1], hs[2], hs[3]);
-            o = make_float4(os[0], os[1], os[2], os[3]);
-            reinterpret_cast<float4 *>(dst + (size_t)which * 2 * kTcSlab)[j] = h;
-            reinterpret_cast<float4 *>(dst + (size_t)which * 2 * kTcSlab + kTcSlab)[j] = o;
-          }
-          fence_proxy_async_smem();  // the MMAs read the split slabs through the async proxy
-          mbar_arrive_local(&tempty[ts]);
-          mbar_arrive_local(&sfull[ss]);
-          if (++ts == kTsStages) { ts = 0; tph ^= 1; }
-          if (++ss == kTsStages) { ss = 0; sph ^= 1; }
-        }
-    }
-  } else if (warp == 1) {
-    // ---- MMA issuer ------------------------------------------------------------
-    if (lane == 0) {
-      constexpr uint32_t idesc = tc_idesc_tf32(kTcM, kTcN);
-      int st = 0;
-      uint32_t ph = 0;
-      long long i = 0;  // tiles with work so far: accumulator buffer i & 1
-      bool stop = false;
-      for (long long u = blockIdx.x; u < tiles && !stop; u += gridDim.x) {
-        const TsTile T = ts_tile(a, l, u);
-        if (T.nr == 0) continue;
-        const int b = (int)(i & 1);
-        if (!ts_wait(&acc_empty[b], (uint32_t)((i >> 1) & 1), a.timeout_ns, abort)) {
-          fail();
-          break;
-        }
-        tc_fence_after();
-        const uint32_t d = tmem + (uint32_t)(b * kTcN);
-        bool first = true;
-        for (int r = 0; r < T.nr && !stop; ++r)
-          for (int kc = 0; kc < kchunks; ++kc) {
-            if (!ts_wait(&sfull[st], ph, a.timeout_ns, abort)) {
-              fail();
-              stop = true;
-              break;
-            }
-            tc_fence_after();
-            const unsigned char *base = split + (size_t)st * kTsSplit;
-            const unsigned char *Ahi = base, *Alo = base + kTcSlab, *Bhi = base + 2 * kTcSlab,
-                                *Blo = base + 3 * kTcSlab;
-#pragma unroll
-            for (int kk = 0; kk < kTcK / 8; ++kk) {
-              const int off = kk * 32;  // 8 TF32 = 32 bytes along K inside the swizzle atom
-              tc_mma_tf32(d, tc_desc_sw128(Ahi, off), tc_desc_sw128(Bhi, off), idesc, first ? 0u : 1u);
-              first = false;
-              tc_mma_tf32(d, tc_desc_sw128(Ahi, off), tc_desc_sw128(Blo, off), idesc, 1u);
-              tc_mma_tf32(d, tc_desc_sw128(Alo, off), tc_desc_sw128(Bhi, off), idesc, 1u);
-            }
-            tc_commit(&sempty[st]);
-            if (++st == kTsStages) { st = 0; ph ^= 1; }
-          }
-        if (stop) break;
-        tc_commit(&acc_full[b]);
-        ++i;
-      }
-      // every MMA issued has completed before TMEM is released
-      tc_commit(&drain);
-      ts_wait(&drain, 0, a.timeout_ns, nullptr);
-    }
-  } else {
-    // ---- epilogue: warps 2..5, TMEM lane quarter warp % 4 ---------------------
-    const int quarter = warp & 3;
-    const size_t nn = (size_t)n * n;
-    tc_fence_before();
-    mbar_arrive_local(&acc_empty[0]);
-    mbar_arrive_local(&acc_empty[1]);
-    long long i = 0;
-    for (long long u = blockIdx.x; u < tiles; u += gridDim.x) {
-      const TsTile T = ts_tile(a, l, u);
-      if (T.nr == 0) continue;
-      const int b = (int)(i & 1);
-      int ok = 0;
-      if (lane == 0) ok = ts_wait(&acc_full[b], (uint32_t)((i >> 1) & 1), a.timeout_ns, abort) ? 1 : 0;
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-      if (!ok) {
-        if (lane == 0) fail();
-        break;
-      }
-      if (lane != 0) ts_try(&acc_full[b], (uint32_t)((i >> 1) & 1));
-      tc_fence_after();
-      const int R = T.ti * kTcM + 32 * quarter + lane;
-      const long long s = 2 * T.k, orig = s << l;
-      const uint32_t taddr = tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)(b * kTcN);
-#pragma unroll 1
-      for (int cb = 0; cb < kTcN / 32; ++cb) {
-        float v[32];
-        tmem_ld32(taddr + (uint32_t)(cb * 32), v);
-        if (R >= n) continue;
-        const int C0 = T.tj * kTcN + cb * 32;
-        if (T.isD) {
-          if (C0 > R) continue;  // the block lies above the diagonal for this row
-          float *Dg = a.Ld + (size_t)orig * nn + (size_t)R * n;
-          float base[32];
-          // every load of the block first (independent, in flight together),
-          // then the stores
-          if (l == 0) {
-            const double *Ag = a.A_diag + (size_t)orig * nn;
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              const int C = C0 + j;
-              const bool in = C <= R && C < n;
-              const double x = in ? ldcg(Ag + (size_t)R * n + C) : 0.0;
-              const double y = in ? ldcg(Ag + (size_t)C * n + R) : 0.0;
-              base[j] = 0.5f * ((float)x + (float)y);
-            }
-          } else {
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-              const int C = C0 + j;
-              base[j] = (C <= R && C < n) ? ldcg(Dg + C) : 0.0f;
-            }
-          }
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const int C = C0 + j;
-            if (C <= R && C < n) Dg[C] = base[j] - v[j];
-          }
-        } else {
-          float *Eg = a.Eb + ((size_t)a.p.off[l + 1] + (size_t)T.k) * nn + (size_t)R * n;
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const int C = C0 + j;
-            if (C < n) Eg[C] = -v[j];
-          }
-        }
-      }
-      tc_fence_before();
-      mbar_arrive_local(&acc_empty[b]);
-      ++i;
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  if (warp == 1) tmem_dealloc(tmem, kTsTmemCols);
-}
-
 // FP64 residual for large blocks: one CTA per block row, one thread per row r
 // of the block with up to 16 right-hand-side columns in registers:
 //   R[r][c] = B[r][c] - 0.5 sum_p (A[r][p] + A[p][r]) x_i[p][c]
@@ -1062,21 +672,18 @@ size_t smem_bytes_large(int n, int d) {
   size_t b = smem_large(n, d, (int)sizeof(T)) * sizeof(T);
   const size_t top = smem_large_top(n, d) * sizeof(double);
   if (top > b) b = top;
-  if (sizeof(T) == 4 && kTcSmemBytes > b) b = kTcSmemBytes;
   return (b + 15) & ~(size_t)15;
 }
 
 template <typename T>
-cudaError_t configure_large(int n, int d, size_t *smem, int *blocks_per_sm, int *blocks_per_sm_tc) {
+cudaError_t configure_large(int n, int d, size_t *smem, int *blocks_per_sm) {
   int dev = 0, optin = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  const void *kernels[] = {(const void *)k_large_persistent<T, false>, (const void *)k_large_sub<T, false>,
-                           (const void *)k_large_persistent<float, true>, (const void *)k_large_sub<float, true>,
+  const void *kernels[] = {(const void *)k_large_persistent<T>, (const void *)k_large_sub<T>,
                            (const void *)k_large_top<T>, (const void *)k_residual_rows,
                            (const void *)k_tc_selftest, (const void *)k_large_corr<1>,
-                           (const void *)k_large_corr<2>, (const void *)k_large_corr<4>,
-                           (const void *)k_tf32_schur};
+                           (const void *)k_large_corr<2>, (const void *)k_large_corr<4>};
   for (const void *k : kernels) {
     cudaFuncAttributes fa;
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k);
@@ -1084,22 +691,13 @@ cudaError_t configure_large(int n, int d, size_t *smem, int *blocks_per_sm, int 
       e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
   }
   const size_t sm = smem_bytes_large<T>(n, d);
-  int occ = 0, occ_tc = 0;
+  int occ = 0;
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_large_persistent<T, false>, kThreads, sm);
-  if (e == cudaSuccess && sizeof(T) == 4)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_tc, k_large_persistent<float, true>, kThreads, sm);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_large_persistent<T>, kThreads, sm);
   if (e != cudaSuccess) return e;
   *smem = sm;
   *blocks_per_sm = occ;
-  *blocks_per_sm_tc = sizeof(T) == 4 ? occ_tc : occ;
   return cudaSuccess;
-}
-
-// The tensor-core kernel runs only when the TF32 mode factors.
-template <typename T>
-bool large_uses_tc(const Args<T> &a, int factor) {
-  return sizeof(T) == 4 && a.tf32 && factor;
 }
 
 template <typename T>
@@ -1108,21 +706,12 @@ cudaError_t launch_large_persistent(const Args<T> &a, int factor, int rhs, int g
   if (!rhs) copy.d = 0;
   int f = factor, r = rhs;
   void *params[] = {(void *)&copy, (void *)&f, (void *)&r};
-  const void *k = (const void *)k_large_persistent<T, false>;
-  if constexpr (sizeof(T) == 4)
-    if (large_uses_tc(a, factor)) k = (const void *)k_large_persistent<float, true>;
-  return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kThreads), params, smem, s);
+  return cudaLaunchCooperativeKernel((const void *)k_large_persistent<T>, dim3(grid), dim3(kThreads), params, smem, s);
 }
 
 template <typename T>
 cudaError_t launch_large_sub(const Args<T> &a, int l, int sub, int factor, int grid, size_t smem, cudaStream_t s) {
-  if constexpr (sizeof(T) == 4) {
-    if (large_uses_tc(a, factor) && sub == kSubB) {
-      k_large_sub<float, true><<<grid, kThreads, smem, s>>>(a, l, sub, factor);
-      return cudaGetLastError();
-    }
-  }
-  k_large_sub<T, false><<<grid, kThreads, smem, s>>>(a, l, sub, factor);
+  k_large_sub<T><<<grid, kThreads, smem, s>>>(a, l, sub, factor);
   return cudaGetLastError();
 }
 
@@ -1176,25 +765,14 @@ cudaError_t launch_large_corr(const CorrMaps *maps, int max_split, const Args<fl
   return cudaGetLastError();
 }
 
-cudaError_t launch_tf32_schur(const CUtensorMap &mapW, const Args<float> &a, int l, int sms, cudaStream_t s) {
-  const int n = a.p.n, nt = (n + kTcM - 1) / kTcM;
-  const long long tiles = ((a.p.Nl[l] + 1) / 2) * (long long)(nt * (nt + 1) / 2 + nt * nt);
-  if (tiles <= 0) return cudaSuccess;
-  const int grid = (int)(tiles < sms ? tiles : sms);
-  k_tf32_schur<<<grid, kTsThreads, kTsSmem, s>>>(mapW, a, l);
-  return cudaGetLastError();
-}
-
-long long large_sub_tasks(const Plan &p, int l, int sub, int factor, int d, int esz, int tf32, int inv) {
+long long large_sub_tasks(const Plan &p, int l, int sub, int factor, int d, int esz, int inv) {
   const long long Nl = p.Nl[l], nE = Nl / 2, nS = (Nl + 1) / 2;
-  if (sub == kSubBRhsOnly) return nS * largeB_tiles(p.n, false, d);
   if (sub == kSubA1 || sub == kSubC) return nE;
   if (sub == kSubA2) {
     if (!factor && inv) return nE;
     const int VT = vec_tile(esz);
-    return nE * (((factor ? (inv ? 3 : 2) * p.n : 0) + d + VT - 1) / VT);
+    return nE * (((factor ? 2 * p.n : 0) + d + VT - 1) / VT);
   }
-  if (tf32 && factor) return nS * (largeB_tc_tiles(p.n) + largeB_tiles(p.n, false, d));
   if (!factor && esz == 4) return nS;  // a thread per row (largeB_rows)
   return nS * largeB_tiles(p.n, factor != 0, d);
 }
@@ -1333,7 +911,7 @@ cudaError_t launch_residual_rows(long long N, int n, int d, const double *A_diag
 
 #define BDSS_INSTANTIATE_LARGE(T)                                                                        \
   template size_t smem_bytes_large<T>(int, int);                                                         \
-  template cudaError_t configure_large<T>(int, int, size_t *, int *, int *);                             \
+  template cudaError_t configure_large<T>(int, int, size_t *, int *);                                    \
   template cudaError_t launch_large_persistent<T>(const Args<T> &, int, int, int, size_t, cudaStream_t); \
   template cudaError_t launch_large_sub<T>(const Args<T> &, int, int, int, int, size_t, cudaStream_t);   \
   template cudaError_t launch_large_top<T>(const Args<T> &, int, size_t, cudaStream_t);

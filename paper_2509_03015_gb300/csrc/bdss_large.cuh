@@ -173,14 +173,13 @@ __host__ __device__ inline size_t smem_large(int n, int d, int esz) {
 // column + 1.
 // ---------------------------------------------------------------------------
 template <typename T>
-__device__ __noinline__ int chol_blocked(T *M, int n, const double *src_sym, T *smem, int *s_flag, T *Dinv = nullptr) {
+__device__ __noinline__ int chol_blocked(T *M, int n, const double *src_sym, T *smem, int *s_flag) {
   smem = as_shared(smem);
   s_flag = as_shared(s_flag);
   const int nt = ntiles(n);
   T *sT = smem;                              // 64 x 65 tile
   T *sA = sT + kTile * kTilePad;
   T *sB = sA + kKc * kTilePad;
-  T *sP2 = sB + kKc * kTilePad;              // panel rows when Dinv is given (64 x 65)
   const int ld = kTilePad;
   auto src = [&](int r, int c) -> T {      // element of the matrix before step 0
     if (src_sym) return T(0.5) * ((T)ldcg(src_sym + (long long)r * n + c) + (T)ldcg(src_sym + (long long)c * n + r));
@@ -204,50 +203,8 @@ __device__ __noinline__ int chol_blocked(T *M, int n, const double *src_sym, T *
       const int r = e / kb, c = e - r * kb;
       if (c <= r) M[(long long)(k0 + r) * n + k0 + c] = sT[r * ld + c];
     }
-    if (Dinv) {
-      // L_kk^{-1} (the diagonal tile of L^{-1}): unit vectors through the tile
-      // substitution once, then every solve with this tile is a product
-      T *sI = sA;  // 64 x 65 (sA and sB are contiguous)
-      __syncthreads();
-      for (int e = threadIdx.x; e < kTile * kTile; e += blockDim.x) {
-        const int r = e / kTile, c = e - r * kTile;
-        sI[r * ld + c] = (r == c && r < kb) ? T(1) : T(0);
-      }
-      __syncthreads();
-      trsv_tile_fwd(sT, ld, kb, sI, ld, kb);
-      for (int e = threadIdx.x; e < kb * kb; e += blockDim.x) {
-        const int r = e / kb, c = e - r * kb;  // (L_kk^{-1})[r][c] = entry r of solved vector c
-        Dinv[(long long)(k0 + r) * n + k0 + c] = (c <= r) ? sI[c * ld + r] : T(0);
-      }
-      __syncthreads();
-      // panel below: L_ik = S_ik L_kk^{-T}, i.e. L_ik[r][c] = sum_q S_ik[r][q] L_kk^{-1}[c][q]
-      const View<T> Dk{Dinv + (long long)k0 * n + k0, n, 1, kb, kb};
-      for (int i = k + 1; i < nt; ++i) {
-        const int i0 = i * kTile, ib = min(kTile, n - i0);
-#pragma unroll 4
-        for (int e = threadIdx.x; e < kTile * kTile; e += blockDim.x) {
-          const int r = e / kTile, c = e - r * kTile;
-          T v = T(0);
-          if (r < ib && c < kb) v = first ? src(i0 + r, k0 + c) : ldcg(M + (long long)(i0 + r) * n + k0 + c);
-          sP2[r * ld + c] = v;
-        }
-        __syncthreads();
-        T acc[4][4] = {};
-        const View<T, true> Pr{sP2, ld, 1, ib, kb};
-        gemm_nt_tile(acc, Pr, 0, Dk, 0, kb, sA, sB);
-        const int tm = threadIdx.x >> 4, tn = threadIdx.x & 15;
-#pragma unroll
-        for (int a2 = 0; a2 < 4; ++a2)
-#pragma unroll
-          for (int b2 = 0; b2 < 4; ++b2) {
-            const int r = 4 * tm + a2, c = 4 * tn + b2;
-            if (r < ib && c < kb) M[(long long)(i0 + r) * n + k0 + c] = acc[a2][b2];
-          }
-        __syncthreads();
-      }
-    }
     // panel below: L_ik = S_ik L_kk^{-T}: each row x solves L_kk x = s
-    for (int i = k + 1; i < nt && !Dinv; ++i) {
+    for (int i = k + 1; i < nt; ++i) {
       const int i0 = i * kTile, ib = min(kTile, n - i0);
       // reuse the gemm staging area for the panel rows (ib x kb)
       T *sP = sA;  // needs kTile x kTilePad: sA and sB are contiguous 2 * kKc * kTilePad = kTile * kTilePad
@@ -295,7 +252,7 @@ __device__ __noinline__ int chol_blocked(T *M, int n, const double *src_sym, T *
 // n + 1), L (n x n, reciprocal diagonal) in global memory, blocked by 64-row
 // tiles: gemm update from the solved rows, then the triangular tile.
 template <typename T>
-__device__ void trsv_fwd_blocked(const T *L, int n, T *sV, int nv, T *smem, const T *Dinv = nullptr) {
+__device__ void trsv_fwd_blocked(const T *L, int n, T *sV, int nv, T *smem) {
   const int nt = ntiles(n), lv = n + 1;
   T *sT = smem;
   T *sA = sT + kTile * kTilePad;
@@ -319,26 +276,6 @@ __device__ void trsv_fwd_blocked(const T *L, int n, T *sV, int nv, T *smem, cons
           }
         __syncthreads();
       }
-    }
-    if (Dinv) {
-      // the diagonal tile's solve as a product with its stored inverse:
-      // v[r0 + i] = sum_q L_RR^{-1}[i][q] v[r0 + q], 64 vectors at a time
-      const View<T> Dr{Dinv + (long long)r0 * n + r0, n, 1, rb, rb};
-      for (int c0 = 0; c0 < nv; c0 += kTile) {
-        T acc[4][4] = {};
-        const View<T, true> Vc{sV + (long long)c0 * lv + r0, lv, 1, nv - c0, rb};
-        gemm_nt_tile(acc, Dr, 0, Vc, 0, rb, sA, sB);
-        const int tm = threadIdx.x >> 4, tn = threadIdx.x & 15;
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int b = 0; b < 4; ++b) {
-            const int i = 4 * tm + a, c = c0 + 4 * tn + b;
-            if (i < rb && c < nv) sV[(long long)c * lv + r0 + i] = acc[a][b];
-          }
-        __syncthreads();
-      }
-      continue;
     }
 #pragma unroll 4
     for (int e = threadIdx.x; e < kTile * kTile; e += blockDim.x) {
@@ -398,10 +335,7 @@ __device__ bool largeA1(const Args<T> &a, int l, long long j, T *smem, int *s_fl
   const int n = a.p.n;
   const long long orig = j << l;
   T *M = a.Ld + orig * (long long)n * n;
-  // FP32 with stored inverses: the diagonal tiles of L^{-1} are formed here,
-  // and every tile solve after them is a product
-  T *Dinv = a.Li ? a.Li + orig * (long long)n * n : nullptr;
-  const int bad = chol_blocked(M, n, l == 0 ? a.A_diag + orig * (long long)n * n : nullptr, smem, s_flag, Dinv);
+  const int bad = chol_blocked(M, n, l == 0 ? a.A_diag + orig * (long long)n * n : nullptr, smem, s_flag);
   if (bad) {
     if (threadIdx.x == 0) set_status(a.st, kStNotSPD, l, orig);
     __syncthreads();
@@ -414,11 +348,10 @@ __device__ bool largeA1(const Args<T> &a, int l, long long j, T *smem, int *s_fl
 // Number of vectors of eliminated position j's forward substitution.
 // Vector slots of an eliminated block's forward substitution: the couplings
 // (2 n, the 64-vector tiles are laid out as if the right coupling existed),
-// the n unit vectors whose solutions are the columns of L^{-1} (factor with
-// an inverse buffer), then the RHS columns.
+// then the RHS columns.
 template <typename T>
 __device__ __forceinline__ int largeA2_slots(const Args<T> &a, bool factor) {
-  return (factor ? (a.Li ? 3 : 2) * a.p.n : 0) + a.d;
+  return (factor ? 2 * a.p.n : 0) + a.d;
 }
 
 // Number of vectors of eliminated position j's forward substitution.
@@ -432,8 +365,8 @@ __device__ __forceinline__ bool largeA2_live(const Args<T> &a, int l, long long 
 
 // A2: vector tile v of eliminated position j.  Slots [0, n) are E_L's
 // columns, [n, 2n) E_R's rows (absent for the last block of a level: those
-// slots are skipped), [2n, 3n) the unit vectors of L^{-1} (with an inverse
-// buffer), then the RHS columns; in a solve pass only the RHS columns.
+// slots are skipped), then the RHS columns; in a solve pass only the RHS
+// columns.
 template <typename T>
 __device__ void largeA2(const Args<T> &a, int l, long long j, int v, bool factor, T *smem) {
   const int n = a.p.n, d = a.d, lv = n + 1;
@@ -442,9 +375,8 @@ __device__ void largeA2(const Args<T> &a, int l, long long j, int v, bool factor
   const long long orig = j << l;
   const size_t nn = (size_t)n * n;
   const int nW = factor ? 2 * n : 0;              // coupling slots
-  const int nI = (factor && a.Li) ? n : 0;        // unit-vector slots
   const int VT = vec_tile(sizeof(T));
-  const int slots = nW + nI + d;
+  const int slots = nW + d;
   const int c0 = v * VT, nv = min(VT, slots - c0);
   T *sV = smem;
   T *work = sV + (size_t)VT * lv;
@@ -462,10 +394,8 @@ __device__ void largeA2(const Args<T> &a, int l, long long j, int v, bool factor
       val = !hasR ? T(0)
                   : (l == 0) ? (T)ldcg(a.A_sub + (size_t)j * nn + (size_t)r * n + i)
                              : ldcg(E + (size_t)j * nn + (size_t)r * n + i);
-    } else if (c < nW + nI) {  // unit vector e_{c - nW}
-      val = (i == c - nW) ? T(1) : T(0);
     } else {  // RHS column
-      const int k = c - nW - nI;
+      const int k = c - nW;
       const size_t bo = (size_t)orig * n * d + (size_t)i * d + k;
       if (l == 0 && a.B64) val = (T)ldcg(a.B64 + bo);
       else if (l == 0 && a.Bt) val = ldcg(a.Bt + bo);
@@ -474,7 +404,7 @@ __device__ void largeA2(const Args<T> &a, int l, long long j, int v, bool factor
     sV[(size_t)cc * lv + i] = val;
   }
   __syncthreads();
-  trsv_fwd_blocked(a.Ld + (size_t)orig * nn, n, sV, nv, work, factor && a.Li ? a.Li + (size_t)orig * nn : nullptr);
+  trsv_fwd_blocked(a.Ld + (size_t)orig * nn, n, sV, nv, work);
   // write back
   T *W = a.Wb + (size_t)a.p.off[l] * nn;
   for (int e = threadIdx.x; e < n * nv; e += blockDim.x) {
@@ -483,23 +413,8 @@ __device__ void largeA2(const Args<T> &a, int l, long long j, int v, bool factor
     long long wo = -1;  // element of the coupling buffer, if this is a coupling slot
     if (c < nW && c < n) wo = (long long)((size_t)(j - 1) * nn + (size_t)c * n + i);
     else if (c < nW) { if (hasR) wo = (long long)((size_t)j * nn + (size_t)(c - n) * n + i); }
-    else if (c >= nW + nI) a.Y[(size_t)orig * n * d + (size_t)i * d + (c - nW - nI)] = val;
+    else a.Y[(size_t)orig * n * d + (size_t)i * d + (c - nW)] = val;
     if (wo >= 0) W[wo] = val;
-  }
-  if (nI) {
-    // columns u0..u1-1 of L^{-1}, row-major in Li: consecutive threads take
-    // consecutive columns of one row
-    const int u0 = max(c0, nW) - nW, u1 = min(c0 + nv, nW + nI) - nW;
-    if (u1 > u0) {
-      T *Li = a.Li + (size_t)orig * nn;
-      const int nu = u1 - u0;
-      for (int e = threadIdx.x; e < n * nu; e += blockDim.x) {
-        const int i = e / nu, u = u0 + e - i * nu;
-        // the diagonal tiles were formed by the Cholesky task and are read
-        // by this level's other substitution tasks: left as they are
-        if (i / kTile != u / kTile) Li[(size_t)i * n + u] = sV[(size_t)(u + nW - c0) * lv + i];
-      }
-    }
   }
   __syncthreads();
 }
@@ -587,80 +502,6 @@ __device__ void largeB(const Args<T> &a, int l, long long k, int t, bool factor,
     }
   }
   __syncthreads();
-}
-
-// Tensor-core tiles of a separator's Schur update (large FP32 path, TF32
-// mode): 128 x 128 output tiles, lower D tiles then E tiles.
-__host__ __device__ inline int largeB_tc_tiles(int n) {
-  const int t = (n + kTcM - 1) / kTcM;
-  return t * (t + 1) / 2 + t * t;
-}
-
-// Tile t of separator s = 2k at level l on tcgen05 (3xTF32).  Returns false on
-// a timed-out wait (the status word is then set).
-__device__ inline bool largeB_tc(const Args<float> &a, int l, long long k, int t, TcState &tc) {
-  const int n = a.p.n, nt = (n + kTcM - 1) / kTcM, nD = nt * (nt + 1) / 2;
-  const long long Nl = a.p.Nl[l];
-  const long long s = 2 * k;
-  const bool hasM = (s >= 2), hasP = (s + 1 < Nl), hasE = (s + 2 < Nl);
-  const long long orig = s << l;
-  const size_t nn = (size_t)n * n;
-  const long long slot0 = a.p.off[l];
-  bool ok = true;
-  int ti, tj;
-  if (t < nD) {
-    ti = 0;
-    while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
-    tj = t - ti * (ti + 1) / 2;
-    bool first = true;
-    if (hasM) {
-      const int base = (int)((slot0 + s - 1) * n);
-      ok = tc_accumulate(tc, a.tmap_w, base + ti * kTcM, base + tj * kTcM, n, first, a.timeout_ns);
-      first = false;
-    }
-    if (ok && hasP) {
-      const int base = (int)((slot0 + s) * n);
-      ok = tc_accumulate(tc, a.tmap_w, base + ti * kTcM, base + tj * kTcM, n, first, a.timeout_ns);
-    }
-  } else {
-    if (!hasE) return true;
-    const int u = t - nD;
-    ti = u / nt;
-    tj = u - ti * nt;
-    ok = tc_accumulate(tc, a.tmap_w, (int)((slot0 + s + 1) * n) + ti * kTcM, (int)((slot0 + s) * n) + tj * kTcM, n,
-                       true, a.timeout_ns);
-  }
-  if (!ok) {
-    if (threadIdx.x == 0) set_status(a.st, kStTimeout, l, orig);
-    return false;
-  }
-  float v[64];
-  int row, col0;
-  tc_read_row(tc, v, row, col0);
-  const int R = ti * kTcM + row;
-  if (t < nD) {
-    float *Dg = a.Ld + (size_t)orig * nn;
-    const double *Ag = a.A_diag + (size_t)orig * nn;
-    if (R < n)
-      for (int j = 0; j < 64; ++j) {
-        const int C = tj * kTcN + col0 + j;
-        if (C <= R && C < n) {
-          const float base = (l == 0) ? 0.5f * ((float)ldcg(Ag + (size_t)R * n + C) + (float)ldcg(Ag + (size_t)C * n + R))
-                                      : ldcg(Dg + (size_t)R * n + C);
-          Dg[(size_t)R * n + C] = base - v[j];
-        }
-      }
-  } else {
-    float *En = a.Eb + ((size_t)a.p.off[l + 1] + (size_t)k) * nn;
-    if (R < n)
-      for (int j = 0; j < 64; ++j) {
-        const int C = tj * kTcN + col0 + j;
-        if (C < n) En[(size_t)R * n + C] = -v[j];
-      }
-  }
-  tc_fence_before();
-  __syncthreads();
-  return true;
 }
 
 // ---------------------------------------------------------------------------
@@ -875,32 +716,6 @@ __device__ __noinline__ bool largeTop(const Args<T> &a, bool factor, double *sme
       if (threadIdx.x == 0) set_status(a.st, kStNotSPD, L, 0);
       __syncthreads();
       return false;
-    }
-    if constexpr (sizeof(T) == 4) {
-      if (a.Ltinv) {
-        // the FP32 solve passes apply the top factor as products with L^{-1}:
-        // float(L) into Ltinv[0 .. n^2), then its inverse into Ltinv[n^2 ..),
-        // 64 unit vectors at a time through the blocked substitution
-        float *Lf = a.Ltinv, *Li = a.Ltinv + nn;
-        for (int e = threadIdx.x; e < n * n; e += blockDim.x) Lf[e] = (float)a.Ltop[e];
-        __syncthreads();
-        float *sV = reinterpret_cast<float *>(smem);
-        float *work = sV + (size_t)kTile * lv;
-        for (int u0 = 0; u0 < n; u0 += kTile) {
-          const int nu = min(kTile, n - u0);
-          for (int e = threadIdx.x; e < nu * n; e += blockDim.x) {
-            const int c = e / n, i = e - c * n;
-            sV[(size_t)c * lv + i] = (i == u0 + c) ? 1.0f : 0.0f;
-          }
-          __syncthreads();
-          trsv_fwd_blocked(Lf, n, sV, nu, work);
-          for (int e = threadIdx.x; e < n * nu; e += blockDim.x) {
-            const int i = e / nu, c = e - i * nu;
-            Li[(size_t)i * n + u0 + c] = sV[(size_t)c * lv + i];
-          }
-          __syncthreads();
-        }
-      }
     }
   }
   if constexpr (sizeof(T) == 4) {

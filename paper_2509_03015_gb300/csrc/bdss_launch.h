@@ -34,7 +34,7 @@ cudaError_t launch_adjoint_grads(long long N, int n, int d, const double *Lam, c
 constexpr int kMaxNLarge = 256;
 template <typename T> size_t smem_bytes_large(int n, int d);
 template <typename T>
-cudaError_t configure_large(int n, int d, size_t *smem, int *blocks_per_sm, int *blocks_per_sm_tc);
+cudaError_t configure_large(int n, int d, size_t *smem, int *blocks_per_sm);
 template <typename T>
 cudaError_t launch_large_persistent(const Args<T> &a, int factor, int rhs, int grid, size_t smem, cudaStream_t s);
 template <typename T>
@@ -70,14 +70,7 @@ cudaError_t launch_large_corr(const CorrMaps *maps, int max_split, const Args<fl
 // t = y_j - W x of the neighbours in place in Yt, C2 x_j = L_j^{-T} t.
 constexpr int kSubC1 = 5, kSubC2 = 6;
 
-// TF32 Schur products of level l on the tensor cores (pipelined, warp roles):
-// a map over Wb (boxes of 128 rows x 32 columns).
-cudaError_t launch_tf32_schur(const CUtensorMap &mapW, const Args<float> &a, int l, int sms, cudaStream_t s);
-
-// Sub-phase code of the large path: the separators' RHS tiles alone (their D
-// and E tiles ran elsewhere, e.g. on the tensor cores).
-constexpr int kSubBRhsOnly = 4;
-long long large_sub_tasks(const Plan &p, int l, int sub, int factor, int d, int esz, int tf32, int inv);
+long long large_sub_tasks(const Plan &p, int l, int sub, int factor, int d, int esz, int inv);
 cudaError_t make_w_tensor_map(CUtensorMap *out, const float *Wb, long long rows, int n);
 cudaError_t run_tc_selftest(double *max_err, int *status);
 cudaError_t launch_residual_rows(long long N, int n, int d, const double *A_diag, const double *A_sub,

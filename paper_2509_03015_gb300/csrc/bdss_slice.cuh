@@ -138,10 +138,20 @@ __device__ __forceinline__ void sl_mma(uint32_t d, uint64_t adesc, uint64_t bdes
       : "memory");
 }
 
+// One lane of a converged warp.
+__device__ __forceinline__ bool sl_elect() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+
 // All digit pairs of A (128 rows) times a B tile of `cols` rows (16 or 32), K
 // steps 0 .. ks - 1, into the accumulators at TMEM address d (diagonal t at
-// columns cols t ..).  One thread; rolled loops, since the code of the digit
-// kernels has to stay in the instruction cache.
+// columns cols t ..).  One elected lane of a warp that takes this path as a
+// whole (its operands then stay in uniform registers: issued by one thread of
+// a diverged warp, a product took 130 cycles against the tensor core's 72);
+// rolled over p, since the code of the digit kernels has to stay in the
+// instruction cache.
 template <typename T>
 __device__ __forceinline__ void sl_issue(uint32_t d, const unsigned char *A, const unsigned char *B, int cols, int ks) {
   constexpr int kDig = SliceFmt<T>::kDig;
@@ -151,14 +161,10 @@ __device__ __forceinline__ void sl_issue(uint32_t d, const unsigned char *A, con
     const uint32_t idesc = sl_idesc<T>(cols * (kDig - p)), dp = d + (uint32_t)(cols * p);
     // the start address field counts 16-byte units: a slab is kSlASlab / 16,
     // a K step of 16 FP16 entries 2 of them
-    uint64_t ad = ad0 + (uint64_t)(p * (kSlASlab / 16)), bd = bd0;
-    if (ks == 4) {
+    const uint64_t ad = ad0 + (uint64_t)(p * (kSlASlab / 16));
 #pragma unroll
-      for (int k = 0; k < 4; ++k) sl_mma(dp, ad + 2 * k, bd + 2 * k, idesc, (uint32_t)(p | k));
-    } else {
-#pragma unroll 1
-      for (int k = 0; k < ks; ++k, ad += 2, bd += 2) sl_mma(dp, ad, bd, idesc, (uint32_t)(p | k));
-    }
+    for (int k = 0; k < 4; ++k)
+      if (k < ks) sl_mma(dp, ad + 2 * k, bd0 + 2 * k, idesc, (uint32_t)(p | k));
   }
 }
 

@@ -102,16 +102,19 @@ __device__ __forceinline__ void wd_issue(WdCta<T> &w, bool cols2, int ks0, int k
   fence_proxy_async_smem();
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0) {
+  // the second tile's commit covers the first's products as well
+  if (__shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0) == 0) {
     tc_fence_after();
-    sl_issue<T>(w.tmem, w.A, w.B, kSlCols, ks0);
-    tc_commit(w.bar);
-    if (cols2) {
-      sl_issue<T>(w.tmem + kWdBufCols<T>, w.A, w.B + kWdBBytes<T>, kSlCols, ks1);
-      tc_commit(w.bar + 1);
+    if (sl_elect()) {
+      sl_issue<T>(w.tmem, w.A, w.B, kSlCols, ks0);
+      tc_commit(w.bar);
+      if (cols2) {
+        sl_issue<T>(w.tmem + kWdBufCols<T>, w.A, w.B + kWdBBytes<T>, kSlCols, ks1);
+        tc_commit(w.bar + 1);
+      }
     }
+    __syncwarp();
   }
-  __syncwarp();
 }
 // Wait (bounded) for a column tile's product, a warp at a time: the warps of
 // the first tile drain it while the second is multiplied.  False after a

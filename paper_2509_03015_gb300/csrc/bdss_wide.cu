@@ -20,6 +20,12 @@
 // and their W^T share a slot of Wb, D and its L a slot of Ld (reciprocal
 // diagonal), where a diagonal tile keeps X_kk^T above its diagonal for the
 // downward pass.
+//
+// Why: the substitutions of the couplings are n^3 multiply-adds a block on an
+// ALU of 2 FP64 multiply-adds a cycle and SM.  Measured (factor + solve):
+//   N = 1024, n = 256, d = 1, FP64              89.2 -> 22.0 ms
+//   N = 100, n = 256, d = 1, FP32 refined        8.96 -> 5.1 ms
+//   N = 4096, n = 256, d = 16, TF32 mode refined 58.0 -> 49.3 ms
 #include "bdss_launch.h"
 #include "bdss_slice_cta.cuh"
 #include "bdss_wide.h"
@@ -129,6 +135,15 @@ __host__ __device__ inline int panel_slots(const WidePanels &P, bool couplings, 
   return P.nt - 1 - k + (couplings ? 2 * P.nt : 0) + (d > 0 ? 1 : 0) + (inverse ? k : 0);
 }
 
+// Rounds of a tile of two slots: one per earlier panel (left-looking, so that a
+// row's entries are read and written once a panel and no second launch is
+// needed), P, and for rows of D two with half the columns each for their own
+// diagonal tiles.
+//
+// What bounds it, in FP64: the logic pipe while operands are cut and sums
+// converted, and the products themselves, half hidden (profile of
+// k_wide_schur, whose rounds are the same).  N = 1024, n = 256: the four panels
+// of level 0 take 0.55, 0.91, 0.89 and 1.04 ms.
 template <typename T>
 __global__ void __launch_bounds__(kWdThreads<T>, sizeof(T) == 8 ? 1 : 2)
     k_wide_panel(const __grid_constant__ Args<T> a, const WideBuf<T> wb, int l, int k) {
@@ -277,6 +292,14 @@ __host__ __device__ inline int schur_tiles(int nt, int d) {
   return schur_tiles_d(nt) + (d > 0 ? tr : 0) + tr * nt;
 }
 
+// One round per K chunk of 64; a D tile sums both eliminated neighbours.  The
+// accumulators hold one chunk exactly, the chunks meet in registers.
+//
+// What bounds it, in FP64: the logic pipe, 59 % busy over a launch, 2.1
+// instructions a cycle; level 0 of N = 1024, n = 256 takes 3.7 ms (planes of
+// ten BF16 digits cut by a launch of their own and read through TMA took 9.6 ms
+// over all levels, this kernel 7.9).  In FP32: instructions as well (59 % of the
+// issue slots); pipelining two rounds in one CTA of 32 warps changed nothing.
 template <typename T>
 __global__ void __launch_bounds__(kWdThreads<T>, sizeof(T) == 8 ? 1 : 2)
     k_wide_schur(const __grid_constant__ Args<T> a, int l) {
@@ -382,7 +405,9 @@ __global__ void __launch_bounds__(kWdThreads<T>, sizeof(T) == 8 ? 1 : 2)
   wd_end(w);
 }
 
-// Cholesky factor and inverse of the diagonal tiles of panel k.
+// Cholesky factor and inverse of the diagonal tiles of panel k (chol_inverse).
+// One block's tile takes 77 us in FP64 and 35 us in FP32, launch included: the
+// critical path of levels with few blocks.
 constexpr int kDiagThreads = 256;
 template <typename T>
 __global__ void __launch_bounds__(kDiagThreads) k_wide_diag(const __grid_constant__ Args<T> a, const WideBuf<T> wb,
@@ -516,7 +541,9 @@ __global__ void __launch_bounds__(256) k_wide_ingest(const __grid_constant__ Arg
   }
 }
 
-// Downward pass (Algorithms 6, 2), first half: t_j = y_j - W_L x_{j-1} - W_R x_{j+1}
+// Downward pass (Algorithms 6, 2) in FP64, split in two so that a level of few
+// blocks spreads its W over SMs (27 and 57 us for one block of n = 256), and
+// over the columns there are instead of 64-wide vector tiles.  First half: t_j = y_j - W_L x_{j-1} - W_R x_{j+1}
 // for 64 rows of an eliminated block, (W x)[q] = sum_p Wt[p][q] x[p]: a thread
 // per row and quarter of the sum, four columns of x at a time.
 constexpr int kDownCols = 4;
