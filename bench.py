@@ -1,5 +1,5 @@
 """Benchmark: factor + solve of the synthetic Kalman-smoother Hessian
-N = 16384 blocks, n = 64, d = 4 (FP64, fused persistent kernel), in
+N = 16384 blocks, n = 64, d = 4 (FP64, level by level), in
 systems/s, with the roofline of the kernel, the FP32 + FP64-refinement path,
 the per-level launch structure, an end-to-end figure through the C ABI with
 host buffers, the SM clocks seen, and the CPU oracle timed on the host.
@@ -115,10 +115,10 @@ def kernel_rooflines(kt, steps, units, N, n, d, mode, sms, mhz, emu=False):
                   FP32 residual: HBM;
       factor      the oracle's block-Thomas tally of factor + solve, on the
                   ALU of the mode's precision;
-      schur_tc    the Schur products of every level as tensor-core tiles
-                  (accounting.tc_tile_flops, one product counted once; the
-                  3xTF32 split executes three), TF32 tensor rate = measured
-                  BF16 x 1/2 (nominal ratio)."""
+      schur_tc    the products of the factorisation (coupling solves, panels,
+                  separator updates; accounting.cr_flops) on the tensor cores,
+                  one product counted once, against the BF16 rate divided by the
+                  16-bit products each takes (36 in FP64, 6 in FP32)."""
     pk = measured_peaks()
     out = {}
     slots = sum(Nl - 1 for Nl in accounting.levels(N)[:-1])
@@ -134,13 +134,6 @@ def kernel_rooflines(kt, steps, units, N, n, d, mode, sms, mhz, emu=False):
         elif cls == "residual":
             work, unit, bound = 6.0 * n * n * d * N, "TFLOP/s", "alu"
             peak, pdef = fp64_peak(sms, mhz), "FP64 ALU (SMs x 2 DFMA/clk x 2 x clock)"
-        elif cls == "slice" and mode == "fp64":
-            work, unit, bound = accounting.emu_wslice_bytes(N, n), "GB/s", "hbm"
-            peak, pdef = pk["hbm_gbs"] * 1e9, f"HBM copy bandwidth ({pk['source']}); coupling blocks sliced"
-        elif cls == "schur_tc" and mode == "fp64":
-            work, unit, bound = accounting.emu_schur_mma_flops(N, n), "TFLOP/s", "tensor"
-            peak = pk["bf16_tflops"] * 1e12
-            pdef = f"BF16 dense ({pk['source']}); digit-slice products executed"
         elif cls == "slice":
             np_ = -(-n // 64) * 64
             work, unit, bound = 16.0 * N * n * n + 20.0 * N * n * 3 * np_, "GB/s", "hbm"
@@ -150,15 +143,21 @@ def kernel_rooflines(kt, steps, units, N, n, d, mode, sms, mhz, emu=False):
             unit, bound = "GB/s", "hbm"
             peak, pdef = pk["hbm_gbs"] * 1e9, f"HBM copy bandwidth ({pk['source']})"
         elif cls == "schur_tc":
-            work, unit, bound = accounting.tc_tile_flops(N, n), "TFLOP/s", "tensor"
-            peak = pk["bf16_tflops"] * 0.5e12
-            pdef = f"TF32 dense = BF16 ({pk['source']}) x 1/2 nominal ratio"
-        elif cls == "factor" and mode == "fp64" and "schur_tc" in kt:
-            # the FP64-ALU share of cyclic reduction: everything but the
-            # Schur products, which ran on the tensor cores
-            c = accounting.cr_flops(N, n, d)
-            work, unit, bound = c["factor"] + c["solve"] - accounting.tc_tile_flops(N, n), "TFLOP/s", "alu"
-            peak, pdef = fp64_peak(sms, mhz), "FP64 ALU; executed CR flops outside the Schur products"
+            # couplings, panels and separator updates: all of the factorisation
+            # but the diagonal tiles; each product is 36 (FP64: digit pairs) or
+            # 6 (FP32: part pairs) products of 16-bit numbers
+            pairs = 36 if mode == "fp64" else 6
+            work, unit, bound = accounting.cr_flops(N, n, d)["factor"], "TFLOP/s", "tensor"
+            peak = pk["bf16_tflops"] * 1e12 / pairs
+            pdef = f"BF16 dense ({pk['source']}) / {pairs} products of 16-bit parts"
+        elif cls == "factor" and "schur_tc" in kt:
+            # diagonal tiles (Cholesky factor and inverse, n^2 nb 2/3 flops a
+            # block), top block, downward pass
+            nt = -(-n // 64)
+            work = N * nt * 2.0 / 3.0 * (n / nt) ** 3 + 10.0 * N * n * n * d
+            unit, bound = "TFLOP/s", "alu"
+            peak = fp64_peak(sms, mhz) if mode == "fp64" else fp32_peak(sms, mhz)
+            pdef = "FP64 ALU" if mode == "fp64" else "FP32 ALU (SMs x 128 FFMA x 2 x clock)"
         elif cls == "factor":
             t = accounting.thomas_flops(N, n, d)
             work, unit, bound = t["factor"] + t["solve"], "TFLOP/s", "alu"
@@ -171,8 +170,6 @@ def kernel_rooflines(kt, steps, units, N, n, d, mode, sms, mhz, emu=False):
         out[cls] = {"bound": bound, "achieved": ach / scale, "peak": peak / scale, "unit": unit,
                     "frac": ach / peak, "ms_per_unit": per * 1e3, "units_per_step": u,
                     "launches_per_step": launches / steps, "work_per_unit": work, "peak_definition": pdef}
-        if cls == "schur_tc" and mode != "fp64":
-            out[cls]["executed_frac"] = 3 * ach / peak
     return out
 
 
@@ -339,7 +336,7 @@ def timed_leg(sol, call, reps, stream, max_over_ranks, N, n, d, mode, sms, mhz):
     # each plain refinement step is one correction
     units = {"factor": 1, "schur_tc": 1, "residual": kt.get("residual", (0, 0))[1] / reps,
              "correction": refs[0] / reps,
-             "slice": 1 if mode == "fp64" else kt.get("slice", (0, 0))[1] / reps}
+             "slice": kt.get("slice", (0, 0))[1] / reps}
     emu = mode != "fp64" and 64 < n <= 256 and d <= 16
     roof = kernel_rooflines(kt, reps, units, N, n, d, mode, sms, mhz, emu=emu)
     dom = max(per_step, key=lambda c: per_step[c]["ms_per_step"]) if per_step else None
@@ -779,8 +776,8 @@ def main():
     }
 
     if launches_per_step > 1:
-        # the FP64 factorisation runs level by level with its Schur products on
-        # the tensor cores: the step is several kernels, so the roofline is the
+        # the FP64 factorisation runs level by level with its products on the
+        # tensor cores: the step is several kernels, so the roofline is the
         # dominant kernel class's, from the library's per-class CUDA events in
         # a separate pass (the timed region above has no events inside)
         K4 = max(3, args.steps // 4)
@@ -797,8 +794,8 @@ def main():
             out["roofline"] = r
         out["kernels"] = kt4
         out["rooflines"] = roof4
-        out["config"]["path"] = ("FP64, per-level factor with the Schur products on the tensor cores "
-                                 "(BF16 digit slices, exact FP32 accumulation) + solve")
+        out["config"]["path"] = ("FP64, per-level factor with its products on the tensor cores (FP16 digits, exact "
+                                 "FP32 accumulation) + solve with the stored inverses")
 
     args.mhz = peak_mhz
     if not args.no_extras:
