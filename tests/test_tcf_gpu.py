@@ -99,3 +99,20 @@ def test_mixed_precision_matches_oracle(oracle_mod, N, n, d, precision):
     for x in (X, X2):
         assert oracle_mod.forward_error(x, Xo) <= 1e-11
         assert oracle_mod.backward_error(s["A_diag"], s["A_sub"], x, s["B"]) <= 1.1e-14
+
+
+# the line of the choice by size, both sides of it (launches of the call: one
+# for the persistent kernel), with the tolerances above
+@pytest.mark.parametrize("N,n,d,tc", [(127, 48, 1, False), (128, 48, 1, True), (128, 47, 1, False), (128, 48, 2, False),
+                                      (1536, 40, 2, True), (1535, 40, 2, False)])
+def test_choice_by_size(oracle_mod, N, n, d, tc):
+    from paper_2509_03015_gb300 import Solver
+    s = inputs.random_btd(N, n, d, seed=N + n)
+    sol = Solver(N, n, d_max=d)
+    X = sol.factor_solve(_dev(s["A_diag"]), _dev(s["A_sub"]), _dev(s["B"])).cpu().numpy()
+    launches = sol.launch_stats()[0]
+    sol.close()
+    assert (launches > 1) == tc
+    Xo = oracle_mod.solve_system(s["A_diag"], s["A_sub"], s["B"])
+    assert oracle_mod.forward_error(X, Xo) <= 1e-12
+    assert oracle_mod.backward_error(s["A_diag"], s["A_sub"], X, s["B"]) <= 1e-14
