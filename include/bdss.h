@@ -142,7 +142,8 @@ typedef enum {
                                    0 = on the FP64 ALU (for n <= 64 the single persistent
                                    launch).  Default 1 for 64 < n <= 256; for n <= 64 by size
                                    (long systems of large blocks).  Setting 1 on a handle
-                                   without it gives BDSS_ERR_UNSUPPORTED */
+                                   without it gives BDSS_ERR_UNSUPPORTED; mixed-precision
+                                   handles accept 0, which changes nothing there */
   BDSS_OPT_RESIDUAL_EMU = 10,   /* mixed precision, 64 < n <= 256 and d_max <= 16: 1 (default)
                                    = the FP64 residual of the refinement on the tensor cores
                                    (BF16 digit slices, exact FP32 accumulation: see

@@ -91,7 +91,7 @@ struct bdss_ctx {
   void *tcfcb = nullptr;  // (N / 2) x 2 x n x d_max (T)
   int tcf_ready = 0;
   bool tcf_factored = false;  // the stored factors are that path's
-  int tcf_opt = -1;       // BDSS_OPT_SCHUR_EMU at n <= 64: -1 by size, 0 off, 1 on
+  int tcf_opt = -1;       // BDSS_OPT_SCHUR_EMU at n <= 64 (FP64): -1 by size, 0 off, 1 on
   // large mixed path: streamed solve passes (maps over Li and Wb)
   CorrMaps corr_maps[3];  // split factors P = 1, 2, 4
   int corr_max_split = 1;
@@ -596,7 +596,7 @@ static cudaError_t run_levels_large(bdss_ctx *h, const Args<T> &a, bool factor, 
   if (!rhs) b.d = 0;
   // solve passes with the stored inverses keep y of the eliminated blocks in Yt
   b.Yt = (!factor && inv) ? (T *)h->Yt : nullptr;
-  if (factor && h->wide_on) return run_levels_wide(h, a, rhs);
+  if (factor && (sizeof(T) == 4 || h->wide_on)) return run_levels_wide(h, a, rhs);
   if constexpr (sizeof(T) == 4) {
     if (!factor && rhs && inv && h->corr_ok && b.d <= kCorrMaxD) return run_corr_passes(h, b);
   }
@@ -951,6 +951,7 @@ bdss_status bdss_set_option(bdss_handle h, bdss_option key, int64_t value) {
     case BDSS_OPT_SCHUR_EMU:
       if (value != 0 && value != 1) return BDSS_ERR_INVALID_ARG;
       if (value && (is_mixed(h) || h->N < 2 || h->n < kTcfMinN)) return BDSS_ERR_UNSUPPORTED;
+      if (is_mixed(h)) return BDSS_OK;  // an FP64 choice: FP32 factors of n > 64 have no other path
       if (h->large) {
         h->wide_on = value && h->wide_ready;
       } else {

@@ -1,0 +1,49 @@
+"""GPU: options that choose between factorisation paths, switched between the
+factorisations and solves of one handle.  Every result is checked against the
+CPU oracle, on systems drawn apart from each other, so that factors left from
+an earlier one cannot pass."""
+import numpy as np
+import pytest
+
+from paper_2509_03015_gb300 import inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).to("cuda:0")
+
+
+def _put(s):
+    return _dev(s["A_diag"]), _dev(s["A_sub"]), _dev(s["B"])
+
+
+# random_btd has kappa(A) below 1e3: 1e-12 forward in FP64, 1e-11 where the call
+# refines to a backward error of 1e-14
+
+
+@pytest.mark.parametrize("N,n,precision", [(40, 32, "fp32_ir"), (40, 32, "tf32_ir"), (9, 128, "fp32_ir"),
+                                           (9, 128, "tf32_ir"), (5, 256, "fp32_ir"), (5, 256, "tf32_ir")])
+@pytest.mark.parametrize("persistent", [1, 0])
+def test_schur_emu_off_changes_nothing_in_mixed_precision(oracle_mod, N, n, precision, persistent):
+    """The option is an FP64 one; on the other handles 0 is accepted and leaves
+    the path, and its results, as they are."""
+    from paper_2509_03015_gb300 import Solver
+    s1, s2 = inputs.random_btd(N, n, 2, seed=1), inputs.random_btd(N, n, 2, seed=2)
+    L, C = oracle_mod.factor(s2["A_diag"], s2["A_sub"])
+    Xo = oracle_mod.solve(L, C, s2["B"])
+    sol = Solver(N, n, d_max=2, precision=precision, persistent=bool(persistent))
+    sol.factor(*_put(s1)[:2])
+    launches = sol.launch_stats()[0]
+    sol.set_option("schur_emu", 0)
+    Ad, As, B = _put(s2)
+    sol.factor(Ad, As)
+    assert sol.launch_stats()[0] == launches
+    ld = sol.logdet()
+    X = sol.solve(B).cpu().numpy()
+    sol.close()
+    # each of the N n pivots' logarithms is within a few FP32 roundings
+    assert abs(ld - oracle_mod.logdet(L)) <= N * n * 2.0 ** -20
+    assert oracle_mod.forward_error(X, Xo) <= 1e-11
+    assert oracle_mod.backward_error(s2["A_diag"], s2["A_sub"], X, s2["B"]) <= 1e-14
