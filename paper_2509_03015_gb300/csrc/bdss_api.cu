@@ -644,7 +644,6 @@ template <typename T>
 static cudaError_t run_levels(bdss_ctx *h, const Args<T> &a, bool factor, bool rhs) {
   const Plan &p = h->plan;
   if (h->large) return run_levels_large<T>(h, a, factor, rhs);
-  if (factor) h->tcf_factored = false;
   if (factor && use_tcf(h)) return run_levels_tcf<T>(h, a, rhs);
   if (!factor && h->tcf_factored && use_tcf(h)) return run_solve_tcf<T>(h, a);
   const int cap = h->bps * h->sms;
@@ -1060,6 +1059,7 @@ static void info_init(bdss_info *info) {
 static bdss_status factor_impl(bdss_ctx *h, const double *A_diag, const double *A_sub, const double *B, double *X,
                                int d, bdss_info *info) {
   h->factored = false;
+  h->tcf_factored = false;  // run_levels_tcf sets it; every other path's factors are without the inverses
   h->launches = 0;
   h->barriers = 0;
   kt_reset(h);

@@ -47,3 +47,23 @@ def test_schur_emu_off_changes_nothing_in_mixed_precision(oracle_mod, N, n, prec
     assert abs(ld - oracle_mod.logdet(L)) <= N * n * 2.0 ** -20
     assert oracle_mod.forward_error(X, Xo) <= 1e-11
     assert oracle_mod.backward_error(s2["A_diag"], s2["A_sub"], X, s2["B"]) <= 1e-14
+
+
+@pytest.mark.parametrize("d", [1, 12])
+def test_factors_of_another_path_are_not_taken_for_the_tensor_core_ones(oracle_mod, d):
+    """Tensor-core factors of one system, then the one-cluster path's factors of
+    another, then a solve with the tensor-core option on again."""
+    from paper_2509_03015_gb300 import Solver
+    N, n = 40, 32
+    s1, s2 = inputs.random_btd(N, n, d, seed=3), inputs.random_btd(N, n, d, seed=4)
+    sol = Solver(N, n, d_max=d)
+    sol.set_option("schur_emu", 1)
+    sol.factor(*_put(s1)[:2])
+    sol.set_option("schur_emu", 0)
+    sol.set_option("small_cluster", 1)
+    Ad, As, B = _put(s2)
+    sol.factor(Ad, As)
+    sol.set_option("schur_emu", 1)
+    X = sol.solve(B).cpu().numpy()
+    sol.close()
+    assert oracle_mod.forward_error(X, oracle_mod.solve_system(s2["A_diag"], s2["A_sub"], s2["B"])) <= 1e-12
