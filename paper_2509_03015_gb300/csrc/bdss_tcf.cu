@@ -529,7 +529,8 @@ __global__ void __launch_bounds__(256) k_tcf_top(const __grid_constant__ Args<T>
 
 // One level of a solve with the stored inverses.
 //   kUp:   separator s: b_s -= Wt(s-1) y_{s-1} + Wt(s) y_{s+1}; if s is eliminated
-//          at the next level, y_s = X_s b_s.  first: no level before the first
+//          at the next level (odd, and that level is not the blocks left for the
+//          top sweep), y_s = X_s b_s.  first: no level before the first
 //          elimination yet, y_j = X_j b_j of level 0.
 //   down:  eliminated j: t = y_j - Wt(j-1)^T x_{j-1} - Wt(j)^T x_{j+1}, x_j = X_j^T t.
 // Thread (i, g): row i of the result, a quarter of either sum; it loads all of
@@ -549,7 +550,8 @@ __global__ void __launch_bounds__(256, 2) k_tcf_solve(const __grid_constant__ Ar
   const long long m = blockIdx.x, Nl = a.p.Nl[l];
   const long long pos = kUp && !first ? 2 * m : 2 * m + 1, orig = pos << l;
   const bool hasM = !first && pos >= 1, hasP = !first && pos + 1 < Nl;
-  const bool tri = !kUp || first || (m & 1);  // a triangular product follows
+  // a triangular product follows, unless the next level is the serial top's
+  const bool tri = !kUp || first || ((m & 1) && l + 1 < a.p.L);
   const bool raw = kUp && l == 0 && (a.B64 || a.Bt);
   // matrix entries: W of slot pos - 1 (g < 2) or pos (g >= 2), X of this block
   T wv[kMaxN / 2], xv[kMaxN / 4];
@@ -655,7 +657,7 @@ __global__ void __launch_bounds__(1024, 1) k_tcf_solve_tc(const __grid_constant_
   for (long long m = blockIdx.x; m < count && ok; m += gridDim.x) {
     const long long pos = kUp && !first ? 2 * m : 2 * m + 1, orig = pos << l;
     const bool hasM = !first && pos >= 1, hasP = !first && pos + 1 < Nl;
-    const bool tri = !kUp || first || (m & 1), raw = kUp && l == 0 && (a.B64 || a.Bt);
+    const bool tri = !kUp || first || ((m & 1) && l + 1 < a.p.L), raw = kUp && l == 0 && (a.B64 || a.Bt);
     const double *W0 = a.Wb + (size_t)(a.p.off[l] + pos - 1) * nn, *W1 = W0 + nn;
     // X (FP64 keeps X^T above the diagonal of Ld): X[i][q] at sX[q kTcLdX + i], q <= i
     double xv[4];

@@ -67,3 +67,23 @@ def test_factors_of_another_path_are_not_taken_for_the_tensor_core_ones(oracle_m
     X = sol.solve(B).cpu().numpy()
     sol.close()
     assert oracle_mod.forward_error(X, oracle_mod.solve_system(s2["A_diag"], s2["A_sub"], s2["B"])) <= 1e-12
+
+
+@pytest.mark.parametrize("N,n,nstar", [(100, 32, 2), (100, 48, 7), (37, 64, 2), (9, 40, 64), (130, 33, 3)])
+@pytest.mark.parametrize("d", [1, 16])
+def test_stored_factors_with_a_serial_top(oracle_mod, N, n, nstar, d):
+    """Tensor-core factors below a serial sweep of up to nstar top blocks: the
+    separators of the last level are that sweep's, not eliminated blocks."""
+    from paper_2509_03015_gb300 import Solver
+    s = inputs.random_btd(N, n, d, seed=N + n + nstar)
+    sol = Solver(N, n, d_max=d)
+    sol.set_option("schur_emu", 1)
+    sol.set_option("nstar", nstar)
+    Ad, As, B = _put(s)
+    X = sol.factor_solve(Ad, As, B).cpu().numpy()
+    X2 = sol.solve(B).cpu().numpy()
+    sol.close()
+    Xo = oracle_mod.solve_system(s["A_diag"], s["A_sub"], s["B"])
+    for x in (X, X2):
+        assert oracle_mod.forward_error(x, Xo) <= 1e-12
+        assert oracle_mod.backward_error(s["A_diag"], s["A_sub"], x, s["B"]) <= 1e-14
