@@ -89,6 +89,7 @@ struct bdss_ctx {
   void *tcfX = nullptr;   // (N / 2) x n x n (T)
   void *tcfC = nullptr;   // (N / 2) x 2 x n x n (T)
   void *tcfcb = nullptr;  // (N / 2) x 2 x n x d_max (T)
+  short *tcfE = nullptr;  // N x 64: exponents of its scaling, kept with the factors
   int tcf_ready = 0;
   bool tcf_factored = false;  // the stored factors are that path's
   int tcf_opt = -1;       // BDSS_OPT_SCHUR_EMU at n <= 64 (FP64): -1 by size, 0 off, 1 on
@@ -326,6 +327,7 @@ static bdss_status tcf_alloc(bdss_ctx *h) {
   bool ok = h->tcfX || ws_alloc(h, &h->tcfX, m * nn * esz);
   ok = ok && (h->tcfC || ws_alloc(h, &h->tcfC, m * 2 * nn * esz));
   ok = ok && (h->tcfcb || ws_alloc(h, &h->tcfcb, m * 2 * h->n * h->d_max * esz));
+  ok = ok && (h->tcfE || ws_alloc(h, (void **)&h->tcfE, (size_t)h->N * h->n * sizeof(int)));
   if (!ok) {
     cudaGetLastError();
     return BDSS_ERR_ALLOC;
@@ -532,7 +534,7 @@ template <typename T>
 static cudaError_t tcf_down(bdss_ctx *h, const Args<T> &b) {
   cudaError_t e = cudaSuccess;
   kt_begin(h, h->kt_cls);
-  for (int l = h->plan.L - 1; l >= 0 && e == cudaSuccess; --l) e = launch_tcf_down<T>(b, l, h->sms, h->stream);
+  for (int l = h->plan.L - 1; l >= 0 && e == cudaSuccess; --l) e = launch_tcf_down<T>(b, h->tcfE, l, h->sms, h->stream);
   kt_end(h, h->plan.L);
   h->launches += h->plan.L;
   return e;
@@ -547,7 +549,7 @@ static cudaError_t run_levels_tcf(bdss_ctx *h, const Args<T> &a, bool rhs) {
   const Plan &p = h->plan;
   Args<T> b = a;
   if (!rhs) b.d = 0;
-  const TcfLevel<T> c{(T *)h->tcfX, (T *)h->tcfC, (T *)h->tcfcb};
+  const TcfLevel<T> c{(T *)h->tcfX, (T *)h->tcfC, (T *)h->tcfcb, h->tcfE};
   cudaError_t e = cudaSuccess;
   for (int l = 0; l < p.L && e == cudaSuccess; ++l) {
     kt_begin(h, h->kt_cls);
@@ -724,6 +726,7 @@ bdss_status bdss_destroy(bdss_handle h) {
   cudaFree(h->tcfX);
   cudaFree(h->tcfC);
   cudaFree(h->tcfcb);
+  cudaFree(h->tcfE);
   cudaFree(h->Li);
   cudaFree(h->Yt);
   cudaFree(h->Ltinv);

@@ -12,8 +12,7 @@
 //   ACC_t = sum_{p+q=t} sum_k d_p(a) d_q(b),
 // and only the diagonals t < 8 are formed: the digit pairs left out weigh
 // below 2^-64 x 64 x 8, i.e. 2^-57 of the product of the two row maxima at
-// worst and 2^-61 for digits of random sign, beneath the rounding of a chain
-// of 64 FP64 multiply-adds.  Every
+// worst and 2^-61 for digits of random sign.  Every
 // |ACC_t| <= 2 x 64 x 64 x 128 + (t - 1) x 64 x 128 x 128 < 2^23, so the FP32
 // accumulation of the tensor cores is exact whatever its order.
 //
@@ -26,6 +25,19 @@
 // products cost three bits against a chain of FP32 multiply-adds; the sum of
 // the products h h is an integer below 2^16 x 64 and exact, and the others'
 // truncation weighs 2^-8 as much.
+//
+// Scaling along K.  These bounds are relative to the row maxima, so they say
+// nothing about a product whose rows have their large entries at different K
+// indices.  State components in different units do that: with the states of a
+// block scaled by s_k a coupling's entry k grows with s_k and that of the
+// inverse factor with 1 / s_k (spread 1e8: 5e-11 of the solution lost).  So
+// before it is cut, entry k of one operand is scaled by 2^-e_k and of the other
+// by 2^e_k, exactly, with 2^e_k about the square root of the diagonal entry
+// that index k belongs to (sl_half_exp).  The rows of an SPD system's
+// off-diagonal blocks are then bounded by the other index's diagonal entry
+// alone, |a_rk| <= sqrt(a_rr a_kk), whatever the units, as the error of a
+// Cholesky factorisation is.  Products of W^T and of y with each other need no
+// scaling: their K indices are rows of L^{-1} A and carry no unit.
 //
 // One tcgen05.mma (kind::f16, M = 128) per A part p and K step of 16 covers
 // the B parts q = 0 .. kDig-1-p of up to 32 B rows at once: the B operand
@@ -60,6 +72,26 @@ template <typename T>
 __device__ __forceinline__ int sl_row_exp(int ex) {
   return sizeof(T) == 8 && ex == 0x7FF ? kSlPoisonEx : ex;
 }
+// e with 2^e <= sqrt(x) < 2^(e+1) for a positive normal x (any bits: -512 <= e <= 512).
+__device__ __forceinline__ int sl_half_exp(double x) { return (sl_exp(x) - 1023) >> 1; }
+__device__ __forceinline__ int sl_half_exp(float x) { return (sl_exp(x) - 127) >> 1; }
+// Entries that count as v 2^e.  FP32 scales them first (sl_prep).  FP64 leaves
+// the bits alone (an FP64 instruction holds a warp's FP64 unit for 64 cycles on
+// this GPU): their exponent fields and shifts are offset instead.
+__device__ __forceinline__ void sl_prep(double &, int) {}
+__device__ __forceinline__ void sl_prep(float &v, int e) { v *= __int_as_float((127 + e) << 23); }
+// Exponent of such an entry, poison included; a row's largest is its row
+// exponent as it is.  A zero counts as 2^(e - 1023) <= 2^-511 in it, which is
+// nothing beside the sqrt(a_rr) that a row of an SPD system's factorisation is
+// rounded against; where rows have no such bound, sl_exp_nz leaves zeros out.
+__device__ __forceinline__ int sl_exp_at(double v, int e) {
+  const int x = sl_exp(v);
+  return x + (x == 0x7FF ? kSlPoisonEx : e);
+}
+__device__ __forceinline__ int sl_exp_at(float v, int) { return sl_exp(v); }
+constexpr int kSlNoEx = -(1 << 13);  // below every exponent
+__device__ __forceinline__ int sl_exp_nz(double v, int e) { return sl_exp(v) == 0 ? kSlNoEx : sl_exp_at(v, e); }
+
 // Biased digits of v under the row exponent field exmax: the byte p from the
 // top is d_p + 128.
 __device__ __forceinline__ unsigned long long sl_biased(double v, int exmax) {
@@ -83,11 +115,13 @@ __device__ __forceinline__ void sl_half_pairs(unsigned c, unsigned &lo, unsigned
 }
 
 // Two consecutive K entries of one row -> 4 bytes of every digit slab.
+// e0, e1: they count as v0 2^e0, v1 2^e1 (FP32: scaled already).
 template <typename T>
-__device__ __forceinline__ void sl_store2(T v0, T v1, int exmax, unsigned char *dst, int stride);
+__device__ __forceinline__ void sl_store2(T v0, T v1, int exmax, unsigned char *dst, int stride, int e0 = 0, int e1 = 0);
 template <>
-__device__ __forceinline__ void sl_store2<double>(double v0, double v1, int exmax, unsigned char *dst, int stride) {
-  const unsigned long long u0 = sl_biased(v0, exmax), u1 = sl_biased(v1, exmax);
+__device__ __forceinline__ void sl_store2<double>(double v0, double v1, int exmax, unsigned char *dst, int stride,
+                                                  int e0, int e1) {
+  const unsigned long long u0 = sl_biased(v0, exmax - e0), u1 = sl_biased(v1, exmax - e1);
   const unsigned h0 = (unsigned)(u0 >> 32), h1 = (unsigned)(u1 >> 32), l0 = (unsigned)u0, l1 = (unsigned)u1;
   unsigned w[8];
   sl_half_pairs(__byte_perm(h0, h1, 0x7632), w[1], w[0]);
@@ -113,7 +147,8 @@ __device__ __forceinline__ void sl_parts(float v0, float v1, int exmax, unsigned
   }
 }
 template <>
-__device__ __forceinline__ void sl_store2<float>(float v0, float v1, int exmax, unsigned char *dst, int stride) {
+__device__ __forceinline__ void sl_store2<float>(float v0, float v1, int exmax, unsigned char *dst, int stride, int,
+                                                 int) {
   unsigned w[3];
   sl_parts(v0, v1, exmax, w);
 #pragma unroll

@@ -48,14 +48,22 @@ __device__ __forceinline__ void load2<float>(const float *p, float &x, float &y)
 }
 
 // Eight consecutive K entries of one row -> 16 bytes of every digit slab.
-template <typename T>
-__device__ __forceinline__ void store8(const T *v, int ex, unsigned char *dst, int stride);
-template <>
-__device__ __forceinline__ void store8<double>(const double *v, int ex, unsigned char *dst, int stride) {
+// kSign = 1 or -1: entry i counts as v[i] 2^(kSign e_i) (FP32: scaled already).
+struct SlScale8 {  // the exponents e of eight K indices
+  unsigned w[4];
+  __device__ __forceinline__ int at(int i) const { return (int)(short)(w[i >> 1] >> (16 * (i & 1))); }
+};
+__device__ __forceinline__ SlScale8 sl_scale8(const short *p) {  // 16-byte aligned; null: zeros
+  const uint4 x = p ? __ldcg(reinterpret_cast<const uint4 *>(p)) : make_uint4(0, 0, 0, 0);
+  return {{x.x, x.y, x.z, x.w}};
+}
+template <int kSign>
+__device__ __forceinline__ void store8_of(const double *v, int ex, unsigned char *dst, int stride, SlScale8 sc) {
   unsigned w[4][8];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const unsigned long long u0 = sl_biased(v[2 * i], ex), u1 = sl_biased(v[2 * i + 1], ex);
+    const unsigned long long u0 = sl_biased(v[2 * i], ex - kSign * sc.at(2 * i)),
+                             u1 = sl_biased(v[2 * i + 1], ex - kSign * sc.at(2 * i + 1));
     const unsigned h0 = (unsigned)(u0 >> 32), h1 = (unsigned)(u1 >> 32), l0 = (unsigned)u0, l1 = (unsigned)u1;
     sl_half_pairs(__byte_perm(h0, h1, 0x7632), w[i][1], w[i][0]);
     sl_half_pairs(__byte_perm(h0, h1, 0x5410), w[i][3], w[i][2]);
@@ -66,14 +74,18 @@ __device__ __forceinline__ void store8<double>(const double *v, int ex, unsigned
   for (int p = 0; p < 8; ++p)
     *reinterpret_cast<uint4 *>(dst + p * stride) = make_uint4(w[0][p], w[1][p], w[2][p], w[3][p]);
 }
-template <>
-__device__ __forceinline__ void store8<float>(const float *v, int ex, unsigned char *dst, int stride) {
+template <int kSign>
+__device__ __forceinline__ void store8_of(const float *v, int ex, unsigned char *dst, int stride, SlScale8) {
   unsigned w[4][3];
 #pragma unroll
   for (int i = 0; i < 4; ++i) sl_parts(v[2 * i], v[2 * i + 1], ex, w[i]);
 #pragma unroll
   for (int p = 0; p < 3; ++p)
     *reinterpret_cast<uint4 *>(dst + p * stride) = make_uint4(w[0][p], w[1][p], w[2][p], w[3][p]);
+}
+template <typename T, int kSign = 0>
+__device__ __forceinline__ void store8(const T *v, int ex, unsigned char *dst, int stride, SlScale8 sc = {}) {
+  store8_of<kSign>(v, ex, dst, stride, sc);
 }
 
 // The A rows from registers: this thread's kWdCols columns of its row.  Contains a

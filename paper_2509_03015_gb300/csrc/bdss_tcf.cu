@@ -7,7 +7,8 @@
 //                (Assemble); an odd position is then factored on the FP64
 //                (FP32) ALU: L = chol(D), y = L^{-1} b, X = L^{-1}.
 //   k_tcf_schur  per eliminated block, on the tensor cores by digit products
-//                (bdss_slice.cuh): P = [W_L^T; W_R^T] = [A_{j,j-1}^T; A_{j+1,j}] X^T,
+//                (bdss_slice.cuh): P = [W_L^T; W_R^T] = [A_{j,j-1}^T; A_{j+1,j}] X^T
+//                (both factors scaled along their common index by D's diagonal),
 //                then the products of P with itself, which hold everything
 //                the elimination leaves behind:
 //                  W_L^T W_L -> left separator's D,  W_R^T W_R -> right one's,
@@ -83,6 +84,10 @@ __global__ void __launch_bounds__(256) k_tcf_diag(const __grid_constant__ Args<T
   }
   __syncthreads();
   T *Lg = a.Ld + (size_t)orig * nn;
+  if ((elim || fold_all) && threadIdx.x < kMaxN) {  // before the factorisation's first barrier and writes
+    const int i = threadIdx.x;
+    w.E[orig * kMaxN + i] = i < n ? (short)sl_half_exp(s[i * ld + i]) : (short)0;
+  }
   if (elim) {
     for (int e = threadIdx.x; e < (np - n) * np; e += blockDim.x) {
       const int i = n + e / np, c = e % np;
@@ -233,15 +238,18 @@ __global__ void __launch_bounds__(kSchurThreads, kSchurCtas<T>)
   // row r of P in the column tiles' space, its pieces permuted by r (free of
   // bank conflicts by rows and by columns)
   auto p_piece = [&](int r, int pc) { return B0 + (size_t)r * (64 * sizeof(T)) + ((pc ^ (r & (kPieces - 1))) << 4); };
-  // exponent of a row from its lanes' entries
-  auto row_exp = [&](Pair<T> v, int *ex_at) {
-    int ex = max(sl_exp(v.x), sl_exp(v.y));
+  // largest exponent of a row from its lanes' entries
+  auto row_max = [&](int ex) {
     if constexpr (LPR == 32) {
-      ex = (int)__reduce_max_sync(0xffffffffu, (unsigned)ex);
+      ex = __reduce_max_sync(0xffffffffu, ex);
     } else {
 #pragma unroll
       for (int o = 1; o < LPR; o <<= 1) ex = max(ex, __shfl_xor_sync(0xffffffffu, ex, o));
     }
+    return ex;
+  };
+  auto row_exp = [&](Pair<T> v, int *ex_at) {
+    const int ex = row_max(max(sl_exp(v.x), sl_exp(v.y)));
     if (k == 0) *ex_at = sl_row_exp<T>(ex);
     return ex;
   };
@@ -258,6 +266,12 @@ __global__ void __launch_bounds__(kSchurThreads, kSchurCtas<T>)
       }
       __syncthreads();
     }
+    // scaling of entries k, k + 1: the couplings' down, X's up
+    short2 ke[G];
+#pragma unroll
+    for (int b = 0; b < G; ++b)
+      ke[b] = m0 + b < nE ? __ldcg(reinterpret_cast<const short2 *>(w.E + ((2 * (m0 + b) + 1) << l) * kMaxN + k))
+                          : make_short2(0, 0);
     // ---- rows 0 .. 127: the couplings; 128 .. 191: X ---------------------------------
     // (level 0: X in a second pass, its digits take the place of the raw couplings)
     for (int r0 = 0; r0 < kSlRows + 64; r0 += 4 * kWarps * RPW) {
@@ -292,8 +306,13 @@ __global__ void __launch_bounds__(kSchurThreads, kSchurCtas<T>)
         const int r = r0 + (u * kWarps + warp) * RPW + sub, i = r - kSlRows;
         if (r >= kSlRows + 64) continue;  // kNP = 32: the same for the whole warp
         unsigned char *at = r < kSlRows ? A + sl_off(r, k >> 3) : B0 + (i >> 5) * kBBytes + sl_off(i & 31, k >> 3);
-        const int ex = row_exp(v[u], ex_row + r);
-        sl_store2<T>(v[u].x, v[u].y, ex, at + 2 * (k & 7), r < kSlRows ? kSlASlab : kSlBSlab);
+        const short2 kb = ke[G > 1 && (r < kSlRows ? r >= 64 : i >= 32) ? G - 1 : 0];
+        const int e0 = r < kSlRows ? -kb.x : kb.x, e1 = r < kSlRows ? -kb.y : kb.y;
+        sl_prep(v[u].x, e0);
+        sl_prep(v[u].y, e1);
+        const int ex = row_max(max(sl_exp_at(v[u].x, e0), sl_exp_at(v[u].y, e1)));
+        if (k == 0) ex_row[r] = ex;
+        sl_store2<T>(v[u].x, v[u].y, ex, at + 2 * (k & 7), r < kSlRows ? kSlASlab : kSlBSlab, e0, e1);
       }
     }
     const long long m = m0 + rblk;
@@ -501,6 +520,11 @@ __global__ void __launch_bounds__(256) k_tcf_top(const __grid_constant__ Args<T>
     v -= ldcg(w.cb + e);
     sB[c * ld + i] = (double)v;
   }
+  __syncthreads();
+  if (threadIdx.x < kMaxN) {
+    const int i = threadIdx.x;
+    w.E[i] = i < n ? (short)sl_half_exp(s[i * ld + i]) : (short)0;
+  }
   if (chol_inverse(s, ld, np, cbuf, s_cnt, &s_flag)) {
     if (threadIdx.x == 0) set_status(a.st, kStNotSPD, L, 0);
     return;
@@ -627,6 +651,9 @@ __global__ void __launch_bounds__(256, 2) k_tcf_solve(const __grid_constant__ Ar
 // multiplied by its own neighbour's vectors (B tile 0 or 1), so the halves of
 // the result are added.
 //
+// On the way down the common index of W x runs over the separators' states:
+// both factors are scaled along it (E; bdss_slice.cuh).
+//
 // With 16 columns the FP64 ALU needs 2.5 n^2 d multiply-adds a block and way
 // (82,000 cycles at n = 64); here cutting W (the same for any d) and 16k cycles
 // of triangular product remain.
@@ -635,7 +662,8 @@ constexpr int kTcLdX = kMaxN + 1;
 constexpr size_t kTcSolveSmem = 8 * kSlASlab + 2 * 8 * kTcRhs * 128 +
                                 (size_t)(kSlRows * kTcRhs + kMaxN * kTcRhs + kMaxN * kTcLdX) * sizeof(double) + 1024;
 template <bool kUp>
-__global__ void __launch_bounds__(1024, 1) k_tcf_solve_tc(const __grid_constant__ Args<double> a, int l, int first) {
+__global__ void __launch_bounds__(1024, 1) k_tcf_solve_tc(const __grid_constant__ Args<double> a, const short *E, int l,
+                                                          int first) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint64_t s_bar[2];
   __shared__ uint32_t s_tmem;
@@ -695,20 +723,23 @@ __global__ void __launch_bounds__(1024, 1) k_tcf_solve_tc(const __grid_constant_
       } else {  // columns of W^T: thread (column, eight K entries)
         const int c = tid & 63, g = (tid >> 6) & 7, half = tid >> 9;
         const double *src = half ? W1 : W0;
+        const bool live = half ? hasP : hasM;
+        const SlScale8 sc = sl_scale8(live ? E + ((half ? pos + 1 : pos - 1) << l) * kMaxN + 8 * g : nullptr);
         double v[8];
-        int ex = 0;
+        int ex = kSlNoEx;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           const int p = 8 * g + i;
-          v[i] = (half ? hasP : hasM) && c < n && p < n ? ldcg(src + (size_t)p * n + c) : 0.0;
-          ex = max(ex, sl_exp(v[i]));
+          v[i] = live && c < n && p < n ? ldcg(src + (size_t)p * n + c) : 0.0;
         }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) ex = max(ex, sl_exp_at(v[i], -sc.at(i)));
         w.exP[g * kSlRows + 64 * half + c] = ex;
         __syncthreads();
 #pragma unroll
         for (int q = 0; q < 8; ++q) ex = max(ex, w.exP[q * kSlRows + 64 * half + c]);
-        if (g == 0) w.exA[64 * half + c] = sl_row_exp<double>(ex);
-        store8<double>(v, ex, w.A + sl_off(64 * half + c, g), kSlASlab);
+        if (g == 0) w.exA[64 * half + c] = ex;
+        store8<double, -1>(v, ex, w.A + sl_off(64 * half + c, g), kSlASlab, sc);
       }
     }
 #pragma unroll
@@ -724,9 +755,13 @@ __global__ void __launch_bounds__(1024, 1) k_tcf_solve_tc(const __grid_constant_
         const double *src = a.Y + (size_t)((side ? pos + 1 : pos - 1) << l) * nd + d0 + r;
         const bool live = (side ? hasP : hasM) && d0 + r < d;
         const double v0 = live && k < n ? src[(size_t)k * d] : 0.0, v1 = live && k + 1 < n ? src[(size_t)(k + 1) * d] : 0.0;
-        const int ex = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(sl_exp(v0), sl_exp(v1)));
-        if (lane == 0) w.exB[warp] = sl_row_exp<double>(ex);
-        sl_store2<double>(v0, v1, ex, w.B + side * kTileB + sl_off(r, k >> 3) + 2 * (k & 7), kTcRhs * 128);
+        short2 ke = make_short2(0, 0);
+        if constexpr (!kUp) {
+          if (live) ke = __ldcg(reinterpret_cast<const short2 *>(E + ((side ? pos + 1 : pos - 1) << l) * kMaxN + k));
+        }
+        const int ex = __reduce_max_sync(0xffffffffu, max(sl_exp_nz(v0, ke.x), sl_exp_nz(v1, ke.y)));
+        if (lane == 0) w.exB[warp] = ex;
+        sl_store2<double>(v0, v1, ex, w.B + side * kTileB + sl_off(r, k >> 3) + 2 * (k & 7), kTcRhs * 128, ke.x, ke.y);
         fence_proxy_async_smem();
         tc_fence_before();
         __syncthreads();
@@ -851,9 +886,10 @@ cudaError_t launch_tcf_top(const Args<T> &a, const TcfLevel<T> &c, cudaStream_t 
 // products (measured at N = 4096, n = 64, both passes: d = 16, see k_tcf_solve_tc).
 constexpr int kTcMinRhs = 8;
 template <bool kUp>
-static cudaError_t launch_solve_tc(const Args<double> &a, int l, int first, long long count, int sms, cudaStream_t s) {
+static cudaError_t launch_solve_tc(const Args<double> &a, const short *E, int l, int first, long long count, int sms,
+                                   cudaStream_t s) {
   const unsigned grid = (unsigned)(count < sms ? count : sms);
-  k_tcf_solve_tc<kUp><<<grid, 1024, kTcSolveSmem, s>>>(a, l, first);
+  k_tcf_solve_tc<kUp><<<grid, 1024, kTcSolveSmem, s>>>(a, E, l, first);
   return cudaGetLastError();
 }
 
@@ -861,17 +897,17 @@ template <typename T>
 cudaError_t launch_tcf_up(const Args<T> &a, int l, int first, int sms, cudaStream_t s) {
   const long long count = first ? a.p.Nl[l] / 2 : (a.p.Nl[l] + 1) / 2;
   if constexpr (sizeof(T) == 8) {
-    if (a.d > kTcMinRhs) return launch_solve_tc<true>(a, l, first, count, sms, s);
+    if (a.d > kTcMinRhs) return launch_solve_tc<true>(a, nullptr, l, first, count, sms, s);
   }
   k_tcf_solve<T, true><<<(unsigned)count, 256, 0, s>>>(a, l, first);
   return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t launch_tcf_down(const Args<T> &a, int l, int sms, cudaStream_t s) {
+cudaError_t launch_tcf_down(const Args<T> &a, const short *E, int l, int sms, cudaStream_t s) {
   const long long count = a.p.Nl[l] / 2;
   if constexpr (sizeof(T) == 8) {
-    if (a.d > kTcMinRhs) return launch_solve_tc<false>(a, l, 0, count, sms, s);
+    if (a.d > kTcMinRhs) return launch_solve_tc<false>(a, E, l, 0, count, sms, s);
   }
   k_tcf_solve<T, false><<<(unsigned)count, 256, 0, s>>>(a, l, 0);
   return cudaGetLastError();
@@ -883,7 +919,7 @@ cudaError_t launch_tcf_down(const Args<T> &a, int l, int sms, cudaStream_t s) {
   template cudaError_t launch_tcf_schur<T>(const Args<T> &, const TcfLevel<T> &, int, int, cudaStream_t);        \
   template cudaError_t launch_tcf_top<T>(const Args<T> &, const TcfLevel<T> &, cudaStream_t);                     \
   template cudaError_t launch_tcf_up<T>(const Args<T> &, int, int, int, cudaStream_t);                                 \
-  template cudaError_t launch_tcf_down<T>(const Args<T> &, int, int, cudaStream_t);
+  template cudaError_t launch_tcf_down<T>(const Args<T> &, const short *, int, int, cudaStream_t);
 BDSS_TCF_INSTANTIATE(double)
 BDSS_TCF_INSTANTIATE(float)
 

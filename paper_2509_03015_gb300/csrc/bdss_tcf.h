@@ -15,6 +15,9 @@ struct TcfLevel {
   T *X;   // [m][n][n], zero above the diagonal
   T *C;   // [m][2][n][n]
   T *cb;  // [m][2][n][d]
+  // every block, by its original index: exponents of sqrt(D_kk) when its turn
+  // comes to be factored (zero from n on), kept with the factors
+  short *E;  // [N][64]
 };
 
 template <typename T> cudaError_t tcf_configure(int n, int d);
@@ -30,8 +33,9 @@ cudaError_t launch_tcf_schur(const Args<T> &a, const TcfLevel<T> &c, int l, int 
 // The top block of the last level (one block): factor, and x_0 if d > 0.
 template <typename T> cudaError_t launch_tcf_top(const Args<T> &a, const TcfLevel<T> &c, cudaStream_t s);
 // One level of a solve pass over stored factors that hold X (after launch_tcf_diag;
-// in FP32 after any factorisation): up (first: y of level 0) and down.
+// in FP32 after any factorisation): up (first: y of level 0) and down.  E: the
+// factorisation's exponents (FP64).
 template <typename T> cudaError_t launch_tcf_up(const Args<T> &a, int l, int first, int sms, cudaStream_t s);
-template <typename T> cudaError_t launch_tcf_down(const Args<T> &a, int l, int sms, cudaStream_t s);
+template <typename T> cudaError_t launch_tcf_down(const Args<T> &a, const short *E, int l, int sms, cudaStream_t s);
 
 }  // namespace bdss
