@@ -80,6 +80,7 @@ struct bdss_ctx {
   // 64 < n <= 256: factorisation with its products on the tensor cores
   // (bdss_wide.cu)
   void *wideX = nullptr;  // inverses of the current panel's diagonal tiles (T)
+  short *wideE = nullptr;    // exponents of their scaling
   float *wideV = nullptr;    // mixed: L^{-T} of the current level's blocks (N / 2 x n x n)
   double *wideTop = nullptr; // mixed: workspace of the FP64 top block
   int wide_ready = 0;
@@ -483,7 +484,7 @@ static cudaError_t run_levels_wide(bdss_ctx *h, const Args<double> &a, bool rhs)
   const Plan &p = h->plan;
   Args<double> b = a;
   if (!rhs) b.d = 0;
-  const WideBuf<double> w{(double *)h->wideX, nullptr, nullptr};
+  const WideBuf<double> w{(double *)h->wideX, h->wideE, nullptr, nullptr};
   cudaError_t e = wide_up<double>(h, b, w);
   if (e == cudaSuccess) e = wide_block<double>(h, b, w, p.L);
   // the solve passes read the top factor from Ltop
@@ -507,7 +508,7 @@ static cudaError_t run_levels_wide(bdss_ctx *h, const Args<float> &a, bool rhs) 
   Args<float> b = a;  // upward: b and y in Yt
   if (!rhs) b.d = 0;
   b.Y = h->Yt;
-  cudaError_t e = wide_up<float>(h, b, WideBuf<float>{(float *)h->wideX, (float *)h->Li, h->wideV});
+  cudaError_t e = wide_up<float>(h, b, WideBuf<float>{(float *)h->wideX, h->wideE, (float *)h->Li, h->wideV});
   double *ws = h->wideTop;  // X, L^{-1}, L^{-T} and y of the top block
   Args<double> t = base_args<double>(h);
   t.Ld = h->Ltop;
@@ -517,7 +518,7 @@ static cudaError_t run_levels_wide(bdss_ctx *h, const Args<float> &a, bool rhs) 
   if (e == cudaSuccess) e = launch_wide_top_in(b, h->Ltop, t.Y, h->stream);
   kt_end(h, 1);
   if (e == cudaSuccess)
-    e = wide_block<double>(h, t, WideBuf<double>{ws, ws + (size_t)64 * 64, ws + (size_t)64 * 64 + nn}, p.L);
+    e = wide_block<double>(h, t, WideBuf<double>{ws, h->wideE, ws + (size_t)64 * 64, ws + (size_t)64 * 64 + nn}, p.L);
   b.Y = a.Y;
   b.Yt = h->Yt;
   kt_begin(h, h->kt_cls);
@@ -721,6 +722,7 @@ bdss_status bdss_destroy(bdss_handle h) {
   cudaFree(h->emu.xexp);
   cudaFree(h->emu.xmax);
   cudaFree(h->wideX);
+  cudaFree(h->wideE);
   cudaFree(h->wideV);
   cudaFree(h->wideTop);
   cudaFree(h->tcfX);
@@ -851,6 +853,7 @@ bdss_status bdss_create(bdss_handle *out, int64_t N, int32_t n, int32_t d_max, b
   }
   if (ok && h->large) {
     ok = ws_alloc(h, &h->wideX, is_mixed(h) ? wide_x_bytes<float>(N) : wide_x_bytes<double>(N));
+    ok = ok && ws_alloc(h, (void **)&h->wideE, (size_t)(N / 2 > 1 ? N / 2 : 1) * 64 * sizeof(short));
     if (is_mixed(h)) {
       ok = ok && ws_alloc(h, (void **)&h->wideV, (size_t)(N / 2 > 1 ? N / 2 : 1) * nn * sizeof(float));
       ok = ok && ws_alloc(h, (void **)&h->wideTop, ((size_t)64 * 64 + 2 * nn + (size_t)n * d_max) * sizeof(double));

@@ -75,11 +75,21 @@ __device__ __forceinline__ int sl_row_exp(int ex) {
 // e with 2^e <= sqrt(x) < 2^(e+1) for a positive normal x (any bits: -512 <= e <= 512).
 __device__ __forceinline__ int sl_half_exp(double x) { return (sl_exp(x) - 1023) >> 1; }
 __device__ __forceinline__ int sl_half_exp(float x) { return (sl_exp(x) - 127) >> 1; }
+// v 2^e, exactly; FP64: on the integer pipe, a subnormal operand or result is
+// zero, as in the cut.
+__device__ __forceinline__ double sl_scale(double v, int e) {
+  const int ex = sl_exp(v), x = ex + e;
+  if ((unsigned)(ex - 1) < 0x7FEu && (unsigned)(x - 1) < 0x7FEu)
+    return __hiloint2double(__double2hiint(v) + (int)((unsigned)e << 20), __double2loint(v));
+  if (ex == 0x7FF) return v;
+  return ex == 0 || x <= 0 ? 0.0 : copysign(__longlong_as_double(0x7FF0000000000000LL), v);
+}
+__device__ __forceinline__ float sl_scale(float v, int e) { return v * __int_as_float((127 + e) << 23); }
 // Entries that count as v 2^e.  FP32 scales them first (sl_prep).  FP64 leaves
 // the bits alone (an FP64 instruction holds a warp's FP64 unit for 64 cycles on
 // this GPU): their exponent fields and shifts are offset instead.
 __device__ __forceinline__ void sl_prep(double &, int) {}
-__device__ __forceinline__ void sl_prep(float &v, int e) { v *= __int_as_float((127 + e) << 23); }
+__device__ __forceinline__ void sl_prep(float &v, int e) { v = sl_scale(v, e); }
 // Exponent of such an entry, poison included; a row's largest is its row
 // exponent as it is.  A zero counts as 2^(e - 1023) <= 2^-511 in it, which is
 // nothing beside the sqrt(a_rr) that a row of an SPD system's factorisation is

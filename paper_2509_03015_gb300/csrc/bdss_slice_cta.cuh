@@ -53,8 +53,8 @@ struct SlScale8 {  // the exponents e of eight K indices
   unsigned w[4];
   __device__ __forceinline__ int at(int i) const { return (int)(short)(w[i >> 1] >> (16 * (i & 1))); }
 };
-__device__ __forceinline__ SlScale8 sl_scale8(const short *p) {  // 16-byte aligned; null: zeros
-  const uint4 x = p ? __ldcg(reinterpret_cast<const uint4 *>(p)) : make_uint4(0, 0, 0, 0);
+__device__ __forceinline__ SlScale8 sl_scale8(const short *p) {  // 16-byte aligned
+  const uint4 x = *reinterpret_cast<const uint4 *>(p);
   return {{x.x, x.y, x.z, x.w}};
 }
 template <int kSign>
@@ -88,21 +88,23 @@ __device__ __forceinline__ void store8(const T *v, int ex, unsigned char *dst, i
   store8_of<kSign>(v, ex, dst, stride, sc);
 }
 
-// The A rows from registers: this thread's kWdCols columns of its row.  Contains a
-// CTA barrier.
-template <typename T>
-__device__ __forceinline__ void wd_cut_regs(const WdCta<T> &w, const T (&v)[kWdCols<T>], int row, int hw) {
+// The A rows from registers: this thread's kWdCols columns of its row, scaled
+// down by sc if kScaled.  Contains a CTA barrier.
+template <typename T, bool kScaled>
+__device__ __forceinline__ void wd_cut_regs(const WdCta<T> &w, const T (&v)[kWdCols<T>],
+                                            const SlScale8 (&sc)[kWdCols<T> / 8], int row, int hw) {
   constexpr int kGroups = kWdCols<T> / 8;
   int ex = 0;
 #pragma unroll
-  for (int i = 0; i < kWdCols<T>; ++i) ex = max(ex, sl_exp(v[i]));
+  for (int i = 0; i < kWdCols<T>; ++i) ex = max(ex, kScaled ? sl_exp_at(v[i], -sc[i >> 3].at(i & 7)) : sl_exp(v[i]));
   w.exP[hw * kSlRows + row] = ex;
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < 64 / kWdCols<T>; ++q) ex = max(ex, w.exP[q * kSlRows + row]);
-  if (hw == 0) w.exA[row] = sl_row_exp<T>(ex);
+  if (hw == 0) w.exA[row] = kScaled ? ex : sl_row_exp<T>(ex);
 #pragma unroll
-  for (int i = 0; i < kGroups; ++i) store8<T>(v + 8 * i, ex, w.A + sl_off(row, kGroups * hw + i), kSlASlab);
+  for (int i = 0; i < kGroups; ++i)
+    store8<T, kScaled ? -1 : 0>(v + 8 * i, ex, w.A + sl_off(row, kGroups * hw + i), kSlASlab, sc[i]);
 }
 
 // Issue the product of the cut operands.  cols2: the second 32 columns as

@@ -724,7 +724,8 @@ __global__ void __launch_bounds__(1024, 1) k_tcf_solve_tc(const __grid_constant_
         const int c = tid & 63, g = (tid >> 6) & 7, half = tid >> 9;
         const double *src = half ? W1 : W0;
         const bool live = half ? hasP : hasM;
-        const SlScale8 sc = sl_scale8(live ? E + ((half ? pos + 1 : pos - 1) << l) * kMaxN + 8 * g : nullptr);
+        SlScale8 sc = {};
+        if (live) sc = sl_scale8(E + ((half ? pos + 1 : pos - 1) << l) * kMaxN + 8 * g);
         double v[8];
         int ex = kSlNoEx;
 #pragma unroll

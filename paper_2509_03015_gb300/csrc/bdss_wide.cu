@@ -9,8 +9,8 @@
 // Per panel k two launches:
 //   k_wide_diag   the diagonal tile on the FP64 (FP32) ALU: L_kk = chol, X_kk
 //                 = L_kk^{-1};
-//   k_wide_panel  every other row v: P_vk = (S_vk - sum_{p<k} P_vp L_kp^T) X_kk^T,
-//                 and for rows of D their own diagonal tile, updated by P P^T.
+//   k_wide_panel  every other row v: P_vk = (S_vk - sum_{p<k} P_vp L_kp^T) X_kk^T
+//                 (scaled along the columns by the tile's diagonal), and for rows of D their own diagonal tile, updated by P P^T.
 // Then one launch forms what the separators receive (k_wide_schur): D, the
 // next level's couplings, b.
 //
@@ -66,13 +66,18 @@ __device__ __forceinline__ void load2_cached(const T *p, T &x, T &y) {
 
 // Digits of the K columns [0, kc) of the slots a0, a1 (A rows 0 .. 63, 64 ..
 // 127; skipped unless do_a) and b (B rows), a warp per row: all loads of the
-// 192 rows first, then the cutting.
-template <typename T>
+// 192 rows first, then the cutting.  kScaled: the A rows scaled down by 2^E
+// along K.
+template <typename T, bool kScaled>
 __device__ __forceinline__ void wd_cut(const WdCta<T> &w, const Slot<T> &a0, const Slot<T> &a1, const Slot<T> &b,
-                                       bool do_a, bool do_b, int kc, bool pairs) {
+                                       bool do_a, bool do_b, int kc, bool pairs, const short *E) {
   constexpr int kR = 64 / kWdWarps<T>;  // rows of a slot per warp
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, k = 2 * lane;
   T v[3 * kR][2];
+  short2 ke = make_short2(0, 0);
+  if constexpr (kScaled) {
+    ke = __ldcg(reinterpret_cast<const short2 *>(E + k));
+  }
 #pragma unroll
   for (int u = 0; u < 3 * kR; ++u) {
     const Slot<T> &s = u < kR ? a0 : u < 2 * kR ? a1 : b;
@@ -92,13 +97,23 @@ __device__ __forceinline__ void wd_cut(const WdCta<T> &w, const Slot<T> &a0, con
   for (int u = 0; u < 3 * kR; ++u) {
     if (!(u < 2 * kR ? do_a : do_b)) continue;
     const int r = (u % kR) * kWdWarps<T> + warp;
-    const int ex = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(sl_exp(v[u][0]), sl_exp(v[u][1])));
+    const bool scaled = kScaled && u < 2 * kR;
+    int ex, rex;
+    if (scaled) {
+      sl_prep(v[u][0], -ke.x);
+      sl_prep(v[u][1], -ke.y);
+      rex = ex = __reduce_max_sync(0xffffffffu, max(sl_exp_at(v[u][0], -ke.x), sl_exp_at(v[u][1], -ke.y)));
+    } else {
+      ex = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(sl_exp(v[u][0]), sl_exp(v[u][1])));
+      rex = sl_row_exp<T>(ex);
+    }
     if (u < 2 * kR) {
       const int ra = 64 * (u / kR) + r;
-      if (lane == 0) w.exA[ra] = sl_row_exp<T>(ex);
-      sl_store2<T>(v[u][0], v[u][1], ex, w.A + sl_off(ra, k >> 3) + 2 * (k & 7), kSlASlab);
+      if (lane == 0) w.exA[ra] = rex;
+      sl_store2<T>(v[u][0], v[u][1], ex, w.A + sl_off(ra, k >> 3) + 2 * (k & 7), kSlASlab, scaled ? -ke.x : 0,
+                   scaled ? -ke.y : 0);
     } else {
-      if (lane == 0) w.exB[r] = sl_row_exp<T>(ex);
+      if (lane == 0) w.exB[r] = rex;
       sl_store2<T>(v[u][0], v[u][1], ex, w.B + (r >> 5) * kWdBBytes<T> + sl_off(r & 31, k >> 3) + 2 * (k & 7),
                    kSlBSlab);
     }
@@ -144,9 +159,14 @@ __host__ __device__ inline int panel_slots(const WidePanels &P, bool couplings, 
 // converted, and the products themselves, half hidden (profile of
 // k_wide_schur, whose rounds are the same).  N = 1024, n = 256: the four panels
 // of level 0 take 0.55, 0.91, 0.89 and 1.04 ms.
-template <typename T>
+//
+// kFirst: panel 0 (its operands are cut, and scaled, as they come from memory;
+// a later panel's from registers).
+template <typename T, bool kFirst>
 __global__ void __launch_bounds__(kWdThreads<T>, sizeof(T) == 8 ? 1 : 2)
-    k_wide_panel(const __grid_constant__ Args<T> a, const WideBuf<T> wb, int l, int k) {
+    k_wide_panel(const __grid_constant__ Args<T> a, const WideBuf<T> wb, int l, int panel) {
+  const int k = kFirst ? 0 : panel;
+  __shared__ __align__(16) short s_E[kWdTile];
   WD_CTA_SETUP(T)
   const int n = a.p.n;
   const WidePanels P = panels_of(n);
@@ -163,6 +183,9 @@ __global__ void __launch_bounds__(kWdThreads<T>, sizeof(T) == 8 ? 1 : 2)
     if (s0.rows == 0 && s1.rows == 0) continue;
     const int nD = P.nt - 1 - k - i0;  // this tile's slots of D
     const T *Lk = a.Ld + ((size_t)(j << l) * n + (size_t)k * P.nb) * n;
+    const short *Ek = wb.E + m * kWdTile;
+    if (!kFirst && threadIdx.x < kWdTile / 2)  // at hand in round k
+      reinterpret_cast<short2 *>(s_E)[threadIdx.x] = __ldcg(reinterpret_cast<const short2 *>(Ek) + threadIdx.x);
     const Slot<T> mine = row < 64 ? s0 : s1;
     const int r = row & 63, wrows = mine.rows - (row0 & 63);  // rows of this warp
     T acc[kWdCols<T>];
@@ -177,10 +200,15 @@ __global__ void __launch_bounds__(kWdThreads<T>, sizeof(T) == 8 ? 1 : 2)
         if (rd < s1.q) c_1.rows = 0;
         Slot<T> b = rd < k ? Slot<T>{const_cast<T *>(Lk) + c0, n, 1, kb}
                            : Slot<T>{wb.X + (size_t)m * kWdTile * kWdTile, kWdTile, 1, kWdTile};
-        wd_cut<T>(w, c_0, c_1, b, rd < k || k == 0, true, rd < k ? P.nb : kb, pairs);
+        wd_cut<T, kFirst>(w, c_0, c_1, b, rd < k || kFirst, true, rd < k ? P.nb : kb, pairs, Ek);
       }
-      if ((rd == k && k > 0) || rd == k + 1) {
-        if (rd == k) {  // S - sum of the products
+      if ((rd == k && !kFirst) || rd == k + 1) {
+        SlScale8 sc[kWdCols<T> / 8] = {};
+        if (!kFirst && rd == k) {
+#pragma unroll
+          for (int i = 0; i < kWdCols<T> / 8; ++i) sc[i] = sl_scale8(s_E + cb + 8 * i);
+        }
+        if (!kFirst && rd == k) {  // S - sum of the products
           const T *src = mine.p + (r * mine.rs + (k * P.nb + cb) * mine.cs);
 #pragma unroll
           for (int i = 0; i < kWdCols<T>; i += 2) {  // (plain loads: a sector serves several of them)
@@ -195,9 +223,11 @@ __global__ void __launch_bounds__(kWdThreads<T>, sizeof(T) == 8 ? 1 : 2)
             }
             acc[i] = x0 - acc[i];
             acc[i + 1] = x1 - acc[i + 1];
+            sl_prep(acc[i], -sc[i >> 3].at(i & 7));
+            sl_prep(acc[i + 1], -sc[(i + 1) >> 3].at((i + 1) & 7));
           }
         }
-        wd_cut_regs<T>(w, acc, row, hw);
+        wd_cut_regs<T, !kFirst>(w, acc, sc, row, hw);
         if (rd == k + 1) __syncthreads();
       }
       if (rd > k) {
@@ -357,7 +387,7 @@ __global__ void __launch_bounds__(kWdThreads<T>, sizeof(T) == 8 ? 1 : 2)
         const T *Bs = isE ? BE : second ? A1 : A0;
         b = {const_cast<T *>(Bs) + (size_t)jb * nb * n + c0, n, 1, bcols};
       }
-      wd_cut<T>(w, s0, s1, b, true, true, kc, pairs);
+      wd_cut<T, false>(w, s0, s1, b, true, true, kc, pairs, nullptr);
       const int ks = (kc + 15) >> 4;
       const bool cols2 = bcols > 32;
       wd_issue<T>(w, cols2, ks, ks);
@@ -431,6 +461,10 @@ __global__ void __launch_bounds__(kDiagThreads) k_wide_diag(const __grid_constan
     const int i = i0 + u * kStep;
     if (i < kp && c <= i) s[i * ld + c] = i < kb ? ldcg(Lg + (size_t)i * n + c) : T(i == c);
   }
+  __syncthreads();
+  // before the factorisation's first barrier and writes
+  const int ec = c < kb ? sl_half_exp(s[c * (ld + 1)]) : 0;
+  if (threadIdx.x < kWdTile) wb.E[m * kWdTile + c] = (short)ec;
   if (chol_inverse(s, ld, kp, cbuf, s_cnt, &s_flag)) {
     if (threadIdx.x == 0) set_status(a.st, kStNotSPD, l, orig);
     return;
@@ -444,7 +478,7 @@ __global__ void __launch_bounds__(kDiagThreads) k_wide_diag(const __grid_constan
     const int i = i0 + u * kStep;
     const bool in = i < kb && c < kb;
     const T x = in && c <= i ? s[c * ld + i] : T(0);  // X[i][c] is in the upper triangle
-    Xg[i * kWdTile + c] = x;
+    Xg[i * kWdTile + c] = sl_scale(x, ec);
     if (in) {
       Lg[(size_t)i * n + c] = s[i * ld + c];
       if (wb.Li) V[(size_t)i * n + c] = i <= c ? s[i * ld + c] : T(0);
@@ -671,11 +705,12 @@ size_t wide_x_bytes(long long N) {
 
 template <typename T>
 cudaError_t wide_configure() {
-  cudaError_t e = cudaFuncSetAttribute((const void *)k_wide_panel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)wd_smem<T>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute((const void *)k_wide_schur<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)wd_smem<T>());
+  const void *kernels[] = {(const void *)k_wide_panel<T, true>, (const void *)k_wide_panel<T, false>,
+                           (const void *)k_wide_schur<T>};
+  cudaError_t e = cudaSuccess;
+  for (const void *k : kernels)
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wd_smem<T>());
   return e;
 }
 
@@ -701,7 +736,9 @@ cudaError_t launch_wide_panel(const Args<T> &a, const WideBuf<T> &w, int l, int 
   const bool top = l == a.p.L;
   const long long tasks = (top ? 1 : a.p.Nl[l] / 2) * ((panel_slots(P, !top, k, a.d, w.Li != nullptr) + 1) / 2);
   if (tasks == 0) return cudaSuccess;  // the last panel of the top block without right-hand sides
-  k_wide_panel<T><<<wd_grid(tasks, sizeof(T) == 8 ? sms : 2 * sms), kWdThreads<T>, wd_smem<T>(), s>>>(a, w, l, k);
+  const unsigned grid = wd_grid(tasks, sizeof(T) == 8 ? sms : 2 * sms);
+  if (k == 0) k_wide_panel<T, true><<<grid, kWdThreads<T>, wd_smem<T>(), s>>>(a, w, l, k);
+  else k_wide_panel<T, false><<<grid, kWdThreads<T>, wd_smem<T>(), s>>>(a, w, l, k);
   return cudaGetLastError();
 }
 

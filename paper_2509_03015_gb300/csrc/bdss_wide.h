@@ -16,6 +16,9 @@ WidePanels wide_panels(int n);
 template <typename T>
 struct WideBuf {
   T *X;  // [m][64][64]: inverse of the current panel's diagonal tile, per eliminated block of the level
+  // [m][64]: exponents of the square roots of the current panel's diagonal; the
+  // columns of X are scaled by 2^E, what it multiplies by 2^-E as it is cut
+  short *E;
   // both or neither (FP32, whose solve passes stream L^{-1}):
   T *Li;  // L^{-1} of every eliminated block (slot of its original index), zero above the diagonal
   T *V;   // [m][n][n]: L^{-T} of the level's blocks, as far as formed

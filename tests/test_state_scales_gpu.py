@@ -52,9 +52,27 @@ def test_blocks_up_to_64(oracle_mod, N, n, d, decades):
         assert oracle_mod.forward_error(x * D[:, :, None], Xo) <= 1e-13
 
 
+@pytest.mark.parametrize("N,n,d", [(1, 100, 1), (9, 96, 2), (5, 130, 17), (6, 256, 16)])
+@pytest.mark.parametrize("decades", DECADES)
+def test_blocks_above_64(oracle_mod, N, n, d, decades):
+    from paper_2509_03015_gb300 import Solver
+    s = inputs.random_btd(N, n, d, seed=N + n)
+    D = _scales(N, n, decades, seed=n)
+    t = _scaled(s, D)
+    As = t["A_sub"] if N > 1 else np.zeros((1, n, n))
+    Xo = oracle_mod.solve_system(s["A_diag"], s["A_sub"], s["B"])
+    sol = Solver(N, n, d_max=d)
+    X = sol.factor_solve(_dev(t["A_diag"]), _dev(As), _dev(t["B"])).cpu().numpy()
+    X2 = sol.solve(_dev(t["B"])).cpu().numpy()
+    sol.close()
+    for x in (X, X2):
+        assert oracle_mod.forward_error(x * D[:, :, None], Xo) <= 1e-13
+
+
 # a target that the FP32 solution meets at once: what the FP32 factors give,
 # unrefined; kappa(A) u_32 is below 1e-4, and 1e-4 is the bar
-@pytest.mark.parametrize("N,n,d,precision", [(40, 24, 1, "fp32_ir"), (40, 64, 4, "fp32_ir")])
+@pytest.mark.parametrize("N,n,d,precision", [(40, 24, 1, "fp32_ir"), (40, 64, 4, "fp32_ir"), (9, 96, 2, "fp32_ir"),
+                                             (6, 256, 16, "tf32_ir")])
 @pytest.mark.parametrize("decades", (3, 8))
 def test_unrefined_fp32_factors(oracle_mod, N, n, d, precision, decades):
     from paper_2509_03015_gb300 import Solver
