@@ -267,9 +267,17 @@ bdss_status bdss_adjoint_grads(bdss_handle h, const double *Lambda, const double
  * The outputs feed bdss_factor / bdss_solve directly.  Sizes: N, n, m >= 1
  * and rinv_diagonal 0 or 1 (else BDSS_ERR_INVALID_ARG); n <= 256, m <= 4096 and N (n/64 rounded up)
  * (n/64 + m/64 rounded up, + 1) < 2^31 (else BDSS_ERR_UNSUPPORTED).  The call
- * allocates N (m n + m + n) doubles of stream-ordered workspace on `cuda_stream`
- * (BDSS_ERR_ALLOC if that fails), runs two kernels and synchronises the stream
- * before it returns.  Outputs must not overlap inputs.
+ * allocates N (m n + m + n) doubles and 2 or 4 bytes per measurement and state
+ * (each rounded up to 64 a step) of stream-ordered workspace on `cuda_stream` (BDSS_ERR_ALLOC if
+ * that fails), runs a few kernels and synchronises the stream before it returns.
+ * The matrix products run on the tensor cores: both operands of Qinv G,
+ * G^T (Qinv G), Rinv H and H^T (Rinv H) are scaled along the summed index by
+ * the square roots of the precisions' diagonals (powers of two; not where these
+ * are within a factor of 16 of each other in every step), cut into digits 62 bits
+ * below the row maxima and multiplied exactly, so that an entry (r, c) of a
+ * product is off by 2^-53 at most, typically 2^-57, of
+ * sqrt(Qinv_rr) max_k sqrt(Qinv_kk) |G_kc| (and likewise for the others),
+ * whatever the units of the states and measurements.  Outputs must not overlap inputs.
  */
 bdss_status bdss_kalman_assemble(int64_t N, int32_t n, int32_t m, int32_t rinv_diagonal,
                                  const double *G, const double *H, const double *Qinv,

@@ -1470,7 +1470,9 @@ bdss_status bdss_kalman_assemble(int64_t N, int32_t n, int32_t m, int32_t rinv_d
   a.A_diag = A_diag;
   a.A_sub = N > 1 ? A_sub : nullptr;
   a.B = B;
-  const size_t words = (size_t)N * ((size_t)m * n + m + n), bytes = words * sizeof(double) + sizeof(DevStatus);
+  const size_t words = (size_t)N * ((size_t)m * n + m + n), eq = (size_t)N * kalman_pad(n),
+               er = (size_t)N * kalman_pad(m);
+  const size_t bytes = (2 * eq + er) * sizeof(short) + words * sizeof(double) + 16 + sizeof(DevStatus);
   int dev = 0, sms = 0, status = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
@@ -1481,11 +1483,15 @@ bdss_status bdss_kalman_assemble(int64_t N, int32_t n, int32_t m, int32_t rinv_d
     cudaGetLastError();
     return BDSS_ERR_ALLOC;
   }
-  a.U = static_cast<double *>(ws);
+  a.EQ = static_cast<short *>(ws);
+  a.EG = a.EQ + eq;
+  a.ER = a.EG + eq;
+  a.U = reinterpret_cast<double *>(a.ER + er);
   a.v = a.U + (size_t)N * m * n;
   a.w = a.v + (size_t)N * m;
-  DevStatus *st = reinterpret_cast<DevStatus *>(a.v + (size_t)N * (m + n));
-  cudaError_t e = cudaMemsetAsync(st, 0, kStatusCoreBytes, s);
+  a.scaled = reinterpret_cast<int *>(a.v + (size_t)N * (m + n));
+  DevStatus *st = reinterpret_cast<DevStatus *>(a.scaled + 4);
+  cudaError_t e = cudaMemsetAsync(a.scaled, 0, 16 + kStatusCoreBytes, s);
   if (e == cudaSuccess) e = launch_kalman_assemble(a, st, sms, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(&status, &st->status, sizeof(int), cudaMemcpyDeviceToHost, s);
   cudaError_t f = cudaFreeAsync(ws, s);

@@ -11,6 +11,16 @@
 //   products  A_{k+1,k} = -Qinv G and, for a full Rinv, U_k = Rinv_k H_k;
 //   diagonal  A_kk = Qinv_k + H_k^T U_k - G_{k+1}^T A_{k+1,k} (a diagonal Rinv
 //             scales the rows of H as they are cut).
+// The products' common index runs over the states of step k + 1 (Qinv G and
+// G^T A_{k+1,k}) or the measurements of step k (Rinv H and H^T U), whose units
+// enter the operands oppositely, so the operands are scaled along it by the
+// exponents of the square roots of the precisions' diagonals (bdss_slice.cuh;
+// without it a spread of units of 1e8 cost nine digits).  An entry is then off by
+// 2^-57 .. 2^-53 of sqrt(Qinv_rr) max_k sqrt(Qinv_kk) |G_kc|, which is nothing beside
+// the geometric mean of the diagonal entries of the normal equations it couples.
+// A small launch finds the exponents; where no step's differ by more than
+// kKmSpread the products run unscaled, at that loss of the 2^-57 (N = 16384,
+// n = 64, m = 32: 7.6 ms, and 8.1 ms scaled).
 // The vectors v_k = Rinv_k z_k, w_k = Qinv_k zeta_k and b_k are two small
 // FP64 launches.
 //
@@ -59,11 +69,16 @@ __device__ __forceinline__ void km_load_col(const KmSlot &s, int ld, int k0, int
     if (s.scale && in) v[i] *= ldcg(s.scale + k);
   }
 }
-__device__ __forceinline__ int km_exp(const double (&v)[8]) {
-  int ex = 0;
+// Exponent of eight entries that count as v 2^(kSign e); kSign = 0: as they are.
+template <int kSign>
+__device__ __forceinline__ int km_exp(const double (&v)[8], const SlScale8 &sc) {
+  int raw = 0, ex = kSlNoEx;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) ex = max(ex, sl_exp(v[i]));
-  return ex;
+  for (int i = 0; i < 8; ++i) {
+    raw = max(raw, sl_exp(v[i]));
+    if (kSign) ex = max(ex, sl_exp(v[i]) + kSign * sc.at(i));
+  }
+  return raw == 0x7FF ? kSlPoisonEx : kSign ? ex : raw;
 }
 
 // What a CTA multiplies: out[c][r] (+)= sum_k A(k, c) B(k, r) over K.
@@ -74,12 +89,15 @@ struct KmProduct {
   int ldb;
   bool brows;    // B read by rows (K contiguous)
   double sign;
+  const short *e[2];  // exponents along K of each
 };
 
 // acc += sign x product: this thread's row and 8 columns.  pair: two steps, 32
 // columns each per round (column 32 h + 4 hw + i at acc[4 h + i]); else 64
-// columns from the first B slot (column 8 hw + i).  ncols: columns in use.
-template <bool kPair>
+// columns from the first B slot (column 8 hw + i).  ncols: columns in use.  The A
+// columns are scaled by 2^(kSign e) along K, the B columns by the inverse (kSign =
+// 0: neither).
+template <bool kPair, int kSign>
 __device__ __forceinline__ bool km_product(WdCta<double> &w, const KmProduct &P, int ncols, int row, int hw,
                                            uint32_t lane_base, int *exK, double (&acc)[8]) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -94,9 +112,17 @@ __device__ __forceinline__ bool km_product(WdCta<double> &w, const KmProduct &P,
     for (int h = 0; h < halves; ++h) {
       double v[8], vb[8], r2[kR][2];
       const KmSlot sa = half ? P.a[1] : P.a[0];
-      if (h == 0) km_load_col(sa, P.lda, k0, P.K, c, g, v);
+      SlScale8 sca = {}, scb = {};
+      short2 ke[2] = {};
+      if (h == 0) {
+        if (kSign) sca = sl_scale8((half ? P.e[1] : P.e[0]) + k0 + 8 * g);
+        km_load_col(sa, P.lda, k0, P.K, c, g, v);
+      }
       // B row rr of 64: column 32 h + (rr & 31) of its step, or column rr
       if (P.brows) {
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+          if (kSign) ke[b] = *reinterpret_cast<const short2 *>(P.e[b] + k0 + 2 * lane);
 #pragma unroll
         for (int u = 0; u < kR; ++u) {
           const int rr = u * kWdWarps<double> + warp, k = 2 * lane;
@@ -111,33 +137,36 @@ __device__ __forceinline__ bool km_product(WdCta<double> &w, const KmProduct &P,
         }
       } else if (half == 0) {
         const KmSlot sb = kPair && c >= 32 ? P.b[1] : P.b[0];
+        if (kSign) scb = sl_scale8((kPair && c >= 32 ? P.e[1] : P.e[0]) + k0 + 8 * g);
         km_load_col(sb, P.ldb, k0, P.K, kPair ? 32 * h + (c & 31) : c, g, vb);
-        exKB[g * 64 + c] = km_exp(vb);
+        exKB[g * 64 + c] = km_exp<-kSign>(vb, scb);
       }
-      if (h == 0) exK[g * kSlRows + 64 * half + c] = km_exp(v);
+      if (h == 0) exK[g * kSlRows + 64 * half + c] = km_exp<kSign>(v, sca);
       __syncthreads();
       if (h == 0) {
-        int ex = 0;
+        int ex = kSlNoEx;
 #pragma unroll
         for (int q = 0; q < kKmGroups; ++q) ex = max(ex, exK[q * kSlRows + 64 * half + c]);
-        if (g == 0) w.exA[64 * half + c] = sl_row_exp<double>(ex);
-        store8<double>(v, ex, w.A + sl_off(64 * half + c, g), kSlASlab);
+        if (g == 0) w.exA[64 * half + c] = ex;
+        store8<double, kSign>(v, ex, w.A + sl_off(64 * half + c, g), kSlASlab, sca);
       }
       if (P.brows) {
 #pragma unroll
         for (int u = 0; u < kR; ++u) {
           const int rr = u * kWdWarps<double> + warp, k = 2 * lane;
-          const int ex = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(sl_exp(r2[u][0]), sl_exp(r2[u][1])));
-          if (lane == 0) w.exB[rr] = sl_row_exp<double>(ex);
+          const short2 kb = ke[kPair && rr >= 32 ? 1 : 0];
+          const int e0 = -kSign * kb.x, e1 = -kSign * kb.y;
+          const int ex = __reduce_max_sync(0xffffffffu, max(sl_exp_at(r2[u][0], e0), sl_exp_at(r2[u][1], e1)));
+          if (lane == 0) w.exB[rr] = ex;
           sl_store2<double>(r2[u][0], r2[u][1], ex,
-                            w.B + (rr >> 5) * kWdBBytes<double> + sl_off(rr & 31, k >> 3) + 2 * (k & 7), kSlBSlab);
+                            w.B + (rr >> 5) * kWdBBytes<double> + sl_off(rr & 31, k >> 3) + 2 * (k & 7), kSlBSlab, e0, e1);
         }
       } else if (half == 0) {
-        int ex = 0;
+        int ex = kSlNoEx;
 #pragma unroll
         for (int q = 0; q < kKmGroups; ++q) ex = max(ex, exKB[q * 64 + c]);
-        if (g == 0) w.exB[c] = sl_row_exp<double>(ex);
-        store8<double>(vb, ex, w.B + (c >> 5) * kWdBBytes<double> + sl_off(c & 31, g), kSlBSlab);
+        if (g == 0) w.exB[c] = ex;
+        store8<double, -kSign>(vb, ex, w.B + (c >> 5) * kWdBBytes<double> + sl_off(c & 31, g), kSlBSlab, scb);
       }
       const bool cols2 = kPair || ncols > 32;
       wd_issue<double>(w, cols2, ks, ks);
@@ -175,15 +204,93 @@ __device__ __forceinline__ bool km_product(WdCta<double> &w, const KmProduct &P,
   return true;
 }
 
+// Exponents for one step, a CTA: EQ and ER from the diagonals, zero beyond n or m.
+// A diagonal entry that is not positive (or not a normal number) gives way to the
+// largest of its row and column; where these are zero, the operand on the other
+// side, on which the product does not depend, is scaled below anything that counts.
+// EG scales Qinv G, whose entries are results: EQ, or nothing where the row
+// maxima of Qinv and column maxima of G are smaller together without it (precisions
+// that differ by orders of magnitude with a G that does not follow them).
+constexpr short kKmDrop = -600;
+constexpr int kKmSpread = 3;
+__device__ short km_half_exp(const double *A, int n, int i) {
+  double x = ldcg(A + (size_t)i * n + i);
+  if (!(x > 0.0) || sl_exp(x) == 0) {
+    x = 0.0;
+    for (int j = 0; j < n; ++j) x = fmax(x, fmax(fabs(A[(size_t)i * n + j]), fabs(A[(size_t)j * n + i])));
+    if (sl_exp(x) == 0) return kKmDrop;
+  }
+  return (short)sl_half_exp(x);
+}
+// Exponents of a finite v as it is and scaled by 2^e, into running maxima.
+__device__ __forceinline__ void km_maxima(double v, int e, int &m0, int &m1) {
+  const int x = sl_exp(v);
+  if (x == 0 || x == 0x7FF) return;
+  m0 = max(m0, x);
+  m1 = max(m1, x + e);
+}
+__global__ void __launch_bounds__(256) k_kalman_scale(const __grid_constant__ KalmanArgs a) {
+  __shared__ int s_lo[2], s_hi[2], s_gain;
+  const int n = a.n, m = a.m, pn = (int)kalman_pad(n), pm = (int)kalman_pad(m), tid = threadIdx.x;
+  const long long k = blockIdx.x;
+  const double *Q = a.Qinv + (size_t)k * n * n, *R = a.Rinv + (size_t)k * (a.rinv_diag ? (size_t)m : (size_t)m * m);
+  short *EQ = a.EQ + k * pn, *EG = a.EG + k * pn, *ER = a.ER + k * pm;
+  if (tid < 2) {
+    s_lo[tid] = 1 << 20;
+    s_hi[tid] = -(1 << 20);
+  }
+  if (tid == 0) s_gain = 0;
+  __syncthreads();
+  for (int i = tid; i < pn + pm; i += blockDim.x) {  // a warp's entries are one matrix's
+    const int which = i >= pn, j = which ? i - pn : i;
+    const bool in = j < (which ? m : n);
+    short e = 0;
+    if (in) {
+      if (!which) {
+        e = km_half_exp(Q, n, j);
+      } else if (a.rinv_diag) {
+        const double x = fabs(R[j]);
+        e = sl_exp(x) == 0 ? kKmDrop : (short)sl_half_exp(x);
+      } else {
+        e = km_half_exp(R, m, j);
+      }
+    }
+    const int lo = __reduce_min_sync(0xffffffffu, in ? (int)e : 1 << 20);
+    const int hi = __reduce_max_sync(0xffffffffu, in ? (int)e : -(1 << 20));
+    if ((tid & 31) == 0) {
+      atomicMin(s_lo + which, lo);
+      atomicMax(s_hi + which, hi);
+    }
+    if (which) ER[j] = e;
+    else EQ[j] = EG[j] = e;
+  }
+  __syncthreads();
+  const bool q = s_hi[0] - s_lo[0] > kKmSpread;
+  if (tid == 0 && (q || s_hi[1] - s_lo[1] > kKmSpread)) atomicExch(a.scaled, 1);
+  if (!q || k == 0) return;
+  const double *G = a.G + (size_t)k * n * n;
+  int gain = 0;  // sum of the maxima's exponents, scaled less unscaled
+  for (int r = tid >> 5; r < n; r += blockDim.x >> 5) {
+    int m0 = -(1 << 20), m1 = m0;
+    for (int c = tid & 31; c < n; c += 32) km_maxima(ldcg(Q + (size_t)r * n + c), -EQ[c], m0, m1);
+    m0 = __reduce_max_sync(0xffffffffu, m0);
+    m1 = __reduce_max_sync(0xffffffffu, m1);
+    if ((tid & 31) == 0) gain += m1 - m0;
+  }
+  for (int c = tid; c < n; c += blockDim.x) {
+    int m0 = -(1 << 20), m1 = m0;
+    for (int r = 0; r < n; ++r) km_maxima(ldcg(G + (size_t)r * n + c), EQ[r], m0, m1);
+    gain += m1 - m0;
+  }
+  atomicAdd(&s_gain, gain);
+  __syncthreads();
+  if (s_gain > 0)
+    for (int i = tid; i < pn; i += blockDim.x) EG[i] = 0;
+}
+
 // kDiag = 0: the products A_{k+1,k} and U_k; 1: the diagonal blocks.
-template <int kDiag, bool kPair>
-__global__ void __launch_bounds__(kWdThreads<double>, 1) k_kalman_tc(const __grid_constant__ KalmanArgs a, DevStatus *st) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ uint64_t s_bar[2];
-  __shared__ uint32_t s_tmem;
-  __shared__ int s_exA[kSlRows], s_exB[64], s_exK[kKmGroups * (kSlRows + 64)];
-  WdCta<double> w;
-  wd_begin(w, smem_raw, s_bar, &s_tmem, s_exA, s_exB, s_exK, kKalmanTimeoutNs);
+template <int kDiag, bool kPair, bool kScaled>
+__device__ __forceinline__ void kalman_tiles(const KalmanArgs &a, DevStatus *st, WdCta<double> &w, int *s_exK) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, hw = warp >> 2, row0 = 32 * (warp & 3), row = row0 + lane;
   const uint32_t lane_base = w.tmem + ((uint32_t)row0 << 16);
   const int n = a.n, m = a.m;
@@ -227,13 +334,18 @@ __global__ void __launch_bounds__(kWdThreads<double>, 1) k_kalman_tc(const __gri
         }
         P.a[b] = sa;
         P.b[b] = sb;
+        // (a slot without a step: any step's)
+        const bool meas = kDiag ? part == 0 : isU;
+        if (kScaled)
+          P.e[b] = meas ? a.ER + min(k, a.N - 1) * kalman_pad(m)
+                        : (kDiag ? a.EQ : a.EG) + min(k + 1, a.N - 1) * kalman_pad(n);
       }
       if (!kPair) P.b[1] = P.b[0];
       P.brows = !kDiag;
       P.K = (kDiag ? part == 0 : isU) ? m : n;
       P.ldb = kDiag ? n : isU ? m : n;
       P.sign = kDiag ? (part == 0 ? 1.0 : -1.0) : isU ? 1.0 : -1.0;
-      ok = km_product<kPair>(w, P, ncols, row, hw, lane_base, s_exK, acc);
+      ok = km_product<kPair, !kScaled ? 0 : kDiag ? -1 : 1>(w, P, ncols, row, hw, lane_base, s_exK, acc);
     }
     if (!ok) {
       if (threadIdx.x == 0) set_status(st, kStTimeout, -1, -1);
@@ -253,6 +365,18 @@ __global__ void __launch_bounds__(kWdThreads<double>, 1) k_kalman_tc(const __gri
       }
     }
   }
+}
+
+template <int kDiag, bool kPair>
+__global__ void __launch_bounds__(kWdThreads<double>, 1) k_kalman_tc(const __grid_constant__ KalmanArgs a, DevStatus *st) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint64_t s_bar[2];
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_exA[kSlRows], s_exB[64], s_exK[kKmGroups * (kSlRows + 64)];
+  WdCta<double> w;
+  wd_begin(w, smem_raw, s_bar, &s_tmem, s_exA, s_exB, s_exK, kKalmanTimeoutNs);
+  if (*a.scaled) kalman_tiles<kDiag, kPair, true>(a, st, w, s_exK);
+  else kalman_tiles<kDiag, kPair, false>(a, st, w, s_exK);
   wd_end(w);
 }
 
@@ -311,6 +435,10 @@ cudaError_t launch_kalman_assemble(const KalmanArgs &a, DevStatus *st, int sms, 
   cudaError_t e = cudaSuccess;
   for (const void *k : kernels)
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kKmSmem);
+  if (e == cudaSuccess) {
+    k_kalman_scale<<<(unsigned)a.N, kalman_pad(a.n) + kalman_pad(a.m) <= 128 ? 128 : 256, 0, s>>>(a);
+    e = cudaGetLastError();
+  }
   for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
     const int tn = (a.n + 63) / 64, tm = i || a.rinv_diag ? 0 : (a.m + 63) / 64;
     const long long tasks = kalman_groups(a.N, a.n) * kalman_row_tiles(a.n) * (tn + tm);

@@ -16,7 +16,13 @@ struct KalmanArgs {
   const double *G, *H, *Qinv, *Rinv, *z, *zeta;
   double *A_diag, *A_sub, *B;
   double *U, *v, *w;
+  // scaling along the products' common index (bdss_kalman.cu), 16-byte aligned:
+  // N x kalman_pad(n) twice, N x kalman_pad(m); whether any step needs it (cleared
+  // by the caller)
+  short *EQ, *EG, *ER;
+  int *scaled;
 };
+__host__ __device__ inline long long kalman_pad(int n) { return ((long long)n + 63) / 64 * 64; }
 // A product whose wait runs out sets st->status (cleared by the caller).
 cudaError_t launch_kalman_assemble(const KalmanArgs &a, DevStatus *st, int sms, cudaStream_t s);
 long long kalman_max_steps(int n, int m);  // largest N whose grids fit one launch

@@ -88,3 +88,59 @@ def test_unrefined_fp32_factors(oracle_mod, N, n, d, precision, decades):
     sol.close()
     for x in (X, X2):
         assert oracle_mod.forward_error(x * D[:, :, None], Xo) <= 1e-4
+
+
+@pytest.mark.parametrize("N,n,m,diag", [(3, 2, 3, False), (4, 24, 12, False), (5, 33, 65, False), (4, 64, 32, True),
+                                        (3, 100, 70, False), (3, 256, 130, True)])
+@pytest.mark.parametrize("decades", DECADES)
+def test_kalman_assembly(N, n, m, diag, decades):
+    """x = S x', z = T z': G -> S_k+1 G S_k^-1, H -> T H S^-1, Qinv -> S^-1 Qinv
+    S^-1, Rinv -> T^-1 Rinv T^-1.  Every entry against the sums of magnitudes it
+    is formed from, as a chain of FP64 multiply-adds would give it."""
+    from paper_2509_03015_gb300 import kalman_assemble
+    mod = inputs.kalman_model(N, n, m, seed=N + n + m)
+    S, T = _scales(N, n, decades, seed=n), _scales(N, m, decades, seed=m + 1)
+    G, H, Q, R = mod["G"].copy(), mod["H"], mod["Qinv"], mod["Rinv"]
+    G[1:] *= S[1:, :, None] / S[:-1, None, :]
+    H = H * T[:, :, None] / S[:, None, :]
+    Q = Q / (S[:, :, None] * S[:, None, :])
+    R = R / (T[:, :, None] * T[:, None, :])
+    if diag:
+        R = np.stack([np.diag(np.diag(r)) for r in R])
+    Rin = np.ascontiguousarray(np.einsum("kii->ki", R)) if diag else R
+    A, E, _ = kalman_assemble(_dev(G), _dev(H), _dev(Q), _dev(Rin))
+    A, E = A.cpu().numpy(), E.cpu().numpy()
+    ld = np.longdouble
+    aG, aH, aQ, aR = np.abs(G), np.abs(H), np.abs(Q), np.abs(R)
+    for k in range(N):
+        want = Q[k].astype(ld) + H[k].T.astype(ld) @ (R[k].astype(ld) @ H[k].astype(ld))
+        mag = aQ[k] + aH[k].T @ (aR[k] @ aH[k])
+        if k + 1 < N:
+            QG = Q[k + 1].astype(ld) @ G[k + 1].astype(ld)
+            want = want + G[k + 1].T.astype(ld) @ QG
+            mag = mag + aG[k + 1].T @ (aQ[k + 1] @ aG[k + 1])
+            # n products each within eps of its own size
+            assert (np.abs(E[k] + QG) <= (n + 4) * 2.0 ** -52 * (aQ[k + 1] @ aG[k + 1])).all()
+        assert (np.abs(A[k] - want) <= 2 * (n + m + 4) * 2.0 ** -52 * mag).all()
+
+
+@pytest.mark.parametrize("n", [5, 48, 80])
+def test_kalman_assembly_with_uneven_diagonal_precisions(n):
+    """Process precisions over eight decades beside a G of O(1): A_{k+1,k} entry by
+    entry.  An entry is one product; G's entries are of one magnitude, and a column
+    is cut 62 bits below its own largest."""
+    from paper_2509_03015_gb300 import kalman_assemble
+    N = 3
+    mod = inputs.kalman_model(N, n, 4, seed=n)
+    rng = np.random.default_rng(n)
+    G = rng.uniform(0.25, 1.0, (N, n, n)) * rng.choice([-1.0, 1.0], (N, n, n)) / np.sqrt(n)
+    q = np.logspace(-4, 4, n)
+    Q = np.stack([np.diag(np.random.default_rng(k).permutation(q)) for k in range(N)])
+    Q[1, 0, 0] = 0.0  # no information at all on one component
+    A, E, _ = kalman_assemble(_dev(G), _dev(mod["H"]), _dev(Q), _dev(mod["Rinv"]))
+    want = -np.matmul(Q[1:], G[1:])
+    assert (np.abs(E.cpu().numpy() - want) <= 8 * 2.0 ** -52 * np.abs(want)).all()
+    Ad = Q + np.matmul(mod["H"].transpose(0, 2, 1), np.matmul(mod["Rinv"], mod["H"]))
+    Ad[:-1] += np.matmul(G[1:].transpose(0, 2, 1), np.matmul(Q[1:], G[1:]))
+    s = np.sqrt(np.einsum("kii->ki", Ad))
+    assert (np.abs(A.cpu().numpy() - Ad) <= 4 * (n + 4) * 2.0 ** -52 * s[:, :, None] * s[:, None, :]).all()
