@@ -328,7 +328,7 @@ static bdss_status tcf_alloc(bdss_ctx *h) {
   bool ok = h->tcfX || ws_alloc(h, &h->tcfX, m * nn * esz);
   ok = ok && (h->tcfC || ws_alloc(h, &h->tcfC, m * 2 * nn * esz));
   ok = ok && (h->tcfcb || ws_alloc(h, &h->tcfcb, m * 2 * h->n * h->d_max * esz));
-  ok = ok && (h->tcfE || ws_alloc(h, (void **)&h->tcfE, (size_t)h->N * h->n * sizeof(int)));
+  ok = ok && (h->tcfE || ws_alloc(h, (void **)&h->tcfE, (size_t)h->N * kMaxN * sizeof(short)));
   if (!ok) {
     cudaGetLastError();
     return BDSS_ERR_ALLOC;

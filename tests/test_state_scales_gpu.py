@@ -90,6 +90,21 @@ def test_unrefined_fp32_factors(oracle_mod, N, n, d, precision, decades):
         assert oracle_mod.forward_error(x * D[:, :, None], Xo) <= 1e-4
 
 
+@pytest.mark.parametrize("N,n,precision", [(257, 20, "fp32_ir"), (257, 24, "fp32_ir"), (130, 31, "tf32_ir"),
+                                           (257, 33, "fp32_ir"), (65, 32, "fp64"), (65, 47, "fp64"), (9, 65, "fp64"),
+                                           (9, 100, "fp32_ir")])
+def test_workspace_guards_hold(N, n, precision):
+    """The exponents' buffers among the others: 64 to a block whatever its size."""
+    from paper_2509_03015_gb300 import Solver
+    s = inputs.random_btd(N, n, 1, seed=n)
+    sol = Solver(N, n, d_max=1, precision=precision)
+    if precision == "fp64":
+        sol.set_option("schur_emu", 1)
+    sol.set_option("debug_guards", 1)
+    sol.factor_solve(_dev(s["A_diag"]), _dev(s["A_sub"]), _dev(s["B"]))
+    sol.close()
+
+
 @pytest.mark.parametrize("N,n,m,diag", [(3, 2, 3, False), (4, 24, 12, False), (5, 33, 65, False), (4, 64, 32, True),
                                         (3, 100, 70, False), (3, 256, 130, True)])
 @pytest.mark.parametrize("decades", DECADES)
