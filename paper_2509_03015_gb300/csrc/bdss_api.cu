@@ -1302,7 +1302,6 @@ static bdss_status krylov_cycle(bdss_ctx *h, const double *B, double *X, int d) 
 // of either kind.
 static bdss_status refine(bdss_ctx *h, const double *B, double *X, int d, bdss_info *info) {
   constexpr int kMaxCgCycles = 4;
-  constexpr double kTargetMargin = 0.95;
   double prev = INFINITY, berr = -1.0;
   int cycles = 0;
   bdss_status result = BDSS_ERR_NO_CONVERGENCE;
@@ -1311,12 +1310,9 @@ static bdss_status refine(bdss_ctx *h, const double *B, double *X, int d, bdss_i
   for (int it = 0;; ++it) {
     bdss_status st = residual_berr(h, B, X, d, &berr);
     if (st != BDSS_OK) return st;
-    // the measured error stands for the true one within a few per cent (a
-    // residual of finite precision, an FP32 norm of A): the target counts as
-    // met with that much to spare, or exactly once refinement has stalled
+    if (berr <= h->target) { result = BDSS_OK; break; }
     const bool stalled = it > 0 && !(berr < 0.5 * prev);
     const bool plain_done = stalled || it >= h->max_refine;
-    if (berr <= (plain_done ? 1.0 : kTargetMargin) * h->target) { result = BDSS_OK; break; }
     // shifted factors are no accurate solver of A: CG from the first correction
     const bool cg = cycles > 0 || h->krylov == 2 || (h->krylov == 1 && (plain_done || h->shift_used > 0));
     if (!cg) {
