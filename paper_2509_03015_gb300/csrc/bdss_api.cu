@@ -319,6 +319,35 @@ static bool use_tcf(const bdss_ctx *h) {
   if (h->tcf_opt >= 0) return h->tcf_opt == 1;
   return h->persistent && !h->skip_barrier && h->nstar == 1 && tcf_by_size(h);
 }
+// Solve passes over its factors: a launch per level and way (bdss_tcf.cu), or the
+// single launch of the persistent kernel, which reads the same L (FP32: L^{-1}) and
+// W.  Measured on GB300, the pass by levels over the single launch:
+//   FP64   d = 1     4     5     8     9    64     (N = 128 .. 8192)
+//   n = 32  1.5-2.4 1.4-1.8 2.3-3.2 1.9-2.4 0.7-0.9 0.6
+//   n = 48  1.1-1.6 1.0-1.1 1.6-1.8 1.2-1.3 0.6     0.4
+//   n = 52  1.0-1.3 0.9     1.2-1.4 1.1     0.6     0.4
+//   n = 56  1.0-1.2 0.9     1.1-1.3 1.0     0.6     0.4
+//   n = 64  0.9-1.1 0.8     1.0-1.2 0.9     0.5     0.3
+// (up to eight columns go through the ALU, four at a time: d = 5 pays for eight;
+// more are digit products, 16 at a time.)
+//   FP32   d = 1     4     5     16      64        (N = 32 .. 4096)
+//   n = 20  1.0     1.0     1.1-1.3 1.1-1.4 1.6-1.8
+//   n = 28  0.9     0.9     1.0-1.1 1.1     1.3
+//   n = 32  0.9     0.9     1.0     0.9     0.7
+//   n = 36  0.8-0.9 0.9     1.0     0.9-1.0 1.0-1.1
+//   n = 64  0.8     0.8     0.8     0.6     0.3-0.5
+static bool tcf_solve_by_size(const bdss_ctx *h, int d) {
+  if (!h->persistent) return true;
+  const int n = h->n;
+  if (is_mixed(h)) return n >= 40 || n == 32 || (n > 32 ? d < 24 : d <= 4);
+  if (d > kTcfMinRhsTc) return true;
+  switch (d) {
+    case 1: case 2: return n >= 60 && h->N <= 2048;
+    case 3: case 4: return n >= 52;
+    case 5: case 6: return false;
+    default: return n >= 56;
+  }
+}
 // Its buffers: with the handle where the size selects the path, else when the
 // option asks for it.
 static bdss_status tcf_alloc(bdss_ctx *h) {
@@ -648,7 +677,7 @@ static cudaError_t run_levels(bdss_ctx *h, const Args<T> &a, bool factor, bool r
   const Plan &p = h->plan;
   if (h->large) return run_levels_large<T>(h, a, factor, rhs);
   if (factor && use_tcf(h)) return run_levels_tcf<T>(h, a, rhs);
-  if (!factor && h->tcf_factored && use_tcf(h)) return run_solve_tcf<T>(h, a);
+  if (!factor && h->tcf_factored && use_tcf(h) && tcf_solve_by_size(h, a.d)) return run_solve_tcf<T>(h, a);
   const int cap = h->bps * h->sms;
   if (h->persistent) {
     long long most = 1;  // tasks of the busiest step

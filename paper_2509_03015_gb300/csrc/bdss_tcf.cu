@@ -883,9 +883,6 @@ cudaError_t launch_tcf_top(const Args<T> &a, const TcfLevel<T> &c, cudaStream_t 
   return cudaGetLastError();
 }
 
-// Solve passes with more than kTcMinRhs right-hand sides take the digit
-// products (measured at N = 4096, n = 64, both passes: d = 16, see k_tcf_solve_tc).
-constexpr int kTcMinRhs = 8;
 template <bool kUp>
 static cudaError_t launch_solve_tc(const Args<double> &a, const short *E, int l, int first, long long count, int sms,
                                    cudaStream_t s) {
@@ -898,7 +895,7 @@ template <typename T>
 cudaError_t launch_tcf_up(const Args<T> &a, int l, int first, int sms, cudaStream_t s) {
   const long long count = first ? a.p.Nl[l] / 2 : (a.p.Nl[l] + 1) / 2;
   if constexpr (sizeof(T) == 8) {
-    if (a.d > kTcMinRhs) return launch_solve_tc<true>(a, nullptr, l, first, count, sms, s);
+    if (a.d > kTcfMinRhsTc) return launch_solve_tc<true>(a, nullptr, l, first, count, sms, s);
   }
   k_tcf_solve<T, true><<<(unsigned)count, 256, 0, s>>>(a, l, first);
   return cudaGetLastError();
@@ -908,7 +905,7 @@ template <typename T>
 cudaError_t launch_tcf_down(const Args<T> &a, const short *E, int l, int sms, cudaStream_t s) {
   const long long count = a.p.Nl[l] / 2;
   if constexpr (sizeof(T) == 8) {
-    if (a.d > kTcMinRhs) return launch_solve_tc<false>(a, E, l, 0, count, sms, s);
+    if (a.d > kTcfMinRhsTc) return launch_solve_tc<false>(a, E, l, 0, count, sms, s);
   }
   k_tcf_solve<T, false><<<(unsigned)count, 256, 0, s>>>(a, l, 0);
   return cudaGetLastError();

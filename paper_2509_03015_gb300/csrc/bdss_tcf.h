@@ -32,6 +32,11 @@ template <typename T>
 cudaError_t launch_tcf_schur(const Args<T> &a, const TcfLevel<T> &c, int l, int sms, cudaStream_t s);
 // The top block of the last level (one block): factor, and x_0 if d > 0.
 template <typename T> cudaError_t launch_tcf_top(const Args<T> &a, const TcfLevel<T> &c, cudaStream_t s);
+// FP64 solve passes with more right-hand sides than this are digit products
+// (n = 64, N = 4096, d = 16, both ways: 4.2 -> 1.74 ms; with nine columns, in a
+// tile of 16, they take 0.5 to 0.9 of the persistent kernel's time from n = 32 on,
+// where the ALU kernel takes 0.9 to 2.4 of it with eight).
+constexpr int kTcfMinRhsTc = 8;
 // One level of a solve pass over stored factors that hold X (after launch_tcf_diag;
 // in FP32 after any factorisation): up (first: y of level 0) and down.  E: the
 // factorisation's exponents (FP64).

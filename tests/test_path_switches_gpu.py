@@ -87,3 +87,43 @@ def test_stored_factors_with_a_serial_top(oracle_mod, N, n, nstar, d):
     for x in (X, X2):
         assert oracle_mod.forward_error(x, Xo) <= 1e-12
         assert oracle_mod.backward_error(s["A_diag"], s["A_sub"], x, s["B"]) <= 1e-14
+
+
+# the choice between the solve passes over tensor-core factors, both sides of its
+# lines (one launch: the persistent kernel, over the other path's factors)
+@pytest.mark.parametrize("N,n,d,one", [(130, 52, 3, False), (130, 51, 4, True), (65, 60, 1, False), (65, 59, 2, True),
+                                       (65, 64, 5, True), (65, 64, 6, True), (65, 56, 7, False), (65, 55, 8, True),
+                                       (65, 32, 9, False), (65, 32, 8, True), (2049, 60, 1, True)])
+def test_choice_of_the_solve_pass(oracle_mod, N, n, d, one):
+    from paper_2509_03015_gb300 import Solver
+    s = inputs.random_btd(N, n, d, seed=N + n)
+    sol = Solver(N, n, d_max=d)
+    sol.set_option("schur_emu", 1)
+    Ad, As, B = _put(s)
+    sol.factor(Ad, As)
+    X = sol.solve(B).cpu().numpy()
+    launches = sol.launch_stats()[0]
+    sol.close()
+    assert (launches == 1) == one
+    Xo = oracle_mod.solve_system(s["A_diag"], s["A_sub"], s["B"])
+    assert oracle_mod.forward_error(X, Xo) <= 1e-12
+    assert oracle_mod.backward_error(s["A_diag"], s["A_sub"], X, s["B"]) <= 1e-14
+
+
+@pytest.mark.parametrize("N,n,d,one", [(40, 20, 4, False), (40, 31, 5, True), (40, 32, 64, False), (40, 33, 23, False),
+                                       (40, 39, 24, True), (40, 40, 24, False)])
+def test_choice_of_the_solve_pass_in_mixed_precision(oracle_mod, N, n, d, one):
+    """With a target that the unrefined solution meets: the pass and one residual."""
+    from paper_2509_03015_gb300 import Solver
+    s = inputs.random_btd(N, n, d, seed=N + n)
+    sol = Solver(N, n, d_max=d, precision="fp32_ir")
+    Ad, As, B = _put(s)
+    sol.factor(Ad, As)
+    X = sol.solve(B).cpu().numpy()
+    sol.set_option("target_berr_e18", 10 ** 18)
+    sol.solve(B)
+    launches = sol.launch_stats()[0]
+    sol.close()
+    assert (launches == 2) == one
+    Xo = oracle_mod.solve_system(s["A_diag"], s["A_sub"], s["B"])
+    assert oracle_mod.forward_error(X, Xo) <= 1e-11
