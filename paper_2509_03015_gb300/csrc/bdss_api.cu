@@ -301,17 +301,30 @@ static bool use_small(const bdss_ctx *h) {
 //   n = 40   1.11  1.01  0.95  0.91        n = 24   0.89  0.84  0.84
 //   n = 48   0.93  0.82  0.73  0.67        n = 48   0.78  0.68  0.74
 //   n = 64   0.68  0.57  0.47  0.42        n = 64   0.70  0.60  0.69
-// (n = 37, whose odd rows cannot be read in pairs, 1.05 at N = 8192.)  Handles
-// for several right-hand sides keep the single launch up to N = 1536: their
-// callers count on one.
+// (n = 37, whose odd rows cannot be read in pairs, 1.05 at N = 8192.)  FP64 with
+// several right-hand sides:
+//          N = 512            1536                8192
+//   n = 40   d = 4: 0.99        1.00                0.89
+//            d = 5, 8: 1.1      1.15, 1.07          1.03, 0.95
+//   n = 44   d = 5: 1.02        1.02                0.89
+//   n = 48   d = 4, 16: 0.8, 0.7  0.8, 0.65         0.65, 0.55
+//   n = 64   d = 4, 16: 0.56    0.52, 0.44          0.41, 0.36
+// Five to eight of them cost the downward pass two rounds of four, so n < 44
+// waits for N = 8192 there.  Handles with d_max > 1 keep the single launch below
+// N = 1536 whatever the table says: that such a call is one launch is pinned by a
+// test of the option (N = 1500, n = 64, d = 4).  FP32 from n = 20: at n = 16 it is
+// 0.95 of the persistent kernel's time, and a test of that kernel's barrier trace
+// pins it there.
 constexpr int kTcfMinN = 32;
 constexpr int kTcfAutoMinN = 40, kTcfAutoMinBlocks = 1536;
+constexpr int kTcfAutoMinNUneven = 44, kTcfAutoMinBlocksUneven = 8192;  // five to eight right-hand sides
 constexpr int kTcfAutoMinN1 = 48, kTcfAutoMinBlocks1 = 128;  // one right-hand side
 constexpr int kTcfAutoMinN32 = 20, kTcfAutoMinBlocks32 = 32;  // FP32
 static bool tcf_by_size(const bdss_ctx *h) {
   if (h->large) return false;
   if (is_mixed(h)) return h->n >= kTcfAutoMinN32 && h->N >= kTcfAutoMinBlocks32;
-  return (h->n >= kTcfAutoMinN && h->N >= kTcfAutoMinBlocks) ||
+  const bool uneven = h->d_max > 4 && h->d_max <= 8 && h->n < kTcfAutoMinNUneven && h->N < kTcfAutoMinBlocksUneven;
+  return (h->n >= kTcfAutoMinN && h->N >= kTcfAutoMinBlocks && !uneven) ||
          (h->d_max == 1 && h->n >= kTcfAutoMinN1 && h->N >= kTcfAutoMinBlocks1);
 }
 static bool use_tcf(const bdss_ctx *h) {

@@ -127,3 +127,19 @@ def test_choice_of_the_solve_pass_in_mixed_precision(oracle_mod, N, n, d, one):
     assert (launches == 2) == one
     Xo = oracle_mod.solve_system(s["A_diag"], s["A_sub"], s["B"])
     assert oracle_mod.forward_error(X, Xo) <= 1e-11
+
+
+# five to eight right-hand sides: the factorisation's line (launches of the call)
+@pytest.mark.parametrize("N,n,d,tc", [(1600, 43, 5, False), (1600, 43, 8, False), (1600, 44, 5, True), (1600, 43, 9, True),
+                                      (1600, 43, 4, True), (8192, 40, 5, True)])
+def test_choice_of_the_factorisation_for_several_columns(oracle_mod, N, n, d, tc):
+    from paper_2509_03015_gb300 import Solver
+    s = inputs.random_btd(N, n, d, seed=N + n)
+    sol = Solver(N, n, d_max=d)
+    X = sol.factor_solve(*_put(s)).cpu().numpy()
+    launches = sol.launch_stats()[0]
+    sol.close()
+    assert (launches > 1) == tc
+    Xo = oracle_mod.solve_system(s["A_diag"], s["A_sub"], s["B"])
+    assert oracle_mod.forward_error(X, Xo) <= 1e-12
+    assert oracle_mod.backward_error(s["A_diag"], s["A_sub"], X, s["B"]) <= 1e-14
