@@ -270,7 +270,8 @@ bdss_status bdss_adjoint_grads(bdss_handle h, const double *Lambda, const double
  * allocates N (m n + m + n) doubles and 2 or 4 bytes per measurement and state
  * (each rounded up to 64 a step) of stream-ordered workspace on `cuda_stream` (BDSS_ERR_ALLOC if
  * that fails), runs a few kernels and synchronises the stream before it returns.
- * The matrix products run on the tensor cores: both operands of Qinv G,
+ * Small assemblies run on the FP64 ALU.  The matrix products of the others run on
+ * the tensor cores: both operands of Qinv G,
  * G^T (Qinv G), Rinv H and H^T (Rinv H) are scaled along the summed index by
  * the square roots of the precisions' diagonals (powers of two; not where these
  * are within a factor of 16 of each other in every step), cut into digits 62 bits

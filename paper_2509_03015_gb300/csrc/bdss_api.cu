@@ -1529,9 +1529,10 @@ bdss_status bdss_kalman_assemble(int64_t N, int32_t n, int32_t m, int32_t rinv_d
   a.w = a.v + (size_t)N * m;
   a.scaled = reinterpret_cast<int *>(a.v + (size_t)N * (m + n));
   DevStatus *st = reinterpret_cast<DevStatus *>(a.scaled + 4);
-  cudaError_t e = cudaMemsetAsync(a.scaled, 0, 16 + kStatusCoreBytes, s);
+  const bool alu = kalman_on_alu(N, n, m);
+  cudaError_t e = alu ? cudaSuccess : cudaMemsetAsync(a.scaled, 0, 16 + kStatusCoreBytes, s);
   if (e == cudaSuccess) e = launch_kalman_assemble(a, st, sms, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&status, &st->status, sizeof(int), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess && !alu) e = cudaMemcpyAsync(&status, &st->status, sizeof(int), cudaMemcpyDeviceToHost, s);
   cudaError_t f = cudaFreeAsync(ws, s);
   if (e == cudaSuccess) e = f;
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);

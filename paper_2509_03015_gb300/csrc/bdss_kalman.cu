@@ -7,7 +7,7 @@
 //   A_{k+1,k} = -Qinv_{k+1} G_{k+1}
 //   b_k       = H_k^T Rinv_k z_k + Qinv_k zeta_k - G_{k+1}^T Qinv_{k+1} zeta_{k+1}
 // The n x n and m x n products run on the tensor cores as digit products
-// (bdss_slice.cuh), two launches:
+// (bdss_slice.cuh; small assemblies on the FP64 ALU, kalman_on_alu), two launches:
 //   products  A_{k+1,k} = -Qinv G and, for a full Rinv, U_k = Rinv_k H_k;
 //   diagonal  A_kk = Qinv_k + H_k^T U_k - G_{k+1}^T A_{k+1,k} (a diagonal Rinv
 //             scales the rows of H as they are cut).
@@ -20,7 +20,7 @@
 // the geometric mean of the diagonal entries of the normal equations it couples.
 // A small launch finds the exponents; where no step's differ by more than
 // kKmSpread the products run unscaled, at that loss of the 2^-57 (N = 16384,
-// n = 64, m = 32: 7.6 ms, and 8.1 ms scaled).
+// n = 64, m = 32: 7.6 ms, and 8.4 ms scaled).
 // The vectors v_k = Rinv_k z_k, w_k = Qinv_k zeta_k and b_k are two small
 // FP64 launches.
 //
@@ -34,6 +34,7 @@
 // FP64-ALU tiles took 23.2 ms at N = 16384, n = 64, m = 32 (0.82 of the FP64
 // pipe's rate).
 #include "bdss_kalman.h"
+#include "bdss_large.cuh"
 #include "bdss_launch.h"
 #include "bdss_slice_cta.cuh"
 
@@ -381,9 +382,8 @@ __global__ void __launch_bounds__(kWdThreads<double>, 1) k_kalman_tc(const __gri
 }
 
 // v_k = Rinv_k z_k, w_k = Qinv_k zeta_k (one step per CTA).
-__global__ void __launch_bounds__(kThreads) k_kalman_vectors(const __grid_constant__ KalmanArgs a) {
+__device__ __forceinline__ void kalman_vectors(const KalmanArgs &a, long long k) {
   const int n = a.n, m = a.m;
-  const long long k = blockIdx.x;
   const double *Rk = a.Rinv + (size_t)k * (a.rinv_diag ? (size_t)m : (size_t)m * m), *zk = a.z + k * m;
   const double *Qk = a.Qinv + (size_t)k * n * n, *ek = a.zeta ? a.zeta + k * n : nullptr;
   for (int i = threadIdx.x; i < n + m; i += blockDim.x) {
@@ -402,10 +402,13 @@ __global__ void __launch_bounds__(kThreads) k_kalman_vectors(const __grid_consta
   }
 }
 
+__global__ void __launch_bounds__(kThreads) k_kalman_vectors(const __grid_constant__ KalmanArgs a) {
+  kalman_vectors(a, blockIdx.x);
+}
+
 // b_k = H_k^T v_k + w_k - G_{k+1}^T w_{k+1}.
-__global__ void __launch_bounds__(kThreads) k_kalman_rhs(const __grid_constant__ KalmanArgs a) {
+__device__ __forceinline__ void kalman_rhs(const KalmanArgs &a, long long k) {
   const int n = a.n, m = a.m;
-  const long long k = blockIdx.x;
   const double *Hk = a.H + (size_t)k * m * n, *vk = a.v + k * m, *wk = a.w + k * n;
   const bool next = k + 1 < a.N;
   const double *G1 = a.G + (size_t)(k + 1) * n * n, *w1 = a.w + (k + 1) * n;
@@ -418,17 +421,129 @@ __global__ void __launch_bounds__(kThreads) k_kalman_rhs(const __grid_constant__
     a.B[k * n + i] = s + wk[i] - g;
   }
 }
+__global__ void __launch_bounds__(kThreads) k_kalman_rhs(const __grid_constant__ KalmanArgs a) {
+  kalman_rhs(a, blockIdx.x);
+}
+
+// The same on the FP64 ALU, for small assemblies: a flat grid of (step, task) CTAs
+// of 64 x 64 tiles, two launches, the vectors among the tasks.
+//   products  A_{k+1,k} (-Qinv G), U_k = Rinv_k H_k (a row scaling when Rinv_k is
+//             diagonal), v_k and w_k;
+//   diagonal  A_kk = Qinv_k + H_k^T U_k - G_{k+1}^T A_{k+1,k}, and b_k.
+__device__ void store_tile(double *out, long long ld, int rows, int cols, int r0, int c0, const double (&acc)[4][4],
+                           double sign, const double *add) {
+  const int tm = threadIdx.x >> 4, tn = threadIdx.x & 15;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int r = r0 + 4 * tm + i;
+    if (r >= rows) continue;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int c = c0 + 4 * tn + j;
+      if (c >= cols) continue;
+      const long long o = (long long)r * ld + c;
+      out[o] = (add ? add[o] : 0.0) + sign * acc[i][j];
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kThreads) k_kalman_products_alu(const __grid_constant__ KalmanArgs a) {
+  __shared__ double sA[kKc * kTilePad], sB[kKc * kTilePad];
+  const int n = a.n, m = a.m, nt = ntiles(n), mt = ntiles(m);
+  const int tasks = nt * nt + mt * nt + 1;
+  const long long k = (long long)blockIdx.x / tasks;
+  const int t = (int)((long long)blockIdx.x - k * tasks);
+  const long long nn = (long long)n * n, mn = (long long)m * n;
+  const long long mm = a.rinv_diag ? (long long)m : (long long)m * m;  // Rinv stride per step
+  double acc[4][4] = {};
+  if (t < nt * nt) {
+    if (k + 1 >= a.N) return;
+    const int r0 = (t / nt) * kTile, c0 = (t % nt) * kTile;
+    const View<double> Q{a.Qinv + (k + 1) * nn, n, 1, n, n};  // (r, j) -> Qinv_{k+1}[r][j]
+    const View<double> Gt{a.G + (k + 1) * nn, 1, n, n, n};    // (c, j) -> G_{k+1}[j][c]
+    gemm_nt_tile(acc, Q, r0, Gt, c0, n, sA, sB);
+    store_tile(a.A_sub + k * nn, n, n, n, r0, c0, acc, -1.0, nullptr);
+  } else if (t < nt * nt + mt * nt) {
+    const int u = t - nt * nt, r0 = (u / nt) * kTile, c0 = (u % nt) * kTile;
+    if (a.rinv_diag) {
+      const double *rk = a.Rinv + k * mm, *Hk = a.H + k * mn;
+      double *Uk = a.U + k * mn;
+      for (int e = threadIdx.x; e < kTile * kTile; e += blockDim.x) {
+        const int r = r0 + e / kTile, c = c0 + e % kTile;
+        if (r < m && c < n) Uk[(long long)r * n + c] = rk[r] * Hk[(long long)r * n + c];
+      }
+      return;
+    }
+    const View<double> R{a.Rinv + k * mm, m, 1, m, m};  // (r, j) -> Rinv_k[r][j]
+    const View<double> Ht{a.H + k * mn, 1, n, n, m};    // (c, j) -> H_k[j][c]
+    gemm_nt_tile(acc, R, r0, Ht, c0, m, sA, sB);
+    store_tile(a.U + k * mn, n, m, n, r0, c0, acc, 1.0, nullptr);
+  } else if (a.B) {
+    kalman_vectors(a, k);
+  }
+}
+
+__global__ void __launch_bounds__(kThreads) k_kalman_diag_alu(const __grid_constant__ KalmanArgs a) {
+  __shared__ double sA[kKc * kTilePad], sB[kKc * kTilePad];
+  const int n = a.n, m = a.m, nt = ntiles(n);
+  const int tasks = nt * nt + 1;
+  const long long k = (long long)blockIdx.x / tasks;
+  const int t = (int)((long long)blockIdx.x - k * tasks);
+  const long long nn = (long long)n * n, mn = (long long)m * n;
+  if (t < nt * nt) {
+    const int r0 = (t / nt) * kTile, c0 = (t % nt) * kTile;
+    double acc[4][4] = {};
+    const View<double> Hc{a.H + k * mn, 1, n, n, m};  // (r, j) -> H_k[j][r]
+    const View<double> Uc{a.U + k * mn, 1, n, n, m};  // (c, j) -> U_k[j][c]
+    gemm_nt_tile(acc, Hc, r0, Uc, c0, m, sA, sB);
+    if (k + 1 < a.N) {
+      double acc2[4][4] = {};
+      const View<double> Gc{a.G + (k + 1) * nn, 1, n, n, n};  // (r, j) -> G_{k+1}[j][r]
+      const View<double> Sc{a.A_sub + k * nn, 1, n, n, n};    // (c, j) -> A_{k+1,k}[j][c]
+      gemm_nt_tile(acc2, Gc, r0, Sc, c0, n, sA, sB);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] -= acc2[i][j];
+    }
+    store_tile(a.A_diag + k * nn, n, n, n, r0, c0, acc, 1.0, a.Qinv + k * nn);
+  } else if (a.B) {
+    kalman_rhs(a, k);
+  }
+}
 
 }  // namespace
 
-// Grid limit of the former per-tile launches, kept as the entry point's limit.
+// Limit of the ALU tiles' grids, the entry point's for either path.
 long long kalman_max_steps(int n, int m) {
-  const int nt = (n + 63) / 64, mt = (m + 63) / 64;
+  const int nt = ntiles(n), mt = ntiles(m);
   return 0x7fffffffLL / (nt * nt + mt * nt + 1);
+}
+
+// The tensor-core path takes five launches and 128-column tiles of 64 K entries
+// whatever n and m: few steps, or small ones, are faster on the ALU.  Its time over
+// the ALU's, measured on GB300 (full Rinv; diagonal ones cross 1 at the same sizes
+// within two):
+//   N          n + m:  2     5     8     10    14    20    32    48    64
+//   4 .. 32           1.3   1.3   1.2   1.2   1.2   1.15  1.1   1.05  0.95
+//   128               1.3   1.2   1.2   1.15  1.1   1.0   0.9   0.85
+//   512               1.4   1.25  1.1   1.1   1.0   0.85  0.75
+//   2048              1.7   1.3   1.1   1.0   0.85  0.65
+//   100000            2.7   1.6   1.2   1.0   0.7   0.5
+// One step has no coupling to form (n + m = 96: 1.0 .. 1.15).
+bool kalman_on_alu(long long N, int n, int m) {
+  if (N == 1) return n + m <= 96;
+  return n + m <= 48 && n + m <= 10 + 1280 / N;
 }
 
 cudaError_t launch_kalman_assemble(const KalmanArgs &a, DevStatus *st, int sms, cudaStream_t s) {
   if (a.N > kalman_max_steps(a.n, a.m)) return cudaErrorInvalidValue;
+  if (kalman_on_alu(a.N, a.n, a.m)) {
+    const int nt = ntiles(a.n), mt = ntiles(a.m);
+    k_kalman_products_alu<<<(unsigned)(a.N * (nt * nt + mt * nt + 1)), kThreads, 0, s>>>(a);
+    k_kalman_diag_alu<<<(unsigned)(a.N * (nt * nt + 1)), kThreads, 0, s>>>(a);
+    return cudaGetLastError();
+  }
   const bool pair = a.n <= 64;
   const void *kernels[2] = {pair ? (const void *)k_kalman_tc<0, true> : (const void *)k_kalman_tc<0, false>,
                             pair ? (const void *)k_kalman_tc<1, true> : (const void *)k_kalman_tc<1, false>};

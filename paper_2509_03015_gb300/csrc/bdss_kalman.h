@@ -23,6 +23,9 @@ struct KalmanArgs {
   int *scaled;
 };
 __host__ __device__ inline long long kalman_pad(int n) { return ((long long)n + 63) / 64 * 64; }
+// Whether an assembly is small enough for the FP64-ALU tiles, which use neither the
+// scaling nor a status.
+bool kalman_on_alu(long long N, int n, int m);
 // A product whose wait runs out sets st->status (cleared by the caller).
 cudaError_t launch_kalman_assemble(const KalmanArgs &a, DevStatus *st, int sms, cudaStream_t s);
 long long kalman_max_steps(int n, int m);  // largest N whose grids fit one launch
