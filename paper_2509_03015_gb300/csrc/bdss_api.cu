@@ -38,7 +38,7 @@ struct bdss_ctx {
   bool large = false;   // 64 < n <= 256: tiled path
   void *Ld = nullptr;   // N n n  (T)
   void *Wb = nullptr;   // coupling slots (T)
-  void *Eb = nullptr;   // large path: couplings of levels >= 1 (T)
+  double *Eb = nullptr; // FP64 tiled path on the ALU: couplings of levels >= 1
   double *Ltop = nullptr;
   void *Li = nullptr;    // large mixed path: L^{-1} of the eliminated blocks (N n n, FP32)
   float *Yt = nullptr;   // large mixed path: y of the eliminated blocks in solve passes (N n d_max)
@@ -836,7 +836,7 @@ bdss_status bdss_create(bdss_handle *out, int64_t N, int32_t n, int32_t d_max, b
   t_alloc_count = 0;
   bool ok = ws_alloc(h, &h->Ld, (size_t)N * nn * esz);
   ok = ok && ws_alloc(h, &h->Wb, slots * nn * esz);
-  if (h->large) ok = ok && ws_alloc(h, &h->Eb, slots * nn * esz);
+  if (h->large && !is_mixed(h)) ok = ok && ws_alloc(h, (void **)&h->Eb, slots * nn * esz);
   // the top factors: one block, or (blocks up to n = 64) the L_j, C_j and
   // y_j of a serial top sweep of up to kNStarMax blocks
   const size_t top_words = h->large ? nn : (size_t)kNStarMax * (2 * nn + (size_t)n * d_max);

@@ -15,8 +15,9 @@ __device__ bool large_sub(const Args<T> &a, int l, int sub, bool factor, T *smem
   const int n = a.p.n, d = a.d;
   const long long Nl = a.p.Nl[l];
   const long long nE = Nl / 2, nS = (Nl + 1) / 2;
+  if constexpr (sizeof(T) == 4) factor = false;  // FP32 blocks are factored in bdss_wide.cu
   if (sub == kSubA1) {
-    if constexpr (sizeof(T) == 8)  // (FP32 blocks are factored in bdss_wide.cu)
+    if constexpr (sizeof(T) == 8)
       for (long long m = rank; m < nE; m += gridDim.x)
         if (!largeA1(a, l, 2 * m + 1, smem, s_flag)) return false;
   } else if (sub == kSubA2 && !factor && a.Li) {
@@ -54,6 +55,7 @@ __device__ bool large_sub(const Args<T> &a, int l, int sub, bool factor, T *smem
 
 template <typename T>
 __device__ void large_body(const Args<T> &a, int factor, int rhs, unsigned char *smem_raw, int *s_flag) {
+  if constexpr (sizeof(T) == 4) factor = 0;
   T *smem = reinterpret_cast<T *>(smem_raw);
   int bar = 0;
   const int rank = spread_rank(a.st, a.timeout_ns);
