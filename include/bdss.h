@@ -335,8 +335,10 @@ bdss_status bdss_last_launch_stats(bdss_handle h, int64_t *kernel_launches, int6
 /* Test hook: the k-th device or page-locked allocation of every following
  * bdss_create, bdss_kalman_assemble or first CG refinement of a handle
  * (counted per call, 1-based) fails as if the memory were exhausted; 0 turns
- * it off.  The call must then return BDSS_ERR_ALLOC; bdss_create frees what
- * it had allocated, a solve keeps its buffers for bdss_destroy. */
+ * it off.  The call must then return BDSS_ERR_ALLOC -- except bdss_create for the
+ * buffers of a path it chose by size, without which it makes the handle --;
+ * bdss_create frees what it had allocated, a solve keeps its buffers for
+ * bdss_destroy. */
 bdss_status bdss_debug_fail_alloc(int32_t k);
 
 /* Relative diagonal shift sigma of the handle's stored factors (mixed

@@ -151,6 +151,19 @@ static bool ws_alloc(bdss_ctx *h, void **p, size_t bytes) {
   return cudaMemset(static_cast<char *>(*p) + bytes, kGuardByte, kGuardBytes) == cudaSuccess;
 }
 
+// Give a workspace buffer back, with its guard's entry.
+template <typename T>
+static void ws_free(bdss_ctx *h, T **p) {
+  if (!*p) return;
+  for (size_t i = 0; i < h->guards.size(); ++i)
+    if (h->guards[i].base == (void *)*p) {
+      h->guards.erase(h->guards.begin() + i);
+      break;
+    }
+  cudaFree(*p);
+  *p = nullptr;
+}
+
 // All guard bands intact?  (Synchronous copies; debug option only.)
 static bool guards_intact(const bdss_ctx *h) {
   unsigned char buf[kGuardBytes];
@@ -367,12 +380,16 @@ static bdss_status tcf_alloc(bdss_ctx *h) {
   if (h->tcf_ready) return BDSS_OK;
   const size_t nn = (size_t)h->n * h->n, m = (size_t)(h->N / 2);
   const size_t esz = is_mixed(h) ? sizeof(float) : sizeof(double);
-  bool ok = h->tcfX || ws_alloc(h, &h->tcfX, m * nn * esz);
-  ok = ok && (h->tcfC || ws_alloc(h, &h->tcfC, m * 2 * nn * esz));
-  ok = ok && (h->tcfcb || ws_alloc(h, &h->tcfcb, m * 2 * h->n * h->d_max * esz));
-  ok = ok && (h->tcfE || ws_alloc(h, (void **)&h->tcfE, (size_t)h->N * kMaxN * sizeof(short)));
+  bool ok = ws_alloc(h, &h->tcfX, m * nn * esz);
+  ok = ok && ws_alloc(h, &h->tcfC, m * 2 * nn * esz);
+  ok = ok && ws_alloc(h, &h->tcfcb, m * 2 * h->n * h->d_max * esz);
+  ok = ok && ws_alloc(h, (void **)&h->tcfE, (size_t)h->N * kMaxN * sizeof(short));
   if (!ok) {
     cudaGetLastError();
+    ws_free(h, &h->tcfX);
+    ws_free(h, &h->tcfC);
+    ws_free(h, &h->tcfcb);
+    ws_free(h, &h->tcfE);
     return BDSS_ERR_ALLOC;
   }
   const cudaError_t e = is_mixed(h) ? tcf_configure<float>(h->n, h->d_max) : tcf_configure<double>(h->n, h->d_max);
@@ -912,8 +929,9 @@ bdss_status bdss_create(bdss_handle *out, int64_t N, int32_t n, int32_t d_max, b
     }
   }
   if (ok && tcf_by_size(h)) {
+    // without the memory for it the handle is the persistent kernel's
     const bdss_status st = tcf_alloc(h);
-    if (st != BDSS_OK) {
+    if (st != BDSS_OK && st != BDSS_ERR_ALLOC) {
       bdss_destroy(h);
       return st;
     }
