@@ -41,8 +41,9 @@ CSRC = os.path.join(ROOT, "paper_2509_03015_gb300", "csrc")
 L2_BYTES = 129 * 2 ** 20
 
 
-# Sources the headline kernel (k_persistent<double>) is compiled from: the
-# DRAM traffic from the committed ncu summary is used only while they match.
+# Sources of the persistent FP64 kernel, the headline's when BDSS_OPT_SCHUR_EMU = 0:
+# its DRAM traffic from the committed ncu summary is used only while they match (the
+# default path is several kernels, whose line carries no traffic).
 KERNEL_SOURCES = ("bdss_device.cuh", "bdss_kernels.cu", "bdss_launch.h")
 
 
@@ -115,8 +116,9 @@ def kernel_rooflines(kt, steps, units, N, n, d, mode, sms, mhz, emu=False):
                   FP32 residual: HBM;
       factor      the oracle's block-Thomas tally of factor + solve, on the
                   ALU of the mode's precision;
+                  with schur_tc beside it: the diagonal tiles and the downward pass;
       schur_tc    the products of the factorisation (coupling solves, panels,
-                  separator updates; accounting.cr_flops) on the tensor cores,
+                  separator updates, upward right-hand sides) on the tensor cores,
                   one product counted once, against the BF16 rate divided by the
                   16-bit products each takes (36 in FP64, 6 in FP32)."""
     pk = measured_peaks()
@@ -143,18 +145,23 @@ def kernel_rooflines(kt, steps, units, N, n, d, mode, sms, mhz, emu=False):
             unit, bound = "GB/s", "hbm"
             peak, pdef = pk["hbm_gbs"] * 1e9, f"HBM copy bandwidth ({pk['source']})"
         elif cls == "schur_tc":
-            # couplings, panels and separator updates: all of the factorisation
-            # but the diagonal tiles; each product is 36 (FP64: digit pairs) or
-            # 6 (FP32: part pairs) products of 16-bit numbers
+            # couplings, panels, separator updates and the upward right-hand sides
+            # (W^T y of two neighbours; n > 64: y as well): all of the way up but the
+            # Cholesky factors of the diagonal tiles; each product is 36 (FP64: digit
+            # pairs) or 6 (FP32: part pairs) products of 16-bit numbers
             pairs = 36 if mode == "fp64" else 6
-            work, unit, bound = accounting.cr_flops(N, n, d)["factor"], "TFLOP/s", "tensor"
+            nt = -(-n // 64)
+            work = (accounting.cr_flops(N, n, d)["factor"] - N * nt * accounting.chol_flops(n / nt)
+                    + (4.0 if n <= 64 else 5.0) * N * n * n * d)
+            unit, bound = "TFLOP/s", "tensor"
             peak = pk["bf16_tflops"] * 1e12 / pairs
             pdef = f"BF16 dense ({pk['source']}) / {pairs} products of 16-bit parts"
         elif cls == "factor" and "schur_tc" in kt:
-            # diagonal tiles (Cholesky factor and inverse, n^2 nb 2/3 flops a
-            # block), top block, downward pass
+            # diagonal tiles (Cholesky factor and inverse, 2/3 nb^3 flops each), top
+            # block, downward pass (W x of two neighbours 4 n^2 d, the triangle n^2 d)
+            # and, for n <= 64, y = X b (n^2 d)
             nt = -(-n // 64)
-            work = N * nt * 2.0 / 3.0 * (n / nt) ** 3 + 10.0 * N * n * n * d
+            work = N * nt * 2.0 / 3.0 * (n / nt) ** 3 + (6.0 if n <= 64 else 5.0) * N * n * n * d
             unit, bound = "TFLOP/s", "alu"
             peak = fp64_peak(sms, mhz) if mode == "fp64" else fp32_peak(sms, mhz)
             pdef = "FP64 ALU" if mode == "fp64" else "FP32 ALU (SMs x 128 FFMA x 2 x clock)"

@@ -21,9 +21,9 @@
  * can read: page-locked memory (cudaHostAlloc, cudaHostRegister) or, on a
  * system whose GPU reads pageable host memory (cudaDevAttrPageableMemoryAccess,
  * e.g. a coherent NVLink-C2C host link), any host memory.  The level-0
- * kernels then read the inputs in place, asking L2 for the next task's blocks
- * one task ahead, so that the transfer overlaps the factorisation; the FP64
- * path reads every input element once per bdss_factor_solve.  The mixed modes
+ * kernels then read the inputs in place, so that the transfer overlaps the
+ * factorisation (the persistent kernel asks L2 for the next task's blocks one
+ * task ahead); the FP64 path reads every input element once per bdss_factor_solve.  The mixed modes
  * read A again for every refinement residual, where device copies are
  * faster.  X must be device (or managed) memory.  A pointer the GPU cannot
  * read is rejected with BDSS_ERR_INVALID_ARG before any launch.
@@ -71,11 +71,13 @@ typedef enum {
 } bdss_status;
 
 typedef enum {
-  BDSS_FP64 = 0,     /* every step in FP64 (DFMA) */
-  BDSS_FP32_IR = 1,  /* factor/solve in FP32, FP64 residual + iterative refinement */
-  BDSS_TF32_IR = 2   /* as FP32_IR; for 64 < n <= 256 (n % 4 == 0) the Schur-update
-                        products run on tcgen05 tensor cores (3xTF32 split, FP32
-                        accumulation); for n <= 64 it equals BDSS_FP32_IR */
+  BDSS_FP64 = 0,     /* FP64 factors and solutions; large products as exact sums of digit
+                        products on the tensor cores, rounded to FP64 (BDSS_OPT_SCHUR_EMU) */
+  BDSS_FP32_IR = 1,  /* factor/solve in FP32 (n > 64, and n >= 20 with N >= 32: the products on
+                        the tensor cores, an operand as three BF16 parts), FP64 residual +
+                        iterative refinement */
+  BDSS_TF32_IR = 2   /* the same as BDSS_FP32_IR; kept for callers that ask for the faster of
+                        the mixed modes */
 } bdss_precision;
 
 typedef struct {
@@ -92,7 +94,11 @@ typedef struct {
 typedef enum {
   BDSS_OPT_TIMEOUT_MS = 0,      /* limit of every device-side wait (default 10000) */
   BDSS_OPT_PERSISTENT = 1,      /* 1 (default): one persistent launch with grid barriers
-                                   per factor / solve; 0: one launch per level and phase
+                                   per factor / solve where the factorisation is not on
+                                   the tensor cores (BDSS_OPT_SCHUR_EMU; mixed precision
+                                   with n > 64, or n >= 20 and N >= 32: a few launches per
+                                   level), and for solve passes over those factors where it
+                                   is the faster pass; 0: one launch per level and phase
                                    (the per-level structure of Algorithms 4 and 7) */
   BDSS_OPT_MAX_REFINE = 2,      /* mixed precision: refinement step limit (default 10) */
   BDSS_OPT_TARGET_BERR_E18 = 3, /* mixed precision: target backward error x 1e18
@@ -135,15 +141,20 @@ typedef enum {
   BDSS_OPT_SCHUR_EMU = 13,      /* FP64, N > 1, 32 <= n <= 256: 1 = the factorisation's products
                                    on the tensor cores (the separator update of Algorithm 3,
                                    D - W^T W and -W^T W of Eq. 5's reduced system; the coupling
-                                   solves of Algorithm 1): each operand row
-                                   cut into digits below its maximum (59 bits or more), every
-                                   digit product summed exactly in FP32, the result rounded
-                                   to FP64; a few launches per level even in persistent mode.
+                                   solves of Algorithm 1): operands scaled along the summed
+                                   index by powers of two from the diagonal, so that the units
+                                   of the states do not matter, each row cut into digits 62
+                                   bits below its maximum (subnormal entries count as zero),
+                                   every digit product summed exactly in FP32, the result
+                                   rounded to FP64; a few launches per level even in persistent
+                                   mode, which record no grid barriers and no trace.
                                    0 = on the FP64 ALU (for n <= 64 the single persistent
                                    launch).  Default 1 for 64 < n <= 256; for n <= 64 by size
-                                   (long systems of large blocks).  Setting 1 on a handle
-                                   without it gives BDSS_ERR_UNSUPPORTED; mixed-precision
-                                   handles accept 0, which changes nothing there */
+                                   (n >= 40 and N >= 1536; with d_max = 1, n >= 48 and
+                                   N >= 128; with d_max 5 .. 8, n < 44 from N = 8192).  Setting
+                                   1 on a handle without it gives BDSS_ERR_UNSUPPORTED;
+                                   mixed-precision handles accept 0, which changes nothing
+                                   there */
   BDSS_OPT_RESIDUAL_EMU = 10,   /* mixed precision, 64 < n <= 256 and d_max <= 16: 1 (default)
                                    = the FP64 residual of the refinement on the tensor cores
                                    (BF16 digit slices, exact FP32 accumulation: see
@@ -175,7 +186,8 @@ typedef enum {
 /* Kernel classes of bdss_last_kernel_times. */
 typedef enum {
   BDSS_KT_FACTOR = 0,      /* factorisation passes (with the first solve when fused) on CUDA cores */
-  BDSS_KT_SCHUR_TC = 1,    /* BDSS_TF32_IR, n > 64: the tensor-core Schur-update launches of a factorisation */
+  BDSS_KT_SCHUR_TC = 1,    /* the launches of a factorisation whose products run on the tensor cores
+                              (coupling solves, panels, Schur products, upward right-hand sides) */
   BDSS_KT_SOLVE = 2,       /* the solve pass of bdss_solve on stored factors */
   BDSS_KT_CORRECTION = 3,  /* mixed precision: refinement corrections X += M^-1 (B - A X) */
   BDSS_KT_RESIDUAL = 4,    /* mixed precision: FP64 residuals B - A X (with the backward-error norms) */
@@ -364,10 +376,12 @@ bdss_status bdss_get_launch_config(bdss_handle h, int32_t *ctas_per_sm, int32_t 
  * one per downward level.  Differences of consecutive stamps are the time of
  * each step.  Writes min(*count, capacity) entries to the host array
  * release_ns and the number recorded (at most 256) to *count (may be NULL).
- * The paper reports wall-clock phases only; this is the per-level split. */
+ * The paper reports wall-clock phases only; this is the per-level split.
+ * Factorisations on the tensor cores (and solve passes over them that go level by
+ * level) have no grid barriers and record nothing. */
 bdss_status bdss_last_trace(bdss_handle h, int64_t *release_ns, int32_t capacity, int32_t *count);
 
-/* Self-check of the tensor-core Schur tile used by BDSS_TF32_IR for n > 64:
+/* Self-check of the TMA and tensor-core plumbing (no solve uses this tile):
  * one 128 x 128 tile C = A B^T with K = 256 computed with TMA-fed
  * tcgen05.mma (3xTF32 split) and compared on the device with an FP64 product
  * of the same FP32 inputs.  *max_rel_err = max |C_tc - C_ref| / sum_k |a b|

@@ -54,9 +54,8 @@ def thomas_flops(N: int, n: int, d: int):
 
 
 def tc_tile_flops(N: int, n: int) -> float:
-    """Flops of the Schur-update products (Algorithm 3, Eq. 5) that the TF32
-    mode of the tiled path runs on the tensor cores, summed over the levels:
-    per separator one symmetric product n^2 (n+1) per eliminated neighbour and
+    """Flops of the Schur-update products (Algorithm 3, Eq. 5), summed over the
+    levels: per separator one symmetric product n^2 (n+1) per eliminated neighbour and
     the new coupling 2 n^3 when it exists (the separator part of cr_flops)."""
     fl = 0.0
     for Nl in levels(N)[:-1]:
@@ -67,8 +66,9 @@ def tc_tile_flops(N: int, n: int) -> float:
 
 
 def emu_schur_mma_flops(N: int, n: int) -> float:
-    """BF16 tensor-core flops the FP64 tiled factorisation executes for its
-    Schur products with the digit-slice engine: per separator, 128 x 16
+    """BF16 tensor-core flops of the Schur products with ten digit planes written
+    to memory (the scheme of the residual; the factorisation cuts its digits in the
+    kernel, bdss_slice.cuh): per separator, 128 x 16
     output tiles of D's lower part (one accumulation round per eliminated
     neighbour) and of the new coupling E (one round); a round is ten
     128 x 160 x np products (np = n rounded up to 64), one per A slice."""
@@ -84,7 +84,8 @@ def emu_schur_mma_flops(N: int, n: int) -> float:
 
 
 def emu_wslice_bytes(N: int, n: int) -> float:
-    """HBM bytes of the coupling-block slicing over the levels: each stored
+    """HBM bytes of writing the ten digit planes of the couplings over the levels (the
+    same scheme): each stored
     n x n FP64 block read once, its ten BF16 digit planes (n x np) written."""
     np_ = -(-n // 64) * 64
     blocks = sum(Nl - 1 for Nl in levels(N)[:-1])

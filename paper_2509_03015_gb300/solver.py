@@ -232,7 +232,8 @@ class Solver:
         """Barrier release times (ns, device clock) of the last persistent
         pass: start-up, then phase A / phase B of each level, then one per
         downward level (grid barriers; on the one-cluster path its cluster
-        barriers, with one more stamp at the end)."""
+        barriers, with one more stamp at the end).  Empty where no pass ran with
+        barriers: factorisations on the tensor cores go level by level."""
         buf = (ctypes.c_int64 * 256)()
         cnt = ctypes.c_int32()
         _lib.check(self.lib.bdss_last_trace(self.h, buf, 256, ctypes.byref(cnt)), "bdss_last_trace")
@@ -263,8 +264,7 @@ def solve(A_diag, A_sub, B, precision="fp64"):
 class BlockTriSolve(torch.autograd.Function):
     """X = A^{-1} B for the SPD block-tridiagonal A(A_diag, A_sub), FP64.
 
-    forward:  factor + solve (one persistent launch); the factors stay in a
-              handle saved for backward.
+    forward:  factor + solve; the factors stay in a handle saved for backward.
     backward: the adjoint solve A Lam = dL/dX reuses the stored factors (A is
               symmetric), then dL/dB = Lam, dL/dA_ii = -sym(Lam_i X_i^T),
               dL/dA_{i+1,i} = -(Lam_{i+1} X_i^T + X_{i+1} Lam_i^T)."""
