@@ -18,11 +18,11 @@
 // without it a spread of units of 1e8 cost nine digits).  An entry is then off by
 // 2^-57 .. 2^-53 of sqrt(Qinv_rr) max_k sqrt(Qinv_kk) |G_kc|, which is nothing beside
 // the geometric mean of the diagonal entries of the normal equations it couples.
-// A small launch finds the exponents; where no step's differ by more than
-// kKmSpread the products run unscaled, at that loss of the 2^-57 (N = 16384,
-// n = 64, m = 32: 7.6 ms, and 8.4 ms scaled).
-// The vectors v_k = Rinv_k z_k, w_k = Qinv_k zeta_k and b_k are two small
-// FP64 launches.
+// A launch before the products (k_kalman_prepare) finds the exponents and forms
+// the vectors v_k = Rinv_k z_k and w_k = Qinv_k zeta_k; where no step's exponents
+// differ by more than kKmSpread the products run unscaled, at that loss of the 2^-57
+// (N = 16384, n = 64, m = 32: 7.6 ms, and 8.4 ms scaled).  b_k is a small launch
+// after them.
 //
 // Every product is formed transposed (TMEM lane = column of the result), so
 // that a warp stores 32 consecutive entries of a row, and its A operand is a
@@ -70,7 +70,8 @@ __device__ __forceinline__ void km_load_col(const KmSlot &s, int ld, int k0, int
     if (s.scale && in) v[i] *= ldcg(s.scale + k);
   }
 }
-// Exponent of eight entries that count as v 2^(kSign e); kSign = 0: as they are.
+// Exponent of eight entries that count as v 2^(kSign e), poison included; kSign = 0:
+// as they are, without it (km_row_exp).
 template <int kSign>
 __device__ __forceinline__ int km_exp(const double (&v)[8], const SlScale8 &sc) {
   int raw = 0, ex = kSlNoEx;
@@ -79,7 +80,11 @@ __device__ __forceinline__ int km_exp(const double (&v)[8], const SlScale8 &sc) 
     raw = max(raw, sl_exp(v[i]));
     if (kSign) ex = max(ex, sl_exp(v[i]) + kSign * sc.at(i));
   }
-  return raw == 0x7FF ? kSlPoisonEx : kSign ? ex : raw;
+  return kSign == 0 ? raw : raw == 0x7FF ? kSlPoisonEx : ex;
+}
+template <int kSign>
+__device__ __forceinline__ int km_row_exp(int ex) {
+  return kSign == 0 ? sl_row_exp<double>(ex) : ex;
 }
 
 // What a CTA multiplies: out[c][r] (+)= sum_k A(k, c) B(k, r) over K.
@@ -145,10 +150,10 @@ __device__ __forceinline__ bool km_product(WdCta<double> &w, const KmProduct &P,
       if (h == 0) exK[g * kSlRows + 64 * half + c] = km_exp<kSign>(v, sca);
       __syncthreads();
       if (h == 0) {
-        int ex = kSlNoEx;
+        int ex = kSign == 0 ? 0 : kSlNoEx;
 #pragma unroll
         for (int q = 0; q < kKmGroups; ++q) ex = max(ex, exK[q * kSlRows + 64 * half + c]);
-        if (g == 0) w.exA[64 * half + c] = ex;
+        if (g == 0) w.exA[64 * half + c] = km_row_exp<kSign>(ex);
         store8<double, kSign>(v, ex, w.A + sl_off(64 * half + c, g), kSlASlab, sca);
       }
       if (P.brows) {
@@ -157,16 +162,18 @@ __device__ __forceinline__ bool km_product(WdCta<double> &w, const KmProduct &P,
           const int rr = u * kWdWarps<double> + warp, k = 2 * lane;
           const short2 kb = ke[kPair && rr >= 32 ? 1 : 0];
           const int e0 = -kSign * kb.x, e1 = -kSign * kb.y;
-          const int ex = __reduce_max_sync(0xffffffffu, max(sl_exp_at(r2[u][0], e0), sl_exp_at(r2[u][1], e1)));
-          if (lane == 0) w.exB[rr] = ex;
+          int ex;
+          if constexpr (kSign != 0) ex = __reduce_max_sync(0xffffffffu, max(sl_exp_at(r2[u][0], e0), sl_exp_at(r2[u][1], e1)));
+          else ex = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(sl_exp(r2[u][0]), sl_exp(r2[u][1])));
+          if (lane == 0) w.exB[rr] = kSign != 0 ? ex : sl_row_exp<double>(ex);
           sl_store2<double>(r2[u][0], r2[u][1], ex,
                             w.B + (rr >> 5) * kWdBBytes<double> + sl_off(rr & 31, k >> 3) + 2 * (k & 7), kSlBSlab, e0, e1);
         }
       } else if (half == 0) {
-        int ex = kSlNoEx;
+        int ex = kSign == 0 ? 0 : kSlNoEx;
 #pragma unroll
         for (int q = 0; q < kKmGroups; ++q) ex = max(ex, exKB[q * 64 + c]);
-        if (g == 0) w.exB[c] = ex;
+        if (g == 0) w.exB[c] = km_row_exp<kSign>(ex);
         store8<double, -kSign>(vb, ex, w.B + (c >> 5) * kWdBBytes<double> + sl_off(c & 31, g), kSlBSlab, scb);
       }
       const bool cols2 = kPair || ncols > 32;
@@ -205,6 +212,27 @@ __device__ __forceinline__ bool km_product(WdCta<double> &w, const KmProduct &P,
   return true;
 }
 
+// v_k = Rinv_k z_k, w_k = Qinv_k zeta_k (one step per CTA).
+__device__ __forceinline__ void kalman_vectors(const KalmanArgs &a, long long k) {
+  const int n = a.n, m = a.m;
+  const double *Rk = a.Rinv + (size_t)k * (a.rinv_diag ? (size_t)m : (size_t)m * m), *zk = a.z + k * m;
+  const double *Qk = a.Qinv + (size_t)k * n * n, *ek = a.zeta ? a.zeta + k * n : nullptr;
+  for (int i = threadIdx.x; i < n + m; i += blockDim.x) {
+    double s = 0.0;
+    if (i < n) {
+      if (ek)
+        for (int j = 0; j < n; ++j) s = fma(Qk[(size_t)i * n + j], ek[j], s);
+      a.w[k * n + i] = s;
+    } else if (a.rinv_diag) {
+      a.v[k * m + i - n] = Rk[i - n] * zk[i - n];
+    } else {
+      const double *r = Rk + (size_t)(i - n) * m;
+      for (int j = 0; j < m; ++j) s = fma(r[j], zk[j], s);
+      a.v[k * m + i - n] = s;
+    }
+  }
+}
+
 // Exponents for one step, a CTA: EQ and ER from the diagonals, zero beyond n or m.
 // A diagonal entry that is not positive (or not a normal number) gives way to the
 // largest of its row and column; where these are zero, the operand on the other
@@ -230,7 +258,7 @@ __device__ __forceinline__ void km_maxima(double v, int e, int &m0, int &m1) {
   m0 = max(m0, x);
   m1 = max(m1, x + e);
 }
-__global__ void __launch_bounds__(256) k_kalman_scale(const __grid_constant__ KalmanArgs a) {
+__global__ void __launch_bounds__(256) k_kalman_prepare(const __grid_constant__ KalmanArgs a) {
   __shared__ int s_lo[2], s_hi[2], s_gain;
   const int n = a.n, m = a.m, pn = (int)kalman_pad(n), pm = (int)kalman_pad(m), tid = threadIdx.x;
   const long long k = blockIdx.x;
@@ -268,6 +296,7 @@ __global__ void __launch_bounds__(256) k_kalman_scale(const __grid_constant__ Ka
   __syncthreads();
   const bool q = s_hi[0] - s_lo[0] > kKmSpread;
   if (tid == 0 && (q || s_hi[1] - s_lo[1] > kKmSpread)) atomicExch(a.scaled, 1);
+  if (a.B) kalman_vectors(a, k);
   if (!q || k == 0) return;
   const double *G = a.G + (size_t)k * n * n;
   int gain = 0;  // sum of the maxima's exponents, scaled less unscaled
@@ -379,31 +408,6 @@ __global__ void __launch_bounds__(kWdThreads<double>, 1) k_kalman_tc(const __gri
   if (*a.scaled) kalman_tiles<kDiag, kPair, true>(a, st, w, s_exK);
   else kalman_tiles<kDiag, kPair, false>(a, st, w, s_exK);
   wd_end(w);
-}
-
-// v_k = Rinv_k z_k, w_k = Qinv_k zeta_k (one step per CTA).
-__device__ __forceinline__ void kalman_vectors(const KalmanArgs &a, long long k) {
-  const int n = a.n, m = a.m;
-  const double *Rk = a.Rinv + (size_t)k * (a.rinv_diag ? (size_t)m : (size_t)m * m), *zk = a.z + k * m;
-  const double *Qk = a.Qinv + (size_t)k * n * n, *ek = a.zeta ? a.zeta + k * n : nullptr;
-  for (int i = threadIdx.x; i < n + m; i += blockDim.x) {
-    double s = 0.0;
-    if (i < n) {
-      if (ek)
-        for (int j = 0; j < n; ++j) s = fma(Qk[(size_t)i * n + j], ek[j], s);
-      a.w[k * n + i] = s;
-    } else if (a.rinv_diag) {
-      a.v[k * m + i - n] = Rk[i - n] * zk[i - n];
-    } else {
-      const double *r = Rk + (size_t)(i - n) * m;
-      for (int j = 0; j < m; ++j) s = fma(r[j], zk[j], s);
-      a.v[k * m + i - n] = s;
-    }
-  }
-}
-
-__global__ void __launch_bounds__(kThreads) k_kalman_vectors(const __grid_constant__ KalmanArgs a) {
-  kalman_vectors(a, blockIdx.x);
 }
 
 // b_k = H_k^T v_k + w_k - G_{k+1}^T w_{k+1}.
@@ -520,7 +524,7 @@ long long kalman_max_steps(int n, int m) {
   return 0x7fffffffLL / (nt * nt + mt * nt + 1);
 }
 
-// The tensor-core path takes five launches and 128-column tiles of 64 K entries
+// The tensor-core path takes four launches and 128-column tiles of 64 K entries
 // whatever n and m: few steps, or small ones, are faster on the ALU.  Its time over
 // the ALU's, measured on GB300 (full Rinv; diagonal ones cross 1 at the same sizes
 // within two):
@@ -551,7 +555,7 @@ cudaError_t launch_kalman_assemble(const KalmanArgs &a, DevStatus *st, int sms, 
   for (const void *k : kernels)
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kKmSmem);
   if (e == cudaSuccess) {
-    k_kalman_scale<<<(unsigned)a.N, kalman_pad(a.n) + kalman_pad(a.m) <= 128 ? 128 : 256, 0, s>>>(a);
+    k_kalman_prepare<<<(unsigned)a.N, kalman_pad(a.n) + kalman_pad(a.m) <= 128 ? 128 : 256, 0, s>>>(a);
     e = cudaGetLastError();
   }
   for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
@@ -562,7 +566,6 @@ cudaError_t launch_kalman_assemble(const KalmanArgs &a, DevStatus *st, int sms, 
     e = cudaLaunchKernel(kernels[i], dim3(grid), dim3(kWdThreads<double>), args, kKmSmem, s);
   }
   if (e != cudaSuccess || !a.B) return e;
-  k_kalman_vectors<<<(unsigned)a.N, kThreads, 0, s>>>(a);
   k_kalman_rhs<<<(unsigned)a.N, kThreads, 0, s>>>(a);
   return cudaGetLastError();
 }
