@@ -10,7 +10,8 @@
 //   k_wide_diag   the diagonal tile on the FP64 (FP32) ALU: L_kk = chol, X_kk
 //                 = L_kk^{-1};
 //   k_wide_panel  every other row v: P_vk = (S_vk - sum_{p<k} P_vp L_kp^T) X_kk^T
-//                 (scaled along the columns by the tile's diagonal), and for rows of D their own diagonal tile, updated by P P^T.
+//                 (scaled along the columns by the tile's diagonal), and for
+//                 rows of D their own diagonal tile, updated by P P^T.
 // Then one launch forms what the separators receive (k_wide_schur): D, the
 // next level's couplings, b.
 //
